@@ -11,6 +11,7 @@
 #include <deque>
 #include <mutex>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -50,6 +51,48 @@ cudaError_t dalloc(T *&p, uint64_t count) {
 }
 
 uint32_t bit_length(uint32_t x) { return x ? 32u - (uint32_t)__builtin_clz(x) : 0u; }
+
+// Cuts the vertices into consecutive ranges of at most `arcs` arcs (a hub
+// counts HEAVY_DEG: longer rows are queued in chunks) and ITEM_SPAN
+// vertices; a single vertex may exceed the arc limit.  Returns the range
+// starts followed by n.  Blocks of CUT_BLOCK vertices are cut side by side
+// on the host's threads.
+std::vector<uint32_t> cut_items(const uint32_t *row_ptr, uint32_t n, uint64_t arcs) {
+    constexpr uint32_t CUT_BLOCK = 1u << 20;
+    const uint32_t blocks = (uint32_t)(((uint64_t)n + CUT_BLOCK - 1) / CUT_BLOCK);
+    std::vector<std::vector<uint32_t>> part(blocks);
+    std::atomic<uint32_t> next{0};
+    auto work = [&] {
+        for (uint32_t b; (b = next.fetch_add(1)) < blocks;) {
+            const uint32_t lo = b * CUT_BLOCK, hi = (uint32_t)std::min<uint64_t>(n, (uint64_t)lo + CUT_BLOCK);
+            std::vector<uint32_t> &at = part[b];
+            uint64_t sum = 0;
+            for (uint32_t v = lo; v < hi; ++v) {
+                const uint32_t d = std::min(row_ptr[v + 1] - row_ptr[v], HEAVY_DEG);
+                if (at.empty() || sum + d > arcs || v - at.back() == ITEM_SPAN) {
+                    at.push_back(v);
+                    sum = 0;
+                }
+                sum += d;
+            }
+        }
+    };
+    std::vector<std::thread> pool;
+    const uint32_t threads = std::min(blocks, std::min(16u, std::max(1u, std::thread::hardware_concurrency())));
+    for (uint32_t t = 1; t < threads; ++t) {
+        try {
+            pool.emplace_back(work);
+        } catch (const std::system_error &) {
+            break;          // fewer threads do the same work
+        }
+    }
+    work();
+    for (auto &t : pool) t.join();
+    std::vector<uint32_t> at;
+    for (auto &p : part) at.insert(at.end(), p.begin(), p.end());
+    at.push_back(n);
+    return at;
+}
 
 uint32_t bits_for(uint32_t n) {
     uint32_t b = 1;
@@ -588,6 +631,23 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     G->geo.sssp_max_blocks = G->geo.sssp_blocks;
     int mst_sm = mst_occupancy(512);
     G->geo.mst_blocks = std::max(1, mst_sm) * G->geo.sm_count;
+    {   // dense work items: some sixteen per warp of the persistent grid
+        const uint64_t warps = (uint64_t)G->geo.sssp_max_blocks * (G->geo.threads / 32);
+        const uint64_t arcs = std::min<uint64_t>(std::max<uint64_t>(n_arcs / (16 * warps), ITEM_ARCS_MIN),
+                                                 ITEM_ARCS_MAX);
+        const std::vector<uint32_t> it = cut_items(irp, n, arcs);
+        const std::vector<uint32_t> sp = cut_items(irp, n, SPARSE_ITEM_FACTOR * arcs);
+        G->g.n_items = (uint32_t)it.size() - 1;
+        G->g.n_sparse_items = (uint32_t)sp.size() - 1;
+        e = dalloc(G->g.items, it.size());
+        if (e == cudaSuccess) e = dalloc(G->g.sparse_items, sp.size());
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(G->g.items, it.data(), it.size() * 4, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(G->g.sparse_items, sp.data(), sp.size() * 4, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return bail(cuda_fail(e, "work items"));
+    }
     // default band width: ~32 average weights spread over the average degree
     double avg_w = 0;
     if (n_arcs) {
@@ -618,7 +678,7 @@ void steiner_free_graph(steiner_graph_t G) {
                     ws.e_key, ws.e_ra, ws.e_rb, ws.e_arc, ws.e_mst, ws.tile_off, ws.comp, ws.hook,
                     ws.best, ws.tree_key, ws.tree_key2, ws.tree_w, ws.tree_w2, G->g.row_ptr,
                     G->g.adj, G->g.heavy_chunks, G->g.orig_row_ptr, G->g.orig_of, G->g.new_of,
-                    G->g.adj_w, G->g.lend};
+                    G->g.adj_w, G->g.lend, G->g.items, G->g.sparse_items};
     for (void *p : bufs)
         if (p) cudaFree(p);
     for (auto &ev : G->ev)

@@ -13,6 +13,16 @@ namespace stn {
 // CHUNK arcs (one warp per chunk) instead of inside a 32-vertex batch.
 constexpr uint32_t HEAVY_DEG = 256;
 constexpr uint32_t CHUNK = 512;
+// Largest vertex range of a dense work item: whatever its alignment it
+// touches at most 32 bitmap words, one per lane.
+constexpr uint32_t ITEM_SPAN = 992;
+// Arcs per dense work item: some sixteen items per warp of the grid, within
+// these bounds (below one relax_group a smaller item saves nothing; above
+// the upper one the slowest item shows).  Voronoi query, R-MAT 22, weights
+// to 10^5, k = 64: 2.76 ms; four items per warp up to 8192 arcs 3.30 ms.
+constexpr uint64_t ITEM_ARCS_MIN = 128, ITEM_ARCS_MAX = 4096;
+// A sparse bitmap's items may hold this many times the arcs (few are set).
+constexpr uint64_t SPARSE_ITEM_FACTOR = 8;
 
 // Resident graph: row offsets and interleaved (neighbour, weight) arcs.
 struct DevGraph {
@@ -39,6 +49,11 @@ struct DevGraph {
     uint2 *adj_w = nullptr;
     uint32_t *lend = nullptr;
     uint32_t part_delta = 0;        // 0: not built
+    // Work items of a dense (bitmap) frontier: consecutive vertex ranges
+    // [items[i], items[i + 1]) of about equal arcs, at most ITEM_SPAN
+    // vertices each; a sparse bitmap is read through the coarser list.
+    uint32_t *items = nullptr, *sparse_items = nullptr;
+    uint32_t n_items = 0, n_sparse_items = 0;
     // Vertices with ids at or above n_big have fewer than HEAVY_DEG arcs
     // (the descending-degree order puts the hubs first; n without it).
     uint32_t n_big = 0;
@@ -75,6 +90,7 @@ struct Control {
     uint32_t err;
     uint32_t near_count[3];
     uint32_t heavy_count[3];
+    uint32_t work_next[3];       // work items handed out on demand
     uint32_t far_count[2];
     uint32_t far_min[2];
     uint32_t iterations;

@@ -81,6 +81,11 @@ struct SsspArgs {
     uint32_t n_words;        // bitmap words, ceil(n / 32)
     uint32_t *nbm0, *nbm1;   // near bitmaps, alternating by iteration
     uint32_t *bbm;           // band bitmap
+    // vertex ranges that dense iterations hand to the warps (n_items of
+    // them), and the coarser ones for a sparse bitmap
+    const uint32_t *__restrict__ items;
+    const uint32_t *__restrict__ sparse_items;
+    uint32_t n_items, n_sparse_items;
     // with the split: end of each row's light part in the weight-partitioned
     // adjacency `adj` (null: rows are unpartitioned and arcs are filtered)
     const uint32_t *lend;
@@ -145,8 +150,6 @@ constexpr uint32_t FAR_STAGE = 1024;   // block staging capacity (far items)
 constexpr uint32_t BAND_STAGE = 2048;  // block staging capacity (band-list items)
 constexpr uint32_t BAND_REGION = BAND_STAGE / SSSP_WARPS;
 constexpr int SPLIT_ILP = 4;           // 32-vertex chunks per warp step in a band split
-constexpr uint32_t DENSE_WORDS = 8;    // bitmap words per dense work item (light arcs)
-constexpr uint32_t DENSE_WORDS_HP = 8; // the same in a heavy-arc pass
 constexpr int PULL_ILP = 4;            // 32-vertex chunks per warp step in a pull pass
 
 // Where the appends of one processing segment go.
@@ -819,6 +822,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         if (first) {
             ctl->near_count[(it + 2) % 3] = 0;
             ctl->heavy_count[(it + 2) % 3] = 0;
+            ctl->work_next[(it + 2) % 3] = 0;
             if (hp && pull) ++ctl->pulls;
             if (it < TRACE_LEN) {
                 ctl->trace[it][0] = n_light;
@@ -874,14 +878,16 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         // (fewer sequential rounds per warp), a thick one packs 32 per warp.
         uint32_t per = (n_light + nwarps - 1) / nwarps;
         uint32_t bsz = per <= 1 ? 1 : per <= 2 ? 2 : per <= 4 ? 4 : per <= 8 ? 8 : per <= 16 ? 16 : 32;
-        // A dense work item is one bitmap word (32 vertices) where vertices
-        // may have many arcs (ids below n_big, in the degree order the high
-        // degrees), else DENSE_WORDS words: balanced work per warp.  A
-        // sparse bitmap (under one set bit per two words) is read 32 words
-        // per item: the sweep itself is then the cost.
-        const uint32_t cw = n_light < a.n_words / 2 ? 32u : hp ? DENSE_WORDS_HP : DENSE_WORDS;
-        const uint32_t fine = min(a.n_words, (a.n_big + 1023) / 1024 * 32);
-        const uint32_t n_work = n_heavy + (dense_in ? fine + (a.n_words - fine + cw - 1) / cw
+        // A dense work item is a vertex range of about equal arcs (a range
+        // of equal vertices gave the first warps 256 rows of nearly
+        // HEAVY_DEG arcs each: on R-MAT 16, k = 16 the slowest warp of an
+        // iteration was busy 1.2 ms against a mean of 11 us, and the query
+        // took 3.6 ms against 0.87).  A sparse
+        // bitmap (under one set bit per two words) is read in the coarser
+        // ranges: the sweep itself is then the cost.
+        const bool sparse = n_light < a.n_words / 2;
+        const uint32_t *items = sparse ? a.sparse_items : a.items;
+        const uint32_t n_work = n_heavy + (dense_in ? (sparse ? a.n_sparse_items : a.n_items)
                                                     : (n_light + bsz - 1) / bsz);
         if (a.trace && lane == 0) trace_snap[threadIdx.x >> 5][3] = global_ns();
         if (hp && pull) {
@@ -896,8 +902,18 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
                               (listed || a.tail) ? nullptr : pile, &ctl->far_count[fc],
                               a.tail != 0, t.nbm, t.qn, t.qn_count, t.hqn, t.hqn_count,
                               attempts, improved, narrow_miss, atomics);
-        } else
-        for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
+        } else {
+        // The last quarter of a long list is handed out on demand (the next
+        // index is fetched while an item is relaxed), so that the iteration
+        // does not end with its slowest warp (R-MAT 26, degree 8, k = 10,000:
+        // the thickest iterations 3.2 ms, all fixed 3.65).
+        const uint32_t n_fixed = n_work < 8 * nwarps ? n_work : n_work / 4 * 3 / nwarps * nwarps;
+        uint32_t grab = 0;
+        for (uint32_t wi = warp; wi < n_work;
+             wi = wi + nwarps < n_fixed || n_fixed == n_work ? wi + nwarps
+                                                             : n_fixed + __shfl_sync(FULL, grab, 0)) {
+            if (wi + nwarps >= n_fixed && n_fixed != n_work && lane == 0)
+                grab = atomicAdd(&ctl->work_next[cs], 1u);
             if (wi < n_heavy) {
                 // one CHUNK of a high-degree vertex per warp
                 uint64_t item = __ldcg(reinterpret_cast<const unsigned long long *>(&hqc[wi]));
@@ -924,15 +940,22 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
                                 improved, narrow_miss, atomics);
                 }
             } else if (dense_in) {
-                // 1 or 32 words of the bitmap, one per lane (read and
-                // cleared); their set bits, 32 at a time, are the vertices
-                const uint32_t di = wi - n_heavy;
-                const uint32_t w0 = di < fine ? di : fine + (di - fine) * cw;
-                const uint32_t nw = di < fine ? 1u : cw;
+                // the words of the item's vertex range, one per lane (the
+                // range's bits are read and cleared; a word may be shared
+                // with the neighbouring items); their set bits, 32 at a
+                // time, are the vertices
+                const uint32_t v0 = __ldg(&items[wi - n_heavy]), v1 = __ldg(&items[wi - n_heavy + 1]);
+                const uint32_t w0 = v0 >> 5, w1 = (v1 - 1) >> 5;
                 uint32_t word = 0;
-                if (lane < nw && w0 + lane < a.n_words) {
-                    word = ldcg_u32(&bm_in[w0 + lane]);
-                    if (word) bm_in[w0 + lane] = 0;
+                if (w0 + lane <= w1) {
+                    uint32_t own = FULL;
+                    if (lane == 0) own <<= v0 & 31;
+                    if (w0 + lane == w1) own &= FULL >> (31 - ((v1 - 1) & 31));
+                    word = ldcg_u32(&bm_in[w0 + lane]) & own;
+                    if (word) {
+                        if (own == FULL) bm_in[w0 + lane] = 0;
+                        else atomicAnd(&bm_in[w0 + lane], ~own);
+                    }
                 }
                 const uint32_t cnt = (uint32_t)__popc(word);
                 const uint32_t incl = warp_inclusive_scan(cnt);
@@ -956,6 +979,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
                 relax_vertices<NARROW>(a, st, t, has, u, hp, track, tag_band, wlo, whi, bsz == 32,
                                        attempts, improved, narrow_miss, atomics);
             }
+        }
         }
         // Local rounds: relax the vertices just staged for the next
         // iteration right away, a hop further per round, instead of waiting
@@ -1130,6 +1154,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         if (first) {
             ctl->near_count[(its + 1) % 3] = 0;
             ctl->heavy_count[(its + 1) % 3] = 0;
+            ctl->work_next[(its + 1) % 3] = 0;
             ctl->band_count = 0;
             ctl->band_hcount = 0;
             ctl->band_hsum = 0;
@@ -1377,6 +1402,10 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.nbm0 = ws.nbm[0];
     a.nbm1 = ws.nbm[1];
     a.bbm = ws.bbm;
+    a.items = g.items;
+    a.sparse_items = g.sparse_items;
+    a.n_items = g.n_items;
+    a.n_sparse_items = g.n_sparse_items;
     a.lend = active_lend(g, p.delta);
     if (a.lend) a.adj = g.adj_w;        // rows partitioned by weight class
     void *args[] = {&a};
