@@ -33,12 +33,18 @@ __host__ __device__ __forceinline__ uint64_t widen_label(uint32_t l, uint32_t sh
     return ((uint64_t)(l >> shift) << 32) | (l & ((1u << shift) - 1u));
 }
 
-// Spin limit of a grid barrier wait (each spin sleeps ~64 ns): ~4 s.
+// Polls of a grid barrier wait before it gives up (after the first few each
+// sleeps ~64 ns).
 constexpr long long BARRIER_SPIN_LIMIT = 1ll << 26;
+constexpr int BARRIER_TIGHT_POLLS = 64;
+// Added to the arrival count by a block that gave up: every wait that sees
+// the count this far beyond its target fails too.
+constexpr uint32_t BARRIER_POISON = 1u << 29;
 
+// Arrival count, zero at the launch of a kernel that uses it.
 struct GridBarrier {
     unsigned int count;
-    unsigned int gen;
+    unsigned int pad;
 };
 
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int *p) {
@@ -47,8 +53,11 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int *p) {
     return v;
 }
 
-__device__ __forceinline__ void red_release_add_u32(unsigned int *p, unsigned int v) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
+__device__ __forceinline__ unsigned int add_acq_rel_u32(unsigned int *p, unsigned int v) {
+    unsigned int old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;"
+                 : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
 }
 
 // Loads that bypass L1: for values written by other blocks of a persistent
@@ -58,46 +67,41 @@ __device__ __forceinline__ uint64_t ldcg_u64(const uint64_t *p) {
 }
 __device__ __forceinline__ uint32_t ldcg_u32(const uint32_t *p) { return __ldcg(p); }
 
-// Grid-wide barrier for cooperatively launched kernels.  Every wait is
-// bounded: a block that waits longer than BARRIER_SPIN_LIMIT spins sets
-// ERR_BARRIER in *err and returns false; callers then leave their loop.
-// Once ERR_BARRIER is set every later barrier returns false too, so all
-// blocks leave within one more bounded wait.  Returns true on a normal
-// release.  Single-block grids use __syncthreads.
-__device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *err) {
-    __shared__ int ok_s;
+// Grid-wide barrier for cooperatively launched kernels.  The arrival count
+// only grows: barrier number i is open once it reaches i * gridDim.x, which
+// each thread tracks in `target` (0 before the first barrier), so the last
+// arrival is itself the release and a wait costs one round trip after it.
+// (A generation word released by the last arrival, with the count reset and
+// an error flag read after every wait, cost four dependent round trips: a
+// 1021 x 733 grid's query, some 560 barriers, 6.68 ms against 5.94.)
+// Every wait is bounded: a block that polls longer than BARRIER_SPIN_LIMIT
+// sets ERR_BARRIER in *err, poisons the count and returns false; every
+// other block's current or next wait then returns false as well.  Returns
+// true on a normal release.  Single-block grids use __syncthreads.
+__device__ __forceinline__ bool grid_sync(GridBarrier *bar, uint32_t *err, uint32_t &target) {
     if (gridDim.x == 1) {
         __syncthreads();
         return true;
     }
+    target += gridDim.x;
     __syncthreads();
+    int ok = 1;
     if (threadIdx.x == 0) {
-        int ok = 1;
-        unsigned int g = ld_acquire_u32(&bar->gen);
-        __threadfence();
-        unsigned int arrived = atomicAdd(&bar->count, 1u) + 1u;
-        if (arrived == gridDim.x) {
-            bar->count = 0;
-            __threadfence();
-            red_release_add_u32(&bar->gen, 1u);
-        } else {
-            long long spins = 0;
-            while (ld_acquire_u32(&bar->gen) == g) {
-                if (++spins > BARRIER_SPIN_LIMIT) {
-                    atomicOr(err, ERR_BARRIER);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
+        uint32_t seen = add_acq_rel_u32(&bar->count, 1u) + 1u;
+        for (long long polls = 0; (int32_t)(seen - target) < 0; ++polls) {
+            if (polls > BARRIER_SPIN_LIMIT) {
+                if (!(atomicOr(err, ERR_BARRIER) & ERR_BARRIER))
+                    atomicAdd(&bar->count, BARRIER_POISON);
+                ok = 0;
+                break;
             }
+            if (polls >= BARRIER_TIGHT_POLLS) __nanosleep(64);
+            seen = ld_acquire_u32(&bar->count);
         }
-        __threadfence();
-        // a block that gave up earlier poisons every later barrier
-        if (ld_acquire_u32(err) & ERR_BARRIER) ok = 0;
-        ok_s = ok;
+        // unpoisoned, the others can be at most one barrier ahead
+        if ((int32_t)(seen - target) >= (int32_t)(BARRIER_POISON / 2)) ok = 0;
     }
-    __syncthreads();
-    return ok_s != 0;
+    return __syncthreads_and(ok) != 0;
 }
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }

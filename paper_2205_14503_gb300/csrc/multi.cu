@@ -424,6 +424,7 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
     }
     __syncthreads();
     uint32_t iters = 0, reason = 0;
+    uint32_t bar_target = 0;
 
     while (infl) {
         const uint32_t cs = it % 3, ns = (it + 1) % 3;
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
         }
         if (threadIdx.x == 0) a.bsum[blockIdx.x] = st.carry;
         unsigned long long tm1 = first ? gtimer() : 0;
-        if (!grid_sync(&ctl->bar, &ctl->err)) { reason = 5; break; }
+        if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; break; }
         unsigned long long tm2 = first ? gtimer() : 0;
         // block offsets and the total
         {
@@ -652,7 +653,7 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
         seg_flush(st, t, ctl, a.n);
         if (first)
             ctl->stop_req[it & 1] = (a.yield && a.doorbell) ? *(volatile const uint32_t *)a.doorbell : 0u;
-        if (!grid_sync(&ctl->bar, &ctl->err)) { reason = 5; break; }
+        if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; break; }
         if (first) {
             unsigned long long tm4 = gtimer();
             ctl->t_part[0] += tm1 - tm0;
@@ -694,7 +695,7 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
         // Split the far pile for the slots in S.  A barrier first: every
         // block has read the decision inputs before the split appends to
         // them.  Near pushes go to this iteration's queue (slot it % 3).
-        if (!grid_sync(&ctl->bar, &ctl->err)) { reason = 5; break; }
+        if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; break; }
         if (threadIdx.x < MQ_SLOTS) {
             uint32_t q = threadIdx.x;
             unsigned long long Tq = st.T[q];
@@ -755,7 +756,7 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
                          &ctl->err);
         }
         seg_flush(st, u, ctl, a.n);
-        if (!grid_sync(&ctl->bar, &ctl->err)) { reason = 5; break; }
+        if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; break; }
         if (first) {
             for (uint32_t q = 0; q < MQ_SLOTS; ++q) {
                 if (!((S >> q) & 1)) {

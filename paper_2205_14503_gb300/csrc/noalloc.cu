@@ -87,7 +87,7 @@ __device__ __forceinline__ uint32_t *queue_of(const NaArgs &a, uint32_t it) {
 __global__ void na_ctl_reset_kernel(NaArgs a) {
     NaControl *c = ctl_of(a);
     c->bar.count = 0;
-    c->bar.gen = 0;
+    c->bar.pad = 0;
     c->err = 0;
     c->count[0] = c->count[1] = c->count[2] = 0;
     c->iterations = 0;
@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(256) na_sssp_kernel(NaArgs a) {
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;   // set by the reset or seed kernel: all blocks agree
+    uint32_t bar_target = 0;
     for (uint32_t it = 0;; ++it) {
         uint32_t nf = min(ldcg_u32(&c->count[it % 3]), a.n);
         if (first) c->count[(it + 2) % 3] = 0;
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(256) na_sssp_kernel(NaArgs a) {
                 if (slot != INF32) qn[slot] = v;
             }
         }
-        if (!grid_sync(&c->bar, &c->err)) return;
+        if (!grid_sync(&c->bar, &c->err, bar_target)) return;
         if (it + 1 >= a.max_iters) {
             if (first) atomicOr(&c->err, ERR_TIMEOUT);
             return;

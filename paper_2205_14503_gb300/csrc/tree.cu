@@ -39,8 +39,9 @@ __global__ void __launch_bounds__(512) mst_kernel(MstArgs a) {
     const uint32_t nth = gridDim.x * blockDim.x;
     const uint32_t E = ldcg_u32(&ctl->n_pairs);
     const bool first = tid == 0;
+    uint32_t bar_target = 0;
     for (uint32_t r = tid; r < a.k; r += nth) a.comp[r] = r;
-    if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+    if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
     for (int round = 0;; ++round) {
         if (round >= 64) {
             if (first) atomicOr(&ctl->err, ERR_TIMEOUT);
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(512) mst_kernel(MstArgs a) {
             a.hook[c] = c;
         }
         if (first) ctl->mst_any = 0;
-        if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+        if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
         // lightest edge leaving every component
         bool any = false;
         for (uint32_t j = tid; j < E; j += nth) {
@@ -63,7 +64,7 @@ __global__ void __launch_bounds__(512) mst_kernel(MstArgs a) {
             any = true;
         }
         if (__any_sync(FULL, any) && lane_id() == 0) atomicExch(&ctl->mst_any, 1u);
-        if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+        if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
         if (ldcg_u32(&ctl->mst_any) == 0) break;
         // hook each component along its lightest edge; mark the edge
         for (uint32_t j = tid; j < E; j += nth) {
@@ -79,13 +80,13 @@ __global__ void __launch_bounds__(512) mst_kernel(MstArgs a) {
                 a.e_mst[j] = 1;
             }
         }
-        if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+        if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
         // two components that chose each other: the smaller id becomes root
         for (uint32_t c = tid; c < a.k; c += nth) {
             uint32_t p = ldcg_u32(&a.hook[c]);
             if (p != c && ldcg_u32(&a.hook[p]) == c && c < p) a.hook[c] = c;
         }
-        if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+        if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
         // relabel every rank with its new root
         for (uint32_t r = tid; r < a.k; r += nth) {
             uint32_t c = ldcg_u32(&a.comp[r]);
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(512) mst_kernel(MstArgs a) {
             }
             a.comp[r] = c;
         }
-        if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+        if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
     }
 }
 
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(RS_THREADS) radix_sort_kernel(SortArgs a) {
     const uint32_t per = (N + gridDim.x - 1) / gridDim.x;
     const uint32_t lo = min(N, blockIdx.x * per), hi = min(N, lo + per);
     const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
+    uint32_t bar_target = 0;
 
     // total distance
     unsigned long long tot = 0;
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(RS_THREADS) radix_sort_kernel(SortArgs a) {
         __syncthreads();
         for (uint32_t d = threadIdx.x; d < 256; d += RS_THREADS)
             a.blk_hist[blockIdx.x * 256 + d] = hist[d];
-        if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+        if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
         // this block's first output position per digit
         if (threadIdx.x < 256) {
             uint32_t d = threadIdx.x, before = 0, total = 0;
@@ -292,7 +294,7 @@ __global__ void __launch_bounds__(RS_THREADS) radix_sort_kernel(SortArgs a) {
             if (threadIdx.x < 256) base[threadIdx.x] += tile_tot[threadIdx.x];
             __syncthreads();
         }
-        if (!grid_sync(&ctl->bar2, &ctl->err)) return;
+        if (!grid_sync(&ctl->bar2, &ctl->err, bar_target)) return;
     }
 }
 

@@ -786,6 +786,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
     __shared__ unsigned long long trace_snap[SSSP_WARPS][4];
     if (threadIdx.x < SSSP_WARPS * 4) (&trace_snap[0][0])[threadIdx.x] = 0;
     uint32_t it = 0, phase = 0, bands = 0;
+    uint32_t bar_target = 0;
     uint64_t T = a.delta;
     bool first = (blockIdx.x == 0 && threadIdx.x == 0);
     bool hp = false;               // this iteration is a band's heavy-arc pass
@@ -1069,7 +1070,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
             }
         }
         flush_stage(st, t, a.n, &ctl->err);
-        if (!grid_sync(&ctl->bar, &ctl->err)) {
+        if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) {
             if (first) ctl->exit_reason = 3;
             break;
         }
@@ -1256,7 +1257,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
             }
         }
         flush_stage(st, u, a.n, &ctl->err);
-        if (!grid_sync(&ctl->bar, &ctl->err)) {
+        if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) {
             if (first) ctl->exit_reason = 4;
             break;
         }
