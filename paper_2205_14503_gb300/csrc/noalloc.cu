@@ -17,10 +17,11 @@
 // the rest, so calls that overlap on the GPU (other streams, other host
 // threads) race with each other and must be serialised by the caller.
 //
-// The kernels here are a simpler variant of the library's Voronoi path:
-// the same packed (distance << 32 | seed rank) 64-bit atomicMin fixed point,
-// run as a plain frontier Bellman-Ford in one cooperative kernel, followed
-// by one pass that derives predecessors and writes the outputs.
+// One cooperative kernel does the whole call: it clears the state and checks
+// the row offsets, seeds the frontier, runs the same packed
+// (distance << 32 | seed rank) 64-bit atomicMin fixed point as the library's
+// Voronoi path as a frontier Bellman-Ford, and derives predecessors and
+// writes the outputs, with a grid barrier between the steps.
 #include <algorithm>
 #include <cstddef>
 #include <mutex>
@@ -37,7 +38,8 @@ constexpr uint32_t NA_MAX_VERTICES = STEINER_NOALLOC_MAX_VERTICES;
 struct NaControl {
     GridBarrier bar;
     uint32_t err;            // ERR_* bits, plus NA_BAD_INPUT
-    uint32_t count[3];       // frontier sizes, rotating by iteration
+    uint32_t count[3];       // frontier: short rows, rotating by iteration
+    uint32_t hubs[3];        // frontier: rows of NA_HUB_DEG arcs or more
     uint32_t iterations;
 };
 
@@ -65,6 +67,7 @@ struct NaArgs {
     uint32_t k;
     unsigned char *scratch;     // device address of g_scratch
     uint32_t max_iters;
+    uint32_t local_rounds;      // hops a warp follows its own pushes per iteration
     int32_t *cell;
     uint32_t *dist;
     int32_t *pred;
@@ -83,156 +86,371 @@ __device__ __forceinline__ uint32_t *queue_of(const NaArgs &a, uint32_t it) {
     return reinterpret_cast<uint32_t *>(a.scratch + ((it & 1) ? Q1_OFF : Q0_OFF));
 }
 
-// Clears the control block of the previous call (one thread).
-__global__ void na_ctl_reset_kernel(NaArgs a) {
-    NaControl *c = ctl_of(a);
-    c->bar.count = 0;
-    c->bar.pad = 0;
-    c->err = 0;
-    c->count[0] = c->count[1] = c->count[2] = 0;
-    c->iterations = 0;
+// Rows of NA_HUB_DEG arcs or more are cut into NA_CHUNK-arc pieces spread
+// over the grid's warps; shorter ones are relaxed 32 rows to a warp.
+constexpr uint32_t NA_HUB_DEG = 256;
+constexpr uint32_t NA_CHUNK = 256;
+constexpr int NA_ILP = 4;                  // arcs in flight per lane
+constexpr uint32_t NA_WARPS = 8;           // per block
+constexpr uint32_t NA_REGION = 512;        // staged pushes per warp
+// Rows of NA_BLOCK_DEG arcs or more take the whole block in the export.
+constexpr uint32_t NA_BLOCK_DEG = 1024;
+
+// A frontier: short rows from the bottom of its queue, hubs from the top
+// (a vertex is queued once, so the two never meet).
+struct NaFront {
+    uint32_t *q;
+    uint32_t *count, *hubs;
+    uint32_t tag;
+};
+
+__device__ __forceinline__ void na_queue(const NaArgs &a, const NaFront &f, bool want, uint32_t v,
+                                         uint32_t *err) {
+    bool hub = false;
+    if (want) {
+        want = atomicExch(&stamp_of(a)[v], f.tag) != f.tag;
+        hub = a.row_ptr[v + 1] - a.row_ptr[v] >= NA_HUB_DEG;
+    }
+    uint32_t g = warp_append(want && !hub, f.count, a.n, err);
+    if (g != INF32) f.q[g] = v;
+    g = warp_append(want && hub, f.hubs, a.n, err);
+    if (g != INF32) f.q[a.n - 1 - g] = v;
 }
 
-// Clears the per-vertex state of the previous call and checks the row
-// offsets (row_ptr[0] = 0, non-decreasing, row_ptr[n] = n_arcs), so that no
-// later kernel reads an arc outside [0, n_arcs).
-__global__ void na_reset_kernel(NaArgs a) {
-    uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
-    NaControl *c = ctl_of(a);
-    if (tid == 0 && (a.row_ptr[0] != 0 || (uint64_t)a.row_ptr[a.n] != a.n_arcs))
-        atomicOr(&c->err, NA_BAD_INPUT);
+// Relaxes up to NA_ILP arcs per lane (arc index and tail label each), the
+// loads and atomics of all of them issued back to back; vertices that
+// improve are staged in the warp's region (a vertex may be staged twice),
+// or queued when it is full.
+__device__ __forceinline__ void na_relax(const NaArgs &a, NaControl *c, const NaFront &f,
+                                         uint32_t *region, uint32_t *region_n,
+                                         const bool (&valid)[NA_ILP],
+                                         const uint32_t (&arc)[NA_ILP],
+                                         const uint64_t (&lab)[NA_ILP]) {
     uint64_t *label = label_of(a);
-    uint32_t *stamp = stamp_of(a);
+    int32_t cv[NA_ILP];
+    uint32_t wt[NA_ILP];
+#pragma unroll
+    for (int i = 0; i < NA_ILP; ++i) {
+        cv[i] = -1;
+        wt[i] = 0;
+        if (valid[i]) {
+            cv[i] = a.col[arc[i]];
+            wt[i] = a.w[arc[i]];
+        }
+    }
+    uint64_t nl[NA_ILP], cur[NA_ILP];
+    bool imp[NA_ILP];
     bool bad = false;
-    for (uint32_t v = tid; v < a.n; v += gridDim.x * blockDim.x) {
-        label[v] = INF64;
-        stamp[v] = 0;
-        bad |= a.row_ptr[v] > a.row_ptr[v + 1];
+#pragma unroll
+    for (int i = 0; i < NA_ILP; ++i) {
+        nl[i] = INF64;
+        cur[i] = 0;
+        if (!valid[i]) continue;
+        if (cv[i] < 0 || (uint32_t)cv[i] >= a.n) {
+            bad = true;
+            continue;
+        }
+        const uint64_t nd = (lab[i] >> 32) + (uint64_t)wt[i];
+        if (nd < INF32) {          // the export reports a distance beyond
+            nl[i] = (nd << 32) | (lab[i] & 0xFFFFFFFFull);
+            cur[i] = ldcg_u64(&label[cv[i]]);
+        }
     }
     if (bad) atomicOr(&c->err, NA_BAD_INPUT);
-}
-
-// Seeds (ascending, distinct, in range) at distance 0 on the first frontier.
-__global__ void na_seed_kernel(NaArgs a) {
-    uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= a.k) return;
-    NaControl *c = ctl_of(a);
-    int32_t s = a.seeds[r];
-    bool ok = s >= 0 && (uint32_t)s < a.n && (r == 0 || a.seeds[r - 1] < s);
-    if (!ok) {
-        atomicOr(&c->err, NA_BAD_INPUT);
-        return;
+#pragma unroll
+    for (int i = 0; i < NA_ILP; ++i) {
+        imp[i] = false;
+        if (nl[i] < cur[i])
+            imp[i] = nl[i] < atomicMin(reinterpret_cast<unsigned long long *>(&label[cv[i]]),
+                                       (unsigned long long)nl[i]);
     }
-    label_of(a)[s] = (uint64_t)r;
-    stamp_of(a)[s] = 1;
-    queue_of(a, 0)[r] = (uint32_t)s;
-    if (r == 0) c->count[0] = a.k;
+    if (!__any_sync(FULL, imp[0] | imp[1] | imp[2] | imp[3])) return;
+#pragma unroll
+    for (int i = 0; i < NA_ILP; ++i) {
+        const uint32_t mask = __ballot_sync(FULL, imp[i]);
+        if (mask == 0) continue;
+        const uint32_t n = *(volatile uint32_t *)region_n;
+        const uint32_t slot = n + (uint32_t)__popc(mask & lanemask_lt());
+        if (imp[i] && slot < NA_REGION) region[slot] = (uint32_t)cv[i];
+        __syncwarp();
+        if (lane_id() == 0) *(volatile uint32_t *)region_n = min(n + (uint32_t)__popc(mask), NA_REGION);
+        __syncwarp();
+        if (n + (uint32_t)__popc(mask) > NA_REGION)
+            na_queue(a, f, imp[i] && slot >= NA_REGION, (uint32_t)cv[i], &c->err);
+    }
 }
 
-// Frontier Bellman-Ford: iteration `it` relaxes the arcs of its frontier,
-// pushing every vertex whose label drops (once per iteration, by stamp).
-__global__ void __launch_bounds__(256) na_sssp_kernel(NaArgs a) {
+// Relaxes the rows of up to 32 vertices (has, u: one per lane), their arcs
+// flattened over the lanes.  Hubs are left to the hub pass of the next
+// iteration (`requeue`) or were queued as such.
+__device__ __forceinline__ void na_relax_rows(const NaArgs &a, NaControl *c, const NaFront &f,
+                                              uint32_t *region, uint32_t *region_n, bool has,
+                                              uint32_t u, bool requeue) {
+    const uint32_t lane = lane_id();
+    uint32_t s = 0, deg = 0;
+    uint64_t lab = INF64;
+    if (has) {
+        s = a.row_ptr[u];
+        deg = a.row_ptr[u + 1] - s;
+        lab = ldcg_u64(&label_of(a)[u]);
+    }
+    if (requeue) {
+        const bool hub = deg >= NA_HUB_DEG;
+        if (__any_sync(FULL, hub)) na_queue(a, f, hub, u, &c->err);
+        if (hub) deg = 0;
+    }
+    const uint32_t incl = warp_inclusive_scan(deg);
+    const uint32_t excl = incl - deg;
+    const uint32_t total = __shfl_sync(FULL, incl, 31);
+    for (uint32_t b = 0; b < total; b += 32 * NA_ILP) {
+        bool valid[NA_ILP];
+        uint32_t arc[NA_ILP];
+        uint64_t labs[NA_ILP];
+#pragma unroll
+        for (int i = 0; i < NA_ILP; ++i) {
+            const uint32_t j = b + lane + 32 * i;
+            valid[i] = j < total;
+            const uint32_t owner = warp_owner_search(excl, valid[i] ? j : 0);
+            const uint32_t so = __shfl_sync(FULL, s, owner);
+            const uint32_t eo = __shfl_sync(FULL, excl, owner);
+            labs[i] = __shfl_sync(FULL, lab, owner);
+            arc[i] = so + (j - eo);
+        }
+        na_relax(a, c, f, region, region_n, valid, arc, labs);
+    }
+}
+
+// pred(v) = smallest-id tight neighbour in v's cell: the first tight arc of
+// the row.  Arc `e` of reached vertex v: its index if tight, else INF32; a
+// reached vertex next to an unreached one means a distance did not fit below
+// 2^32 - 1.
+__device__ __forceinline__ uint32_t na_tight(const NaArgs &a, uint64_t lv, uint32_t e,
+                                             bool &overflow) {
+    const int32_t cu = a.col[e];
+    const uint32_t wt = a.w[e];
+    if (cu < 0 || (uint32_t)cu >= a.n) return INF32;
+    const uint64_t lu = ldcg_u64(&label_of(a)[cu]);
+    if (lu == INF64) {
+        overflow = true;
+        return INF32;
+    }
+    return (uint32_t)lu == (uint32_t)lv && (lu >> 32) + wt == lv >> 32 ? e : INF32;
+}
+
+__device__ __forceinline__ void na_write(const NaArgs &a, uint32_t v, uint64_t lv, uint32_t arc) {
+    const bool reached = lv != INF64;
+    if (a.cell) a.cell[v] = reached ? a.seeds[(uint32_t)lv] : -1;
+    if (a.dist) a.dist[v] = reached ? (uint32_t)(lv >> 32) : INF32;
+    if (a.pred) a.pred[v] = !reached ? -1 : (lv >> 32) == 0 ? (int32_t)v
+                                          : arc != INF32 ? a.col[arc] : -1;
+}
+
+// The whole call.  What bounds it: on small-world graphs the relaxations of
+// a few thick iterations (balanced by cutting hub rows over the grid), on
+// high-diameter ones the chain of hops, a barrier each; local_rounds lets a
+// warp follow its own pushes several hops between barriers.
+// R-MAT of 200,003 vertices, k = 300: 0.97 ms (12.7 with a hub's row walked
+// by one warp, and by one thread for its predecessor); grid 499 x 401,
+// k = 25: 0.87 ms (3.5 with a barrier per hop of 1216 blocks).
+__global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
+    __shared__ uint32_t region_s[NA_WARPS][NA_REGION];
+    __shared__ uint32_t region_n_s[NA_WARPS];
+    __shared__ uint32_t first_s[NA_WARPS][32];      // export: first tight arc per row
+    __shared__ uint32_t big_s[256], big_n, big_arc;
     NaControl *c = ctl_of(a);
     uint64_t *label = label_of(a);
-    uint32_t *stamp = stamp_of(a);
-    const uint32_t lane = lane_id();
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
-    if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;   // set by the reset or seed kernel: all blocks agree
+    const uint32_t lane = lane_id(), wib = threadIdx.x >> 5;
+    const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    const uint32_t warp = gtid >> 5, nwarps = nth >> 5;
+    const bool first = gtid == 0;
+    uint32_t *region = region_s[wib], *region_n = &region_n_s[wib];
     uint32_t bar_target = 0;
+
+    // Clear the previous call's state; check the row offsets (row_ptr[0] =
+    // 0, non-decreasing, row_ptr[n] = n_arcs), so that no arc outside
+    // [0, n_arcs) is read later.
+    {
+        bool bad = first && (a.row_ptr[0] != 0 || (uint64_t)a.row_ptr[a.n] != a.n_arcs);
+        uint32_t *stamp = stamp_of(a);
+        for (uint32_t v = gtid; v < a.n; v += nth) {
+            label[v] = INF64;
+            stamp[v] = 0;
+            bad |= a.row_ptr[v] > a.row_ptr[v + 1];
+        }
+        if (bad) atomicOr(&c->err, NA_BAD_INPUT);
+    }
+    if (!grid_sync(&c->bar, &c->err, bar_target)) return;
+    // set before the barrier: all blocks agree
+    if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;
+    // Seeds (ascending, distinct, in range) at distance 0 on the first
+    // frontier (iteration 0, tag 1).
+    for (uint32_t r0 = warp * 32; r0 < a.k; r0 += nwarps * 32) {
+        const uint32_t r = r0 + lane;
+        int32_t s = 0;
+        bool ok = r < a.k;
+        if (ok) {
+            s = a.seeds[r];
+            if (s < 0 || (uint32_t)s >= a.n || (r && a.seeds[r - 1] >= s)) {
+                atomicOr(&c->err, NA_BAD_INPUT);
+                ok = false;
+            } else {
+                label[s] = (uint64_t)r;
+            }
+        }
+        na_queue(a, NaFront{queue_of(a, 0), &c->count[0], &c->hubs[0], 1u}, ok, (uint32_t)s, &c->err);
+    }
+    if (!grid_sync(&c->bar, &c->err, bar_target)) return;
+    if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;
+
+    // Frontier Bellman-Ford: iteration `it` relaxes the arcs of its frontier,
+    // queueing every vertex whose label drops (once per iteration, by stamp).
+    uint32_t nf = min(ldcg_u32(&c->count[0]), a.n), nh = min(ldcg_u32(&c->hubs[0]), a.n);
     for (uint32_t it = 0;; ++it) {
-        uint32_t nf = min(ldcg_u32(&c->count[it % 3]), a.n);
-        if (first) c->count[(it + 2) % 3] = 0;
+        if (first) c->count[(it + 2) % 3] = c->hubs[(it + 2) % 3] = 0;
         const uint32_t *qc = queue_of(a, it);
-        uint32_t *qn = queue_of(a, it + 1);
-        uint32_t *cn = &c->count[(it + 1) % 3];
-        const uint32_t tag = it + 2;
-        for (uint32_t b0 = warp * 32; b0 < nf; b0 += nwarps * 32) {
-            uint32_t i = b0 + lane;
+        const NaFront f{queue_of(a, it + 1), &c->count[(it + 1) % 3], &c->hubs[(it + 1) % 3], it + 2};
+        if (lane == 0) *region_n = 0;
+        __syncwarp();
+        // hubs: 32 at a time, one per lane; piece p of hub h goes to warp
+        // (p + 97 h) mod nwarps
+        for (uint32_t h0 = 0; h0 < nh; h0 += 32) {
             uint32_t s = 0, deg = 0;
             uint64_t lab = INF64;
-            if (i < nf) {
-                uint32_t u = ldcg_u32(&qc[i]);
+            if (h0 + lane < nh) {
+                const uint32_t u = ldcg_u32(&qc[a.n - 1 - (h0 + lane)]);
                 s = a.row_ptr[u];
                 deg = a.row_ptr[u + 1] - s;
                 lab = ldcg_u64(&label[u]);
             }
-            uint32_t incl = warp_inclusive_scan(deg);
-            uint32_t excl = incl - deg;
-            uint32_t total = __shfl_sync(FULL, incl, 31);
-            for (uint32_t b = 0; b < total; b += 32) {
-                uint32_t j = b + lane;
-                bool valid = j < total;
-                uint32_t owner = warp_owner_search(excl, valid ? j : 0);
-                uint32_t so = __shfl_sync(FULL, s, owner);
-                uint32_t eo = __shfl_sync(FULL, excl, owner);
-                uint64_t lo = __shfl_sync(FULL, lab, owner);
-                bool push = false;
-                uint32_t v = 0;
-                if (valid) {
-                    uint32_t arc = so + (j - eo);
-                    int32_t cv = a.col[arc];
-                    if (cv < 0 || (uint32_t)cv >= a.n) {
-                        atomicOr(&c->err, NA_BAD_INPUT);
-                    } else {
-                        v = (uint32_t)cv;
-                        uint64_t nd = (lo >> 32) + (uint64_t)a.w[arc];
-                        if (nd < INF32) {
-                            uint64_t nl = (nd << 32) | (lo & 0xFFFFFFFFull);
-                            uint64_t old = atomicMin(reinterpret_cast<unsigned long long *>(&label[v]),
-                                                     (unsigned long long)nl);
-                            if (nl < old) push = atomicExch(&stamp[v], tag) != tag;
+            const uint32_t pieces = (deg + NA_CHUNK - 1) / NA_CHUNK;
+            const uint32_t p0 = (warp + nwarps - (h0 + lane) * 97u % nwarps) % nwarps;
+            for (uint32_t m = __ballot_sync(FULL, p0 < pieces); m; m &= m - 1) {
+                const uint32_t l = __ffs(m) - 1;
+                const uint32_t sl = __shfl_sync(FULL, s, l), dl = __shfl_sync(FULL, deg, l);
+                const uint64_t ll = __shfl_sync(FULL, lab, l);
+                for (uint64_t p = __shfl_sync(FULL, p0, l); p * NA_CHUNK < dl; p += nwarps) {
+                    const uint32_t lo = (uint32_t)p * NA_CHUNK, hi = min(dl, lo + NA_CHUNK);
+                    for (uint32_t b = lo; b < hi; b += 32 * NA_ILP) {
+                        bool valid[NA_ILP];
+                        uint32_t arc[NA_ILP];
+                        uint64_t labs[NA_ILP];
+#pragma unroll
+                        for (int i = 0; i < NA_ILP; ++i) {
+                            const uint32_t j = b + lane + 32 * i;
+                            valid[i] = j < hi;
+                            arc[i] = sl + j;
+                            labs[i] = ll;
                         }
+                        na_relax(a, c, f, region, region_n, valid, arc, labs);
                     }
                 }
-                uint32_t slot = warp_append(push, cn, a.n, &c->err);
-                if (slot != INF32) qn[slot] = v;
             }
+        }
+        // short rows: a thin frontier is spread over all warps
+        const uint32_t per = (nf + nwarps - 1) / nwarps;
+        const uint32_t bsz = per <= 1 ? 1 : per <= 2 ? 2 : per <= 4 ? 4 : per <= 8 ? 8 : per <= 16 ? 16 : 32;
+        for (uint32_t b0 = warp * bsz; b0 < nf; b0 += nwarps * bsz) {
+            const bool has = lane < bsz && b0 + lane < nf;
+            const uint32_t u = has ? ldcg_u32(&qc[b0 + lane]) : 0;
+            na_relax_rows(a, c, f, region, region_n, has, u, false);
+        }
+        // the warp follows its own pushes, a hop per round
+        uint32_t lo = 0;
+        for (uint32_t r = 0; r < a.local_rounds; ++r) {
+            __syncwarp();
+            const uint32_t hi = *(volatile uint32_t *)region_n;
+            if (lo >= hi) break;
+            for (uint32_t b0 = lo; b0 < hi; b0 += 32) {
+                const bool has = b0 + lane < hi;
+                na_relax_rows(a, c, f, region, region_n, has, has ? region[b0 + lane] : 0, true);
+            }
+            lo = hi;
+        }
+        __syncwarp();
+        const uint32_t staged = *(volatile uint32_t *)region_n;
+        for (uint32_t b0 = lo; b0 < staged; b0 += 32) {
+            const bool has = b0 + lane < staged;
+            na_queue(a, f, has, has ? region[b0 + lane] : 0, &c->err);
         }
         if (!grid_sync(&c->bar, &c->err, bar_target)) return;
         if (it + 1 >= a.max_iters) {
             if (first) atomicOr(&c->err, ERR_TIMEOUT);
             return;
         }
-        if (ldcg_u32(&c->count[(it + 1) % 3]) == 0) {
+        nf = min(ldcg_u32(&c->count[(it + 1) % 3]), a.n);
+        nh = min(ldcg_u32(&c->hubs[(it + 1) % 3]), a.n);
+        if ((nf | nh) == 0) {
             if (first) c->iterations = it + 1;
-            return;
+            break;
         }
     }
-}
 
-// pred(v) = smallest-id tight neighbour in v's cell; outputs in the
-// steiner_voronoi format.  A reached vertex next to an unreached one means
-// a distance did not fit below 2^32 - 1 (ERR_OVERFLOW).
-// A rejected input (NA_BAD_INPUT) leaves the caller's outputs untouched.
-__global__ void na_export_kernel(NaArgs a) {
-    NaControl *c = ctl_of(a);
+    // Predecessors and outputs in the steiner_voronoi format.  A rejected
+    // input leaves the caller's outputs untouched.  A block takes 256 rows,
+    // a warp 32 of them with their arcs flattened over its lanes; rows of
+    // NA_BLOCK_DEG arcs or more are then scanned by the whole block.
     if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;
-    const uint64_t *label = label_of(a);
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < a.n; v += gridDim.x * blockDim.x) {
-        uint64_t lv = label[v];
-        int32_t p = -1;
-        bool overflow = false;
-        if (lv != INF64) {
-            uint64_t dv = lv >> 32;
-            if (dv == 0) p = (int32_t)v;
-            for (uint32_t e = a.row_ptr[v]; e < a.row_ptr[v + 1]; ++e) {
-                int32_t cu = a.col[e];
-                if (cu < 0 || (uint32_t)cu >= a.n) continue;
-                uint64_t lu = label[cu];
-                if (lu == INF64) {
-                    overflow = true;
-                    continue;
-                }
-                if (p < 0 && (uint32_t)lu == (uint32_t)lv && (lu >> 32) + a.w[e] == dv) p = cu;
+    bool overflow = false;
+    for (uint32_t v0 = blockIdx.x * 256; v0 < a.n; v0 += gridDim.x * 256) {
+        if (threadIdx.x == 0) big_n = 0;
+        first_s[wib][lane] = INF32;
+        __syncthreads();
+        const uint32_t v = v0 + threadIdx.x;
+        uint32_t s = 0, deg = 0;
+        uint64_t lv = INF64;
+        bool big = false;
+        if (v < a.n) {
+            lv = ldcg_u64(&label[v]);
+            if (lv != INF64) {
+                s = a.row_ptr[v];
+                deg = a.row_ptr[v + 1] - s;
+                big = deg >= NA_BLOCK_DEG;
             }
         }
-        if (overflow) atomicOr(&c->err, ERR_OVERFLOW);
-        if (a.cell) a.cell[v] = lv == INF64 ? -1 : a.seeds[(uint32_t)lv];
-        if (a.dist) a.dist[v] = lv == INF64 ? INF32 : (uint32_t)(lv >> 32);
-        if (a.pred) a.pred[v] = p;
+        if (big) {
+            big_s[atomicAdd(&big_n, 1u)] = v;
+            deg = 0;
+        }
+        const uint32_t incl = warp_inclusive_scan(deg);
+        const uint32_t excl = incl - deg;
+        const uint32_t total = __shfl_sync(FULL, incl, 31);
+        for (uint32_t b = 0; b < total; b += 32 * NA_ILP) {
+#pragma unroll
+            for (int i = 0; i < NA_ILP; ++i) {
+                const uint32_t j = b + lane + 32 * i;
+                const uint32_t owner = warp_owner_search(excl, j < total ? j : 0);
+                const uint32_t so = __shfl_sync(FULL, s, owner), eo = __shfl_sync(FULL, excl, owner);
+                const uint64_t lo = __shfl_sync(FULL, lv, owner);
+                if (j >= total) continue;
+                const uint32_t t = na_tight(a, lo, so + (j - eo), overflow);
+                if (t != INF32) atomicMin(&first_s[wib][owner], t);
+            }
+        }
+        __syncwarp();
+        if (v < a.n && !big) na_write(a, v, lv, first_s[wib][lane]);
+        __syncthreads();
+        for (uint32_t i = 0; i < big_n; ++i) {
+            const uint32_t u = big_s[i];
+            if (threadIdx.x == 0) big_arc = INF32;
+            __syncthreads();
+            const uint64_t lu = ldcg_u64(&label[u]);
+            const uint32_t r1 = a.row_ptr[u + 1];
+            uint32_t best = INF32;
+            for (uint32_t e0 = a.row_ptr[u] + threadIdx.x; e0 < r1; e0 += 256 * NA_ILP) {
+#pragma unroll
+                for (int q = 0; q < NA_ILP; ++q) {
+                    const uint64_t e = (uint64_t)e0 + 256u * q;
+                    if (e < r1) best = min(best, na_tight(a, lu, (uint32_t)e, overflow));
+                }
+            }
+            best = __reduce_min_sync(FULL, best);
+            if (lane == 0 && best != INF32) atomicMin(&big_arc, best);
+            __syncthreads();
+            if (threadIdx.x == 0) na_write(a, u, lu, big_arc);
+        }
+        __syncthreads();
     }
+    if (__any_sync(FULL, overflow) && lane == 0) atomicOr(&c->err, ERR_OVERFLOW);
 }
 
 // Per-device set-up: the device address of g_scratch (host code cannot use
@@ -258,7 +476,7 @@ static int setup_device(int dev, DeviceSetup &out, const char **why) {
             return STEINER_ECUDA;
         }
         int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, na_sssp_kernel, 256, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, na_kernel, 256, 0);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess || per_sm < 1) {
             *why = e != cudaSuccess ? cudaGetErrorString(e) : "kernel does not fit on an SM";
@@ -310,17 +528,18 @@ extern "C" int steiner_voronoi_noalloc(const uint32_t *row_ptr, const int32_t *c
         return rc;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    NaArgs a{row_ptr, col, w, n, n_arcs, seeds, k, su.scratch, 1u << 22, cell, dist, pred};
-    unsigned grid = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)su.sms * 16);
-    na_ctl_reset_kernel<<<1, 1, 0, s>>>(a);
-    na_reset_kernel<<<grid, 256, 0, s>>>(a);
-    na_seed_kernel<<<(k + 255) / 256, 256, 0, s>>>(a);
-    void *args[] = {&a};
-    e = cudaLaunchCooperativeKernel((const void *)na_sssp_kernel, dim3(su.blocks), dim3(256), args,
-                                    0, s);
+    // A warp per 256 arcs or 32 vertices and at least one block: a small
+    // graph's iterations end at a barrier of fewer blocks.  Graphs of few
+    // arcs per vertex have a high diameter (grids, paths, trees): there a
+    // warp follows its own pushes up to 16 hops between barriers.
+    const uint64_t warps = std::max<uint64_t>(n_arcs / 256, (n + 31) / 32);
+    const unsigned blocks = (unsigned)std::min<uint64_t>((warps + 7) / 8, (uint64_t)su.blocks);
+    NaArgs a{row_ptr, col, w, n, n_arcs, seeds, k, su.scratch, 1u << 22,
+             n_arcs <= 8ull * n ? 16u : 0u, cell, dist, pred};
+    e = cudaMemsetAsync(su.scratch, 0, sizeof(NaControl), s);
     if (e == cudaSuccess) {
-        na_export_kernel<<<grid, 256, 0, s>>>(a);
-        e = cudaGetLastError();
+        void *args[] = {&a};
+        e = cudaLaunchCooperativeKernel((const void *)na_kernel, dim3(blocks), dim3(256), args, 0, s);
     }
     uint32_t err = 0;
     if (e == cudaSuccess)

@@ -45,3 +45,38 @@ def test_dense_items_cover_every_vertex(n, degree):
     g = G.random_graph(n, max(1, n * degree // 2), 1, 100, 7 * n + degree)
     seeds = G.seeds_from(np.arange(n), min(n, 9), n)
     _check(g, seeds, [("delta", 20)])
+
+
+def _noalloc_graphs():
+    for n in (2, 33, 257, 258, 1025, 1026):             # hub rows around 256 and 1024 arcs
+        yield f"star{n}", G.star(n, 1, 9, n)
+    yield "path", G.path(5000, 1, 9, 3)                 # a warp follows its own pushes
+    yield "grid", wl.grid(190, 140, 1000, seed=4)
+    yield "tree", G.random_tree(6000, 1, 50, 5)
+    yield "disconnected", G.random_graph(4000, 3000, 1, 20, 6)
+    yield "dense", G.complete(300, 1, 40, 7)            # every row a hub
+    yield "rmat", wl.rmat(12, 16, wmax=1000, seed=8)    # hubs of several pieces
+
+
+NOALLOC = list(_noalloc_graphs())
+
+
+@pytest.mark.parametrize("name,g", NOALLOC, ids=[c[0] for c in NOALLOC])
+def test_noalloc_rows_and_rounds(name, g):
+    """steiner_voronoi_noalloc against the oracle where its split of the work
+    changes: short rows, hubs in pieces, rows a whole block derives the
+    predecessor of, and warp-local rounds on graphs of few arcs per vertex."""
+    import torch
+
+    def dev(a):
+        return torch.from_numpy(np.ascontiguousarray(a).view(np.int32).copy()).cuda()
+
+    for k in sorted({1, min(7, g.n), g.n}):
+        seeds = np.sort(G.seeds_from(np.arange(g.n), k, k))
+        ref = oracle.voronoi(g, seeds)
+        out = [torch.full((g.n,), -7, dtype=torch.int32, device="cuda") for _ in range(3)]
+        rc = st.steiner_voronoi_noalloc(dev(g.row_ptr), dev(g.col), dev(g.w), dev(seeds), *out)
+        assert rc == st.STEINER_OK, st.last_error()
+        np.testing.assert_array_equal(out[0].cpu().numpy(), ref.cell)
+        np.testing.assert_array_equal(out[1].cpu().numpy().view(np.uint32), ref.dist)
+        np.testing.assert_array_equal(out[2].cpu().numpy(), ref.pred)
