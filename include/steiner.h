@@ -204,7 +204,9 @@ int steiner_serve_stop(steiner_graph_t g);
  *                  co-resident block; at most "sssp_max_blocks")
  *   "local_rounds" local relaxation rounds per frontier iteration
  *                  (0 = off): each warp keeps relaxing the vertices it
- *                  just queued, a hop per round, before the grid barrier
+ *                  just queued, a hop per round, before the grid barrier.
+ *                  At 0, with the far pile, a frontier too thin for the grid
+ *                  still takes some on graphs of few arcs per vertex
  *   "batch_delta"  band width of the multi-query engine (0 = w_max / 8 when
  *                  "delta" is at most the largest weight w_max, else "delta")
  *   "batch_pull"   1 (default): a query's first heavy-arc pass in the

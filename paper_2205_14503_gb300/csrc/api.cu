@@ -54,26 +54,34 @@ uint32_t bit_length(uint32_t x) { return x ? 32u - (uint32_t)__builtin_clz(x) : 
 
 // Cuts the vertices into consecutive ranges of at most `arcs` arcs (a hub
 // counts HEAVY_DEG: longer rows are queued in chunks) and ITEM_SPAN
-// vertices; a single vertex may exceed the arc limit.  Returns the range
+// vertices, and into coarser ones of SPARSE_ITEM_FACTOR times the arcs; a
+// single vertex may exceed the arc limit.  at[0] / at[1] receive the range
 // starts followed by n.  Blocks of CUT_BLOCK vertices are cut side by side
 // on the host's threads.
-std::vector<uint32_t> cut_items(const uint32_t *row_ptr, uint32_t n, uint64_t arcs) {
-    constexpr uint32_t CUT_BLOCK = 1u << 20;
+void cut_items(const uint32_t *row_ptr, uint32_t n, uint64_t arcs, std::vector<uint32_t> (&at)[2]) {
+    constexpr uint32_t CUT_BLOCK = 1u << 17;
+    struct Part {
+        std::vector<uint32_t> at[2];
+    };
     const uint32_t blocks = (uint32_t)(((uint64_t)n + CUT_BLOCK - 1) / CUT_BLOCK);
-    std::vector<std::vector<uint32_t>> part(blocks);
+    std::vector<Part> part(blocks);
     std::atomic<uint32_t> next{0};
     auto work = [&] {
         for (uint32_t b; (b = next.fetch_add(1)) < blocks;) {
             const uint32_t lo = b * CUT_BLOCK, hi = (uint32_t)std::min<uint64_t>(n, (uint64_t)lo + CUT_BLOCK);
-            std::vector<uint32_t> &at = part[b];
-            uint64_t sum = 0;
+            const uint64_t limit[2] = {arcs, SPARSE_ITEM_FACTOR * arcs};
+            uint64_t sum[2] = {0, 0};
+            uint32_t from[2] = {lo, lo};
+            for (int i = 0; i < 2; ++i) part[b].at[i].push_back(lo);
             for (uint32_t v = lo; v < hi; ++v) {
                 const uint32_t d = std::min(row_ptr[v + 1] - row_ptr[v], HEAVY_DEG);
-                if (at.empty() || sum + d > arcs || v - at.back() == ITEM_SPAN) {
-                    at.push_back(v);
-                    sum = 0;
+                for (int i = 0; i < 2; ++i) {
+                    if (v > from[i] && (sum[i] + d > limit[i] || v - from[i] == ITEM_SPAN)) {
+                        part[b].at[i].push_back(from[i] = v);
+                        sum[i] = 0;
+                    }
+                    sum[i] += d;
                 }
-                sum += d;
             }
         }
     };
@@ -88,10 +96,10 @@ std::vector<uint32_t> cut_items(const uint32_t *row_ptr, uint32_t n, uint64_t ar
     }
     work();
     for (auto &t : pool) t.join();
-    std::vector<uint32_t> at;
-    for (auto &p : part) at.insert(at.end(), p.begin(), p.end());
-    at.push_back(n);
-    return at;
+    for (int i = 0; i < 2; ++i) {
+        for (auto &p : part) at[i].insert(at[i].end(), p.at[i].begin(), p.at[i].end());
+        at[i].push_back(n);
+    }
 }
 
 uint32_t bits_for(uint32_t n) {
@@ -415,9 +423,9 @@ int query_locked(steiner_graph *G, const int32_t *seeds, uint32_t k, steiner_res
             double us = t1 > c.trace_ns[i] ? 1e-3 * (double)(t1 - c.trace_ns[i]) : -1.0;
             const double nw = (double)(G->geo.sssp_blocks * (G->geo.threads / 32));
             fprintf(stderr, "[steiner]   it %d: near %u heavy %u far %u T %u  %.1f us  relax %llu "
-                    "improved %llu atomics %llu  warp busy mean %.1f max %.1f us\n",
+                    "improved %llu  warp busy mean %.1f max %.1f us\n",
                     i, c.trace[i][0], c.trace[i][1], c.trace[i][2], c.trace[i][3], us,
-                    c.trace_relax[i][0], c.trace_relax[i][1], c.trace_relax[i][2],
+                    c.trace_relax[i][0], c.trace_relax[i][1],
                     1e-3 * (double)c.trace_busy[i][0] / nw, 1e-3 * (double)c.trace_busy[i][1]);
         }
     }
@@ -635,16 +643,17 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
         const uint64_t warps = (uint64_t)G->geo.sssp_max_blocks * (G->geo.threads / 32);
         const uint64_t arcs = std::min<uint64_t>(std::max<uint64_t>(n_arcs / (16 * warps), ITEM_ARCS_MIN),
                                                  ITEM_ARCS_MAX);
-        const std::vector<uint32_t> it = cut_items(irp, n, arcs);
-        const std::vector<uint32_t> sp = cut_items(irp, n, SPARSE_ITEM_FACTOR * arcs);
-        G->g.n_items = (uint32_t)it.size() - 1;
-        G->g.n_sparse_items = (uint32_t)sp.size() - 1;
-        e = dalloc(G->g.items, it.size());
-        if (e == cudaSuccess) e = dalloc(G->g.sparse_items, sp.size());
+        std::vector<uint32_t> at[2];
+        cut_items(irp, n, arcs, at);
+        G->g.n_items = (uint32_t)at[0].size() - 1;
+        G->g.n_sparse_items = (uint32_t)at[1].size() - 1;
+        e = dalloc(G->g.items, at[0].size());
+        if (e == cudaSuccess) e = dalloc(G->g.sparse_items, at[1].size());
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(G->g.items, it.data(), it.size() * 4, cudaMemcpyHostToDevice, s);
+            e = cudaMemcpyAsync(G->g.items, at[0].data(), at[0].size() * 4, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(G->g.sparse_items, sp.data(), sp.size() * 4, cudaMemcpyHostToDevice, s);
+            e = cudaMemcpyAsync(G->g.sparse_items, at[1].data(), at[1].size() * 4,
+                                cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return bail(cuda_fail(e, "work items"));
     }

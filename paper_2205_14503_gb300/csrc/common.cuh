@@ -238,6 +238,49 @@ __device__ __forceinline__ void region_append(bool want, uint32_t v, uint32_t *r
     __syncwarp();
 }
 
+// As region_append for N vertices per lane at once (want[i] appends v[i]):
+// one look at the fill count and, if the region is full, one move.
+template <int N>
+__device__ __forceinline__ void region_append_n(const bool (&want)[N], const uint32_t (&v)[N],
+                                                uint32_t *region, uint32_t *cnt, uint32_t cap,
+                                                bool flush, uint32_t *gq, uint32_t *gcount,
+                                                uint32_t gcap, uint32_t *err,
+                                                uint32_t *stamp = nullptr, uint32_t tag = 0) {
+    uint32_t mask[N], k = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        mask[i] = __ballot_sync(FULL, want[i]);
+        k += (uint32_t)__popc(mask[i]);
+    }
+    if (k == 0) return;
+    const uint32_t n = *(volatile uint32_t *)cnt;
+    if (n + k > cap) {
+#pragma unroll 1
+        for (int i = 0; i < N; ++i) {
+            // (a dynamic index would put the arrays in local memory)
+            bool wi = false;
+            uint32_t vi = 0;
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+                if (j == i) {
+                    wi = want[j];
+                    vi = v[j];
+                }
+            region_append(wi, vi, region, cnt, cap, flush, gq, gcount, gcap, err, stamp, tag);
+        }
+        return;
+    }
+    uint32_t at = n;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        if (want[i]) region[at + (uint32_t)__popc(mask[i] & lanemask_lt())] = v[i];
+        at += (uint32_t)__popc(mask[i]);
+    }
+    __syncwarp();
+    if (lane_id() == 0) *(volatile uint32_t *)cnt = at;
+    __syncwarp();
+}
+
 // Slot of the seed pair (a, b), a < b < k, in the upper-triangle table:
 // ascending slot order is ascending (a, b) order.
 __host__ __device__ __forceinline__ uint64_t pair_slot(uint64_t a, uint64_t b, uint64_t k) {

@@ -91,8 +91,8 @@ struct Control {
     uint32_t near_count[3];
     uint32_t heavy_count[3];
     uint32_t work_next[3];       // work items handed out on demand
-    uint32_t far_count[2];
-    uint32_t far_min[2];
+    uint32_t far_count[3];       // by phase % 3 (the piles alternate by phase & 1)
+    uint32_t far_min[3];
     uint32_t iterations;
     uint32_t phases;
     unsigned long long relax_attempts;
@@ -120,7 +120,7 @@ struct Control {
     unsigned long long pull_hsum;
     uint32_t trace[TRACE_LEN][4];  // first iterations: near items, heavy chunks, far pile, T
     unsigned long long trace_ns[TRACE_LEN];   // their start times (global timer, ns)
-    unsigned long long trace_relax[TRACE_LEN][3];   // relaxations, improvements, atomics (traced)
+    unsigned long long trace_relax[TRACE_LEN][2];   // relaxations, improvements (traced)
     unsigned long long trace_busy[TRACE_LEN][2];    // warps' relaxation time: sum, max (ns)
     unsigned long long end_ns;                // end of the last iteration
 };

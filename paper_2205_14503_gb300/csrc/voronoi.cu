@@ -48,6 +48,8 @@ struct SsspArgs {
     uint32_t *label32;       // narrow labels (the narrow kernel)
     uint32_t lshift;         // rank bits of a narrow label
     uint32_t ldmax;          // largest distance a narrow label holds
+    uint32_t lstep;          // 1 << lshift: a narrow label's step per unit of distance
+    uint64_t lmiss;          // sums of label and step at or above this do not fit
     uint32_t *stamp_near;
     uint32_t *stamp_far;
     uint32_t *q0, *q1;
@@ -65,7 +67,6 @@ struct SsspArgs {
     uint64_t *band_hq;       // heavy-row chunks of listed high-degree vertices
     uint32_t base_band;
     uint32_t defer;          // light/heavy arc split on
-    uint32_t far_scan;       // no far pile: splits find far vertices by scanning the labels
     uint32_t trace;          // record per-iteration relaxation counts
     // Dense frontiers (with the far scan, without local rounds): a large
     // frontier is a bitmap (one bit per vertex, set with a fire-and-forget
@@ -75,6 +76,8 @@ struct SsspArgs {
     // above it have fewer (the degree order makes this a bound).
     uint32_t dense;
     uint32_t pull;           // heavy-arc passes: 0 push, 1 by cost, 2 pull
+    uint32_t thin;           // far pile: a frontier below this size splits the pile early
+    uint32_t thin_rounds;    // ... and takes this many warp-local rounds
     uint32_t tail;           // 1: after a pull pass the rest runs as one unbounded band
     uint64_t m;              // arcs (the first bound on a pull pass's cost)
     uint32_t n_big;
@@ -117,6 +120,7 @@ __global__ void init_seeds_kernel(const uint32_t *__restrict__ row_ptr,
     if (r == 0) {
         ctl->far_min[0] = INF32;
         ctl->far_min[1] = INF32;
+        ctl->far_min[2] = INF32;
     }
     if (r >= k) return;
     uint32_t s = internal_id(new_of, (uint32_t)seeds[r]);
@@ -150,6 +154,8 @@ constexpr uint32_t FAR_STAGE = 1024;   // block staging capacity (far items)
 constexpr uint32_t BAND_STAGE = 2048;  // block staging capacity (band-list items)
 constexpr uint32_t BAND_REGION = BAND_STAGE / SSSP_WARPS;
 constexpr int SPLIT_ILP = 4;           // 32-vertex chunks per warp step in a band split
+constexpr uint32_t SUB_CHUNKS = 4;     // pieces of a hub chunk while hub chunks are few
+static_assert(CHUNK / SUB_CHUNKS >= 32 * ILP, "a piece is at least one relax_group");
 constexpr int PULL_ILP = 4;            // 32-vertex chunks per warp step in a pull pass
 
 // Where the appends of one processing segment go.
@@ -165,10 +171,7 @@ struct PushTargets {
     uint32_t *band_count;
     uint32_t tag_next;
     uint32_t tag_far;
-    uint64_t T;
-    // A full warp region may move to the global queue mid-segment (not
-    // during the warp-local rounds, which index into the region).
-    bool flush;
+    uint64_t Tl;         // the threshold as a label of the kernel's width
     // Near pushes of light vertices set bits of nbm (the next iteration
     // reads the bitmap) instead of going through the queue.
     bool dense;
@@ -230,30 +233,39 @@ __device__ __forceinline__ void flush_stage(Stage &st, const PushTargets &t, uin
                                             uint32_t *err) {
     __syncthreads();
     const uint32_t nf = min(st.far_n, FAR_STAGE);
-    if (threadIdx.x == 0) {
-        uint32_t nn = 0;
-        for (uint32_t w = 0; w < SSSP_WARPS; ++w) {
+    if (threadIdx.x < 32) {
+        // lane w < SSSP_WARPS sums up warp w's region; the atomics whose
+        // results are needed go out together, from different lanes
+        const uint32_t w = threadIdx.x;
+        uint32_t nn = 0, dnn = 0, dnb = 0, hs = 0;
+        if (w < SSSP_WARPS) {
             const uint32_t hi = min(st.near_n[w], NEAR_REGION), lo = st.local_lo[w];
-            st.near_off[w] = nn;
-            if (!t.nostamp) nn += hi > lo ? hi - lo : 0;
+            nn = !t.nostamp && hi > lo ? hi - lo : 0;
+            // bits set in the bitmaps count as items (a vertex set twice
+            // counts twice): the counts only size the next iteration and
+            // show that a frontier or band list is non-empty
+            dnn = st.dn_near[w];
+            dnb = st.dn_band[w];
+            hs = st.hs[w];
         }
-        st.base_near = nn ? atomicAdd(t.qn_count, nn) : 0;
-        st.base_far = nf ? atomicAdd(t.far_count, nf) : 0;
-        if (st.far_min != INF32) atomicMin(t.far_min, st.far_min);
-        // bits set in the bitmaps count as items (a vertex set twice counts
-        // twice): the counts only size the next iteration and show that a
-        // frontier or band list is non-empty
-        uint32_t dnn = 0, dnb = 0;
-        for (uint32_t w = 0; w < SSSP_WARPS; ++w) {
-            dnn += st.dn_near[w];
-            dnb += st.dn_band[w];
-        }
-        if (dnn) atomicAdd(t.qn_count, dnn);
-        if (dnb) atomicAdd(t.band_count, dnb);
+        const uint32_t incl = warp_inclusive_scan(nn);
+        if (w < SSSP_WARPS) st.near_off[w] = incl - nn;
+        nn = __shfl_sync(FULL, incl, 31);
+        dnn = __reduce_add_sync(FULL, dnn);
+        dnb = __reduce_add_sync(FULL, dnb);
+        unsigned long long hsum = hs;
         if (t.hsum) {
-            unsigned long long hs = 0;
-            for (uint32_t w = 0; w < SSSP_WARPS; ++w) hs += st.hs[w];
-            if (hs) atomicAdd(t.hsum, hs);
+#pragma unroll
+            for (int o = SSSP_WARPS / 2; o >= 1; o >>= 1) hsum += __shfl_xor_sync(FULL, hsum, o);
+        }
+        if (w == 0) {
+            if (dnn) atomicAdd(t.qn_count, dnn);
+            if (dnb) atomicAdd(t.band_count, dnb);
+            if (t.hsum && hsum) atomicAdd(t.hsum, hsum);
+            if (st.far_min != INF32) atomicMin(t.far_min, st.far_min);
+            st.base_near = nn ? atomicAdd(t.qn_count, nn) : 0;
+        } else if (w == 1) {
+            st.base_far = nf ? atomicAdd(t.far_count, nf) : 0;
         }
     }
     __syncthreads();
@@ -291,37 +303,66 @@ __device__ __forceinline__ void flush_stage(Stage &st, const PushTargets &t, uin
     }
 }
 
-// Near appends: high-degree vertices become CHUNK-arc items of the heavy
-// queue (per-lane atomics; rare), the rest go through the staging buffer.
+// Near appends of N vertices per lane: high-degree vertices become CHUNK-arc
+// items of the heavy queue (one atomicAdd for the warp's), the rest go
+// through the staging buffer.  `flush`: a full warp region may move to the
+// global queue (not during the warp-local rounds, which index into it).
+template <int N>
 __device__ __forceinline__ void push_near(const SsspArgs &a, Stage &st, const PushTargets &t,
-                                          bool want, uint32_t v, uint32_t deg) {
-    bool heavy = want && deg >= HEAVY_DEG;
-    const uint32_t w = threadIdx.x >> 5;
-    region_append(want && !heavy, v, st.near_buf + w * NEAR_REGION, &st.near_n[w], NEAR_REGION,
-                  t.flush, t.qn, t.qn_count, a.n, &a.ctl->err,
-                  t.nostamp ? a.stamp_near : nullptr, t.tag_next);
-    if (heavy) {
-        uint32_t nc = (deg + CHUNK - 1) / CHUNK;
-        uint32_t base = atomicAdd(t.hqn_count, nc);
-        if (base + nc > a.heavy_cap) {
-            atomicOr(&a.ctl->err, ERR_CAPACITY);
-        } else {
-            for (uint32_t c = 0; c < nc; ++c) t.hqn[base + c] = ((uint64_t)v << 32) | c;
-        }
+                                          bool flush, const bool (&want)[N],
+                                          const uint32_t (&v)[N], const uint32_t (&deg)[N]) {
+    bool light[N];
+    uint32_t nc = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        light[i] = want[i] && deg[i] < HEAVY_DEG;
+        if (want[i] && !light[i]) nc += (deg[i] + CHUNK - 1) / CHUNK;
     }
+    const uint32_t w = threadIdx.x >> 5;
+    region_append_n<N>(light, v, st.near_buf + w * NEAR_REGION, &st.near_n[w], NEAR_REGION,
+                       flush, t.qn, t.qn_count, a.n, &a.ctl->err,
+                       t.nostamp ? a.stamp_near : nullptr, t.tag_next);
+    if (!__any_sync(FULL, nc)) return;
+    const uint32_t incl = warp_inclusive_scan(nc);
+    uint32_t at = 0;
+    if (lane_id() == 31) at = atomicAdd(t.hqn_count, incl);
+    at = __shfl_sync(FULL, at, 31);
+    if (at + __shfl_sync(FULL, incl, 31) > a.heavy_cap) {
+        if (lane_id() == 0) atomicOr(&a.ctl->err, ERR_CAPACITY);
+        return;
+    }
+    at += incl - nc;
+    // the chunk lists, one hub after another: the whole warp writes each
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        for (uint32_t m = __ballot_sync(FULL, want[i] && !light[i]); m; m &= m - 1) {
+            const uint32_t l = __ffs(m) - 1;
+            const uint32_t vl = __shfl_sync(FULL, v[i], l), base = __shfl_sync(FULL, at, l);
+            const uint32_t n = (__shfl_sync(FULL, deg[i], l) + CHUNK - 1) / CHUNK;
+            for (uint32_t c = lane_id(); c < n; c += 32) t.hqn[base + c] = ((uint64_t)vl << 32) | c;
+            if (lane_id() == l) at += n;
+        }
 }
 
-// Far appends: `want` appends v to the pile (first time this phase);
-// `cand` marks every far proposal, so far_min bounds the pile from below
-// even for vertices already in it.
+// Far appends of N vertices per lane: want[i] appends v[i] to the pile
+// (first time this phase); cand[i] marks every far proposal, so far_min
+// bounds the pile from below even for vertices already in it.
+template <bool SCAN, int N, class Dist>
 __device__ __forceinline__ void push_far(const SsspArgs &a, Stage &st, const PushTargets &t,
-                                         bool want, bool cand, uint32_t v, uint32_t d) {
-    stage_append(want, v, st.far_buf, &st.far_n, FAR_STAGE, t.farq, t.far_count, a.n, &a.ctl->err);
-    if (__any_sync(FULL, cand)) {
-        uint32_t m = cand ? d : INF32;
+                                         const bool (&want)[N], const bool (&cand)[N],
+                                         const uint32_t (&v)[N], Dist dist) {
+    uint32_t m = INF32;
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) m = min(m, __shfl_xor_sync(FULL, m, o));
-        if (lane_id() == 0 && m != INF32) atomicMin(&st.far_min, m);
+    for (int i = 0; i < N; ++i)
+        if (cand[i]) m = min(m, dist(i));
+    m = __reduce_min_sync(FULL, m);
+    if (m == INF32) return;              // nothing far
+    if (lane_id() == 0) atomicMin(&st.far_min, m);
+    if constexpr (!SCAN) {               // (no pile with the scan)
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            stage_append(want[i], v[i], st.far_buf, &st.far_n, FAR_STAGE, t.farq, t.far_count, a.n,
+                         &a.ctl->err);
     }
 }
 
@@ -332,91 +373,113 @@ __device__ __forceinline__ uint64_t sssp_label(const SsspArgs &a, uint32_t v) {
     return ldcg_u64(&a.label[v]);
 }
 
-// Relaxes up to ILP arcs per lane.  For arc u of this lane: valid[u], the
-// arc index and the tail's label; only arcs with wlo <= weight < whi are
-// relaxed.  The loads and atomics of the ILP arcs are issued back to back
-// so their latencies overlap.
+// Labels in the width of the kernel: the hot relaxation compares and sends
+// them as stored.  A narrow proposal is one multiply-add, lab + (w << shift)
+// in 64 bits, whose order and overflow tell everything; widening every
+// label to 64 bits cost twice the instructions.
+template <bool NARROW>
+struct LabelOf {
+    using T = uint64_t;
+};
+template <>
+struct LabelOf<true> {
+    using T = uint32_t;
+};
+
+template <bool NARROW>
+__device__ __forceinline__ typename LabelOf<NARROW>::T raw_label(const SsspArgs &a, uint32_t v) {
+    if constexpr (NARROW) return ldcg_u32(&a.label32[v]);
+    else return ldcg_u64(&a.label[v]);
+}
+
+// The smallest label of a distance at or above T (saturating: with the far
+// side empty every label is below it but the unreached one).
+template <bool NARROW>
+__device__ __forceinline__ uint64_t threshold_label(const SsspArgs &a, uint64_t T) {
+    if (NARROW) return T >= (1ull << (32 - a.lshift)) ? INF32 : T << a.lshift;
+    return T >= INF32 ? INF64 : T << 32;
+}
+
+// One group of up to ILP arcs per lane: the arc records and their tails'
+// labels (`valid`: this lane has arc u).
+template <bool NARROW>
+struct ArcGroup {
+    uint2 e[ILP];
+    typename LabelOf<NARROW>::T lab[ILP];
+    bool valid[ILP];
+};
+
+// Relaxes a group's arcs of weight in [wlo, whi).  The loads and atomics of
+// the ILP arcs are issued back to back so their latencies overlap.
 // With `precheck` a plain load of the head's label comes first and only
 // improving proposals issue the atomic: right for thick frontiers, where
 // L2 atomic throughput is the limit; thin frontiers are latency-bound and
 // skip the extra dependent load.
-// The tail labels lab[] are in the 64-bit form; NARROW kernels keep the
-// head labels in 32 bits and flag (narrow_miss) any proposal whose distance
-// does not fit one, which the host answers with a 64-bit rerun.
-template <bool NARROW>
+// NARROW kernels flag (narrow_miss) any proposal whose distance does not fit
+// a 32-bit label, which the host answers with a 64-bit rerun.
+template <bool NARROW, bool SCAN>
 __device__ __forceinline__ void relax_group(const SsspArgs &a, Stage &st, const PushTargets &t,
-                                            const bool (&valid)[ILP], const uint32_t (&arc)[ILP],
-                                            const uint64_t (&lab)[ILP], bool precheck,
-                                            bool stream, uint32_t wlo, uint32_t whi,
-                                            unsigned long long &attempts,
-                                            unsigned long long &improved, bool &narrow_miss,
-                                            unsigned long long &atomics) {
-    uint2 e[ILP];
+                                            const ArcGroup<NARROW> &g, bool flush, bool precheck, uint32_t wlo,
+                                            uint32_t whi, uint32_t &attempts,
+                                            uint32_t &improved, bool &narrow_miss) {
+    using L = typename LabelOf<NARROW>::T;
+    L nl[ILP], cur[ILP];
+    bool want[ILP];
 #pragma unroll
     for (int u = 0; u < ILP; ++u) {
-        e[u] = make_uint2(0, 0);
-        // heavy-row chunks are streamed (evict first); short rows may be
-        // re-read by later hops and stay cacheable
-        if (valid[u]) e[u] = stream ? __ldcs(&a.adj[arc[u]]) : __ldg(&a.adj[arc[u]]);
+        want[u] = g.valid[u] && g.e[u].y >= wlo && g.e[u].y < whi;
+        attempts += want[u];
+        cur[u] = (L)~0ull;
+        if constexpr (NARROW) {
+            const uint64_t sum = (uint64_t)g.e[u].y * a.lstep + g.lab[u];
+            if (want[u] && sum >= a.lmiss) {
+                narrow_miss = true;
+                want[u] = false;
+            }
+            nl[u] = (uint32_t)sum;
+        } else {
+            // proposals at or above 2^32 - 1 are skipped; the scan reports the overflow
+            const uint64_t nd = (g.lab[u] >> 32) + (uint64_t)g.e[u].y;
+            want[u] = want[u] && nd < INF32;
+            nl[u] = (nd << 32) | (g.lab[u] & 0xFFFFFFFFull);
+        }
+        if (precheck && want[u]) cur[u] = raw_label<NARROW>(a, g.e[u].x);
     }
-    uint64_t nd[ILP];
     bool imp[ILP], fr[ILP];
+    bool any = false;
 #pragma unroll
     for (int u = 0; u < ILP; ++u) {
         imp[u] = fr[u] = false;
-        nd[u] = INF32;
-        if (valid[u] && e[u].y >= wlo && e[u].y < whi) {
-            ++attempts;
-            nd[u] = (lab[u] >> 32) + (uint64_t)e[u].y;
-            if (NARROW) {
-                if (nd[u] > a.ldmax) {
-                    narrow_miss = true;
-                } else {
-                    const uint32_t nl = ((uint32_t)nd[u] << a.lshift) | (uint32_t)lab[u];
-                    if (!precheck || nl < ldcg_u32(&a.label32[e[u].x])) {
-                        ++atomics;
-                        if (a.far_scan && nd[u] >= t.T) {
-                            // a far proposal needs no answer (nothing is queued
-                            // for it): a fire-and-forget reduction
-                            atomicMin(&a.label32[e[u].x], nl);
-                            fr[u] = true;
-                        } else {
-                            const uint32_t old = atomicMin(&a.label32[e[u].x], nl);
-                            imp[u] = nl < old;
-                        }
-                    }
-                }
-            } else if (nd[u] < INF32) {
-                // proposals at or above 2^32 - 1 are skipped; the scan reports the overflow
-                uint64_t nl = (nd[u] << 32) | (lab[u] & 0xFFFFFFFFull);
-                if (!precheck || nl < ldcg_u64(&a.label[e[u].x])) {
-                    ++atomics;
-                    if (a.far_scan && nd[u] >= t.T) {
-                        atomicMin(reinterpret_cast<unsigned long long *>(&a.label[e[u].x]),
-                                  (unsigned long long)nl);
-                        fr[u] = true;
-                    } else {
-                        uint64_t old = atomicMin(reinterpret_cast<unsigned long long *>(&a.label[e[u].x]),
-                                                 (unsigned long long)nl);
-                        imp[u] = nl < old;
-                    }
-                }
+        if (want[u] && nl[u] < cur[u]) {
+            const bool far = SCAN && nl[u] >= (L)t.Tl;
+            if constexpr (NARROW) {
+                // a far proposal needs no answer (nothing is queued for it):
+                // a fire-and-forget reduction
+                if (far) atomicMin(&a.label32[g.e[u].x], nl[u]);
+                else imp[u] = nl[u] < atomicMin(&a.label32[g.e[u].x], nl[u]);
+            } else {
+                auto *dst = reinterpret_cast<unsigned long long *>(&a.label[g.e[u].x]);
+                if (far) atomicMin(dst, (unsigned long long)nl[u]);
+                else imp[u] = nl[u] < atomicMin(dst, (unsigned long long)nl[u]);
             }
+            fr[u] = far;
         }
+        any |= imp[u] | fr[u];
     }
     // rounds that improve nothing skip the append machinery
-    if (!__any_sync(FULL, imp[0] | imp[1] | imp[2] | imp[3] | fr[0] | fr[1] | fr[2] | fr[3])) return;
-    bool to_near[ILP], to_far[ILP], cand[ILP], dn[ILP];
-    uint32_t deg[ILP];
+    if (!__any_sync(FULL, any)) return;
+    bool to_near[ILP], to_far[ILP], cand[ILP];
+    uint32_t deg[ILP], vs[ILP];
+    uint32_t dn = 0;
 #pragma unroll
     for (int u = 0; u < ILP; ++u) {
-        to_near[u] = to_far[u] = dn[u] = false;
+        to_near[u] = to_far[u] = false;
         cand[u] = fr[u];         // a fire-and-forget far proposal still bounds far_min
         deg[u] = 0;
+        const uint32_t v = vs[u] = g.e[u].x;
         if (!imp[u]) continue;
         ++improved;
-        uint32_t v = e[u].x;
-        if (nd[u] < t.T && t.dense) {
+        if (SCAN && nl[u] < (L)t.Tl && t.dense) {
             // a light vertex sets its bit; a possible hub (id below n_big)
             // reads its degree first and, if it is one, joins the chunk queue
             if (v < a.n_big) {
@@ -427,37 +490,30 @@ __device__ __forceinline__ void relax_group(const SsspArgs &a, Stage &st, const 
                 to_near[u] = atomicExch(&a.stamp_near[v], t.tag_next) != t.tag_next;
             } else {
                 atomicOr(&t.nbm[v >> 5], 1u << (v & 31));
-                dn[u] = true;
+                ++dn;
             }
-        } else if (nd[u] < t.T && t.nostamp) {
+        } else if (nl[u] < (L)t.Tl) {
             // ids at or above n_big cannot be hubs: no look at the row
             if (v < a.n_big) {
-                const uint32_t r0 = a.row_ptr[v];
+                const uint32_t r0 = a.row_ptr[v];                 // independent of the exchange
                 deg[u] = (t.lend ? t.lend[v] : a.row_ptr[v + 1]) - r0;
             }
-            to_near[u] = deg[u] < HEAVY_DEG ||     // hubs join the chunk queue once
+            // without stamps only hubs join the chunk queue once
+            to_near[u] = (t.nostamp && deg[u] < HEAVY_DEG) ||
                          atomicExch(&a.stamp_near[v], t.tag_next) != t.tag_next;
-        } else if (nd[u] < t.T) {
-            uint32_t r0 = a.row_ptr[v];                           // independent of the exchange
-            uint32_t r1 = t.lend ? t.lend[v] : a.row_ptr[v + 1];  // end of the part relaxed near
-            to_near[u] = atomicExch(&a.stamp_near[v], t.tag_next) != t.tag_next;
-            deg[u] = r1 - r0;
         } else {
             cand[u] = true;      // bounds far_min
             // with the far scan, the split finds far vertices by their labels
-            if (!a.far_scan) to_far[u] = atomicExch(&a.stamp_far[v], t.tag_far) != t.tag_far;
+            if (!SCAN) to_far[u] = atomicExch(&a.stamp_far[v], t.tag_far) != t.tag_far;
         }
     }
-#pragma unroll
-    for (int u = 0; u < ILP; ++u) {
-        push_near(a, st, t, to_near[u], e[u].x, deg[u]);
-        push_far(a, st, t, to_far[u], cand[u], e[u].x, (uint32_t)nd[u]);
-    }
-    if (t.dense) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) c += (uint32_t)__popc(__ballot_sync(FULL, dn[u]));
-        if (lane_id() == 0 && c) st.dn_near[threadIdx.x >> 5] += c;
+    push_far<SCAN, ILP>(a, st, t, to_far, cand, vs, [&](int u) {
+        return (uint32_t)(NARROW ? nl[u] >> a.lshift : (uint64_t)nl[u] >> 32);
+    });
+    push_near<ILP>(a, st, t, flush, to_near, vs, deg);
+    if (SCAN && t.dense) {
+        dn = __reduce_add_sync(FULL, dn);
+        if (lane_id() == 0 && dn) st.dn_near[threadIdx.x >> 5] += dn;
     }
 }
 
@@ -485,85 +541,18 @@ __device__ __forceinline__ void band_track(const SsspArgs &a, Stage &st, bool wa
     if (lane_id() == 0 && listed) st.hs[w] += listed;
     region_append(add && !big, u, st.band_buf + w * BAND_REGION, &st.band_n[w], BAND_REGION, true,
                   a.band_q, &a.ctl->band_count, a.n, &a.ctl->err);
-    if (big) {
-        const uint32_t nc = (hdeg + CHUNK - 1) / CHUNK;
-        const uint32_t base = atomicAdd(&a.ctl->band_hcount, nc);
+    for (uint32_t m = __ballot_sync(FULL, big); m; m &= m - 1) {     // chunk lists: the whole warp
+        const uint32_t l = __ffs(m) - 1;
+        const uint32_t ul = __shfl_sync(FULL, u, l);
+        const uint32_t nc = (__shfl_sync(FULL, hdeg, l) + CHUNK - 1) / CHUNK;
+        uint32_t base = 0;
+        if (lane_id() == 0) base = atomicAdd(&a.ctl->band_hcount, nc);
+        base = __shfl_sync(FULL, base, 0);
         if (base + nc > a.heavy_cap || base + nc < base) {
-            atomicOr(&a.ctl->err, ERR_CAPACITY);
-        } else {
-            for (uint32_t c = 0; c < nc; ++c) a.band_hq[base + c] = ((uint64_t)u << 32) | c;
+            if (lane_id() == 0) atomicOr(&a.ctl->err, ERR_CAPACITY);
+            continue;
         }
-    }
-}
-
-// Lists high-degree vertex u (warp-uniform; deg arcs in its heavy part) in
-// the current band once, as its CHUNK-arc pieces.
-__device__ __forceinline__ void band_track_heavy(const SsspArgs &a, Stage &st, uint32_t u,
-                                                 uint32_t deg, uint32_t tag) {
-    const uint32_t lane = lane_id();
-    if (deg == 0) return;
-    uint32_t add = 0;
-    if (lane == 0) add = atomicExch(&a.stamp_band[u], tag) != tag;
-    if (!__shfl_sync(FULL, add, 0)) return;
-    if (lane == 0) st.hs[threadIdx.x >> 5] += deg;
-    const uint32_t nc = (deg + CHUNK - 1) / CHUNK;
-    uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(&a.ctl->band_hcount, nc);
-    base = __shfl_sync(FULL, base, 0);
-    if (base + nc > a.heavy_cap || base + nc < base) {
-        if (lane == 0) atomicOr(&a.ctl->err, ERR_CAPACITY);
-        return;
-    }
-    for (uint32_t c = lane; c < nc; c += 32) a.band_hq[base + c] = ((uint64_t)u << 32) | c;
-}
-
-// Relaxes the arcs of up to 32 frontier vertices, one per lane (has, u),
-// flattened over the lanes: their light parts (their heavy parts in a
-// band's closing pass, hp), listing them for the band when tracked.
-template <bool NARROW>
-__device__ __forceinline__ void relax_vertices(const SsspArgs &a, Stage &st, const PushTargets &t,
-                                               bool has, uint32_t u, bool hp, bool track,
-                                               uint32_t tag_band, uint32_t wlo, uint32_t whi,
-                                               bool precheck, unsigned long long &attempts,
-                                               unsigned long long &improved, bool &narrow_miss,
-                                               unsigned long long &atomics) {
-    const uint32_t lane = lane_id();
-    uint32_t s = 0, deg = 0, hdeg = 0;
-    uint64_t lab = INF64;
-    if (has) {
-        const uint32_t r0 = a.row_ptr[u], r1 = a.row_ptr[u + 1];
-        const uint32_t le = t.lend ? t.lend[u] : r1;
-        if (hp) {                       // the heavy part (or the whole row)
-            s = t.lend ? le : r0;
-            deg = r1 - s;
-        } else {                        // the light part
-            s = r0;
-            deg = le - r0;
-            hdeg = t.lend ? r1 - le : r1 - r0;
-        }
-        lab = sssp_label<NARROW>(a, u);
-        if (lab == INF64) deg = 0;
-    }
-    if (track) band_track(a, st, has, u, hdeg, tag_band);
-    const uint32_t incl = warp_inclusive_scan(deg);
-    const uint32_t excl = incl - deg;
-    const uint32_t total = __shfl_sync(FULL, incl, 31);
-    for (uint32_t b = 0; b < total; b += 32 * ILP) {
-        bool valid[ILP];
-        uint32_t arc[ILP];
-        uint64_t labs[ILP];
-#pragma unroll
-        for (int q = 0; q < ILP; ++q) {
-            const uint32_t j = b + lane + 32 * q;
-            valid[q] = j < total;
-            const uint32_t owner = warp_owner_search(excl, valid[q] ? j : 0);
-            const uint32_t so = __shfl_sync(FULL, s, owner);
-            const uint32_t eo = __shfl_sync(FULL, excl, owner);
-            labs[q] = __shfl_sync(FULL, lab, owner);
-            arc[q] = so + (j - eo);
-        }
-        relax_group<NARROW>(a, st, t, valid, arc, labs, precheck, false, wlo, whi, attempts,
-                            improved, narrow_miss, atomics);
+        for (uint32_t c = lane_id(); c < nc; c += 32) a.band_hq[base + c] = ((uint64_t)ul << 32) | c;
     }
 }
 
@@ -580,6 +569,63 @@ __device__ __forceinline__ uint32_t nth_set_bit(uint32_t x, uint32_t t) {
         }
     }
     return pos;
+}
+
+// Relaxes the arcs of up to 32 rows, one per lane ([s, s + deg), tail label
+// lab; lanes without work deg = 0), flattened over the lanes.  The lanes'
+// rows are first compacted (no empty row in between), so that the row of
+// position j is the number of row starts at or before it: one mask per 32
+// positions, not a search by shuffles.  The next group's arc records are
+// loaded before this group is relaxed.
+template <bool NARROW, bool SCAN>
+__device__ __forceinline__ void relax_rows(const SsspArgs &a, Stage &st, const PushTargets &t,
+                                           uint32_t s, uint32_t deg,
+                                           typename LabelOf<NARROW>::T lab, bool flush,
+                                           bool precheck, bool stream, uint32_t wlo, uint32_t whi,
+                                           uint32_t &attempts, uint32_t &improved,
+                                           bool &narrow_miss) {
+    const uint32_t lane = lane_id();
+    const uint32_t mask = __ballot_sync(FULL, deg != 0);
+    if (mask == 0) return;
+    const uint32_t rows = (uint32_t)__popc(mask);
+    if (mask != FULL) {
+        const uint32_t from = nth_set_bit(mask, lane < rows ? lane : 0);
+        s = __shfl_sync(FULL, s, from);
+        lab = __shfl_sync(FULL, lab, from);
+        deg = __shfl_sync(FULL, deg, from);
+        if (lane >= rows) deg = 0;
+    }
+    const uint32_t incl = warp_inclusive_scan(deg);
+    const uint32_t total = __shfl_sync(FULL, incl, 31);
+    const uint32_t excl = lane < rows ? incl - deg : INF32;
+    const uint32_t base = s - excl;      // arc of position j in row r: base(r) + j
+    auto load = [&](uint32_t b, ArcGroup<NARROW> &g) {
+#pragma unroll
+        for (int q = 0; q < ILP; ++q) {
+            const uint32_t b0 = b + 32 * q, j = b0 + lane;
+            // rows that start in this window, and those before it
+            const uint32_t before = (uint32_t)__popc(__ballot_sync(FULL, excl < b0));
+            const uint32_t at = excl - b0;
+            const uint32_t starts = __reduce_or_sync(FULL, at < 32 ? 1u << at : 0u);
+            const uint32_t row = before + (uint32_t)__popc(starts & (FULL >> (31 - lane))) - 1;
+            const uint32_t arc = __shfl_sync(FULL, base, row) + j;
+            g.lab[q] = __shfl_sync(FULL, lab, row);
+            g.valid[q] = j < total;
+            g.e[q] = make_uint2(0, 0);
+            // hub chunks are streamed (evict first); short rows may be
+            // re-read by later hops and stay cacheable
+            if (g.valid[q]) g.e[q] = stream ? __ldcs(&a.adj[arc]) : __ldg(&a.adj[arc]);
+        }
+    };
+    ArcGroup<NARROW> g;
+    load(0, g);
+    for (uint32_t b = 0; b < total; b += 32 * ILP) {
+        ArcGroup<NARROW> next;
+        const bool more = b + 32 * ILP < total;
+        if (more) load(b + 32 * ILP, next);
+        relax_group<NARROW, SCAN>(a, st, t, g, flush, precheck, wlo, whi, attempts, improved, narrow_miss);
+        if (more) g = next;
+    }
 }
 
 // Pull form of a band's heavy-arc pass (threshold T, every label below T
@@ -603,9 +649,8 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
                                        const uint32_t *list, uint32_t count, uint32_t *out,
                                        uint32_t *out_count, bool tail, uint32_t *nbm,
                                        uint32_t *qn, uint32_t *qn_count, uint64_t *hqn,
-                                       uint32_t *hqn_count, unsigned long long &attempts,
-                                       unsigned long long &improved, bool &narrow_miss,
-                                       unsigned long long &atomics) {
+                                       uint32_t *hqn_count, uint32_t &attempts,
+                                       uint32_t &improved, bool &narrow_miss) {
     const uint32_t lane = lane_id();
     const uint32_t wib = threadIdx.x >> 5;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -617,7 +662,6 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
     t.qn_count = qn_count;
     t.hqn = hqn;
     t.hqn_count = hqn_count;
-    t.flush = true;
     t.dense = a.dense != 0;
     t.nbm = nbm;
     t.nostamp = false;
@@ -726,8 +770,12 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
         }
         __syncwarp();
         // each lane settles its own vertices: one atomic per improved one
+        bool push[PULL_ILP];
+        uint32_t pdeg[PULL_ILP];
 #pragma unroll
         for (int c = 0; c < PULL_ILP; ++c) {
+            push[c] = false;
+            pdeg[c] = 0;
             const uint64_t best = pm[32 * c + lane];
             uint64_t now = lab[c];
             if (uns[c] && best < lab[c]) {
@@ -737,8 +785,7 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
                 else
                     atomicMin(reinterpret_cast<unsigned long long *>(&a.label[vs[c]]),
                               (unsigned long long)best);
-                ++atomics;
-                ++improved;
+                    ++improved;
                 fmin = min(fmin, (uint32_t)(best >> 32));
                 now = best;
             }
@@ -754,9 +801,11 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
                     atomicOr(&t.nbm[vs[c] >> 5], 1u << (vs[c] & 31));
                 }
                 if (lane == 0 && word) st.dn_near[wib] += (uint32_t)__popc(word);
-                push_near(a, st, t, want && !bit, vs[c], deg);
+                push[c] = want && !bit;
+                pdeg[c] = deg;
             }
         }
+        if (tail) push_near<PULL_ILP>(a, st, t, true, push, vs, pdeg);
         __syncwarp();
     }
     met = __reduce_add_sync(FULL, met);
@@ -771,23 +820,23 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
 // the persistent near/far kernel
 // ---------------------------------------------------------------------------
 
-template <bool NARROW>
-__global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
+// SCAN: splits scan the labels (a.far_scan), else there is a far pile.
+template <bool NARROW, bool SCAN>
+__global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ SsspArgs a) {
     __shared__ Stage st;
+    __shared__ PushTargets t;      // this iteration's (shared: off the hot loops' registers)
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     Control *ctl = a.ctl;
-    unsigned long long attempts = 0, improved = 0;
+    uint32_t attempts = 0, improved = 0;      // this thread's
     bool narrow_miss = false;
-    unsigned long long atomics = 0;
     // trace: each warp's counter sums at the start of the iteration (lane 0
     // keeps them in shared memory, off the registers of the hot loops)
-    __shared__ unsigned long long trace_snap[SSSP_WARPS][4];
-    if (threadIdx.x < SSSP_WARPS * 4) (&trace_snap[0][0])[threadIdx.x] = 0;
+    __shared__ unsigned long long trace_snap[SSSP_WARPS][3];
+    if (threadIdx.x < SSSP_WARPS * 3) (&trace_snap[0][0])[threadIdx.x] = 0;
     uint32_t it = 0, phase = 0, bands = 0;
-    uint32_t bar_target = 0;
-    uint64_t T = a.delta;
+    uint64_t T = a.delta, T_old = 0;
     bool first = (blockIdx.x == 0 && threadIdx.x == 0);
     bool hp = false;               // this iteration is a band's heavy-arc pass
     bool pull = false;             // ... in the pull form
@@ -810,16 +859,16 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
     if (threadIdx.x == 0) pull_bound = a.m;
     bool cur_dense = false;        // this iteration's light items are the bits of a near bitmap
 
+    // This iteration's frontier, read when its last push was known to be in;
+    // split: it also splits the far pile, whose sizes are n_far and f_min.
+    uint32_t n_light = min(ldcg_u32(&ctl->near_count[0]), a.n);
+    uint32_t n_heavy = min(ldcg_u32(&ctl->heavy_count[0]), a.heavy_cap);
+    uint32_t n_far = 0;
+    bool split = false;
+    uint32_t bar_target = 0;
+
     for (;;) {
         const uint32_t cs = it % 3, ns = (it + 1) % 3;
-        uint32_t n_light, n_heavy;
-        if (hp) {
-            n_light = min(ldcg_u32(&ctl->band_count), a.n);
-            n_heavy = min(ldcg_u32(&ctl->band_hcount), a.heavy_cap);
-        } else {
-            n_light = min(ldcg_u32(&ctl->near_count[cs]), a.n);
-            n_heavy = min(ldcg_u32(&ctl->heavy_count[cs]), a.heavy_cap);
-        }
         if (first) {
             ctl->near_count[(it + 2) % 3] = 0;
             ctl->heavy_count[(it + 2) % 3] = 0;
@@ -828,30 +877,18 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
             if (it < TRACE_LEN) {
                 ctl->trace[it][0] = n_light;
                 ctl->trace[it][1] = n_heavy;
-                ctl->trace[it][2] = ldcg_u32(&ctl->far_count[phase & 1]);
+                ctl->trace[it][2] = split ? n_far : ldcg_u32(&ctl->far_count[phase % 3]);
                 ctl->trace[it][3] = (uint32_t)T;
                 ctl->trace_ns[it] = global_ns();
             }
         }
-        stage_reset(st);
         const bool odd = it & 1;
         const uint32_t *qc = hp ? a.band_q : (odd ? a.q1 : a.q0);
         const uint64_t *hqc = hp ? a.band_hq : (odd ? a.hq1 : a.hq0);
-        const uint32_t fc = phase & 1;
-        PushTargets t;
-        t.qn = odd ? a.q0 : a.q1;
-        t.qn_count = &ctl->near_count[ns];
-        t.hqn = odd ? a.hq0 : a.hq1;
-        t.hqn_count = &ctl->heavy_count[ns];
-        t.farq = fc ? a.far1 : a.far0;
-        t.far_count = &ctl->far_count[fc];
-        t.far_min = &ctl->far_min[fc];
-        t.bandq = a.band_q;
-        t.band_count = &ctl->band_count;
-        t.tag_next = a.base_near + it + 1;
-        t.tag_far = a.base_far + phase;
-        t.T = T;
-        t.flush = true;
+        // fc: which of the two piles takes this phase's far vertices; fs: its
+        // counters (three, so that one can be cleared while the piles of two
+        // phases are in use)
+        const uint32_t fc = phase & 1, fs = phase % 3;
         // dense in: light items from this iteration's near bitmap (or, in a
         // dense heavy-arc pass, the band bitmap); dense out: a large
         // frontier (a fraction of the graph, or many hub chunks) pushes its
@@ -861,20 +898,42 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         const bool push_dense =
             a.dense && !hp && (n_light >= a.n / 128 || n_heavy >= a.n / 4096);
         uint32_t *bm_in = hp ? a.bbm : ((it & 1) ? a.nbm1 : a.nbm0);
-        t.dense = push_dense;
-        t.nbm = (it & 1) ? a.nbm0 : a.nbm1;
-        t.nostamp = a.local_rounds != 0 && !hp;
-        t.nostamp_stamp = a.stamp_near;
         // arcs relaxed by this iteration: all; light ones while a band
         // iterates under the split; heavy ones in the band's closing pass
         // (in the tail every relaxation covers whole rows)
         const uint32_t wlo = hp ? a.delta : 0u;
         const uint32_t whi = (a.defer && !hp && !tail) ? a.delta : 0xFFFFFFFFu;
         const bool track = a.defer && !hp && !tail;
-        t.lend = tail ? nullptr : a.lend;
+        const uint32_t *lend = tail ? nullptr : a.lend;
+        // warp-local rounds; a frontier thinner than the grid takes some in
+        // any case (with the far pile and whole rows)
+        const uint32_t local_rounds =
+            hp ? 0u : a.local_rounds ? a.local_rounds
+                    : !SCAN && !a.defer && n_light + n_heavy < a.thin ? a.thin_rounds : 0u;
         const uint32_t tag_band = a.base_band + bands;
-        t.hsum = track ? &ctl->band_hsum : (hp && pull ? &ctl->pull_hsum : nullptr);
-
+        if (threadIdx.x == 0) {
+            t.qn = odd ? a.q0 : a.q1;
+            t.qn_count = &ctl->near_count[ns];
+            t.hqn = odd ? a.hq0 : a.hq1;
+            t.hqn_count = &ctl->heavy_count[ns];
+            t.farq = fc ? a.far1 : a.far0;
+            t.far_count = &ctl->far_count[fs];
+            t.far_min = &ctl->far_min[fs];
+            // a pull pass without a list yet sweeps every id and lists the
+            // unsettled ones as this phase's pile (empty with the far scan)
+            t.bandq = hp && pull ? t.farq : a.band_q;
+            t.band_count = hp && pull ? t.far_count : &ctl->band_count;
+            t.tag_next = a.base_near + it + 1;
+            t.tag_far = a.base_far + phase;
+            t.Tl = threshold_label<NARROW>(a, T);
+            t.dense = push_dense;
+            t.nbm = odd ? a.nbm0 : a.nbm1;
+            t.nostamp = local_rounds != 0;
+            t.nostamp_stamp = a.stamp_near;
+            t.lend = lend;
+            t.hsum = track ? &ctl->band_hsum : (hp && pull ? &ctl->pull_hsum : nullptr);
+        }
+        stage_reset(st);
         // Vertices per warp batch: a thin frontier is spread over all warps
         // (fewer sequential rounds per warp), a thick one packs 32 per warp.
         uint32_t per = (n_light + nwarps - 1) / nwarps;
@@ -888,182 +947,196 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         // ranges: the sweep itself is then the cost.
         const bool sparse = n_light < a.n_words / 2;
         const uint32_t *items = sparse ? a.sparse_items : a.items;
-        const uint32_t n_work = n_heavy + (dense_in ? (sparse ? a.n_sparse_items : a.n_items)
-                                                    : (n_light + bsz - 1) / bsz);
-        if (a.trace && lane == 0) trace_snap[threadIdx.x >> 5][3] = global_ns();
-        if (hp && pull) {
-            // without a list yet, the pass sweeps every id and lists the
-            // unsettled ones as this phase's pile (empty with the far scan)
+        // Few hub chunks are cut in SUB_CHUNKS pieces of one relax_group each.
+        const uint32_t subs = n_heavy * SUB_CHUNKS <= nwarps ? SUB_CHUNKS : 1u;
+        const uint32_t n_hitems = n_heavy * subs;
+        const uint32_t n_work = n_hitems + (dense_in ? (sparse ? a.n_sparse_items : a.n_items)
+                                                     : (n_light + bsz - 1) / bsz);
+        if (a.trace && lane == 0) trace_snap[threadIdx.x >> 5][2] = global_ns();
+        if (SCAN && hp && pull) {
             uint32_t *pile = fc ? a.far1 : a.far0;
-            t.bandq = pile;
-            t.band_count = &ctl->far_count[fc];
             // with the tail to follow, the pass pushes its first frontier
             pull_pass<NARROW>(a, st, pmin, T, listed ? pile : nullptr,
-                              listed ? min(ldcg_u32(&ctl->far_count[fc]), a.n) : a.n,
-                              (listed || a.tail) ? nullptr : pile, &ctl->far_count[fc],
+                              listed ? min(ldcg_u32(&ctl->far_count[fs]), a.n) : a.n,
+                              (listed || a.tail) ? nullptr : pile, &ctl->far_count[fs],
                               a.tail != 0, t.nbm, t.qn, t.qn_count, t.hqn, t.hqn_count,
-                              attempts, improved, narrow_miss, atomics);
+                              attempts, improved, narrow_miss);
         } else {
-        // The last quarter of a long list is handed out on demand (the next
-        // index is fetched while an item is relaxed), so that the iteration
-        // does not end with its slowest warp (R-MAT 26, degree 8, k = 10,000:
-        // the thickest iterations 3.2 ms, all fixed 3.65).
-        const uint32_t n_fixed = n_work < 8 * nwarps ? n_work : n_work / 4 * 3 / nwarps * nwarps;
-        uint32_t grab = 0;
-        for (uint32_t wi = warp; wi < n_work;
-             wi = wi + nwarps < n_fixed || n_fixed == n_work ? wi + nwarps
-                                                             : n_fixed + __shfl_sync(FULL, grab, 0)) {
-            if (wi + nwarps >= n_fixed && n_fixed != n_work && lane == 0)
-                grab = atomicAdd(&ctl->work_next[cs], 1u);
-            if (wi < n_heavy) {
-                // one CHUNK of a high-degree vertex per warp
-                uint64_t item = __ldcg(reinterpret_cast<const unsigned long long *>(&hqc[wi]));
-                uint32_t u = (uint32_t)(item >> 32), c = (uint32_t)item;
-                uint32_t r0 = a.row_ptr[u], r1 = a.row_ptr[u + 1];
-                const uint32_t le = t.lend ? t.lend[u] : r1;      // light part [r0, le)
-                // a band's heavy pass covers the heavy part, else the light one
-                const uint32_t base = hp && t.lend ? le : r0, end = hp ? r1 : le;
-                uint32_t s = base + c * CHUNK;
-                uint32_t e = min(end, s + CHUNK);
-                uint64_t lab = sssp_label<NARROW>(a, u);
-                if (track && c == 0) band_track_heavy(a, st, u, t.lend ? r1 - le : r1 - r0, tag_band);
-                for (uint32_t b = s; b < e; b += 32 * ILP) {
-                    bool valid[ILP];
-                    uint32_t arc[ILP];
-                    uint64_t labs[ILP];
-#pragma unroll
-                    for (int q = 0; q < ILP; ++q) {
-                        arc[q] = b + lane + 32 * q;
-                        valid[q] = arc[q] < e;
-                        labs[q] = lab;
-                    }
-                    relax_group<NARROW>(a, st, t, valid, arc, labs, true, true, wlo, whi, attempts,
-                                improved, narrow_miss, atomics);
-                }
-            } else if (dense_in) {
-                // the words of the item's vertex range, one per lane (the
-                // range's bits are read and cleared; a word may be shared
-                // with the neighbouring items); their set bits, 32 at a
-                // time, are the vertices
-                const uint32_t v0 = __ldg(&items[wi - n_heavy]), v1 = __ldg(&items[wi - n_heavy + 1]);
-                const uint32_t w0 = v0 >> 5, w1 = (v1 - 1) >> 5;
-                uint32_t word = 0;
-                if (w0 + lane <= w1) {
-                    uint32_t own = FULL;
-                    if (lane == 0) own <<= v0 & 31;
-                    if (w0 + lane == w1) own &= FULL >> (31 - ((v1 - 1) & 31));
-                    word = ldcg_u32(&bm_in[w0 + lane]) & own;
-                    if (word) {
-                        if (own == FULL) bm_in[w0 + lane] = 0;
-                        else atomicAnd(&bm_in[w0 + lane], ~own);
-                    }
-                }
-                const uint32_t cnt = (uint32_t)__popc(word);
-                const uint32_t incl = warp_inclusive_scan(cnt);
-                const uint32_t excl = incl - cnt;
-                const uint32_t total = __shfl_sync(FULL, incl, 31);
-                for (uint32_t b = 0; b < total; b += 32) {
-                    const uint32_t j = b + lane;
-                    const bool has = j < total;
-                    const uint32_t owner = warp_owner_search(excl, has ? j : 0);
-                    const uint32_t wo = __shfl_sync(FULL, word, owner);
-                    const uint32_t eo = __shfl_sync(FULL, excl, owner);
-                    const uint32_t u = has ? (w0 + owner) * 32 + nth_set_bit(wo, j - eo) : 0;
-                    relax_vertices<NARROW>(a, st, t, has, u, hp, track, tag_band, wlo, whi, true,
-                                           attempts, improved, narrow_miss, atomics);
-                }
-            } else {
-                // bsz frontier vertices per warp, their arcs flattened over the lanes
-                const uint32_t i = (wi - n_heavy) * bsz + lane;
-                const bool has = lane < bsz && i < n_light;
-                const uint32_t u = has ? ldcg_u32(&qc[i]) : 0;
-                relax_vertices<NARROW>(a, st, t, has, u, hp, track, tag_band, wlo, whi, bsz == 32,
-                                       attempts, improved, narrow_miss, atomics);
-            }
-        }
-        }
-        // Local rounds: relax the vertices just staged for the next
-        // iteration right away, a hop further per round, instead of waiting
-        // for the grid barrier; what is left is flushed.  (A heavy-arc pass
-        // stages nothing near.)
-        if (a.local_rounds && !hp) {
-            // Warp-local rounds: each warp relaxes the vertices it staged
-            // itself, a hop per round, with no block barrier between hops.
+            // The last quarter of a long list is handed out on demand (the
+            // next index is fetched while an item is relaxed), so that the
+            // iteration does not end with its slowest warp (R-MAT 26, degree
+            // 8, k = 10,000: the thickest iterations 3.2 ms, all fixed 3.65).
+            // After the list come the warp-local rounds (the vertices this
+            // warp staged for the next iteration, relaxed right away, a hop
+            // further per round, without a barrier; what is left is
+            // flushed).  One loop for all of them: the relaxation is
+            // expanded once.
+            const uint32_t n_fixed = n_work < 8 * nwarps ? n_work : n_work / 4 * 3 / nwarps * nwarps;
             const uint32_t wib = threadIdx.x >> 5;
-            t.flush = false;            // the loop below indexes into the region
-            uint32_t *region = st.near_buf + wib * NEAR_REGION;
-            uint32_t lo = 0;
-            for (uint32_t r = 0; r < a.local_rounds; ++r) {
-                __syncwarp();
-                const uint32_t hi = min(*(volatile uint32_t *)&st.near_n[wib], NEAR_REGION);
-                if (lo >= hi) break;
-                for (uint32_t b0 = lo; b0 < hi; b0 += 32) {
-                    const uint32_t i = b0 + lane;
-                    const bool has = i < hi;
-                    uint32_t s = 0, deg = 0, u = 0, hdeg = 0;
-                    uint64_t lab = INF64;
-                    if (has) {
-                        u = region[i];
-                        // row offsets and the label in one round trip: every
-                        // later improvement of u appends u again (to the
-                        // improving warp's region), so the current label is
-                        // all a round needs
-                        s = a.row_ptr[u];
-                        const uint32_t r1 = a.row_ptr[u + 1];
-                        const uint32_t le = t.lend ? t.lend[u] : r1;
-                        deg = le - s;
-                        hdeg = t.lend ? r1 - le : r1 - s;
-                        lab = sssp_label<NARROW>(a, u);
-                    }
-                    if (track) band_track(a, st, has, u, hdeg, tag_band);
-                    uint32_t incl = warp_inclusive_scan(deg);
-                    uint32_t excl = incl - deg;
-                    uint32_t total = __shfl_sync(FULL, incl, 31);
-                    for (uint32_t b = 0; b < total; b += 32 * ILP) {
-                        bool valid[ILP];
-                        uint32_t arc[ILP];
-                        uint64_t labs[ILP];
-#pragma unroll
-                        for (int q = 0; q < ILP; ++q) {
-                            uint32_t j = b + lane + 32 * q;
-                            valid[q] = j < total;
-                            uint32_t owner = warp_owner_search(excl, valid[q] ? j : 0);
-                            uint32_t so = __shfl_sync(FULL, s, owner);
-                            uint32_t eo = __shfl_sync(FULL, excl, owner);
-                            labs[q] = __shfl_sync(FULL, lab, owner);
-                            arc[q] = so + (j - eo);
+            const uint32_t *region = st.near_buf + wib * NEAR_REGION;
+            uint32_t rounds = local_rounds;
+            uint32_t wi = warp, grab = 0, local_lo = 0;
+            for (;;) {
+                // this item: nb batches of up to 32 vertices
+                const bool hub = wi < n_hitems, local = wi >= n_work;
+                uint32_t nb = 1, word = 0, excl = 0, total = 0, w0 = 0, local_hi = 0;
+                if (local) {
+                    if (rounds == 0) break;
+                    --rounds;
+                    __syncwarp();
+                    local_hi = min(*(volatile uint32_t *)&st.near_n[wib], NEAR_REGION);
+                    if (local_lo >= local_hi) break;
+                    nb = (local_hi - local_lo + 31) / 32;
+                } else {
+                    if (wi + nwarps >= n_fixed && n_fixed != n_work && lane == 0)
+                        grab = atomicAdd(&ctl->work_next[cs], 1u);
+                    if (SCAN && dense_in && !hub) {
+                        // the words of the item's vertex range, one per lane
+                        // (the range's bits are read and cleared; a word may
+                        // be shared with the neighbouring items); their set
+                        // bits, 32 at a time, are the vertices
+                        const uint32_t v0 = __ldg(&items[wi - n_hitems]);
+                        const uint32_t v1 = __ldg(&items[wi - n_hitems + 1]);
+                        const uint32_t w1 = (v1 - 1) >> 5;
+                        w0 = v0 >> 5;
+                        if (w0 + lane <= w1) {
+                            uint32_t own = FULL;
+                            if (lane == 0) own <<= v0 & 31;
+                            if (w0 + lane == w1) own &= FULL >> (31 - ((v1 - 1) & 31));
+                            word = ldcg_u32(&bm_in[w0 + lane]) & own;
+                            if (word) {
+                                if (own == FULL) bm_in[w0 + lane] = 0;
+                                else atomicAnd(&bm_in[w0 + lane], ~own);
+                            }
                         }
-                        relax_group<NARROW>(a, st, t, valid, arc, labs, false, false, wlo, whi,
-                                    attempts, improved, narrow_miss, atomics);
+                        const uint32_t cnt = (uint32_t)__popc(word);
+                        excl = warp_inclusive_scan(cnt);
+                        total = __shfl_sync(FULL, excl, 31);
+                        excl -= cnt;
+                        nb = (total + 31) / 32;
                     }
                 }
-                lo = hi;
+                for (uint32_t b = 0; b < nb; ++b) {
+                    // one vertex per lane; a hub chunk (or a piece of one) is
+                    // part of one row, on lane 0
+                    bool has;
+                    uint32_t u = 0, c = 0, sub = 0;
+                    if (local) {
+                        const uint32_t i = local_lo + 32 * b + lane;
+                        has = i < local_hi;
+                        if (has) u = region[i];
+                    } else if (hub) {
+                        has = lane == 0;
+                        if (has) {
+                            const uint64_t item = __ldcg(reinterpret_cast<const unsigned long long *>(
+                                &hqc[subs > 1 ? wi / SUB_CHUNKS : wi]));
+                            sub = subs > 1 ? wi % SUB_CHUNKS : 0u;
+                            u = (uint32_t)(item >> 32);
+                            c = (uint32_t)item;
+                        }
+                    } else if (SCAN && dense_in) {
+                        const uint32_t j = 32 * b + lane;
+                        has = j < total;
+                        const uint32_t owner = warp_owner_search(excl, has ? j : 0);
+                        const uint32_t wo = __shfl_sync(FULL, word, owner);
+                        const uint32_t eo = __shfl_sync(FULL, excl, owner);
+                        if (has) u = (w0 + owner) * 32 + nth_set_bit(wo, j - eo);
+                    } else {
+                        // bsz frontier vertices per warp
+                        const uint32_t i = (wi - n_hitems) * bsz + lane;
+                        has = lane < bsz && i < n_light;
+                        if (has) u = ldcg_u32(&qc[i]);
+                    }
+                    uint32_t s = 0, deg = 0, hdeg = 0;
+                    auto lab = (typename LabelOf<NARROW>::T)~0ull;
+                    if (has) {
+                        const uint32_t r0 = a.row_ptr[u], r1 = a.row_ptr[u + 1];
+                        const uint32_t le = lend ? lend[u] : r1;      // light part [r0, le)
+                        // (a warp-local round needs no more than the current
+                        // label: every later improvement of u appends u
+                        // again, to the improving warp's region)
+                        lab = raw_label<NARROW>(a, u);
+                        // the closing pass of a band covers the heavy part
+                        // (or the whole row), else the light one
+                        s = hp && lend ? le : r0;
+                        deg = (hp ? r1 : le) - s;
+                        if (!hp) hdeg = lend ? r1 - le : r1 - r0;
+                        if (hub) {
+                            const uint32_t at = c * CHUNK + sub * (CHUNK / SUB_CHUNKS);
+                            s += at;
+                            deg = deg > at ? min(deg - at, CHUNK / subs) : 0u;
+                        }
+                        if (lab == (typename LabelOf<NARROW>::T)~0ull) deg = 0;
+                    }
+                    if (track) band_track(a, st, has && (c | sub) == 0, u, hdeg, tag_band);
+                    relax_rows<NARROW, SCAN>(a, st, t, s, deg, lab, !local,
+                                             hub || (SCAN && dense_in) || (!local && bsz == 32), hub,
+                                             wlo, whi, attempts, improved, narrow_miss);
+                }
+                if (local) local_lo = local_hi;
+                else wi = wi + nwarps < n_fixed || n_fixed == n_work ? wi + nwarps
+                                                                     : n_fixed + __shfl_sync(FULL, grab, 0);
             }
-            if (lane == 0) st.local_lo[wib] = lo;
+            if (lane == 0) st.local_lo[wib] = local_lo;
+        }
+        if (!SCAN && split) {
+            // The pile of the phase that this iteration ended (see the
+            // decision below): a vertex below the old threshold was settled
+            // while parked; one below the new threshold joins the next
+            // frontier, the rest the new pile.  Vertices that this
+            // iteration's relaxations push as well are kept apart by the
+            // stamps (a region without stamps may hold a vertex twice).
+            // After the warp-local rounds: only the warps that read the pile
+            // would follow its vertices there, and the others wait (grid
+            // 4096 x 4096, 32 rounds: Voronoi phase 11.4 against 8.5 ms).
+            const uint32_t *pile = fc ? a.far0 : a.far1;
+            for (uint32_t b = warp * 32 * SPLIT_ILP; b < n_far; b += nwarps * 32 * SPLIT_ILP) {
+                uint32_t v[SPLIT_ILP], deg[SPLIT_ILP];
+                uint64_t d[SPLIT_ILP];
+                bool to_near[SPLIT_ILP], keep[SPLIT_ILP], to_far[SPLIT_ILP];
+#pragma unroll
+                for (int c = 0; c < SPLIT_ILP; ++c) {
+                    const uint32_t i = b + 32u * c + lane;
+                    v[c] = i < n_far ? ldcg_u32(&pile[i]) : INF32;
+                }
+#pragma unroll
+                for (int c = 0; c < SPLIT_ILP; ++c)
+                    d[c] = v[c] != INF32 ? sssp_label<NARROW>(a, v[c]) >> 32 : 0ull;
+#pragma unroll
+                for (int c = 0; c < SPLIT_ILP; ++c) {
+                    to_near[c] = d[c] >= T_old && d[c] < T;
+                    deg[c] = 0;
+                    if (to_near[c]) {
+                        if (v[c] < a.n_big) deg[c] = a.row_ptr[v[c] + 1] - a.row_ptr[v[c]];
+                        if (!t.nostamp || deg[c] >= HEAVY_DEG)
+                            to_near[c] = atomicExch(&a.stamp_near[v[c]], t.tag_next) != t.tag_next;
+                    }
+                    keep[c] = d[c] >= T;
+                    to_far[c] = keep[c] && atomicExch(&a.stamp_far[v[c]], t.tag_far) != t.tag_far;
+                }
+                push_far<SCAN, SPLIT_ILP>(a, st, t, to_far, keep, v, [&](int c) { return (uint32_t)d[c]; });
+                push_near<SPLIT_ILP>(a, st, t, !t.nostamp, to_near, v, deg);
+            }
         }
         if (a.trace && it < TRACE_LEN) {
             // per warp: busy time of this iteration's relaxation (sum, max)
-            unsigned long long da = attempts, di = improved, dm = atomics;
+            unsigned long long da = attempts, di = improved;
 #pragma unroll
             for (int o = 16; o >= 1; o >>= 1) {
                 da += __shfl_xor_sync(FULL, da, o);
                 di += __shfl_xor_sync(FULL, di, o);
-                dm += __shfl_xor_sync(FULL, dm, o);
             }
             if (lane == 0) {
                 unsigned long long *snap = trace_snap[threadIdx.x >> 5];
-                const unsigned long long busy = global_ns() - snap[3];
-                const unsigned long long sa = da, si = di, sm = dm;
+                const unsigned long long busy = global_ns() - snap[2];
+                const unsigned long long sa = da, si = di;
                 da -= snap[0];
                 di -= snap[1];
-                dm -= snap[2];
                 snap[0] = sa;
                 snap[1] = si;
-                snap[2] = sm;
                 if (da | di) {
                     atomicAdd(&ctl->trace_relax[it][0], da);
                     atomicAdd(&ctl->trace_relax[it][1], di);
-                    atomicAdd(&ctl->trace_relax[it][2], dm);
                 }
                 atomicAdd(&ctl->trace_busy[it][0], busy);
                 atomicMax(&ctl->trace_busy[it][1], busy);
@@ -1103,8 +1176,41 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
             }
             break;
         }
-        uint32_t next = ldcg_u32(&ctl->near_count[ns]) + ldcg_u32(&ctl->heavy_count[ns]);
-        if (next != 0) continue;
+        n_light = min(ldcg_u32(&ctl->near_count[ns]), a.n);
+        n_heavy = min(ldcg_u32(&ctl->heavy_count[ns]), a.heavy_cap);
+        const uint32_t far_now = ldcg_u32(&ctl->far_count[fs]);   // stable if the pile is split next
+        const uint32_t fmin_now = ldcg_u32(&ctl->far_min[fs]);
+        split = false;
+        if (!SCAN && !a.defer) {
+            // Far pile, no light/heavy split: the next iteration splits the
+            // pile as well (no iteration and barrier of its own) when the
+            // frontier drained, and already when it is thin (a.thin): the
+            // grid's warps would idle through the last hops of every band.  Every block decides on near_count, which no
+            // iteration writes before all have read it.  A thin frontier
+            // always ends the phase (the threshold stays if the pile is
+            // empty): an ended phase's pile takes no more pushes, so every
+            // block reads the same count and minimum of it.
+            if (n_light + n_heavy >= a.thin) continue;
+            const bool drained = (n_light | n_heavy) == 0;
+            n_far = min(far_now, a.n);
+            if (drained && n_far == 0) {
+                if (first) ctl->exit_reason = 1;       // converged
+                break;
+            }
+            ++phase;
+            if (first) {           // last read a phase ago, next used a phase from now
+                ctl->far_count[(phase + 1) % 3] = 0;
+                ctl->far_min[(phase + 1) % 3] = INF32;
+            }
+            if (n_far) {
+                T_old = T;
+                T = (fmin_now != INF32 && (uint64_t)fmin_now > T ? (uint64_t)fmin_now : T) +
+                    a.delta;
+                split = true;
+            }
+            continue;
+        }
+        if (n_light | n_heavy) continue;
         if (tail) {                    // the tail's frontier drained: converged
             if (first) ctl->exit_reason = 1;
             break;
@@ -1121,11 +1227,13 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         if (a.defer && !was_hp && !tail &&
             (ldcg_u32(&ctl->band_count) | ldcg_u32(&ctl->band_hcount)) != 0) {
             hp = true;
+            n_light = min(ldcg_u32(&ctl->band_count), a.n);
+            n_heavy = min(ldcg_u32(&ctl->band_hcount), a.heavy_cap);
             const unsigned long long listed_hs =
                 ldcg_u64(reinterpret_cast<const uint64_t *>(&ctl->band_hsum));
             const unsigned long long rest = pull_bound > listed_hs ? pull_bound - listed_hs : 0ull;
             const uint32_t sweep =
-                listed ? min(ldcg_u32(&ctl->far_count[phase & 1]), a.n) : a.n;
+                listed ? min(far_now, a.n) : a.n;
             pull = a.pull == 2 || (a.pull == 1 && listed_hs > rest + sweep / 8);
             continue;
         }
@@ -1141,16 +1249,16 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         // With the far scan there is no pile: every label at or above the
         // threshold came from a proposal (or a split) that lowered far_min,
         // so an infinite far_min means no vertex is left unsettled.
-        uint32_t nf = min(ldcg_u32(&ctl->far_count[fc]), a.n);
-        uint32_t fmin = ldcg_u32(&ctl->far_min[fc]);
-        if (a.far_scan ? fmin == INF32 : nf == 0) {           // converged
+        const uint32_t nf = min(far_now, a.n), fmin = fmin_now;
+        if (SCAN ? fmin == INF32 : nf == 0) {           // converged
             if (first) ctl->exit_reason = 1;
             break;
         }
-        uint64_t T_old = T;
+        T_old = T;
         T = (fmin != INF32 && (uint64_t)fmin > T ? (uint64_t)fmin : T) + a.delta;
         ++phase;
-        const uint32_t *fs = fc ? a.far1 : a.far0;
+        const uint32_t *pile = fc ? a.far1 : a.far0;
+        const uint32_t fsn = phase % 3;        // the new phase's far counters
         const uint32_t its = it + 1;
         if (first) {
             ctl->near_count[(its + 1) % 3] = 0;
@@ -1159,39 +1267,40 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
             ctl->band_count = 0;
             ctl->band_hcount = 0;
             ctl->band_hsum = 0;
+            ctl->far_count[(phase + 1) % 3] = 0;   // last read a phase ago
+            ctl->far_min[(phase + 1) % 3] = INF32;
         }
-        stage_reset(st);
-        PushTargets u;
-        u.qn = (its & 1) ? a.q1 : a.q0;
-        u.qn_count = &ctl->near_count[its % 3];
-        u.hqn = (its & 1) ? a.hq1 : a.hq0;
-        u.hqn_count = &ctl->heavy_count[its % 3];
-        u.farq = fc ? a.far0 : a.far1;
-        u.far_count = &ctl->far_count[fc ^ 1];
-        u.far_min = &ctl->far_min[fc ^ 1];
-        // With the far scan the split rebuilds the pile as the candidate
-        // list: every vertex at or above T_old (the new band's frontier and
-        // all later ones; unreached vertices with arcs too), staged in the
-        // band regions, which no band listing uses during a split.
-        u.bandq = a.far_scan ? (fc ? a.far0 : a.far1) : a.band_q;
-        u.band_count = a.far_scan ? &ctl->far_count[fc ^ 1] : &ctl->band_count;
-        u.tag_next = a.base_near + its;
-        u.tag_far = a.base_far + phase;
-        u.T = T;
-        u.flush = true;
         // the first split sweeps every id, and sets whole bitmap words;
         // a split over the list sets bits, and only for a list long enough
         // that the next iteration's sweep of the bitmap pays
-        const bool from_list = a.far_scan && listed;
+        const bool from_list = SCAN && listed;
         const bool dense_out = a.dense && (!from_list || nf >= a.n / 64);
-        u.dense = dense_out;
-        u.nbm = (its & 1) ? a.nbm1 : a.nbm0;
-        u.nostamp = false;             // the split visits each vertex once
-        u.nostamp_stamp = a.stamp_near;
-        u.hsum = nullptr;
-        u.lend = tail ? nullptr : a.lend;
+        if (threadIdx.x == 0) {
+            t.qn = (its & 1) ? a.q1 : a.q0;
+            t.qn_count = &ctl->near_count[its % 3];
+            t.hqn = (its & 1) ? a.hq1 : a.hq0;
+            t.hqn_count = &ctl->heavy_count[its % 3];
+            t.farq = fc ? a.far0 : a.far1;
+            t.far_count = &ctl->far_count[fsn];
+            t.far_min = &ctl->far_min[fsn];
+            // With the far scan the split rebuilds the pile as the candidate
+            // list: every vertex at or above T_old (the new band's frontier
+            // and all later ones; unreached vertices with arcs too), staged
+            // in the band regions, which no band listing uses during a
+            // split.
+            t.bandq = SCAN ? t.farq : a.band_q;
+            t.band_count = SCAN ? t.far_count : &ctl->band_count;
+            t.tag_next = a.base_near + its;
+            t.tag_far = a.base_far + phase;
+            t.dense = dense_out;
+            t.nbm = (its & 1) ? a.nbm1 : a.nbm0;
+            t.nostamp = false;             // the split visits each vertex once
+            t.hsum = nullptr;
+            t.lend = a.lend;
+        }
+        stage_reset(st);
         // the far pile (or list), or with the far scan first every vertex
-        const uint32_t n_split = (a.far_scan && !from_list) ? a.n : nf;
+        const uint32_t n_split = (SCAN && !from_list) ? a.n : nf;
         // SPLIT_ILP chunks of 32 per warp step, their loads issued together.
         // A vertex is met once here (the pile holds it once, the scan visits
         // each id once) and nothing relaxes during the split, so its near
@@ -1206,7 +1315,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
                 in[c] = i < n_split;
                 v[c] = 0;
                 d[c] = INF32;
-                if (in[c]) v[c] = (a.far_scan && !from_list) ? i : ldcg_u32(&fs[i]);
+                if (in[c]) v[c] = (SCAN && !from_list) ? i : ldcg_u32(&pile[i]);
             }
 #pragma unroll
             for (int c = 0; c < SPLIT_ILP; ++c)
@@ -1220,11 +1329,11 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
                 // dense: ids at or above n_big are light without a look at the row
                 if (to_near[c] && (!a.dense || v[c] < a.n_big)) {
                     const uint32_t r0 = a.row_ptr[v[c]];
-                    const uint32_t r1 = u.lend ? u.lend[v[c]] : a.row_ptr[v[c] + 1];
-                    a.stamp_near[v[c]] = u.tag_next;
+                    const uint32_t r1 = t.lend ? t.lend[v[c]] : a.row_ptr[v[c] + 1];
+                    a.stamp_near[v[c]] = t.tag_next;
                     deg[c] = r1 - r0;
                 }
-                if (a.far_scan) {
+                if (SCAN) {
                     // the list keeps to_near and cand vertices, and unreached
                     // ones with arcs (isolated vertices are never reached)
                     keep[c] = to_near[c] || cand[c];
@@ -1232,9 +1341,10 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
                         keep[c] = from_list || a.row_ptr[v[c] + 1] != a.row_ptr[v[c]];
                 } else {
                     keep[c] = cand[c] &&
-                              atomicExch(&a.stamp_far[v[c]], u.tag_far) != u.tag_far;
+                              atomicExch(&a.stamp_far[v[c]], t.tag_far) != t.tag_far;
                 }
             }
+            bool push[SPLIT_ILP];
 #pragma unroll
             for (int c = 0; c < SPLIT_ILP; ++c) {
                 // dense: light vertices as bits; from the id sweep a chunk is
@@ -1242,33 +1352,34 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
                 const bool bit = dense_out && to_near[c] && deg[c] < HEAVY_DEG;
                 const uint32_t word = __ballot_sync(FULL, bit);
                 if (from_list) {
-                    if (bit) atomicOr(&u.nbm[v[c] >> 5], 1u << (v[c] & 31));
+                    if (bit) atomicOr(&t.nbm[v[c] >> 5], 1u << (v[c] & 31));
                 } else if (lane == 0 && word) {
-                    u.nbm[(b + 32u * c) >> 5] = word;
+                    t.nbm[(b + 32u * c) >> 5] = word;
                 }
                 if (lane == 0 && word) st.dn_near[threadIdx.x >> 5] += (uint32_t)__popc(word);
-                push_near(a, st, u, to_near[c] && !bit, v[c], deg[c]);
-                if (a.far_scan) {
+                push[c] = to_near[c] && !bit;
+                if (SCAN) {
                     const uint32_t w = threadIdx.x >> 5;
                     region_append(keep[c], v[c], st.band_buf + w * BAND_REGION, &st.band_n[w],
-                                  BAND_REGION, true, u.bandq, u.band_count, a.n, &ctl->err);
+                                  BAND_REGION, true, t.bandq, t.band_count, a.n, &ctl->err);
                 }
-                push_far(a, st, u, keep[c] && !a.far_scan, cand[c], v[c], (uint32_t)d[c]);
             }
+            push_far<SCAN, SPLIT_ILP>(a, st, t, keep, cand, v, [&](int c) { return (uint32_t)d[c]; });
+            push_near<SPLIT_ILP>(a, st, t, true, push, v, deg);
         }
-        flush_stage(st, u, a.n, &ctl->err);
+        flush_stage(st, t, a.n, &ctl->err);
         if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) {
             if (first) ctl->exit_reason = 4;
             break;
         }
+        n_light = min(ldcg_u32(&ctl->near_count[its % 3]), a.n);
+        n_heavy = min(ldcg_u32(&ctl->heavy_count[its % 3]), a.heavy_cap);
         if (first) {
-            ctl->far_count[fc] = 0;
-            ctl->far_min[fc] = INF32;
             ctl->pull_hsum = 0;      // read after the pass's barrier, before this one
         }
         it = its;
         cur_dense = dense_out;        // the split set the next frontier's bits
-        listed = a.far_scan != 0;
+        listed = SCAN;
         if (it >= a.max_iters) {
             if (first) {
                 atomicOr(&ctl->err, ERR_TIMEOUT);
@@ -1278,14 +1389,15 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(SsspArgs a) {
         }
     }
     // counters
+    unsigned long long sum_a = attempts, sum_i = improved;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) {
-        attempts += __shfl_xor_sync(FULL, attempts, o);
-        improved += __shfl_xor_sync(FULL, improved, o);
+        sum_a += __shfl_xor_sync(FULL, sum_a, o);
+        sum_i += __shfl_xor_sync(FULL, sum_i, o);
     }
     if (lane == 0) {
-        atomicAdd(&ctl->relax_attempts, attempts);
-        atomicAdd(&ctl->relax_improved, improved);
+        atomicAdd(&ctl->relax_attempts, sum_a);
+        atomicAdd(&ctl->relax_improved, sum_i);
     }
     if (NARROW && __any_sync(FULL, narrow_miss) && lane == 0) atomicOr(&ctl->err, ERR_NARROW);
     if (first) {
@@ -1351,15 +1463,18 @@ cudaError_t launch_init(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t d
     return cudaGetLastError();
 }
 
-// Co-resident blocks per SM that both label widths of the kernel reach.
+// Co-resident blocks per SM that every form of the kernel reaches.
 int sssp_occupancy(int threads) {
-    int nw = 0, nn = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nw, sssp_kernel<false>, threads, 0) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nn, sssp_kernel<true>, threads, 0) !=
-            cudaSuccess)
-        return 0;
-    return nw < nn ? nw : nn;
+    const void *forms[] = {(const void *)sssp_kernel<false, false>, (const void *)sssp_kernel<false, true>,
+                           (const void *)sssp_kernel<true, false>, (const void *)sssp_kernel<true, true>};
+    int least = 0;
+    for (const void *fn : forms) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, 0) != cudaSuccess) return 0;
+        least = least ? (n < least ? n : least) : n;
+        if (least < 1) return 0;
+    }
+    return least;
 }
 
 cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
@@ -1372,6 +1487,8 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.label32 = ws.label32;
     a.lshift = ws.lshift;
     a.ldmax = (uint32_t)((1ull << (32 - ws.lshift)) - 2);
+    a.lstep = 1u << ws.lshift;
+    a.lmiss = ((uint64_t)a.ldmax + 1) << ws.lshift;
     a.stamp_near = ws.stamp_near;
     a.stamp_far = ws.stamp_far;
     a.q0 = ws.q[0];
@@ -1392,12 +1509,25 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.band_hq = ws.band_hq;
     a.base_band = p.base_band;
     a.defer = p.delta <= g.max_w ? 1u : 0u;
-    a.far_scan = p.far_scan;
     a.trace = p.trace;
     a.dense = p.dense;
     a.pull = p.far_scan ? p.pull : 0u;
     a.tail = p.tail;
     a.m = g.m;
+    // Thin frontiers with the far pile (see the kernel).  Few arcs per vertex
+    // mean a high diameter (grids, paths, trees): below eight vertices per
+    // warp a frontier there also takes 16 warp-local rounds, so that a
+    // barrier is paid every 16 hops (grid 1021 x 733, k = 37: 2.4 ms; split
+    // early without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.64
+    // against 1.21).  On denser graphs a warp's own rounds would relax hub
+    // rows alone (R-MAT 12: 0.93 ms against 0.20); there a frontier below
+    // one vertex per warp only splits early (0.29 against 0.31 ms).  With
+    // local rounds asked for the frontier is rarely latency-bound, and the
+    // early split only unsettles it (grid 4096 x 4096: 9.7 against 9.25 ms).
+    const uint32_t warps = (uint32_t)(geo.sssp_blocks * (geo.threads / 32));
+    const bool sparse_rows = g.m <= 8ull * g.n;
+    a.thin = p.local_rounds ? 1u : sparse_rows ? 8 * warps : warps;
+    a.thin_rounds = sparse_rows ? 16u : 0u;
     a.n_big = g.n_big;
     a.n_words = (g.n + 31) / 32;
     a.nbm0 = ws.nbm[0];
@@ -1410,7 +1540,10 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.lend = active_lend(g, p.delta);
     if (a.lend) a.adj = g.adj_w;        // rows partitioned by weight class
     void *args[] = {&a};
-    const void *fn = ws.narrow ? (const void *)sssp_kernel<true> : (const void *)sssp_kernel<false>;
+    const void *fn = ws.narrow ? (p.far_scan ? (const void *)sssp_kernel<true, true>
+                                             : (const void *)sssp_kernel<true, false>)
+                               : (p.far_scan ? (const void *)sssp_kernel<false, true>
+                                             : (const void *)sssp_kernel<false, false>);
     return cudaLaunchCooperativeKernel(fn, dim3(geo.sssp_blocks), dim3(geo.threads), args, 0, s);
 }
 

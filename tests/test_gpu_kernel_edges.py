@@ -80,3 +80,35 @@ def test_noalloc_rows_and_rounds(name, g):
         np.testing.assert_array_equal(out[0].cpu().numpy(), ref.cell)
         np.testing.assert_array_equal(out[1].cpu().numpy().view(np.uint32), ref.dist)
         np.testing.assert_array_equal(out[2].cpu().numpy(), ref.pred)
+
+
+def _sparse_graphs():
+    yield "grid", wl.grid(150, 111, 1000, seed=21), 30
+    yield "grid_unit", wl.grid(64, 65, 1, seed=22), 9
+    yield "path", G.path(3000, 1, 50, 23), 4
+    yield "tree", G.random_tree(4000, 1, 100, 24), 20
+    yield "connected", G.random_connected(3000, 6000, 1, 50, 25), 15
+    yield "rmat", wl.rmat(11, 16, wmax=60, seed=26), 11      # not sparse: split only
+
+
+SPARSE = list(_sparse_graphs())
+
+
+@pytest.mark.parametrize("label_bits", [32, 64])
+@pytest.mark.parametrize("delta", [3, 61, 1001, 20000])
+@pytest.mark.parametrize("name,g,k", SPARSE, ids=[c[0] for c in SPARSE])
+def test_thin_frontiers_split_early_and_take_rounds(name, g, k, delta, label_bits):
+    """The far pile is split while the frontier is thin, and on sparse graphs
+    a thin frontier takes warp-local rounds: band widths from one hop to the
+    whole graph (with the pile forced below the largest weight too)."""
+    seeds = G.seeds_from(np.arange(g.n), k, 5)
+    _check(g, seeds, [("delta", delta), ("label_bits", label_bits), ("far_scan", 0)])
+
+
+@pytest.mark.parametrize("n", [256, 257, 513, 640, 1026, 2050])
+def test_hub_chunk_pieces(n):
+    """A few hub chunks are relaxed in pieces: stars whose hub row ends at,
+    before and after a piece, with whole rows and with the light/heavy split."""
+    g = G.star(n, 1, 40, n)
+    for delta in (7, 1000):
+        _check(g, G.seeds_from(np.arange(1, n), 5, n), [("delta", delta)])
