@@ -17,17 +17,28 @@
 //
 // Load balance: vertices with degree < HEAVY_DEG are processed 32 per warp
 // with their arcs flattened over the lanes (labels of 32 consecutive
-// vertices are one coalesced load); higher-degree rows are split into
-// CHUNK-arc pieces listed once at graph load.
+// vertices are one coalesced load), in the vertex ranges of about equal
+// arcs that the dense frontiers use; higher-degree rows are split into
+// CHUNK-arc pieces listed once at graph load (smaller ones while they are
+// too few for the grid).  With 32 consecutive rows to a warp the first
+// batches after the hubs held up to 32 x 255 arcs, read 32 at a time: pairs
+// and predecessors of R-MAT 16 took 0.19 ms, 0.034 in ranges; R-MAT of 10^6
+// vertices 0.26 against 0.14; R-MAT 26 (degree 8) 5.9 against 5.6.
 #include "internal.h"
 
 namespace stn {
+
+// Pieces of a hub chunk while chunks are few: 128 arcs, four steps.
+constexpr uint32_t SCAN_SUBS = 4;
 
 struct ScanArgs {
     const uint32_t *__restrict__ row_ptr;
     const uint2 *__restrict__ adj;
     const uint64_t *__restrict__ heavy_chunks;
     uint32_t n_heavy_chunks;
+    uint32_t subs;                   // pieces a chunk is cut into (1 or SCAN_SUBS)
+    const uint32_t *__restrict__ items;   // vertex ranges [items[i], items[i + 1])
+    uint32_t n_items;
     uint32_t n;
     const uint64_t *label;
     const uint32_t *label32;         // narrow labels (the narrow kernel)
@@ -86,16 +97,16 @@ __global__ void __launch_bounds__(256) scan_kernel(ScanArgs a) {
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t n_batches = (a.n + 31) / 32;
-    const uint32_t n_work = a.n_heavy_chunks + n_batches;
+    const uint32_t n_hub = a.n_heavy_chunks * a.subs;
+    const uint32_t n_work = n_hub + a.n_items;
     bool overflow = false;
     for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
-        if (wi < a.n_heavy_chunks) {
-            uint64_t item = a.heavy_chunks[wi];
+        if (wi < n_hub) {
+            uint64_t item = a.heavy_chunks[wi / a.subs];
             uint32_t v = (uint32_t)(item >> 32), c = (uint32_t)item;
             uint32_t rs = a.row_ptr[v];
-            uint32_t s = rs + c * CHUNK;
-            uint32_t e = min(a.row_ptr[v + 1], s + CHUNK);
+            uint32_t s = rs + c * CHUNK + wi % a.subs * (CHUNK / SCAN_SUBS);
+            uint32_t e = min(a.row_ptr[v + 1], s + CHUNK / a.subs);
             uint64_t lv = scan_label<NARROW>(a, v);
             uint32_t cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, rs);
             // the next 32 arcs' records are loaded while these are scanned
@@ -106,11 +117,14 @@ __global__ void __launch_bounds__(256) scan_kernel(ScanArgs a) {
                 if (b + 32 + lane < e) en = __ldcs(&a.adj[b + 32 + lane]);
                 scan_arc<NARROW>(a, b + lane < e, v, lv, cbase, b + lane, ec, overflow);
             }
-        } else {
-            uint32_t v = (wi - a.n_heavy_chunks) * 32 + lane;
+            continue;
+        }
+        const uint32_t v1 = __ldg(&a.items[wi - n_hub + 1]);
+        for (uint32_t vb = __ldg(&a.items[wi - n_hub]); vb < v1; vb += 32) {
+            uint32_t v = vb + lane;
             uint32_t s = 0, deg = 0, cbase = 0;
             uint64_t lv = INF64;
-            if (v < a.n) {
+            if (v < v1) {
                 s = a.row_ptr[v];
                 deg = a.row_ptr[v + 1] - s;
                 if (deg >= HEAVY_DEG) deg = 0;          // covered by the chunk list
@@ -138,7 +152,7 @@ __global__ void __launch_bounds__(256) scan_kernel(ScanArgs a) {
                 if (jn < total) en = __ldcs(&a.adj[sn + (jn - xn)]);
                 const uint64_t lo = __shfl_sync(FULL, lv, owner);
                 const uint32_t co = __shfl_sync(FULL, cbase, owner);
-                const uint32_t vo = (wi - a.n_heavy_chunks) * 32 + owner;
+                const uint32_t vo = vb + owner;
                 scan_arc<NARROW>(a, valid, vo, lo, co, arc, ec, overflow);
             }
         }
@@ -268,9 +282,13 @@ cudaError_t launch_scan(const DevGraph &g, Workspace &ws, uint32_t k, bool pairs
         cudaError_t e = cudaMemsetAsync(ws.pairtab, 0xFF, slots * sizeof(uint64_t), s);
         if (e != cudaSuccess) return e;
     }
-    uint64_t work = (uint64_t)g.n_heavy_chunks + (g.n + 31) / 32;
-    uint64_t blocks = (work + 7) / 8;          // 8 warps per block
     const uint64_t cap = (uint64_t)current_sm_count() * 32;
+    // hub chunks in pieces while they leave most of the grid's warps idle
+    a.subs = g.n_heavy_chunks * (uint64_t)SCAN_SUBS <= cap * 8 ? SCAN_SUBS : 1u;
+    a.items = g.items;
+    a.n_items = g.n_items;
+    uint64_t work = (uint64_t)g.n_heavy_chunks * a.subs + g.n_items;
+    uint64_t blocks = (work + 7) / 8;          // 8 warps per block
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     if (ws.narrow) scan_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(a);

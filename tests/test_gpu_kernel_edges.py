@@ -112,3 +112,11 @@ def test_hub_chunk_pieces(n):
     g = G.star(n, 1, 40, n)
     for delta in (7, 1000):
         _check(g, G.seeds_from(np.arange(1, n), 5, n), [("delta", delta)])
+
+
+@pytest.mark.parametrize("n,degree", [(40, 3), (991, 2), (1985, 30), (3000, 300)])
+def test_scan_ranges_and_hub_pieces(n, degree):
+    """The bridge scan walks vertex ranges cut anywhere and hub rows in
+    pieces: maximal ties (unit weights), every vertex near a bridge."""
+    g = G.random_graph(n, n * degree // 2, 1, 2, n)
+    _check(g, G.seeds_from(np.arange(n), max(2, n // 8), n))
