@@ -98,7 +98,8 @@ typedef struct {
     /* device time per phase (CUDA events on the library's stream, ms):
      * init = labels and seeds, voronoi = the near/far SSSP kernel alone,
      * bridges = pred + bridge scan and pair compaction, mst = Boruvka,
-     * tree = expansion, sort and total */
+     * tree = expansion, sort and total; seed sets of up to 181 run all of
+     * the steps after the scan as one kernel, counted as tree */
     float ms_init, ms_voronoi, ms_bridges, ms_mst, ms_tree;
 } steiner_stats_t;
 

@@ -144,7 +144,8 @@ struct steiner_graph {
     uint32_t narrow_fail_dbits = 0;   // most distance bits a narrow attempt ran out of
     uint32_t last_label_bits = 0;
     uint64_t narrow_reruns = 0;
-    Control *h_ctl = nullptr;      // pinned
+    ResultBlock *h_result = nullptr;   // pinned
+    Control *h_ctl = nullptr;          // &h_result->ctl
     cudaEvent_t ev[6] = {};
     BatchEngine *batch = nullptr;
     ServeEngine *serve = nullptr;
@@ -179,7 +180,9 @@ int ensure_n_workspace(steiner_graph *G) {
     CK(dalloc(ws.hq[1], G->g.heavy_chunk_cap));
     CK(dalloc(ws.far[0], n));
     CK(dalloc(ws.far[1], n));
-    CK(dalloc(ws.ctl, 1));
+    CK(dalloc(ws.result, 1));
+    ws.ctl = &ws.result->ctl;
+    ws.small_tree = &ws.result->tree;
     uint64_t tcap = std::max<uint64_t>(n, 2);
     CK(dalloc(ws.tree_key, tcap));
     CK(dalloc(ws.tree_key2, tcap));
@@ -283,6 +286,22 @@ cudaError_t ensure_partition(steiner_graph *G, uint32_t delta) {
     return cudaSuccess;
 }
 
+// Reads the control block back (after the small tail with its edges, or, if
+// the tree outgrew them, after sorting it) and waits for it.
+int read_result(steiner_graph *G, Workspace &ws, bool small) {
+    cudaStream_t s = G->stream;
+    CK(cudaMemcpyAsync(G->h_result, ws.result, small ? sizeof(ResultBlock) : sizeof(Control),
+                       cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (small && G->h_ctl->n_tree > SMALL_TREE) {
+        CK(launch_sort_keys(ws.tree_key, ws.tree_key2, ws.tree_w, ws.tree_w2, ws.tile_off,
+                            ws.tree_cap, 2 * G->nbits, ws.ctl, s));
+        CK(cudaMemcpyAsync(G->h_ctl, ws.ctl, sizeof(Control), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+    }
+    return STEINER_OK;
+}
+
 // Runs Steps 1 (and, with `full`, 2-7) of Algorithm 2 for one sorted seed
 // list with the label width in G->ws.narrow.  Leaves the control block in
 // G->h_ctl.
@@ -305,28 +324,35 @@ int run_pipeline_once(steiner_graph *G, const std::vector<int32_t> &ss, bool ful
     SsspParams p{G->delta, G->max_iters, ws.epoch_near, ws.epoch_far, G->local_rounds,
                  ws.epoch_band, far_scan, trace ? 1u : 0u, dense, far_scan ? G->pull : 0u,
                  G->tail};
-    CK(cudaEventRecord(G->ev[0], s));
+    // phase times only where they are asked for
+    auto mark = [&](int i) { return ms ? cudaEventRecord(G->ev[i], s) : cudaSuccess; };
+    CK(mark(0));
     CK(ensure_partition(G, G->delta));
     CK(launch_init(G->g, ws, k, G->delta, s));
-    CK(cudaEventRecord(G->ev[1], s));
+    CK(mark(1));
     CK(launch_sssp(G->g, ws, G->geo, p, s));
-    CK(cudaEventRecord(G->ev[2], s));
+    CK(mark(2));
     CK(launch_scan(G->g, ws, k, full, s));
     uint32_t launches = 4;      // init labels, init seeds, SSSP, scan
-    if (full) {
+    const bool small = full && small_tail(k);
+    if (full && !small) {
         CK(launch_compact_pairs(ws, k, s));
-        CK(cudaEventRecord(G->ev[3], s));
+        CK(mark(3));
         CK(launch_mst(ws, k, G->geo, s));
-        CK(cudaEventRecord(G->ev[4], s));
+        CK(mark(4));
         CK(launch_tree(G->g, ws, k, ws.epoch_mark, G->nbits, s));
         if (k > 1) launches += 3 + 1 + 2;   // compaction, MST, expansion + sort
     } else {
-        CK(cudaEventRecord(G->ev[3], s));
-        CK(cudaEventRecord(G->ev[4], s));
+        CK(mark(3));
+        CK(mark(4));
+        if (small) {
+            CK(launch_small_tail(G->g, ws, k, ws.epoch_mark, G->nbits, s));
+            ++launches;
+        }
     }
-    CK(cudaEventRecord(G->ev[5], s));
-    CK(cudaMemcpyAsync(G->h_ctl, ws.ctl, sizeof(Control), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    CK(mark(5));
+    rc = read_result(G, ws, small);
+    if (rc) return rc;
     if (ms) {
         for (int i = 0; i < 5; ++i) cudaEventElapsedTime(&ms[i], G->ev[i], G->ev[i + 1]);
         ms[5] = (float)launches;
@@ -365,17 +391,25 @@ int run_pipeline(steiner_graph *G, const std::vector<int32_t> &ss, bool full, fl
     return rc;
 }
 
-int fetch_tree(steiner_graph *G, steiner_result_t *out) {
+int fetch_tree(steiner_graph *G, uint32_t k, steiner_result_t *out) {
     const Control &c = *G->h_ctl;
     uint32_t nt = std::min(c.n_tree, G->ws.tree_cap);
-    std::vector<uint64_t> keys(nt);
-    std::vector<uint32_t> ws(nt);
-    if (nt) {
-        CK(cudaMemcpyAsync(keys.data(), G->ws.tree_key, (size_t)nt * 8, cudaMemcpyDeviceToHost,
-                           G->stream));
-        CK(cudaMemcpyAsync(ws.data(), G->ws.tree_w, (size_t)nt * 4, cudaMemcpyDeviceToHost,
-                           G->stream));
-        CK(cudaStreamSynchronize(G->stream));
+    std::vector<uint64_t> far_keys;
+    std::vector<uint32_t> far_ws;
+    const uint64_t *keys = G->h_result->tree.key;
+    const uint32_t *ws = G->h_result->tree.w;
+    if (!small_tail(k) || nt > SMALL_TREE) {
+        far_keys.resize(nt);
+        far_ws.resize(nt);
+        keys = far_keys.data();
+        ws = far_ws.data();
+        if (nt) {
+            CK(cudaMemcpyAsync(far_keys.data(), G->ws.tree_key, (size_t)nt * 8,
+                               cudaMemcpyDeviceToHost, G->stream));
+            CK(cudaMemcpyAsync(far_ws.data(), G->ws.tree_w, (size_t)nt * 4, cudaMemcpyDeviceToHost,
+                               G->stream));
+            CK(cudaStreamSynchronize(G->stream));
+        }
     }
     out->edges = nt ? (steiner_edge_t *)malloc((size_t)nt * sizeof(steiner_edge_t)) : nullptr;
     if (nt && !out->edges) return fail(STEINER_ENOMEM, "host allocation of the result failed");
@@ -399,7 +433,7 @@ int query_locked(steiner_graph *G, const int32_t *seeds, uint32_t k, steiner_res
     int rc = sorted_seed_list(G, seeds, k, ss);
     if (rc) return out->status = rc;
     float ms[6] = {0, 0, 0, 0, 0, 0};
-    rc = run_pipeline(G, ss, true, ms);
+    rc = run_pipeline(G, ss, true, stats ? ms : nullptr);
     if (rc) return out->status = rc;
     const Control c = *G->h_ctl;
     rc = status_from(c, k, true);
@@ -430,7 +464,7 @@ int query_locked(steiner_graph *G, const int32_t *seeds, uint32_t k, steiner_res
         }
     }
     if (rc == STEINER_OK || rc == STEINER_EDISCONNECTED) {
-        int rc2 = fetch_tree(G, out);
+        int rc2 = fetch_tree(G, k, out);
         if (rc2) return out->status = rc2;
     }
     if (pairs && (rc == STEINER_OK || rc == STEINER_EDISCONNECTED)) {
@@ -522,8 +556,9 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaStreamCreate"));
     for (auto &ev : G->ev)
         if ((e = cudaEventCreate(&ev)) != cudaSuccess) return bail(cuda_fail(e, "cudaEventCreate"));
-    if ((e = cudaMallocHost((void **)&G->h_ctl, sizeof(Control))) != cudaSuccess)
+    if ((e = cudaMallocHost((void **)&G->h_result, sizeof(ResultBlock))) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMallocHost"));
+    G->h_ctl = &G->h_result->ctl;
     // Internal vertex order: on a skewed degree distribution, descending
     // degree (ties by caller id), so the hubs' labels, which most arcs
     // point to, share L2 sectors.  STEINER_RELABEL=0/1 forces it off/on.
@@ -683,7 +718,7 @@ void steiner_free_graph(steiner_graph_t G) {
     Workspace &ws = G->ws;
     void *bufs[] = {ws.label, ws.label32, ws.nbm[0], ws.nbm[1], ws.bbm, ws.pred_arc, ws.stamp_near, ws.stamp_far, ws.stamp_band, ws.band_q,
                     ws.band_hq, ws.mark, ws.q[0], ws.q[1],
-                    ws.hq[0], ws.hq[1], ws.far[0], ws.far[1], ws.ctl, ws.seeds, ws.pairtab,
+                    ws.hq[0], ws.hq[1], ws.far[0], ws.far[1], ws.result, ws.seeds, ws.pairtab,
                     ws.e_key, ws.e_ra, ws.e_rb, ws.e_arc, ws.e_mst, ws.tile_off, ws.comp, ws.hook,
                     ws.best, ws.tree_key, ws.tree_key2, ws.tree_w, ws.tree_w2, G->g.row_ptr,
                     G->g.adj, G->g.heavy_chunks, G->g.orig_row_ptr, G->g.orig_of, G->g.new_of,
@@ -692,7 +727,7 @@ void steiner_free_graph(steiner_graph_t G) {
         if (p) cudaFree(p);
     for (auto &ev : G->ev)
         if (ev) cudaEventDestroy(ev);
-    if (G->h_ctl) cudaFreeHost(G->h_ctl);
+    if (G->h_result) cudaFreeHost(G->h_result);
     if (G->stream) cudaStreamDestroy(G->stream);
     delete G;
 }
@@ -847,11 +882,15 @@ int api_run_tail(steiner_graph *G, uint64_t *pairtab, uint32_t *pred_base, uint3
     v.pred_stride = pred_stride;
     cudaStream_t s = G->stream;
     CK(cudaMemsetAsync(v.ctl, 0, sizeof(Control), s));
-    CK(launch_compact_pairs(v, k, s));
-    CK(launch_mst(v, k, G->geo, s));
-    CK(launch_tree(G->g, v, k, G->ws.epoch_mark, G->nbits, s));
-    CK(cudaMemcpyAsync(G->h_ctl, v.ctl, sizeof(Control), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    if (small_tail(k)) {
+        CK(launch_small_tail(G->g, v, k, G->ws.epoch_mark, G->nbits, s));
+    } else {
+        CK(launch_compact_pairs(v, k, s));
+        CK(launch_mst(v, k, G->geo, s));
+        CK(launch_tree(G->g, v, k, G->ws.epoch_mark, G->nbits, s));
+    }
+    rc = read_result(G, v, small_tail(k));
+    if (rc) return out->status = rc;
     G->ws.epoch_mark += 1;
     if (G->ws.epoch_mark > 0x7FFFFFFFu) {
         CK(cudaMemsetAsync(G->ws.mark, 0, (size_t)G->ws.n * 4, s));
@@ -860,7 +899,7 @@ int api_run_tail(steiner_graph *G, uint64_t *pairtab, uint32_t *pred_base, uint3
     const Control c = *G->h_ctl;
     rc = status_from(c, k, true);
     if (rc == STEINER_OK || rc == STEINER_EDISCONNECTED) {
-        int rc2 = fetch_tree(G, out);
+        int rc2 = fetch_tree(G, k, out);
         if (rc2) return out->status = rc2;
     }
     return out->status = rc;

@@ -125,6 +125,25 @@ struct Control {
     unsigned long long end_ns;                // end of the last iteration
 };
 
+// Seed sets whose pair table has at most SMALL_TAIL_SLOTS entries (181 seeds)
+// run compaction, MST, expansion and sort as one kernel of one block; a tree
+// of up to SMALL_TREE edges is returned beside the control block (a larger
+// one goes through the radix sort).
+constexpr uint32_t SMALL_TAIL_SLOTS = 16384;
+constexpr uint32_t SMALL_TREE = 2048;
+struct SmallTree {
+    uint64_t key[SMALL_TREE];
+    uint32_t w[SMALL_TREE];
+};
+// The control block and the small tree, read back in one copy.
+struct ResultBlock {
+    Control ctl;
+    SmallTree tree;
+};
+inline bool small_tail(uint32_t k) {
+    return k > 1 && (uint64_t)k * (k - 1) / 2 <= SMALL_TAIL_SLOTS;
+}
+
 // Per-query device workspace for the single-query path.
 struct Workspace {
     uint32_t n = 0;
@@ -149,7 +168,9 @@ struct Workspace {
     uint32_t *q[2] = {nullptr, nullptr};      // light frontier
     uint64_t *hq[2] = {nullptr, nullptr};     // heavy-chunk frontier
     uint32_t *far[2] = {nullptr, nullptr};
-    Control *ctl = nullptr;
+    ResultBlock *result = nullptr;
+    Control *ctl = nullptr;         // &result->ctl
+    SmallTree *small_tree = nullptr;   // &result->tree
     int32_t *seeds = nullptr;       // sorted seed ids (rank order)
     uint32_t seeds_cap = 0;
     uint64_t *pairtab = nullptr;    // k (k - 1) / 2 packed (b << 32 | arc)
@@ -218,6 +239,8 @@ cudaError_t launch_compact_pairs(Workspace &ws, uint32_t k, cudaStream_t s);
 cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, cudaStream_t s);
 cudaError_t launch_tree(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t tag,
                         uint32_t n_bits, cudaStream_t s);
+cudaError_t launch_small_tail(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t tag,
+                              uint32_t n_bits, cudaStream_t s);
 int mst_occupancy(int threads);
 cudaError_t launch_sort_keys(uint64_t *key0, uint64_t *key1, uint32_t *w0, uint32_t *w1,
                              uint32_t *blk_hist, uint32_t cap, uint32_t key_bits, Control *ctl,

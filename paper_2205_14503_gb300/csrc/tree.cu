@@ -299,6 +299,230 @@ __global__ void __launch_bounds__(RS_THREADS) radix_sort_kernel(SortArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// the whole tail for a small seed set: one block
+// ---------------------------------------------------------------------------
+//
+// Compaction, Boruvka, expansion, sort and total are a handful of short
+// dependent steps: as separate launches (six kernels, two of them
+// cooperative, and two clears) they took 0.09 ms on R-MAT 12, k = 12,
+// nearly all of it launch gaps and grid barriers; one block of 1024 threads
+// takes the steps with block barriers.  The bound on the pair table keeps a
+// thread's share of it to ST_PER_THREAD entries.
+
+constexpr uint32_t ST_THREADS = 1024;
+constexpr uint32_t ST_PER_THREAD = 16;
+static_assert(SMALL_TAIL_SLOTS == ST_THREADS * ST_PER_THREAD, "one pass over the pair table");
+constexpr uint32_t ST_MAX_K = 182;       // 181 * 182 / 2 > SMALL_TAIL_SLOTS
+
+struct SmallTailArgs {
+    const uint64_t *pairtab;
+    uint32_t slots, k;
+    uint64_t *e_key;
+    uint32_t *e_ra, *e_rb, *e_arc, *e_mst;
+    const uint32_t *__restrict__ row_ptr;
+    const uint2 *__restrict__ adj;
+    const uint32_t *__restrict__ orig_of, *__restrict__ new_of, *__restrict__ orig_row_ptr;
+    uint32_t n;
+    const uint32_t *pred_arc;
+    uint32_t pred_stride;
+    uint32_t *mark;
+    uint32_t tag, nbits;
+    uint64_t *key;
+    uint32_t *w;
+    uint32_t cap;
+    Control *ctl;
+    SmallTree *out;
+};
+
+// Inclusive scan over the block (wsum: one entry per warp); returns the
+// thread's prefix, the block's total in `total`.
+__device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t *wsum, uint32_t &total) {
+    const uint32_t w = threadIdx.x >> 5;
+    const uint32_t incl = warp_inclusive_scan(x);
+    if (lane_id() == 31) wsum[w] = incl;
+    __syncthreads();
+    if (w == 0) wsum[lane_id()] = warp_inclusive_scan(wsum[lane_id()]);
+    __syncthreads();
+    total = wsum[31];
+    return incl + (w ? wsum[w - 1] : 0);
+}
+
+__global__ void __launch_bounds__(ST_THREADS) small_tail_kernel(SmallTailArgs a) {
+    __shared__ uint32_t wsum[32];
+    __shared__ uint32_t comp[ST_MAX_K], hook[ST_MAX_K];
+    __shared__ unsigned long long best[ST_MAX_K];
+    __shared__ uint32_t mst_arc[ST_MAX_K];
+    __shared__ uint32_t n_mst, n_tree;
+    __shared__ unsigned long long sk[SMALL_TREE];
+    __shared__ uint32_t sw[SMALL_TREE];
+    __shared__ unsigned long long total_s;
+    const uint32_t tid = threadIdx.x;
+    if (tid == 0) {
+        n_mst = n_tree = 0;
+        total_s = 0;
+    }
+
+    // ordered compaction of the pair table
+    uint32_t E = 0;
+    {
+        const uint32_t base = tid * ST_PER_THREAD;
+        uint32_t c = 0;
+#pragma unroll 4
+        for (uint32_t i = 0; i < ST_PER_THREAD; ++i)
+            c += base + i < a.slots && a.pairtab[base + i] != INF64;
+        uint32_t out = block_scan(c, wsum, E) - c;
+        for (uint32_t i = 0; c && i < ST_PER_THREAD; ++i) {
+            if (base + i >= a.slots) break;
+            const uint64_t x = a.pairtab[base + i];
+            if (x == INF64) continue;
+            uint32_t ra, rb;
+            slot_to_pair(base + i, a.k, ra, rb);
+            a.e_key[out] = (x & 0xFFFFFFFF00000000ull) | (base + i);
+            a.e_ra[out] = ra;
+            a.e_rb[out] = rb;
+            a.e_arc[out] = (uint32_t)x;
+            a.e_mst[out] = 0;
+            ++out;
+        }
+    }
+    for (uint32_t r = tid; r < a.k; r += ST_THREADS) comp[r] = r;
+
+    // Boruvka: at least half of the components that still have an edge
+    // merge per round
+    for (uint32_t round = 0; round < 32; ++round) {
+        __syncthreads();
+        for (uint32_t c = tid; c < a.k; c += ST_THREADS) {
+            best[c] = INF64;
+            hook[c] = c;
+        }
+        __syncthreads();
+        bool any = false;
+        for (uint32_t j = tid; j < E; j += ST_THREADS) {
+            const uint32_t ca = comp[a.e_ra[j]], cb = comp[a.e_rb[j]];
+            if (ca == cb) continue;
+            const unsigned long long key = a.e_key[j];
+            if (key < *(volatile unsigned long long *)&best[ca]) atomicMin(&best[ca], key);
+            if (key < *(volatile unsigned long long *)&best[cb]) atomicMin(&best[cb], key);
+            any = true;
+        }
+        if (!__syncthreads_or(any)) break;
+        for (uint32_t j = tid; j < E; j += ST_THREADS) {
+            const uint32_t ca = comp[a.e_ra[j]], cb = comp[a.e_rb[j]];
+            if (ca == cb) continue;
+            const unsigned long long key = a.e_key[j];
+            const bool xa = best[ca] == key, xb = best[cb] == key;
+            if (xa) hook[ca] = cb;
+            if (xb) hook[cb] = ca;
+            if (xa || xb) {
+                a.e_mst[j] = 1;
+                mst_arc[atomicAdd(&n_mst, 1u)] = a.e_arc[j];     // at most k - 1 in all
+            }
+        }
+        __syncthreads();
+        // two components that chose each other: the smaller id becomes root
+        bool root = false;
+        if (tid < a.k) root = hook[tid] != tid && hook[hook[tid]] == tid && tid < hook[tid];
+        __syncthreads();
+        if (root) hook[tid] = tid;
+        __syncthreads();
+        uint32_t c = 0;
+        if (tid < a.k) {
+            c = comp[tid];
+            for (uint32_t steps = 0; steps < a.k && hook[c] != c; ++steps) c = hook[c];
+        }
+        __syncthreads();
+        if (tid < a.k) comp[tid] = c;
+    }
+    __syncthreads();
+
+    // expansion: two walkers per MST pair (see expand_kernel)
+    auto emit = [&](uint32_t x, uint32_t y, uint32_t wt) {
+        const uint32_t slot = atomicAdd(&n_tree, 1u);
+        if (slot >= a.cap) {
+            atomicOr(&a.ctl->err, ERR_CAPACITY);
+            return;
+        }
+        x = caller_id(a.orig_of, x);
+        y = caller_id(a.orig_of, y);
+        const uint64_t key = ((uint64_t)min(x, y) << a.nbits) | max(x, y);
+        a.key[slot] = key;
+        a.w[slot] = wt;
+        if (slot < SMALL_TREE) {
+            sk[slot] = key;
+            sw[slot] = wt;
+        }
+    };
+    for (uint32_t t = tid; t < 2 * n_mst; t += ST_THREADS) {
+        const uint32_t carc = mst_arc[t >> 1];
+        uint32_t tail, arc;
+        if (a.orig_of) {
+            const uint32_t ct = arc_owner(a.orig_row_ptr, a.n, carc);
+            tail = a.new_of[ct];
+            arc = a.row_ptr[tail] + (carc - a.orig_row_ptr[ct]);
+        } else {
+            tail = arc_owner(a.row_ptr, a.n, carc);
+            arc = carc;
+        }
+        const uint2 e = a.adj[arc];
+        uint32_t x = e.x;
+        if ((t & 1) == 0) {
+            x = tail;
+            emit(x, e.x, e.y);
+        }
+        for (uint32_t steps = 0; steps < a.n; ++steps) {
+            const uint32_t pa = a.pred_arc[(uint64_t)x * a.pred_stride];
+            if (pa == SEED_ARC || pa == INF32) break;
+            const uint32_t old = atomicExch(&a.mark[x], a.tag);
+            const uint2 pe = a.adj[pa];              // independent of the exchange's result
+            if (old == a.tag) break;                 // the rest of the chain is another walker's
+            emit(x, pe.x, pe.y);
+            x = pe.x;
+        }
+    }
+    __syncthreads();
+    const uint32_t N = min(n_tree, a.cap);
+    if (tid == 0) {
+        a.ctl->n_pairs = E;
+        a.ctl->n_mst = n_mst;
+        a.ctl->n_tree = n_tree;
+    }
+    if (N > SMALL_TREE) return;          // the host launches the radix sort
+
+    // bitonic sort by key (keys are distinct), padded to a power of two
+    uint32_t P = 2;
+    while (P < N) P *= 2;
+    for (uint32_t i = N + tid; i < P; i += ST_THREADS) {
+        sk[i] = INF64;
+        sw[i] = 0;
+    }
+    unsigned long long tot = 0;
+    for (uint32_t i = tid; i < N; i += ST_THREADS) tot += sw[i];
+    if (tot) atomicAdd(&total_s, tot);
+    for (uint32_t size = 2; size <= P; size *= 2)
+        for (uint32_t d = size / 2; d >= 1; d /= 2) {
+            __syncthreads();
+            for (uint32_t i = tid; i < P / 2; i += ST_THREADS) {
+                const uint32_t lo = 2 * d * (i / d) + i % d, hi = lo + d;
+                const bool up = (lo & size) == 0;
+                if ((sk[lo] > sk[hi]) == up) {
+                    const unsigned long long x = sk[lo];
+                    sk[lo] = sk[hi];
+                    sk[hi] = x;
+                    const uint32_t y = sw[lo];
+                    sw[lo] = sw[hi];
+                    sw[hi] = y;
+                }
+            }
+        }
+    __syncthreads();
+    for (uint32_t i = tid; i < N; i += ST_THREADS) {
+        a.out->key[i] = sk[i];
+        a.out->w[i] = sw[i];
+    }
+    if (tid == 0) a.ctl->total = total_s;
+}
+
+// ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
 
@@ -307,6 +531,37 @@ int mst_occupancy(int threads) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, mst_kernel, threads, 0) != cudaSuccess)
         return 0;
     return nb;
+}
+
+cudaError_t launch_small_tail(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t tag,
+                              uint32_t n_bits, cudaStream_t s) {
+    SmallTailArgs a;
+    a.pairtab = ws.pairtab;
+    a.slots = k * (k - 1) / 2;
+    a.k = k;
+    a.e_key = ws.e_key;
+    a.e_ra = ws.e_ra;
+    a.e_rb = ws.e_rb;
+    a.e_arc = ws.e_arc;
+    a.e_mst = ws.e_mst;
+    a.row_ptr = g.row_ptr;
+    a.adj = g.adj;
+    a.orig_of = g.orig_of;
+    a.new_of = g.new_of;
+    a.orig_row_ptr = g.orig_row_ptr;
+    a.n = g.n;
+    a.pred_arc = ws.pred_arc;
+    a.pred_stride = ws.pred_stride;
+    a.mark = ws.mark;
+    a.tag = tag;
+    a.nbits = n_bits;
+    a.key = ws.tree_key;
+    a.w = ws.tree_w;
+    a.cap = ws.tree_cap;
+    a.ctl = ws.ctl;
+    a.out = ws.small_tree;
+    small_tail_kernel<<<1, ST_THREADS, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 static int sort_blocks_cache = -1;

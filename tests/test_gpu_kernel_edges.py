@@ -120,3 +120,14 @@ def test_scan_ranges_and_hub_pieces(n, degree):
     pieces: maximal ties (unit weights), every vertex near a bridge."""
     g = G.random_graph(n, n * degree // 2, 1, 2, n)
     _check(g, G.seeds_from(np.arange(n), max(2, n // 8), n))
+
+
+@pytest.mark.parametrize("k", [2, 3, 32, 33, 180, 181, 182])
+def test_small_seed_set_tail(k):
+    """Up to 181 seeds the steps after the scan run in one block: seed counts
+    around its limit, with ties, and trees beside it that outgrow its sort
+    (a long path) or fall apart (a forest)."""
+    g = wl.rmat(11, 8, wmax=2, seed=41)
+    _check(g, wl.sample_distinct(wl.largest_cc(g), k, k))
+    for g in (G.path(5000, 1, 9, 42), G.path(2049, 1, 9, 43), G.random_graph(700, 500, 1, 9, 44)):
+        _check(g, np.unique(np.concatenate([[0, g.n - 1], G.seeds_from(np.arange(g.n), k - 2, k)])))
