@@ -21,16 +21,19 @@
 //    a per-vertex mask records which slots relaxed the vertex in their
 //    current band (vertices with any bit set are kept in a band list), and
 //    when a slot's near work drains its heavy arcs are relaxed once, in the
-//    next shared iteration, for the listed vertices with its bit.
+//    next shared iteration, for the listed vertices with its bit;
+//  * a slot whose first heavy-arc pass ran in the pull form finishes as one
+//    unbounded band over whole rows (its tail), as in the single-query
+//    kernel.
 #include "multi.h"
 
 namespace stn {
 
-// (arc, slot) pairs in flight per lane.  Two, at six 256-thread blocks per
-// SM (40 registers), beat four at four blocks (64 registers): the kernel is
-// bound by the latency of each item's chain of L2 round trips, so more
-// resident warps pay more than more pairs per warp.
+// (arc, slot) pairs in flight per lane, and blocks per SM: R-MAT 22, 64 queries
+// 51 ms at two and six, 55 at four and four to six.
 constexpr int MQ_ILP = 2;
+constexpr int MQ_BLOCKS = 6;
+constexpr uint32_t MQ_HOLD = 16;   // iterations a drained first band waits for others
 constexpr uint32_t MQ_NEAR_STAGE = 1024;
 constexpr uint32_t MQ_FAR_STAGE = 512;
 
@@ -59,6 +62,8 @@ struct MqArgs {
     // adjacency `adj` (null: rows are unpartitioned and arcs are filtered)
     const uint32_t *lend;
     uint32_t pull;           // first heavy-arc pass of a slot in the pull form
+    const uint64_t *__restrict__ heavy_chunks;   // hub rows in CHUNK-arc pieces
+    uint32_t n_heavy_chunks;
 };
 
 __device__ __forceinline__ uint32_t *band_list(const MqArgs &a, uint32_t i) {
@@ -203,71 +208,102 @@ __device__ __forceinline__ void mq_push_near(const MqArgs &a, MqStage &st, const
                  &a.ctl->err);
 }
 
-// Relaxes up to MQ_ILP (arc, slot) pairs per lane.
-// Pair i is arc arc[i] for slot qs[i]; heavy[i] marks a heavy-arc pass
-// item (only arcs of weight >= delta), else only lighter arcs are relaxed
-// when the split is on.
+// One slot served by a lane: its number, its label's rank bits and the label
+// (as stored) of the vertex being relaxed.
+struct MqLane {
+    uint32_t q, sh, lab;
+};
+
+// Sums of label and weight step at or above this do not fit slot labels of
+// `sh` rank bits.
+__device__ __forceinline__ uint64_t mq_label_limit(uint32_t sh) { return (1ull << 32) - (1ull << sh); }
+
+// The smallest label of a distance at or above T (saturating).
+__device__ __forceinline__ uint32_t mq_threshold_label(unsigned long long T, uint32_t sh) {
+    return T >= (1ull << (32 - sh)) ? INF32 : (uint32_t)T << sh;
+}
+
+// Relaxes up to MQ_ILP (arc, slot) pairs per lane: arc record e[i] (weight 0:
+// no pair) for the lane's slot s0, or with TWO slots per lane s0 and s1 in
+// turn.  Only arcs of weight in [wlo, whi) are relaxed.  Labels are compared
+// and sent as stored: lab + (weight << rank bits), in 64 bits for the
+// overflow.  UNIFORM: at every i all lanes have the same arc, so the masks
+// and the stamp of its head take one atomic for the warp.
+template <bool TWO, bool UNIFORM>
 __device__ __forceinline__ void mq_relax(const MqArgs &a, MqStage &st, const MqTargets &t,
-                                         const bool (&valid)[MQ_ILP],
-                                         const uint32_t (&arc)[MQ_ILP],
-                                         const uint32_t (&qs)[MQ_ILP],
-                                         const uint64_t (&lab)[MQ_ILP],
-                                         const bool (&heavy)[MQ_ILP],
-                                         unsigned long long &attempts,
-                                         unsigned long long &improved,
-                                         unsigned long long &narrow_miss) {
-    uint2 e[MQ_ILP];
+                                         const uint2 (&e)[MQ_ILP], const MqLane &s0,
+                                         const MqLane &s1, uint32_t wlo, uint32_t whi, uint32_t &attempts,
+                                         uint32_t &improved, unsigned long long &narrow_miss) {
+    uint32_t nl[MQ_ILP], cur[MQ_ILP];
 #pragma unroll
     for (int i = 0; i < MQ_ILP; ++i) {
-        e[i] = make_uint2(0, 0);
-        if (valid[i]) e[i] = __ldg(&a.adj[arc[i]]);
-    }
-    uint64_t nd[MQ_ILP];
-    bool imp[MQ_ILP];
-#pragma unroll
-    for (int i = 0; i < MQ_ILP; ++i) {
-        imp[i] = false;
-        nd[i] = INF32;
-        if (!valid[i] || lab[i] == INF64) continue;
-        if (heavy[i] ? e[i].y < a.delta : (a.defer && e[i].y >= a.delta)) continue;
+        const MqLane &s = TWO && (i & 1) ? s1 : s0;
+        nl[i] = INF32;
+        cur[i] = 0;
+        if (e[i].y < wlo || e[i].y >= whi || s.lab == INF32) continue;
         ++attempts;
-        nd[i] = (lab[i] >> 32) + (uint64_t)e[i].y;
-        const uint32_t sh = st.lshift[qs[i]];
-        if (nd[i] > (uint64_t)((1ull << (32 - sh)) - 2)) {
-            narrow_miss |= 1ull << qs[i];        // the slot is answered by the single-query path
+        const uint64_t sum = ((uint64_t)e[i].y << s.sh) + s.lab;
+        if (sum >= mq_label_limit(s.sh)) {
+            narrow_miss |= 1ull << s.q;          // the slot is answered by the single-query path
         } else {
             // read first: most proposals do not improve, and a load costs far
             // less L2 throughput than an atomic
-            const uint32_t nl = ((uint32_t)nd[i] << sh) | (uint32_t)lab[i];
-            uint32_t *dst = &a.label[(uint64_t)e[i].x * MQ_SLOTS + qs[i]];
-            if (nl < ldcg_u32(dst)) {
-                const uint32_t old = atomicMin(dst, nl);
-                imp[i] = nl < old;
-            }
+            nl[i] = (uint32_t)sum;
+            cur[i] = ldcg_u32(&a.label[(uint64_t)e[i].x * MQ_SLOTS + s.q]);
         }
     }
-    // most rounds improve nothing: skip the append machinery then
-    bool any_imp = false;
+    bool imp[MQ_ILP], any_imp = false;
 #pragma unroll
-    for (int i = 0; i < MQ_ILP; ++i) any_imp |= imp[i];
+    for (int i = 0; i < MQ_ILP; ++i) {
+        const MqLane &s = TWO && (i & 1) ? s1 : s0;
+        imp[i] = nl[i] < cur[i] &&
+                 nl[i] < atomicMin(&a.label[(uint64_t)e[i].x * MQ_SLOTS + s.q], nl[i]);
+        any_imp |= imp[i];
+    }
+    // most rounds improve nothing: skip the append machinery then
     if (!__any_sync(FULL, any_imp)) return;
     bool to_near[MQ_ILP], to_far[MQ_ILP];
     unsigned long long act = 0;
 #pragma unroll
     for (int i = 0; i < MQ_ILP; ++i) {
+        const MqLane &s = TWO && (i & 1) ? s1 : s0;
         to_near[i] = to_far[i] = false;
-        if (!imp[i]) continue;
-        ++improved;
-        uint32_t v = e[i].x, q = qs[i];
-        unsigned long long bit = 1ull << q;
-        if (nd[i] < st.T[q]) {
+        const uint32_t v = e[i].x;
+        const unsigned long long bit = 1ull << s.q;
+        const bool near = imp[i] && (nl[i] >> s.sh) < st.T[s.q], far = imp[i] && !near;
+        if (imp[i]) ++improved;
+        if (near) act |= bit;
+        if (UNIFORM) {
+            if (!__any_sync(FULL, imp[i])) continue;
+            const unsigned long long nb = warp_or64(near ? bit : 0ull);
+            const unsigned long long fb = warp_or64(far ? bit : 0ull);
+            // the lowest lane with an improvement speaks for the warp
+            const uint32_t lead = __ffs(__ballot_sync(FULL, imp[i])) - 1;
+            unsigned long long old = 0;
+            if (lane_id() == lead) {
+                if (nb) {
+                    atomicOr(&a.nmask[v], nb);
+                    to_near[i] = atomicExch(&a.stamp_near[v], t.tag_next) != t.tag_next;
+                }
+                if (fb) {
+                    old = atomicOr(&a.fmask[v], fb);
+                    to_far[i] = atomicExch(&a.in_far[v], 1u) == 0;
+                }
+            }
+            if (fb) {
+                old = __shfl_sync(FULL, old, lead);
+                if (far) {
+                    if (!(old & bit)) atomicAdd(&st.fpend[s.q], 1);
+                    atomicMin(&st.fmin[s.q], nl[i] >> s.sh);
+                }
+            }
+        } else if (near) {
             atomicOr(&a.nmask[v], bit);
             to_near[i] = atomicExch(&a.stamp_near[v], t.tag_next) != t.tag_next;
-            act |= bit;
-        } else {
-            unsigned long long old = atomicOr(&a.fmask[v], bit);
-            if (!(old & bit)) atomicAdd(&st.fpend[q], 1);
-            atomicMin(&st.fmin[q], (uint32_t)nd[i]);
+        } else if (far) {
+            const unsigned long long old = atomicOr(&a.fmask[v], bit);
+            if (!(old & bit)) atomicAdd(&st.fpend[s.q], 1);
+            atomicMin(&st.fmin[s.q], nl[i] >> s.sh);
             to_far[i] = atomicExch(&a.in_far[v], 1u) == 0;
         }
     }
@@ -287,19 +323,103 @@ __device__ __forceinline__ void mq_relax(const MqArgs &a, MqStage &st, const MqT
 // still at or above it only a proposal at or above it.  So instead of
 // pushing the heavy arcs of the band's vertices, every vertex unsettled in
 // some slot of P reads its own heavy arcs and, per arc, the label run of the
-// other end.  Warps sweep the vertices one at a time, lane l serving slots
-// l and l + 32; each lane keeps its slots' best proposal from settled ends
-// in registers and, after the row, sends one atomicMin per improved
-// (vertex, slot) and does the bookkeeping of mq_relax for it (a far
-// proposal: far mask, far pending count, far minimum, far pile).  Only
-// this warp writes these labels during the iteration: the band items of
-// the iteration leave out the slots of P, and those slots have no near
-// work.
+// other end.  Lane l serves slots 2l and 2l + 1 (one 8-byte load of a run per
+// arc), keeps their best proposals from settled ends in registers and, after
+// the row, sends one atomicMin per improved (vertex, slot) and does the
+// bookkeeping of mq_relax for it (a far proposal: far mask, far pending
+// count, far minimum, far pile).  No frontier or band item relaxes those
+// slots in the iteration: the band items leave out the slots of P, and those
+// slots have no near work.
+// What bounds it: the latency of the label runs, so PULL_ARCS of them are in
+// flight per warp (the arc records come 32 at a time, a lane each), and hub
+// rows are cut in pieces over the grid: one arc after another, a hub left
+// unsettled in some slot held up the whole sweep (R-MAT 22, 64 queries: the
+// batch took 100 or 205 ms, by whether the draw of seeds left one).  With one
+// shared sweep and the tails behind it the same batch takes 51 ms: Voronoi
+// part 70 -> 31 ms, 66 -> 23 iterations, 6 -> 1 sweeps.
+constexpr int PULL_ARCS = 4;
+constexpr int PULL_ROWS = 4;       // vertices whose labels are loaded together
+
+__device__ __forceinline__ void mq_pull_row(const MqArgs &a, MqStage &st, const MqTargets &t,
+                                            uint32_t v, uint32_t s, uint32_t r1, uint2 mine,
+                                            uint2 lv, bool ua,
+                                            bool ub, uint32_t sha, uint32_t shb, uint32_t Ta,
+                                            uint32_t Tb, uint32_t &attempts, uint32_t &improved,
+                                            unsigned long long &narrow_miss) {
+    const uint32_t lane = lane_id(), qa = 2 * lane, qb = qa + 1;
+    uint32_t ba = INF32, bb = INF32;
+    for (uint32_t w0 = s; w0 < r1; w0 += 32) {
+        if (w0 != s) mine = w0 + lane < r1 ? __ldcs(&a.adj[w0 + lane]) : make_uint2(0, 0);
+        const uint32_t cnt = min(32u, r1 - w0);
+        for (uint32_t i = 0; i < cnt; i += PULL_ARCS) {
+            uint2 x[PULL_ARCS];
+#pragma unroll
+            for (int k = 0; k < PULL_ARCS; ++k) {
+                const uint32_t head = __shfl_sync(FULL, mine.x, i + k);
+                const uint32_t w = __shfl_sync(FULL, mine.y, i + k);
+                x[k] = make_uint2(INF32, INF32);
+                if (w >= a.delta && (ua || ub))      // (past the row's end w = 0; light arcs
+                                                     // only on unpartitioned rows)
+                    x[k] = __ldcg(reinterpret_cast<const uint2 *>(
+                        &a.label[(uint64_t)head * MQ_SLOTS + qa]));
+            }
+#pragma unroll
+            for (int k = 0; k < PULL_ARCS; ++k) {
+                const uint32_t w = __shfl_sync(FULL, mine.y, i + k);
+                if (ua && x[k].x < Ta) {             // a settled end proposes
+                    ++attempts;
+                    const uint64_t sum = ((uint64_t)w << sha) + x[k].x;
+                    if (sum < mq_label_limit(sha)) ba = min(ba, (uint32_t)sum);
+                    else if (lv.x == INF32) narrow_miss |= 1ull << qa;
+                }
+                if (ub && x[k].y < Tb) {
+                    ++attempts;
+                    const uint64_t sum = ((uint64_t)w << shb) + x[k].y;
+                    if (sum < mq_label_limit(shb)) bb = min(bb, (uint32_t)sum);
+                    else if (lv.y == INF32) narrow_miss |= 1ull << qb;
+                }
+            }
+        }
+    }
+    uint32_t *dst = &a.label[(uint64_t)v * MQ_SLOTS + qa];
+    const bool ia = ua && ba < lv.x && ba < atomicMin(dst, ba);
+    const bool ib = ub && bb < lv.y && bb < atomicMin(dst + 1, bb);
+    const bool fa = ia && ba >= Ta, fb = ib && bb >= Tb;
+    const unsigned long long nbits = warp_or64((ia && !fa ? 1ull << qa : 0ull) | (ib && !fb ? 1ull << qb : 0ull));
+    const unsigned long long fbits = warp_or64((fa ? 1ull << qa : 0ull) | (fb ? 1ull << qb : 0ull));
+    if (!(nbits | fbits)) return;
+    improved += (ia ? 1u : 0u) + (ib ? 1u : 0u);
+    unsigned long long fold = 0;
+    bool to_far = false, to_near = false;
+    if (lane == 0) {
+        if (fbits) {
+            fold = atomicOr(&a.fmask[v], fbits);
+            to_far = atomicExch(&a.in_far[v], 1u) == 0;
+        }
+        if (nbits) {
+            atomicOr(&a.nmask[v], nbits);
+            to_near = atomicExch(&a.stamp_near[v], t.tag_next) != t.tag_next;
+            atomicOr(&st.act, nbits);
+        }
+    }
+    fold = __shfl_sync(FULL, fold, 0);
+    if (fa) {
+        if (!((fold >> qa) & 1ull)) atomicAdd(&st.fpend[qa], 1);
+        atomicMin(&st.fmin[qa], ba >> sha);
+    }
+    if (fb) {
+        if (!((fold >> qb) & 1ull)) atomicAdd(&st.fpend[qb], 1);
+        atomicMin(&st.fmin[qb], bb >> shb);
+    }
+    mq_push_near(a, st, t, to_near, v);
+    stage_append(to_far, v, st.far_buf, &st.far_n, MQ_FAR_STAGE, t.farq, t.far_count, a.n,
+                 &a.ctl->err);
+}
+
 __device__ __noinline__ void mq_pull_sweep(const MqArgs &a, MqStage &st, unsigned long long P,
                                            uint32_t *qn, uint32_t *qn_count, uint32_t *farq,
                                            uint32_t *far_count, uint32_t tag_next,
-                                           unsigned long long &attempts,
-                                           unsigned long long &improved,
+                                           uint32_t &attempts, uint32_t &improved,
                                            unsigned long long &narrow_miss) {
     MqTargets t;
     t.qn = qn;
@@ -312,91 +432,75 @@ __device__ __noinline__ void mq_pull_sweep(const MqArgs &a, MqStage &st, unsigne
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t q0 = lane, q1 = lane + 32;
-    const bool p0 = (P >> q0) & 1ull, p1 = (P >> q1) & 1ull;
-    const uint32_t sh0 = st.lshift[q0], sh1 = st.lshift[q1];
-    const unsigned long long T0 = st.T[q0], T1 = st.T[q1];
-    const uint64_t lm0 = (1ull << (32 - sh0)) - 2, lm1 = (1ull << (32 - sh1)) - 2;
-    for (uint32_t v = warp; v < a.n; v += nwarps) {
-        const uint64_t base = (uint64_t)v * MQ_SLOTS;
-        const uint64_t la = p0 ? widen_label(ldcg_u32(&a.label[base + q0]), sh0) : 0ull;
-        const uint64_t lb = p1 ? widen_label(ldcg_u32(&a.label[base + q1]), sh1) : 0ull;
-        const bool ua = p0 && (la == INF64 || (la >> 32) >= T0);
-        const bool ub = p1 && (lb == INF64 || (lb >> 32) >= T1);
-        if (!__any_sync(FULL, ua || ub)) continue;
-        const uint32_t r1 = a.row_ptr[v + 1];
-        const uint32_t s = a.lend ? a.lend[v] : a.row_ptr[v];
-        uint64_t ba = INF64, bb = INF64;
-        for (uint32_t j = s; j < r1; ++j) {
-            const uint2 e = a.adj[j];                  // one record, every lane
-            if (e.y < a.delta) continue;               // light (unpartitioned rows only)
-            const uint64_t ub_ = (uint64_t)e.x * MQ_SLOTS;
-            const uint32_t xa = ua ? ldcg_u32(&a.label[ub_ + q0]) : INF32;
-            const uint32_t xb = ub ? ldcg_u32(&a.label[ub_ + q1]) : INF32;
-            if (xa != INF32) {
-                const uint64_t lu = widen_label(xa, sh0);
-                if ((lu >> 32) < T0) {                 // a settled end proposes
-                    ++attempts;
-                    const uint64_t nd = (lu >> 32) + (uint64_t)e.y;
-                    if (nd > lm0) {
-                        if (la == INF64) narrow_miss |= 1ull << q0;
-                    } else {
-                        ba = min(ba, (uint64_t)((nd << 32) | (lu & 0xFFFFFFFFull)));
-                    }
-                }
-            }
-            if (xb != INF32) {
-                const uint64_t lu = widen_label(xb, sh1);
-                if ((lu >> 32) < T1) {
-                    ++attempts;
-                    const uint64_t nd = (lu >> 32) + (uint64_t)e.y;
-                    if (nd > lm1) {
-                        if (lb == INF64) narrow_miss |= 1ull << q1;
-                    } else {
-                        bb = min(bb, (uint64_t)((nd << 32) | (lu & 0xFFFFFFFFull)));
-                    }
-                }
-            }
+    const uint32_t qa = 2 * lane, qb = qa + 1;
+    const uint32_t sha = st.lshift[qa], shb = st.lshift[qb];
+    // a slot outside P is settled everywhere: threshold label INF32 + nothing
+    const bool pa = (P >> qa) & 1ull, pb = (P >> qb) & 1ull;
+    const uint32_t Ta = mq_threshold_label(st.T[qa], sha), Tb = mq_threshold_label(st.T[qb], shb);
+    const uint32_t n_items = a.n_heavy_chunks + (a.n + PULL_ROWS - 1) / PULL_ROWS;
+    // Row offsets of an item's vertices, one per lane (starts and the last
+    // end in lanes 0..PULL_ROWS, starts of the heavy parts from lane 8 on),
+    // fetched an item ahead.
+    auto offsets = [&](uint32_t wi) {
+        if (wi >= n_items) return 0u;
+        const uint32_t v0 = wi < a.n_heavy_chunks ? (uint32_t)(a.heavy_chunks[wi] >> 32)
+                                                  : (wi - a.n_heavy_chunks) * PULL_ROWS;
+        const uint32_t r = lane & 7u, v = min(v0 + r, a.n);
+        if (lane < 8) return r <= PULL_ROWS ? a.row_ptr[v] : 0u;
+        if (lane >= 16 || r >= PULL_ROWS || v >= a.n) return 0u;
+        return a.lend ? a.lend[v] : a.row_ptr[v];
+    };
+    uint32_t next = offsets(warp);
+    for (uint32_t wi = warp; wi < n_items; wi += nwarps) {
+        const uint32_t off = next;
+        next = offsets(wi + nwarps);
+        const bool hub = wi < a.n_heavy_chunks;
+        uint32_t v0, c = 0, rows = 1;
+        if (hub) {
+            const uint64_t item = a.heavy_chunks[wi];
+            v0 = (uint32_t)(item >> 32);
+            c = (uint32_t)item;
+        } else {
+            v0 = (wi - a.n_heavy_chunks) * PULL_ROWS;
+            rows = min((uint32_t)PULL_ROWS, a.n - v0);
         }
-        const bool ia = ua && ba < la, ib = ub && bb < lb;
-        if (ia) atomicMin(&a.label[base + q0], ((uint32_t)(ba >> 32) << sh0) | (uint32_t)ba);
-        if (ib) atomicMin(&a.label[base + q1], ((uint32_t)(bb >> 32) << sh1) | (uint32_t)bb);
-        const bool fa = ia && (ba >> 32) >= T0, fb = ib && (bb >> 32) >= T1;
-        unsigned long long nbits = (ia && !fa ? 1ull << q0 : 0ull) | (ib && !fb ? 1ull << q1 : 0ull);
-        unsigned long long fbits = (fa ? 1ull << q0 : 0ull) | (fb ? 1ull << q1 : 0ull);
-        nbits = warp_or64(nbits);
-        fbits = warp_or64(fbits);
-        if (!(nbits | fbits)) continue;
-        improved += (ia ? 1u : 0u) + (ib ? 1u : 0u);
-        unsigned long long fold = 0;
-        bool to_far = false, to_near = false;
-        if (lane == 0) {
-            if (fbits) {
-                fold = atomicOr(&a.fmask[v], fbits);
-                to_far = atomicExch(&a.in_far[v], 1u) == 0;
+        // rows without heavy arcs (isolated vertices above all) need no look
+        // at their labels; hub rows are covered by their pieces
+        uint32_t s[PULL_ROWS], e[PULL_ROWS];
+        uint2 lv[PULL_ROWS], mine[PULL_ROWS];
+#pragma unroll
+        for (int r = 0; r < PULL_ROWS; ++r) {
+            const uint32_t r0 = __shfl_sync(FULL, off, r);
+            e[r] = __shfl_sync(FULL, off, r + 1);
+            s[r] = __shfl_sync(FULL, off, 8 + r);
+            if (hub) {
+                s[r] += c * CHUNK;
+                e[r] = r == 0 && s[r] < e[r] ? min(e[r], s[r] + CHUNK) : s[r];
+            } else if ((uint32_t)r >= rows || e[r] - r0 >= HEAVY_DEG) {
+                e[r] = s[r];
             }
-            if (nbits) {
-                atomicOr(&a.nmask[v], nbits);
-                to_near = atomicExch(&a.stamp_near[v], tag_next) != tag_next;
-                atomicOr(&st.act, nbits);
-            }
+            lv[r] = make_uint2(0, 0);
+            if (e[r] > s[r] && (pa || pb))
+                lv[r] = __ldcg(reinterpret_cast<const uint2 *>(&a.label[(uint64_t)(v0 + r) * MQ_SLOTS + qa]));
         }
-        fold = __shfl_sync(FULL, fold, 0);
-        if (fa) {
-            if (!((fold >> q0) & 1ull)) atomicAdd(&st.fpend[q0], 1);
-            atomicMin(&st.fmin[q0], (uint32_t)(ba >> 32));
+        bool ua[PULL_ROWS], ub[PULL_ROWS];
+#pragma unroll
+        for (int r = 0; r < PULL_ROWS; ++r) {
+            ua[r] = e[r] > s[r] && pa && lv[r].x >= Ta;
+            ub[r] = e[r] > s[r] && pb && lv[r].y >= Tb;
+            mine[r] = make_uint2(0, 0);
+            if (!__any_sync(FULL, ua[r] || ub[r])) e[r] = s[r];
+            else if (s[r] + lane < e[r]) mine[r] = __ldcs(&a.adj[s[r] + lane]);
         }
-        if (fb) {
-            if (!((fold >> q1) & 1ull)) atomicAdd(&st.fpend[q1], 1);
-            atomicMin(&st.fmin[q1], (uint32_t)(bb >> 32));
-        }
-        mq_push_near(a, st, t, to_near, v);
-        stage_append(to_far, v, st.far_buf, &st.far_n, MQ_FAR_STAGE, t.farq, t.far_count, a.n,
-                     &a.ctl->err);
+#pragma unroll
+        for (int r = 0; r < PULL_ROWS; ++r)
+            if (e[r] > s[r])
+                mq_pull_row(a, st, t, v0 + r, s[r], e[r], mine[r], lv[r], ua[r], ub[r], sha, shb,
+                            Ta, Tb, attempts, improved, narrow_miss);
     }
 }
 
-__global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
+__global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_constant__ MqArgs a) {
     __shared__ MqStage st;
     MqControl *ctl = a.ctl;
     const uint32_t lane = lane_id();
@@ -404,7 +508,8 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const bool first = gtid == 0;
-    unsigned long long attempts = 0, improved = 0, narrow_miss = 0;
+    uint32_t attempts = 0, improved = 0;     // this thread's
+    unsigned long long narrow_miss = 0;
     uint32_t it = ldcg_u32(&ctl->it), fc = ldcg_u32(&ctl->fc);
     unsigned long long infl = __ldcg(&ctl->inflight) & ~__ldcg(&ctl->converged);
     unsigned long long conv_total = 0;
@@ -412,6 +517,8 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
     unsigned long long H = __ldcg(&ctl->hpass) & infl;
     unsigned long long hp_done = __ldcg(&ctl->hp_done);
     unsigned long long band0 = __ldcg(&ctl->band0);
+    unsigned long long tails = __ldcg(&ctl->tails);     // slots in their unbounded tail
+    uint32_t held = ldcg_u32(&ctl->held);               // iterations that drained slots waited
     uint32_t pull_sweeps = 0;
     uint32_t bc = ldcg_u32(&ctl->blist);
     if (threadIdx.x < MQ_SLOTS) {
@@ -469,7 +576,7 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
                     u = ldcg_u32(&qc[i]);
                     M = atomicExch(&a.nmask[u], 0ull);
                     // first slot to relax u in its band lists u
-                    if (a.defer && M) listed = atomicOr(&a.bmask[u], M) == 0ull;
+                    if (a.defer && (M & ~tails)) listed = atomicOr(&a.bmask[u], M & ~tails) == 0ull;
                 } else {
                     u = ldcg_u32(&blo[i - n_items]);
                     const unsigned long long old = atomicAnd(&a.bmask[u], ~H);
@@ -477,9 +584,11 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
                     listed = (old & ~H) != 0ull; // still in other slots' bands
                 }
                 a.item_mask[i] = M;
-                // frontier items relax the light part, band items the heavy one
+                // frontier items relax the light part (the whole row for a
+                // slot in its tail, and then for the item's other slots too:
+                // relaxing an arc early does no harm), band items the heavy one
                 const uint32_t r0 = a.row_ptr[u], r1 = a.row_ptr[u + 1];
-                const uint32_t le = a.lend ? a.lend[u] : r1;
+                const uint32_t le = a.lend && !(M & tails) ? a.lend[u] : r1;
                 const uint32_t deg = i < n_items ? le - r0 : (a.lend ? r1 - le : r1 - r0);
                 w = (uint64_t)deg * (uint64_t)popc64(M);
             }
@@ -563,13 +672,14 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
                     c = (uint32_t)popc64(M);
                 }
                 const bool hv = idx >= n_items;        // heavy-arc pass item
+                const bool whole = !hv && (M & tails); // whole row
                 const uint64_t wend = i0 + 32 < n_all ? gpre(i0 + 32) : W;
                 const uint64_t stop = min(p1, wend);
                 // The window's items one after another: an item's pairs are
                 // (arc j, slot t) -> j * c + t; the lanes take fixed slots
                 // (and, for c <= 16, several arcs per step), so a lane finds
                 // its slot and loads the tail's label once per item and then
-                // steps over the arcs with one broadcast arc load per arc.
+                // steps over the arcs.
                 for (uint32_t w = 0; w < 32; ++w) {
                     const uint64_t pre_w = __shfl_sync(FULL, pre, w);
                     if (pre_w >= stop) break;
@@ -580,63 +690,56 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
                     const uint32_t uw = __shfl_sync(FULL, u, w);
                     const uint32_t sw = __shfl_sync(FULL, s0, w);
                     const unsigned long long Mw = __shfl_sync(FULL, M, w);
-                    const bool hw = __shfl_sync(FULL, hv, w);
+                    const bool hw = __shfl_sync(FULL, hv, w), ww = __shfl_sync(FULL, whole, w);
+                    const uint32_t wlo = hw ? a.delta : 1u;          // (weight 0: no pair)
+                    const uint32_t whi = a.defer && !hw && !ww ? a.delta : 0xFFFFFFFFu;
                     // the item's pairs inside this chunk: [lo, hi)
                     const uint32_t lo = (uint32_t)((p > pre_w ? p : pre_w) - pre_w);
                     const uint32_t hi = (uint32_t)(end_w - pre_w);
                     const uint64_t mw = st.mag[cw];
                     const uint32_t jlo = cw > 1 ? (uint32_t)__umul64hi((uint64_t)lo, mw << 24) : lo;
                     const uint32_t jhi = cw > 1 ? (uint32_t)__umul64hi((uint64_t)(hi - 1), mw << 24) : hi - 1;
-                    if (cw <= 32) {
+                    auto lane_slot = [&](uint32_t tq) {
+                        MqLane s{0, 0, INF32};
+                        if (tq < cw) {
+                            s.q = cw == MQ_SLOTS ? tq : nth_bit64(Mw, tq);
+                            s.sh = st.lshift[s.q];
+                            s.lab = ldcg_u32(&a.label[(uint64_t)uw * MQ_SLOTS + s.q]);
+                        }
+                        return s;
+                    };
+                    if (cw > 32) {
+                        // 33..64 slots: each lane takes slots lane and lane + 32
+                        const MqLane s0 = lane_slot(lane), s1 = lane_slot(lane + 32);
+                        for (uint32_t j0 = jlo; j0 <= jhi; j0 += MQ_ILP / 2) {
+                            uint2 e[MQ_ILP];
+#pragma unroll
+                            for (int k = 0; k < MQ_ILP; k += 2) {
+                                const uint32_t jj = j0 + (uint32_t)(k >> 1), l = jj * cw + lane;
+                                uint2 x = make_uint2(0, 0);
+                                if (jj <= jhi) x = __ldg(&a.adj[sw + jj]);
+                                e[k] = e[k + 1] = x;
+                                if (l < lo || l >= hi) e[k].y = 0;
+                                if (lane + 32 >= cw || l + 32 < lo || l + 32 >= hi) e[k + 1].y = 0;
+                            }
+                            mq_relax<true, true>(a, st, t, e, s0, s1, wlo, whi, attempts, improved, narrow_miss);
+                        }
+                    } else {
                         // g lanes per arc (g = c rounded up to a power of two),
                         // 32 / g arcs per step
                         const uint32_t gsh = cw <= 1 ? 0u : 32u - __clz(cw - 1);
                         const uint32_t A = 32u >> gsh;
                         const uint32_t tq = lane & ((1u << gsh) - 1u), aoff = lane >> gsh;
-                        const bool tok = tq < cw;
-                        const uint32_t q = tok ? nth_bit64(Mw, tq) : 0u;
-                        const uint64_t lab = tok ? mq_label(a.label, uw, q, st.lshift[q]) : INF64;
+                        const MqLane s0 = lane_slot(tq);
                         for (uint32_t j0 = jlo; j0 <= jhi; j0 += MQ_ILP * A) {
-                            bool valid[MQ_ILP], heavy[MQ_ILP];
-                            uint32_t arc[MQ_ILP], qs[MQ_ILP];
-                            uint64_t labs[MQ_ILP];
+                            uint2 e[MQ_ILP];
 #pragma unroll
                             for (int k = 0; k < MQ_ILP; ++k) {
-                                const uint32_t jj = j0 + (uint32_t)k * A + aoff;
-                                const uint32_t l = jj * cw + tq;
-                                valid[k] = tok && jj <= jhi && l >= lo && l < hi;
-                                heavy[k] = hw;
-                                arc[k] = sw + jj;
-                                qs[k] = q;
-                                labs[k] = lab;
+                                const uint32_t jj = j0 + (uint32_t)k * A + aoff, l = jj * cw + tq;
+                                e[k] = make_uint2(0, 0);
+                                if (tq < cw && jj <= jhi && l >= lo && l < hi) e[k] = __ldg(&a.adj[sw + jj]);
                             }
-                            mq_relax(a, st, t, valid, arc, qs, labs, heavy, attempts, improved, narrow_miss);
-                        }
-                    } else {
-                        // 33..64 slots: each lane takes slots lane and lane + 32
-                        const uint32_t t1 = lane + 32;
-                        const bool tok1 = t1 < cw;
-                        const uint32_t q0 = cw == MQ_SLOTS ? lane : nth_bit64(Mw, lane);
-                        const uint32_t q1 = tok1 ? (cw == MQ_SLOTS ? t1 : nth_bit64(Mw, t1)) : 0u;
-                        const uint64_t lab0 = mq_label(a.label, uw, q0, st.lshift[q0]);
-                        const uint64_t lab1 = tok1 ? mq_label(a.label, uw, q1, st.lshift[q1]) : INF64;
-                        for (uint32_t j0 = jlo; j0 <= jhi; j0 += MQ_ILP / 2) {
-                            bool valid[MQ_ILP], heavy[MQ_ILP];
-                            uint32_t arc[MQ_ILP], qs[MQ_ILP];
-                            uint64_t labs[MQ_ILP];
-#pragma unroll
-                            for (int k = 0; k < MQ_ILP; ++k) {
-                                const uint32_t jj = j0 + (uint32_t)(k >> 1);
-                                const bool second = k & 1;
-                                const uint32_t tq = second ? t1 : lane;
-                                const uint32_t l = jj * cw + tq;
-                                valid[k] = (second ? tok1 : true) && jj <= jhi && l >= lo && l < hi;
-                                heavy[k] = hw;
-                                arc[k] = sw + jj;
-                                qs[k] = second ? q1 : q0;
-                                labs[k] = second ? lab1 : lab0;
-                            }
-                            mq_relax(a, st, t, valid, arc, qs, labs, heavy, attempts, improved, narrow_miss);
+                            mq_relax<false, false>(a, st, t, e, s0, s0, wlo, whi, attempts, improved, narrow_miss);
                         }
                     }
                 }
@@ -674,7 +777,17 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
         unsigned long long act_next = __ldcg(&ctl->act[it % 3]);
         hp_done &= ~act_next;
         unsigned long long idle = infl & ~act_next, S = 0, conv = 0;
-        H = a.defer ? (idle & ~hp_done) : 0ull;
+        H = a.defer ? (idle & ~hp_done & ~tails) : 0ull;
+        // A pull sweep visits every vertex however few slots it serves, so
+        // drained first bands wait (up to MQ_HOLD iterations) for the other
+        // slots' and share one sweep.
+        if (a.pull && (H & band0) && (infl & band0 & act_next) && held < MQ_HOLD) {
+            idle &= ~(H & band0);
+            H &= ~band0;
+            ++held;
+        } else if (H & band0) {
+            held = 0;
+        }
         hp_done |= H;
         for (unsigned long long m = idle & ~H; m; m &= m - 1) {
             uint32_t q = __ffsll((long long)m) - 1;
@@ -682,6 +795,8 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
             else S |= 1ull << q;
         }
         hp_done &= ~S;                      // a split opens a new band
+        const unsigned long long to_tail = a.pull ? S & band0 : 0ull;
+        tails |= to_tail;
         band0 &= ~S;
         infl &= ~conv;
         conv_total |= conv;
@@ -702,7 +817,8 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
             if ((S >> q) & 1) {
                 uint32_t fm = __ldcg(&ctl->fmin[fc][q]);
                 unsigned long long base = (fm != INF32 && (unsigned long long)fm > Tq) ? fm : Tq;
-                st.Tnew[q] = base + a.delta;
+                // (a tail has no far side: every parked vertex joins the frontier)
+                st.Tnew[q] = (to_tail >> q) & 1 ? 1ull << 40 : base + a.delta;
             } else {
                 st.Tnew[q] = Tq;
             }
@@ -773,14 +889,15 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
         if (first) ctl->t_part[4] += gtimer() - tm5;
     }
     if (!infl && reason == 0) reason = 1;
+    unsigned long long sum_a = attempts, sum_i = improved;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) {
-        attempts += __shfl_xor_sync(FULL, attempts, o);
-        improved += __shfl_xor_sync(FULL, improved, o);
+        sum_a += __shfl_xor_sync(FULL, sum_a, o);
+        sum_i += __shfl_xor_sync(FULL, sum_i, o);
     }
     if (lane == 0) {
-        atomicAdd(&ctl->relax_attempts, attempts);
-        atomicAdd(&ctl->relax_improved, improved);
+        atomicAdd(&ctl->relax_attempts, sum_a);
+        atomicAdd(&ctl->relax_improved, sum_i);
     }
     narrow_miss = warp_or64(narrow_miss);
     if (lane == 0 && narrow_miss) atomicOr(&ctl->slot_narrow, narrow_miss);
@@ -790,6 +907,8 @@ __global__ void __launch_bounds__(256, 6) mq_sssp_kernel(MqArgs a) {
         ctl->hpass = H & infl;
         ctl->hp_done = hp_done;
         ctl->band0 = band0;
+        ctl->tails = tails;
+        ctl->held = held;
         ctl->pull_sweeps += pull_sweeps;
         ctl->blist = bc;
         ctl->converged |= conv_total;
@@ -846,6 +965,7 @@ __global__ void mq_seed_kernel(const uint32_t *__restrict__ row_ptr, uint32_t n,
         ctl->hp_done &= ~bit;
         ctl->hpass &= ~bit;
         ctl->band0 |= bit;
+        ctl->tails &= ~bit;
     }
     if (r >= k) return;
     uint32_t s = internal_id(new_of, (uint32_t)seeds[r]);
@@ -871,6 +991,8 @@ struct MqScanArgs {
     const uint2 *__restrict__ adj;
     const uint64_t *__restrict__ heavy_chunks;
     uint32_t n_heavy_chunks;
+    const uint32_t *__restrict__ items;   // vertex ranges [items[i], items[i + 1])
+    uint32_t n_items;
     uint32_t n;
     const uint32_t *label;
     const uint32_t *lshift;          // rank bits of each slot's labels
@@ -888,45 +1010,49 @@ struct MqScanArgs {
 // v's cell's row of the upper triangle (pair_slot(cv, cv + 1, k)), so that
 // the entry of pair (cv, cu) is tab[cu - cv - 1].
 struct ScanSlot {
-    uint64_t lv;
+    uint32_t lv;        // as stored
+    uint32_t sh;        // rank bits
     uint64_t *tab;
     uint32_t pmin;      // running minimum of v's pred arc
     uint32_t q;
 };
 
-__device__ __forceinline__ ScanSlot mq_row_slot(const MqScanArgs &a, uint32_t v, uint32_t q,
-                                                uint64_t *tab, uint32_t k, uint64_t lv) {
+__device__ __forceinline__ ScanSlot mq_row_slot(uint32_t q, uint64_t *tab, uint32_t k, uint32_t sh,
+                                                uint32_t lv) {
     ScanSlot r;
     r.lv = lv;
+    r.sh = sh;
     r.q = q;
     r.pmin = INF32;
-    const uint32_t cv = (uint32_t)lv;
-    r.tab = lv == INF64 ? tab : tab + pair_slot(cv, cv + 1, k);
+    const uint32_t cv = lv & ((1u << sh) - 1u);
+    r.tab = lv == INF32 ? tab : tab + pair_slot(cv, cv + 1, k);
     return r;
 }
 
-// Arc `arc` = (v, e.x, e.y) for one slot, with lu the slot's label of e.x
+// Arc `arc` = (v, head, w) for one slot, with lu the slot's label of the head
 // and cbase + arc the caller's index of the arc (bridge keys carry it, as in
-// the single-query scan).  A tight same-cell arc lowers r.pmin.
-__device__ __forceinline__ void mq_scan_eval(ScanSlot &r, uint32_t arc, uint2 e, uint64_t lu,
+// the single-query scan).  A tight same-cell arc lowers r.pmin.  Labels are
+// compared as stored.
+__device__ __forceinline__ void mq_scan_eval(ScanSlot &r, uint32_t arc, uint32_t w, uint32_t lu,
                                              uint32_t cbase, unsigned long long &overflow) {
-    if (r.lv == INF64 || lu == INF64) {
+    if (r.lv == INF32 || lu == INF32) {
         if (r.lv != lu) overflow |= 1ull << r.q;
         return;
     }
-    const uint32_t cv = (uint32_t)r.lv, cu = (uint32_t)lu;
-    const uint64_t dv = r.lv >> 32, du = lu >> 32;
-    if (cu == cv) {
-        if (du + e.y == dv) r.pmin = min(r.pmin, arc);
+    const uint32_t mask = (1u << r.sh) - 1u, cv = r.lv & mask, cu = lu & mask;
+    const uint64_t sum = ((uint64_t)w << r.sh) + lu;       // the head's distance + w, its cell
+    if (sum == r.lv) {
+        r.pmin = min(r.pmin, arc);
     } else if (cv < cu) {
-        uint64_t b = dv + e.y + du;
+        const uint64_t b = (r.lv >> r.sh) + (sum >> r.sh);
         if (b >= INF32) {
             overflow |= 1ull << r.q;
             return;
         }
-        uint64_t key = (b << 32) | (uint32_t)(cbase + arc);
+        const uint64_t key = (b << 32) | (uint32_t)(cbase + arc);
         uint64_t *slot = r.tab + (cu - cv - 1);
-        if (key < ldcg_u64(slot))
+        // a cached read may be stale, i.e. larger: at worst one atomic more
+        if (key < __ldg(reinterpret_cast<const unsigned long long *>(slot)))
             atomicMin(reinterpret_cast<unsigned long long *>(slot), (unsigned long long)key);
     }
 }
@@ -939,7 +1065,11 @@ __device__ __forceinline__ void mq_store_pred(const MqScanArgs &a, uint32_t v, c
     else atomicMin(pp, r.pmin);
 }
 
-constexpr int SCAN_PAIR_ILP = 2;   // arcs in flight per lane in the slot-pair mode
+// Label runs in flight per warp in the slot-pair mode.  The scan is bound by
+// the evaluation of (arc, slot) pairs and the probes of the pair tables (R-MAT
+// 22 x 64 queries: 17.1 ms; 7.6 with the label runs alone): labels compared
+// as stored and cached probes took it down from 22.4.
+constexpr int SCAN_ARCS = 4;
 
 // The slots a lane serves for the whole launch, with their pair tables and
 // sizes loaded once.
@@ -966,25 +1096,31 @@ __device__ __forceinline__ void mq_scan_row(const MqScanArgs &a, const LaneSlots
     const uint32_t cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, rs);
     const uint32_t *lrow = &a.label[(uint64_t)v * MQ_SLOTS];
     if (cnt > 32) {
-        if (!ls.h0 && !ls.h1) return;
         const uint2 lv = __ldg(reinterpret_cast<const uint2 *>(&lrow[ls.q0]));
-        ScanSlot r0 = mq_row_slot(a, v, ls.q0, ls.t0, ls.k0, widen_label(lv.x, ls.sh0));
-        ScanSlot r1 = mq_row_slot(a, v, ls.q0 + 1, ls.t1, ls.k1, widen_label(lv.y, ls.sh1));
-        for (uint32_t j0 = s0; j0 < s1; j0 += SCAN_PAIR_ILP) {
-            uint2 e[SCAN_PAIR_ILP];
-            uint2 lu[SCAN_PAIR_ILP];
+        ScanSlot r0 = mq_row_slot(ls.q0, ls.t0, ls.k0, ls.sh0, lv.x);
+        ScanSlot r1 = mq_row_slot(ls.q0 + 1, ls.t1, ls.k1, ls.sh1, lv.y);
+        // the arc records 32 at a time, one per lane, streamed
+        for (uint32_t w0 = s0; w0 < s1; w0 += 32) {
+            uint2 mine = make_uint2(0, 0);
+            if (w0 + lane < s1) mine = __ldcs(&a.adj[w0 + lane]);
+            const uint32_t got = min(32u, s1 - w0);
+            for (uint32_t i = 0; i < got; i += SCAN_ARCS) {
+                uint2 lu[SCAN_ARCS];
 #pragma unroll
-            for (int k = 0; k < SCAN_PAIR_ILP; ++k)
-                if (j0 + k < s1) e[k] = __ldg(&a.adj[j0 + k]);
+                for (int k = 0; k < SCAN_ARCS; ++k) {
+                    const uint32_t head = __shfl_sync(FULL, mine.x, i + k);
+                    lu[k] = make_uint2(INF32, INF32);
+                    if (i + k < got)
+                        lu[k] = __ldg(reinterpret_cast<const uint2 *>(
+                            &a.label[(uint64_t)head * MQ_SLOTS + ls.q0]));
+                }
 #pragma unroll
-            for (int k = 0; k < SCAN_PAIR_ILP; ++k)
-                if (j0 + k < s1)
-                    lu[k] = __ldg(reinterpret_cast<const uint2 *>(&a.label[(uint64_t)e[k].x * MQ_SLOTS + ls.q0]));
-#pragma unroll
-            for (int k = 0; k < SCAN_PAIR_ILP; ++k) {
-                if (j0 + k >= s1) break;
-                if (ls.h0) mq_scan_eval(r0, j0 + k, e[k], widen_label(lu[k].x, ls.sh0), cbase, overflow);
-                if (ls.h1) mq_scan_eval(r1, j0 + k, e[k], widen_label(lu[k].y, ls.sh1), cbase, overflow);
+                for (int k = 0; k < SCAN_ARCS; ++k) {
+                    const uint32_t w = __shfl_sync(FULL, mine.y, i + k);
+                    if (i + k >= got) break;
+                    if (ls.h0) mq_scan_eval(r0, w0 + i + k, w, lu[k].x, cbase, overflow);
+                    if (ls.h1) mq_scan_eval(r1, w0 + i + k, w, lu[k].y, cbase, overflow);
+                }
             }
         }
         if (ls.h0) mq_store_pred(a, v, r0, whole_row);
@@ -993,16 +1129,15 @@ __device__ __forceinline__ void mq_scan_row(const MqScanArgs &a, const LaneSlots
     }
     const uint32_t g = 1u << gsh, apr = 32 >> gsh, grp = lane >> gsh;
     const bool has_slot = ls.h0;
-    ScanSlot r = mq_row_slot(a, v, ls.q0, ls.t0, ls.k0,
-                             has_slot ? widen_label(__ldg(&lrow[ls.q0]), ls.sh0) : INF64);
+    ScanSlot r = mq_row_slot(ls.q0, ls.t0, ls.k0, ls.sh0, has_slot ? __ldg(&lrow[ls.q0]) : INF32);
     for (uint32_t j0 = s0; j0 < s1; j0 += apr * 4) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             uint32_t arc = j0 + k * apr + grp;
             if (has_slot && arc < s1) {
                 uint2 e = __ldg(&a.adj[arc]);
-                uint64_t lu = widen_label(__ldg(&a.label[(uint64_t)e.x * MQ_SLOTS + ls.q0]), ls.sh0);
-                mq_scan_eval(r, arc, e, lu, cbase, overflow);
+                const uint32_t lu = __ldg(&a.label[(uint64_t)e.x * MQ_SLOTS + ls.q0]);
+                mq_scan_eval(r, arc, e.y, lu, cbase, overflow);
             }
         }
     }
@@ -1034,8 +1169,7 @@ __global__ void __launch_bounds__(256, 5) mq_scan_kernel(MqScanArgs a) {
     ls.k1 = ls.h1 ? a.k[ls.q0 + 1] : 0;
     ls.sh0 = ls.h0 ? a.lshift[ls.q0] : 1;
     ls.sh1 = ls.h1 ? a.lshift[ls.q0 + 1] : 1;
-    const uint32_t n_batches = (a.n + 31) / 32;
-    const uint32_t n_work = a.n_heavy_chunks + n_batches;
+    const uint32_t n_work = a.n_heavy_chunks + a.n_items;
     unsigned long long overflow = 0;
     for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
         if (wi < a.n_heavy_chunks) {
@@ -1046,14 +1180,17 @@ __global__ void __launch_bounds__(256, 5) mq_scan_kernel(MqScanArgs a) {
             uint32_t e = min(a.row_ptr[v + 1], s + CHUNK);
             mq_scan_row(a, ls, v, rs, s, e, false, cnt, gsh, overflow);
         } else {
-            uint32_t v0 = (wi - a.n_heavy_chunks) * 32;
-            uint32_t vl = v0 + lane;
-            uint32_t rs = vl < a.n ? a.row_ptr[vl] : 0;
-            uint32_t re = vl < a.n ? a.row_ptr[vl + 1] : 0;
-            for (uint32_t l = 0; l < 32 && v0 + l < a.n; ++l) {
-                uint32_t s = __shfl_sync(FULL, rs, l), e = __shfl_sync(FULL, re, l);
-                if (e - s >= HEAVY_DEG) continue;          // covered by the chunk list
-                mq_scan_row(a, ls, v0 + l, s, s, e, true, cnt, gsh, overflow);
+            const uint32_t v1 = __ldg(&a.items[wi - a.n_heavy_chunks + 1]);
+            for (uint32_t v0 = __ldg(&a.items[wi - a.n_heavy_chunks]); v0 < v1; v0 += 32) {
+                const uint32_t vl = v0 + lane;
+                const uint32_t rs = vl < v1 ? a.row_ptr[vl] : 0;
+                const uint32_t re = vl < v1 ? a.row_ptr[vl + 1] : 0;
+                for (uint32_t l = 0; l < 32 && v0 + l < v1; ++l) {
+                    const uint32_t s = __shfl_sync(FULL, rs, l), e = __shfl_sync(FULL, re, l);
+                    // hubs are covered by the chunk list; no arcs, nothing to scan
+                    if (e - s >= HEAVY_DEG || e == s) continue;
+                    mq_scan_row(a, ls, v0 + l, s, s, e, true, cnt, gsh, overflow);
+                }
             }
         }
     }
@@ -1181,6 +1318,8 @@ cudaError_t mq_launch_sssp(const DevGraph &g, MqState &m, int blocks, uint32_t d
     a.lend = active_lend(g, delta);
     if (a.lend) a.adj = g.adj_w;        // rows partitioned by weight class
     a.pull = a.defer ? pull : 0u;
+    a.heavy_chunks = g.heavy_chunks;
+    a.n_heavy_chunks = g.n_heavy_chunks;
     a.ctl = m.ctl;
     a.doorbell = doorbell;
     a.delta = delta;
@@ -1203,6 +1342,8 @@ cudaError_t mq_launch_scan(const DevGraph &g, MqState &m, unsigned long long slo
     a.adj = g.adj;
     a.heavy_chunks = g.heavy_chunks;
     a.n_heavy_chunks = g.n_heavy_chunks;
+    a.items = g.items;
+    a.n_items = g.n_items;
     a.n = g.n;
     a.label = m.label;
     a.lshift = m.ctl->lshift;
@@ -1213,7 +1354,7 @@ cudaError_t mq_launch_scan(const DevGraph &g, MqState &m, unsigned long long slo
     a.ctl = m.ctl;
     a.orig_of = g.orig_of;
     a.orig_row_ptr = g.orig_row_ptr;
-    uint64_t work = (uint64_t)g.n_heavy_chunks + (g.n + 31) / 32;
+    uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_items;
     uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>((work + 7) / 8, (uint64_t)current_sm_count() * 32));
     mq_scan_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
     return cudaGetLastError();

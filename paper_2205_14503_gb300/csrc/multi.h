@@ -56,6 +56,10 @@ struct MqControl {
     // slots still in their first band (set at admission, cleared by the
     // slot's first split): their heavy-arc pass may run in the pull form
     unsigned long long band0;
+    // slots in their tail: after the pull-form pass the rest runs as one
+    // unbounded band over whole rows
+    unsigned long long tails;
+    uint32_t held;                      // iterations drained first bands waited for others
     uint32_t pull_sweeps;               // pull-form passes run (accumulated)
 };
 

@@ -131,3 +131,25 @@ def test_small_seed_set_tail(k):
     _check(g, wl.sample_distinct(wl.largest_cc(g), k, k))
     for g in (G.path(5000, 1, 9, 42), G.path(2049, 1, 9, 43), G.random_graph(700, 500, 1, 9, 44)):
         _check(g, np.unique(np.concatenate([[0, g.n - 1], G.seeds_from(np.arange(g.n), k - 2, k)])))
+
+
+@pytest.mark.parametrize("queries", [1, 31, 33, 64, 70])
+@pytest.mark.parametrize("batch_delta", [1, 4, 60, 1000])
+def test_batch_pull_pieces_and_tails(queries, batch_delta):
+    """The multi-query engine around its slot counts: the pull sweep's hub
+    pieces (seeds on leaves leave hubs unsettled in narrow first bands),
+    first bands that wait for each other, and the unbounded tails."""
+    g = wl.rmat(10, 24, wmax=500, seed=51)
+    pool = wl.largest_cc(g)
+    deg = np.diff(g.row_ptr.astype(np.int64))[pool]
+    leaves = pool[np.argsort(deg, kind="stable")[:200]]
+    sets = [wl.sample_distinct(leaves if i % 2 else pool, 2 + i % 29, 600 + i) for i in range(queries)]
+    with st.SteinerGraph(g) as Gd:
+        Gd.set_param("delta", max(1, batch_delta))
+        Gd.set_param("batch_delta", batch_delta)
+        rc, res = Gd.query_batch(sets)
+    assert rc == st.STEINER_OK
+    for s, r in zip(sets, res):
+        ref = oracle.steiner(g, s)
+        np.testing.assert_array_equal(r.edges, ref.edges)
+        assert r.total == ref.total
