@@ -701,6 +701,7 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     }
     double d = 32.0 * std::max(1.0, avg_w) / std::max(1.0, avg_deg);
     G->delta = (uint32_t)std::min(std::max(d, 1.0), 1.0e9);
+    G->g.delta0 = G->delta;
     if (const char *env = getenv("STEINER_DELTA")) G->delta = (uint32_t)std::max(1L, atol(env));
     *out = G;
     return STEINER_OK;

@@ -34,6 +34,7 @@ struct DevGraph {
     uint32_t n_heavy_chunks = 0;
     uint32_t heavy_chunk_cap = 0;   // bound on chunk entries a frontier can hold
     uint32_t max_w = 0;             // largest arc weight
+    uint32_t delta0 = 0;            // default band width
     // Internal vertex order.  On a skewed degree distribution the vertices
     // are renumbered by descending degree (ties by id), so the labels of
     // the hubs that most arcs point to share L2 sectors; rows keep the

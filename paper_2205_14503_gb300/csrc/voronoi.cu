@@ -76,6 +76,7 @@ struct SsspArgs {
     // above it have fewer (the degree order makes this a bound).
     uint32_t dense;
     uint32_t pull;           // heavy-arc passes: 0 push, 1 by cost, 2 pull
+    uint32_t step0;          // first threshold inside the first band (0: the band)
     uint32_t thin;           // far pile: a frontier below this size splits the pile early
     uint32_t thin_rounds;    // ... and takes this many warp-local rounds
     uint32_t tail;           // 1: after a pull pass the rest runs as one unbounded band
@@ -836,7 +837,9 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
     __shared__ unsigned long long trace_snap[SSSP_WARPS][3];
     if (threadIdx.x < SSSP_WARPS * 3) (&trace_snap[0][0])[threadIdx.x] = 0;
     uint32_t it = 0, phase = 0, bands = 0;
-    uint64_t T = a.delta, T_old = 0;
+    // T: the threshold; Tb: the end of the band (T is below it in the first
+    // band's first step)
+    uint64_t Tb = a.delta, T = a.step0 && a.step0 < a.delta ? a.step0 : a.delta, T_old = 0;
     bool first = (blockIdx.x == 0 && threadIdx.x == 0);
     bool hp = false;               // this iteration is a band's heavy-arc pass
     bool pull = false;             // ... in the pull form
@@ -1215,6 +1218,12 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
             if (first) ctl->exit_reason = 1;
             break;
         }
+        // The first band is reached in two steps (a.step0, then its end): a
+        // vertex reached by long light paths is then relaxed when the nearer
+        // ones have settled, not once per improvement.  The band's listings
+        // go on; its heavy arcs follow at its end.
+        const bool step = SCAN && !was_hp && T < Tb && fmin_now < Tb;
+        if (SCAN && T < Tb && !step) T = Tb;           // nothing is left below the band's end
         // Band drained: its heavy arcs first (one more iteration), then the
         // split.  The band lists are cleared in the split, so no block can
         // still be reading their counts here.
@@ -1224,7 +1233,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
         // as n / 8 arcs: coalesced, against one random label per arc).
         // Listings count a vertex once per relaxation, which leans to the
         // pull only when the band is large.
-        if (a.defer && !was_hp && !tail &&
+        if (a.defer && !was_hp && !tail && !step &&
             (ldcg_u32(&ctl->band_count) | ldcg_u32(&ctl->band_hcount)) != 0) {
             hp = true;
             n_light = min(ldcg_u32(&ctl->band_count), a.n);
@@ -1255,7 +1264,11 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
             break;
         }
         T_old = T;
-        T = (fmin != INF32 && (uint64_t)fmin > T ? (uint64_t)fmin : T) + a.delta;
+        if (step) {
+            T = Tb;
+        } else {
+            T = Tb = (fmin != INF32 && (uint64_t)fmin > T ? (uint64_t)fmin : T) + a.delta;
+        }
         ++phase;
         const uint32_t *pile = fc ? a.far1 : a.far0;
         const uint32_t fsn = phase % 3;        // the new phase's far counters
@@ -1264,9 +1277,11 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
             ctl->near_count[(its + 1) % 3] = 0;
             ctl->heavy_count[(its + 1) % 3] = 0;
             ctl->work_next[(its + 1) % 3] = 0;
-            ctl->band_count = 0;
-            ctl->band_hcount = 0;
-            ctl->band_hsum = 0;
+            if (!step) {
+                ctl->band_count = 0;
+                ctl->band_hcount = 0;
+                ctl->band_hsum = 0;
+            }
             ctl->far_count[(phase + 1) % 3] = 0;   // last read a phase ago
             ctl->far_min[(phase + 1) % 3] = INF32;
         }
@@ -1337,7 +1352,8 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
                     // the list keeps to_near and cand vertices, and unreached
                     // ones with arcs (isolated vertices are never reached)
                     keep[c] = to_near[c] || cand[c];
-                    if (in[c] && !valid)
+                    if (step && !from_list) keep[c] = false;       // the band's closing lists them
+                    else if (in[c] && !valid)
                         keep[c] = from_list || a.row_ptr[v[c] + 1] != a.row_ptr[v[c]];
                 } else {
                     keep[c] = cand[c] &&
@@ -1379,7 +1395,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
         }
         it = its;
         cur_dense = dense_out;        // the split set the next frontier's bits
-        listed = SCAN;
+        listed = SCAN && (listed || !step);
         if (it >= a.max_iters) {
             if (first) {
                 atomicOr(&ctl->err, ERR_TIMEOUT);
@@ -1524,6 +1540,20 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     // one vertex per warp only splits early (0.29 against 0.31 ms).  With
     // local rounds asked for the frontier is rarely latency-bound, and the
     // early split only unsettles it (grid 4096 x 4096: 9.7 against 9.25 ms).
+    // The first band's inner threshold (the default band width is 32 mean
+    // weights over the mean degree): on R-MAT graphs the hubs and most of the
+    // core settle below half a mean weight over the mean degree, and with
+    // them settled the rest of the band improves most vertices once.  R-MAT
+    // of 10^6 vertices, k = 101, default band: 54 -> 26 M relaxations, 1.72
+    // -> 1.10 ms (1.06 at a 48th, 1.35 at a 96th of the default width);
+    // R-MAT 24, k = 700: 11.2 -> 6.6 ms.  Bands narrowed by tuning gain less
+    // and take an eighth of themselves: R-MAT 26 (degree 8), k = 10,000 14.2
+    // -> 13.4 ms, R-MAT 22, weights to 10^5, k = 64 2.35 -> 2.04.
+    a.step0 = 0;
+    if (a.defer && p.far_scan) {
+        a.step0 = p.delta > g.delta0 / 8 ? g.delta0 / 64 : p.delta / 8;
+        if (a.step0 < 2) a.step0 = 2;
+    }
     const uint32_t warps = (uint32_t)(geo.sssp_blocks * (geo.threads / 32));
     const bool sparse_rows = g.m <= 8ull * g.n;
     a.thin = p.local_rounds ? 1u : sparse_rows ? 8 * warps : warps;

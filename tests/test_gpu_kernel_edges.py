@@ -153,3 +153,14 @@ def test_batch_pull_pieces_and_tails(queries, batch_delta):
         ref = oracle.steiner(g, s)
         np.testing.assert_array_equal(r.edges, ref.edges)
         assert r.total == ref.total
+
+
+@pytest.mark.parametrize("tail,pull", [(1, 1), (0, 1), (0, 0), (1, 2)])
+@pytest.mark.parametrize("wmax,delta", [(1, 1), (3, 2), (3, 3), (60, 9), (1000, 1000), (70000, 8000)])
+def test_first_band_in_two_steps(wmax, delta, tail, pull):
+    """The inner threshold of the first band: bands no wider than it, just
+    wider, and of the whole weight range, with every form of the heavy pass
+    and with later bands and the tail behind it."""
+    g = wl.rmat(11, 12, wmax=wmax, seed=61)
+    seeds = wl.sample_distinct(wl.largest_cc(g), 24, 62)
+    _check(g, seeds, [("delta", delta), ("tail", tail), ("pull", pull)])
