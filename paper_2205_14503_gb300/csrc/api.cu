@@ -610,6 +610,9 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
         while (nb < n && irp[nb + 1] - irp[nb] >= HEAVY_DEG) ++nb;
         G->g.n_big = nb;
     }
+    G->g.n_live = n;
+    if (relabel)
+        G->g.n_live = (uint32_t)(std::lower_bound(irp, irp + n, (uint32_t)n_arcs) - irp);
     G->g.heavy_chunk_cap = (uint32_t)std::max<uint64_t>(cap, 1);
     if ((e = dalloc(G->g.row_ptr, (uint64_t)n + 1)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     if ((e = dalloc(G->g.adj, n_arcs)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
@@ -679,7 +682,7 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
         const uint64_t arcs = std::min<uint64_t>(std::max<uint64_t>(n_arcs / (16 * warps), ITEM_ARCS_MIN),
                                                  ITEM_ARCS_MAX);
         std::vector<uint32_t> at[2];
-        cut_items(irp, n, arcs, at);
+        cut_items(irp, std::max(G->g.n_live, 1u), arcs, at);
         G->g.n_items = (uint32_t)at[0].size() - 1;
         G->g.n_sparse_items = (uint32_t)at[1].size() - 1;
         e = dalloc(G->g.items, at[0].size());

@@ -58,6 +58,9 @@ struct DevGraph {
     // Vertices with ids at or above n_big have fewer than HEAVY_DEG arcs
     // (the descending-degree order puts the hubs first; n without it).
     uint32_t n_big = 0;
+    // Vertices with ids at or above n_live have no arcs (the degree order
+    // puts them last; n without it).
+    uint32_t n_live = 0;
 };
 
 // The weight-partitioned rows to use for band width delta: built for that

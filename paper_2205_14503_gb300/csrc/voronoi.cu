@@ -82,6 +82,7 @@ struct SsspArgs {
     uint32_t tail;           // 1: after a pull pass the rest runs as one unbounded band
     uint64_t m;              // arcs (the first bound on a pull pass's cost)
     uint32_t n_big;
+    uint32_t n_live;         // ids at or above it have no arcs
     uint32_t n_words;        // bitmap words, ceil(n / 32)
     uint32_t *nbm0, *nbm1;   // near bitmaps, alternating by iteration
     uint32_t *bbm;           // band bitmap
@@ -629,34 +630,49 @@ __device__ __forceinline__ void relax_rows(const SsspArgs &a, Stage &st, const P
     }
 }
 
+// Shared-memory scratch of a pull pass, one per warp, for the 32 * PULL_ILP
+// vertices of a step.
+template <bool NARROW>
+struct PullScratch {
+    typename LabelOf<NARROW>::T best[32 * PULL_ILP];   // best label so far
+    uint2 row[32 * PULL_ILP];       // compacted rows: arc base, vertex of the step
+    uint8_t near[32 * PULL_ILP];    // the vertex has an unsettled neighbour
+};
+
 // Pull form of a band's heavy-arc pass (threshold T, every label below T
-// final).  Warps sweep the vertex ids 32 at a time (coalesced labels), or
-// the candidate list; a vertex at or above T (unreached included) reads
-// the arcs of its heavy part, flattened over the warp, and the labels at
-// their other ends.  The best proposal (d(u) + w, rank(u)) from a settled
-// neighbour u is gathered per vertex in shared memory (pmin: one slot per
-// vertex of the warp's step) and, if it beats the vertex's label, sent as
-// one fire-and-forget atomicMin; it bounds far_min as a far push proposal
-// does.  The sweep also clears the band bitmap that the push form would
-// have read.  The warps' sums of the heavy arcs met go to st.hs (the pass's
-// cost).
+// final).  Warps sweep the vertex ids (coalesced labels), or the candidate
+// list, 32 * PULL_ILP at a step; a vertex at or above T (unreached included)
+// reads the arcs of its heavy part and the labels at their other ends.  The
+// step's rows are flattened over the lanes as in relax_rows, the next group's
+// arc records loaded before this group's labels are waited for.  The best
+// proposal (d(u) + w, rank(u)) from a settled neighbour u is gathered per
+// vertex in shared memory and, if it beats the vertex's label, sent as one
+// fire-and-forget atomicMin; it bounds far_min as a far push proposal does.
+// The sweep also clears the band bitmap that the push form would have read.
+// The warps' sums of the heavy arcs met go to st.hs (the pass's cost).
 // `out` (sweep of every id, no tail): the unsettled vertices with arcs are
 // listed there, the candidates of the split that follows.
-// `tail`: the pass starts the unbounded tail band: every unsettled vertex
-// whose label is now finite joins the next frontier (t), with its whole row.
+// `tail`: the pass starts the unbounded tail band.  A vertex whose neighbours
+// are all settled can improve nothing, so the pass reads whole rows, notes
+// which vertices have an unsettled neighbour, and pushes those of them that
+// are reached (R-MAT 26, degree 8, k = 10,000: 18.5 -> 3.6 M vertices, the
+// first tail iteration 0.89 -> 0.48 ms, the pass 2.49 -> 1.31 ms with the
+// flattened steps).
 template <bool NARROW>
-__device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
-                                       unsigned long long (*pmin)[32 * PULL_ILP], uint64_t T,
-                                       const uint32_t *list, uint32_t count, uint32_t *out,
-                                       uint32_t *out_count, bool tail, uint32_t *nbm,
-                                       uint32_t *qn, uint32_t *qn_count, uint64_t *hqn,
-                                       uint32_t *hqn_count, uint32_t &attempts,
+__device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st, PullScratch<NARROW> *scratch,
+                                       uint64_t T, const uint32_t *list, uint32_t count,
+                                       uint32_t *out, uint32_t *out_count, bool tail,
+                                       uint32_t *nbm, uint32_t *qn, uint32_t *qn_count,
+                                       uint64_t *hqn, uint32_t *hqn_count, uint32_t &attempts,
                                        uint32_t &improved, bool &narrow_miss) {
+    using L = typename LabelOf<NARROW>::T;
+    constexpr L UNREACHED = (L)~0ull;
     const uint32_t lane = lane_id();
     const uint32_t wib = threadIdx.x >> 5;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    unsigned long long *pm = pmin[wib];
+    PullScratch<NARROW> &sc = scratch[wib];
+    const L Tl = (L)threshold_label<NARROW>(a, T);
     // where the tail's first frontier goes (light vertices as bits when dense)
     PushTargets t;
     t.qn = qn;
@@ -671,42 +687,42 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
     t.hsum = nullptr;
     t.lend = nullptr;
     uint32_t met = 0;
-    uint32_t fmin = INF32;
-    // the vertices: every id, or the candidate list (then the band bitmap
-    // is cleared by a sweep of its own)
+    L fmin = UNREACHED;
+    // the vertices: every id that may have arcs, or the candidate list (then
+    // the band bitmap is cleared by a sweep of its own)
     if (list && a.dense)
         for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n_words;
              i += gridDim.x * blockDim.x)
             if (ldcg_u32(&a.bbm[i])) a.bbm[i] = 0;
-    const uint32_t nv = list ? count : a.n;
-    // PULL_ILP chunks of 32 vertices per warp step, their loads issued together
+    const uint32_t nv = list ? count : a.n_live;
     for (uint32_t b = warp * 32 * PULL_ILP; b < nv; b += nwarps * 32 * PULL_ILP) {
         if (!list && a.dense && lane < PULL_ILP && (b >> 5) + lane < a.n_words &&
             ldcg_u32(&a.bbm[(b >> 5) + lane]))
             a.bbm[(b >> 5) + lane] = 0;
         uint32_t vs[PULL_ILP];
-        uint64_t lab[PULL_ILP];
+        L lab[PULL_ILP];
         uint32_t s[PULL_ILP], r1[PULL_ILP], r0[PULL_ILP];
 #pragma unroll
         for (int c = 0; c < PULL_ILP; ++c) {
             const uint32_t i = b + 32u * c + lane;
             vs[c] = i < nv ? (list ? ldcg_u32(&list[i]) : i) : INF32;
-            pm[32 * c + lane] = INF64;
         }
 #pragma unroll
         for (int c = 0; c < PULL_ILP; ++c)    // past the end: taken as settled
-            lab[c] = vs[c] != INF32 ? sssp_label<NARROW>(a, vs[c]) : 0ull;
+            lab[c] = vs[c] != INF32 ? raw_label<NARROW>(a, vs[c]) : (L)0;
         bool uns[PULL_ILP];
 #pragma unroll
         for (int c = 0; c < PULL_ILP; ++c) {
             const uint32_t v = vs[c];
             s[c] = r1[c] = r0[c] = 0;
-            uns[c] = lab[c] == INF64 || (lab[c] >> 32) >= T;
+            uns[c] = lab[c] >= Tl;
             if (uns[c]) {
                 r1[c] = a.row_ptr[v + 1];
                 r0[c] = a.row_ptr[v];
                 s[c] = a.lend ? a.lend[v] : r0[c];
             }
+            sc.best[32 * c + lane] = lab[c];
+            sc.near[32 * c + lane] = 0;
         }
         if (out) {
             // the sweep over every id lists the unsettled vertices with arcs
@@ -718,54 +734,94 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
                               &st.band_n[wib], BAND_REGION, true, out, out_count, a.n,
                               &a.ctl->err);
         }
-        __syncwarp();
+        // the step's rows, compacted: rows with arcs in order, their first
+        // positions in excl
+        uint32_t excl[PULL_ILP], rows = 0, total = 0;
 #pragma unroll
         for (int c = 0; c < PULL_ILP; ++c) {
-            const uint32_t deg = r1[c] - s[c];
-            met += deg;
+            met += r1[c] - s[c];
+            const uint32_t from = tail ? r0[c] : s[c], deg = r1[c] - from;
+            const uint32_t m = __ballot_sync(FULL, deg != 0);
             const uint32_t incl = warp_inclusive_scan(deg);
-            const uint32_t excl = incl - deg;
-            const uint32_t total = __shfl_sync(FULL, incl, 31);
-            for (uint32_t j0 = 0; j0 < total; j0 += 32 * ILP) {
-                bool valid[ILP];
-                uint32_t slot[ILP];
-                uint64_t hl[ILP];
-                uint2 e[ILP];
+            excl[c] = deg ? total + incl - deg : INF32;
+            if (deg)
+                sc.row[rows + (uint32_t)__popc(m & lanemask_lt())] =
+                    make_uint2(from - excl[c], 32u * c + lane);
+            rows += (uint32_t)__popc(m);
+            total += __shfl_sync(FULL, incl, 31);
+        }
+        __syncwarp();
+        uint32_t before = 0;           // rows that start before the window
+        auto load = [&](uint32_t j0, uint2 (&e)[ILP], uint32_t (&slot)[ILP]) {
 #pragma unroll
-                for (int q = 0; q < ILP; ++q) {
-                    const uint32_t j = j0 + lane + 32 * q;
-                    valid[q] = j < total;
-                    const uint32_t owner = warp_owner_search(excl, valid[q] ? j : 0);
-                    const uint32_t so = __shfl_sync(FULL, s[c], owner);
-                    const uint32_t eo = __shfl_sync(FULL, excl, owner);
-                    hl[q] = __shfl_sync(FULL, lab[c], owner);
-                    slot[q] = 32u * c + owner;
-                    e[q] = make_uint2(0, 0);
-                    // the unsettled rows are read once per pass: streamed
-                    if (valid[q]) e[q] = __ldcs(&a.adj[so + (j - eo)]);
+            for (int q = 0; q < ILP; ++q) {
+                const uint32_t w0 = j0 + 32 * q, j = w0 + lane;
+                uint32_t starts = 0;
+#pragma unroll
+                for (int c = 0; c < PULL_ILP; ++c)
+                    if (excl[c] - w0 < 32) starts |= 1u << (excl[c] - w0);
+                starts = __reduce_or_sync(FULL, starts);
+                const uint32_t row = before + (uint32_t)__popc(starts & (FULL >> (31 - lane))) - 1;
+                before += (uint32_t)__popc(starts);
+                e[q] = make_uint2(0, 0);                  // weight 0: no arc
+                slot[q] = 0;
+                if (j < total) {
+                    const uint2 r = sc.row[row];
+                    slot[q] = r.y;
+                    e[q] = __ldcs(&a.adj[r.x + j]);       // read once per pass: streamed
                 }
-                uint64_t tl[ILP];
+            }
+        };
+        uint2 e[ILP];
+        uint32_t slot[ILP];
+        if (total) load(0, e, slot);
+        for (uint32_t j0 = 0; j0 < total; j0 += 32 * ILP) {
+            L tl[ILP];
 #pragma unroll
-                for (int q = 0; q < ILP; ++q) {
-                    tl[q] = INF64;
-                    if (valid[q] && e[q].y >= a.delta) tl[q] = sssp_label<NARROW>(a, e[q].x);
-                }
+            for (int q = 0; q < ILP; ++q) {
+                tl[q] = 0;
+                if (e[q].y && (tail || e[q].y >= a.delta)) tl[q] = raw_label<NARROW>(a, e[q].x);
+            }
+            uint2 en[ILP];
+            uint32_t sn[ILP];
+            const bool more = j0 + 32 * ILP < total;
+            if (more) load(j0 + 32 * ILP, en, sn);
 #pragma unroll
-                for (int q = 0; q < ILP; ++q) {
-                    // an unsettled (or unreached) neighbour proposes nothing yet
-                    if (!valid[q] || tl[q] == INF64 || (tl[q] >> 32) >= T) continue;
+            for (int q = 0; q < ILP; ++q) {
+                // an unsettled (or unreached) neighbour proposes nothing yet
+                if (tl[q] >= Tl) {
+                    sc.near[slot[q]] = 1;
+                } else if (e[q].y && e[q].y >= a.delta) {
                     ++attempts;
-                    const uint64_t nd = (tl[q] >> 32) + (uint64_t)e[q].y;
-                    if (NARROW && nd > a.ldmax) {
-                        // only an unreached vertex could take it (a narrow
-                        // label's distance is at most ldmax): the host
-                        // reruns the query with 64-bit labels
-                        if (hl[q] == INF64) narrow_miss = true;
-                        continue;
+                    L nl;
+                    if constexpr (NARROW) {
+                        const uint64_t sum = (uint64_t)e[q].y * a.lstep + tl[q];
+                        nl = (uint32_t)sum;
+                        if (sum >= a.lmiss) {
+                            // only an unreached vertex could take it (a narrow
+                            // label's distance is at most ldmax): the host
+                            // reruns the query with 64-bit labels
+                            if (sc.best[slot[q]] == UNREACHED) narrow_miss = true;
+                            continue;
+                        }
+                    } else {
+                        const uint64_t nd = (tl[q] >> 32) + (uint64_t)e[q].y;
+                        if (nd >= INF32) continue;        // the scan reports the overflow
+                        nl = (nd << 32) | (tl[q] & 0xFFFFFFFFull);
                     }
-                    if (nd >= INF32) continue;         // the scan reports the overflow
-                    const uint64_t nl64 = (nd << 32) | (tl[q] & 0xFFFFFFFFull);
-                    if (nl64 < hl[q]) atomicMin(&pm[slot[q]], (unsigned long long)nl64);
+                    if constexpr (NARROW) {
+                        if (nl < *(volatile uint32_t *)&sc.best[slot[q]]) atomicMin(&sc.best[slot[q]], nl);
+                    } else {
+                        auto *best = reinterpret_cast<unsigned long long *>(&sc.best[slot[q]]);
+                        if (nl < *(volatile unsigned long long *)best) atomicMin(best, (unsigned long long)nl);
+                    }
+                }
+            }
+            if (more) {
+#pragma unroll
+                for (int q = 0; q < ILP; ++q) {
+                    e[q] = en[q];
+                    slot[q] = sn[q];
                 }
             }
         }
@@ -777,22 +833,18 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
         for (int c = 0; c < PULL_ILP; ++c) {
             push[c] = false;
             pdeg[c] = 0;
-            const uint64_t best = pm[32 * c + lane];
-            uint64_t now = lab[c];
+            const L best = sc.best[32 * c + lane];
             if (uns[c] && best < lab[c]) {
-                if (NARROW)
-                    atomicMin(&a.label32[vs[c]],
-                              ((uint32_t)(best >> 32) << a.lshift) | (uint32_t)best);
-                else
-                    atomicMin(reinterpret_cast<unsigned long long *>(&a.label[vs[c]]),
-                              (unsigned long long)best);
-                    ++improved;
-                fmin = min(fmin, (uint32_t)(best >> 32));
-                now = best;
+                if constexpr (NARROW) atomicMin(&a.label32[vs[c]], best);
+                else atomicMin(reinterpret_cast<unsigned long long *>(&a.label[vs[c]]),
+                               (unsigned long long)best);
+                ++improved;
+                fmin = min(fmin, best);
             }
             if (tail) {
-                // reached and unsettled: the tail's first frontier, whole rows
-                const bool want = uns[c] && now != INF64 && r1[c] != r0[c];
+                // reached, unsettled and next to an unsettled vertex: the
+                // tail's first frontier, whole rows
+                const bool want = uns[c] && best != UNREACHED && sc.near[32 * c + lane];
                 const uint32_t deg = r1[c] - r0[c];
                 const bool bit = t.dense && want && deg < HEAVY_DEG;
                 const uint32_t word = __ballot_sync(FULL, bit);
@@ -810,10 +862,11 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st,
         __syncwarp();
     }
     met = __reduce_add_sync(FULL, met);
-    fmin = __reduce_min_sync(FULL, fmin);
+    uint32_t fd = fmin == UNREACHED ? INF32 : (uint32_t)(NARROW ? fmin >> a.lshift : (uint64_t)fmin >> 32);
+    fd = __reduce_min_sync(FULL, fd);
     if (lane == 0) {
         st.hs[wib] += met;
-        if (fmin != INF32) atomicMin(&st.far_min, fmin);
+        if (fd != INF32) atomicMin(&st.far_min, fd);
     }
 }
 
@@ -854,7 +907,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
     // by short chains, and a few iterations reach the fixed point that a
     // band per delta would approach in many splits.
     bool tail = false;
-    __shared__ unsigned long long pmin[SSSP_WARPS][32 * PULL_ILP];   // pull pass minima
+    __shared__ PullScratch<NARROW> pull_scratch[SCAN ? SSSP_WARPS : 1];
     // heavy arcs a pull pass would read now, bounded from above: all arcs
     // at first, then what the last pull pass met (the unsettled set only
     // shrinks)
@@ -959,7 +1012,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
         if (SCAN && hp && pull) {
             uint32_t *pile = fc ? a.far1 : a.far0;
             // with the tail to follow, the pass pushes its first frontier
-            pull_pass<NARROW>(a, st, pmin, T, listed ? pile : nullptr,
+            pull_pass<NARROW>(a, st, pull_scratch, T, listed ? pile : nullptr,
                               listed ? min(ldcg_u32(&ctl->far_count[fs]), a.n) : a.n,
                               (listed || a.tail) ? nullptr : pile, &ctl->far_count[fs],
                               a.tail != 0, t.nbm, t.qn, t.qn_count, t.hqn, t.hqn_count,
@@ -1315,7 +1368,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
         }
         stage_reset(st);
         // the far pile (or list), or with the far scan first every vertex
-        const uint32_t n_split = (SCAN && !from_list) ? a.n : nf;
+        const uint32_t n_split = (SCAN && !from_list) ? a.n_live : nf;
         // SPLIT_ILP chunks of 32 per warp step, their loads issued together.
         // A vertex is met once here (the pile holds it once, the scan visits
         // each id once) and nothing relaxes during the split, so its near
@@ -1559,6 +1612,7 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.thin = p.local_rounds ? 1u : sparse_rows ? 8 * warps : warps;
     a.thin_rounds = sparse_rows ? 16u : 0u;
     a.n_big = g.n_big;
+    a.n_live = g.n_live;
     a.n_words = (g.n + 31) / 32;
     a.nbm0 = ws.nbm[0];
     a.nbm1 = ws.nbm[1];

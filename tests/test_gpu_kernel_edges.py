@@ -164,3 +164,24 @@ def test_first_band_in_two_steps(wmax, delta, tail, pull):
     g = wl.rmat(11, 12, wmax=wmax, seed=61)
     seeds = wl.sample_distinct(wl.largest_cc(g), 24, 62)
     _check(g, seeds, [("delta", delta), ("tail", tail), ("pull", pull)])
+
+
+@pytest.mark.parametrize("relabel", ["0", "1"])
+@pytest.mark.parametrize("n", [64, 127, 128, 129, 641, 3000])
+def test_pull_steps_and_tail_frontier(n, relabel, monkeypatch):
+    """The pull pass takes 128 vertices a step and skips ids without arcs;
+    the tail starts from the vertices with an unsettled neighbour: sizes
+    around a step, isolated vertices, a leaf chain behind the core, and both
+    vertex orders and label widths."""
+    monkeypatch.setenv("STEINER_RELABEL", relabel)
+    r = G.rng(n)
+    core = max(8, n // 3)
+    u = list(r.integers(0, core, 6 * core)) + list(range(core, 2 * core - 1))
+    v = list(r.integers(0, core, 6 * core)) + list(range(core + 1, 2 * core))
+    w = list(r.integers(1, 200, 6 * core)) + list(r.integers(1, 400, core - 1))
+    g = wl.from_edges(n, np.array(u + [0]), np.array(v + [core]), np.array(w + [300]))
+    for tail in (0, 1):
+        for bits in (32, 64):
+            _check(g, G.seeds_from(np.arange(2 * core), 5, n),
+                   [("delta", 30), ("pull", 2), ("tail", tail), ("label_bits", bits)])
+
