@@ -115,7 +115,8 @@ typedef struct {
  * result (tree edges, pair arcs, cell/dist/pred) is still in the caller's
  * vertex ids and arc indices, and the tie rules use the caller's order.
  * The environment variable STEINER_RELABEL=0 or 1, read here, forces this
- * internal order off or on; STEINER_DELTA=<n> sets the initial band width
+ * internal order off or on, STEINER_TREE_SCAN=0 or 1 steiner_query's scan of
+ * only the arcs that the tree can need; STEINER_DELTA=<n> sets the initial band width
  * (default 32 x mean weight / mean degree; "delta" below changes it later).
  * With STEINER_TRACE set, each single query prints its Voronoi loop's exit
  * reason and its first iterations' frontier sizes to stderr.

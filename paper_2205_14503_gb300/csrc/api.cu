@@ -225,6 +225,7 @@ int ensure_k_workspace(steiner_graph *G, uint32_t k, bool with_pairtab = true) {
         CK(dalloc(ws.tile_off, tiles));
         ws.tile_cap = (uint32_t)tiles;
     }
+    if (!ws.hub) CK(dalloc(ws.hub, 1));
     if (k > ws.comp_cap) {
         CK(dalloc(ws.comp, k));
         CK(dalloc(ws.hook, k));
@@ -303,9 +304,11 @@ int read_result(steiner_graph *G, Workspace &ws, bool small) {
 }
 
 // Runs Steps 1 (and, with `full`, 2-7) of Algorithm 2 for one sorted seed
-// list with the label width in G->ws.narrow.  Leaves the control block in
+// list with the label width in G->ws.narrow; `tree_only`: the tree is all the
+// caller wants of it.  Leaves the control block in
 // G->h_ctl.
-int run_pipeline_once(steiner_graph *G, const std::vector<int32_t> &ss, bool full, float *ms) {
+int run_pipeline_once(steiner_graph *G, const std::vector<int32_t> &ss, bool full, bool tree_only,
+                      float *ms) {
     uint32_t k = (uint32_t)ss.size();
     int rc = ensure_n_workspace(G);
     if (rc) return rc;
@@ -332,15 +335,17 @@ int run_pipeline_once(steiner_graph *G, const std::vector<int32_t> &ss, bool ful
     CK(mark(1));
     CK(launch_sssp(G->g, ws, G->geo, p, s));
     CK(mark(2));
-    CK(launch_scan(G->g, ws, k, full, s));
+    const bool pruned = full && tree_only && tree_scan_applies(G->g, ws, k, G->delta);
+    if (pruned) CK(launch_tree_scan(G->g, ws, k, G->delta, G->geo, s));
+    else CK(launch_scan(G->g, ws, k, full, s));
     uint32_t launches = 4;      // init labels, init seeds, SSSP, scan
     const bool small = full && small_tail(k);
     if (full && !small) {
         CK(launch_compact_pairs(ws, k, s));
         CK(mark(3));
-        CK(launch_mst(ws, k, G->geo, s));
+        CK(launch_mst(ws, k, G->geo, INF64, s));
         CK(mark(4));
-        CK(launch_tree(G->g, ws, k, ws.epoch_mark, G->nbits, s));
+        CK(launch_tree(G->g, ws, k, ws.epoch_mark, G->nbits, pruned ? G->delta : 0u, s));
         if (k > 1) launches += 3 + 1 + 2;   // compaction, MST, expansion + sort
     } else {
         CK(mark(3));
@@ -367,7 +372,8 @@ int run_pipeline_once(steiner_graph *G, const std::vector<int32_t> &ss, bool ful
 // (dist << rank bits) | rank; if a distance did not fit (ERR_NARROW) the
 // query runs again with 64-bit labels, so the result never depends on the
 // width.  ms[] (if given) sums both attempts.
-int run_pipeline(steiner_graph *G, const std::vector<int32_t> &ss, bool full, float *ms) {
+int run_pipeline(steiner_graph *G, const std::vector<int32_t> &ss, bool full, bool tree_only,
+                 float *ms) {
     const uint32_t k = (uint32_t)ss.size();
     const uint32_t rbits = bits_for(k);
     const uint32_t dbits = 32 - rbits;
@@ -377,7 +383,7 @@ int run_pipeline(steiner_graph *G, const std::vector<int32_t> &ss, bool full, fl
     else narrow = dbits >= bit_length(G->g.max_w) + 8 && dbits > G->narrow_fail_dbits;
     G->ws.narrow = narrow;
     G->ws.lshift = rbits;
-    int rc = run_pipeline_once(G, ss, full, ms);
+    int rc = run_pipeline_once(G, ss, full, tree_only, ms);
     G->last_label_bits = narrow ? 32 : 64;
     if (rc || !narrow || !(G->h_ctl->err & ERR_NARROW)) return rc;
     ++G->narrow_reruns;
@@ -385,7 +391,7 @@ int run_pipeline(steiner_graph *G, const std::vector<int32_t> &ss, bool full, fl
     G->ws.narrow = false;
     G->last_label_bits = 64;
     float ms2[6] = {0, 0, 0, 0, 0, 0};
-    rc = run_pipeline_once(G, ss, full, ms ? ms2 : nullptr);
+    rc = run_pipeline_once(G, ss, full, tree_only, ms ? ms2 : nullptr);
     if (ms)
         for (int i = 0; i < 6; ++i) ms[i] += ms2[i];
     return rc;
@@ -433,7 +439,8 @@ int query_locked(steiner_graph *G, const int32_t *seeds, uint32_t k, steiner_res
     int rc = sorted_seed_list(G, seeds, k, ss);
     if (rc) return out->status = rc;
     float ms[6] = {0, 0, 0, 0, 0, 0};
-    rc = run_pipeline(G, ss, true, stats ? ms : nullptr);
+    // the counters and G'_1 need every pair of adjacent cells
+    rc = run_pipeline(G, ss, true, !pairs && !stats, stats ? ms : nullptr);
     if (rc) return out->status = rc;
     const Control c = *G->h_ctl;
     rc = status_from(c, k, true);
@@ -705,6 +712,7 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     double d = 32.0 * std::max(1.0, avg_w) / std::max(1.0, avg_deg);
     G->delta = (uint32_t)std::min(std::max(d, 1.0), 1.0e9);
     G->g.delta0 = G->delta;
+    if (const char *env = getenv("STEINER_TREE_SCAN")) G->g.tree_scan = atoi(env) != 0;
     if (const char *env = getenv("STEINER_DELTA")) G->delta = (uint32_t)std::max(1L, atol(env));
     *out = G;
     return STEINER_OK;
@@ -723,7 +731,7 @@ void steiner_free_graph(steiner_graph_t G) {
     void *bufs[] = {ws.label, ws.label32, ws.nbm[0], ws.nbm[1], ws.bbm, ws.pred_arc, ws.stamp_near, ws.stamp_far, ws.stamp_band, ws.band_q,
                     ws.band_hq, ws.mark, ws.q[0], ws.q[1],
                     ws.hq[0], ws.hq[1], ws.far[0], ws.far[1], ws.result, ws.seeds, ws.pairtab,
-                    ws.e_key, ws.e_ra, ws.e_rb, ws.e_arc, ws.e_mst, ws.tile_off, ws.comp, ws.hook,
+                    ws.e_key, ws.e_ra, ws.e_rb, ws.e_arc, ws.e_mst, ws.tile_off, ws.comp, ws.hook, ws.hub,
                     ws.best, ws.tree_key, ws.tree_key2, ws.tree_w, ws.tree_w2, G->g.row_ptr,
                     G->g.adj, G->g.heavy_chunks, G->g.orig_row_ptr, G->g.orig_of, G->g.new_of,
                     G->g.adj_w, G->g.lend, G->g.items, G->g.sparse_items};
@@ -822,7 +830,7 @@ int steiner_voronoi(steiner_graph_t G, const int32_t *seeds, uint32_t k, int32_t
     std::vector<int32_t> ss;
     int rc = sorted_seed_list(G, seeds, k, ss);
     if (rc) return rc;
-    rc = run_pipeline(G, ss, false, nullptr);
+    rc = run_pipeline(G, ss, false, false, nullptr);
     if (rc) return rc;
     Control c = *G->h_ctl;
     rc = status_from(c, k, false);
@@ -890,8 +898,8 @@ int api_run_tail(steiner_graph *G, uint64_t *pairtab, uint32_t *pred_base, uint3
         CK(launch_small_tail(G->g, v, k, G->ws.epoch_mark, G->nbits, s));
     } else {
         CK(launch_compact_pairs(v, k, s));
-        CK(launch_mst(v, k, G->geo, s));
-        CK(launch_tree(G->g, v, k, G->ws.epoch_mark, G->nbits, s));
+        CK(launch_mst(v, k, G->geo, INF64, s));
+        CK(launch_tree(G->g, v, k, G->ws.epoch_mark, G->nbits, 0u, s));
     }
     rc = read_result(G, v, small_tail(k));
     if (rc) return out->status = rc;

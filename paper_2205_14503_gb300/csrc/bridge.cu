@@ -161,6 +161,245 @@ __global__ void __launch_bounds__(256) scan_kernel(ScanArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// the scan of a query that returns the tree alone
+// ---------------------------------------------------------------------------
+//
+// A tree needs the MST of G'_1, not all of G'_1, and predecessors only along
+// tight arcs, which are no heavier than their head's distance.  With rows
+// split at band width delta, most arcs of a large graph are heavy arcs
+// between vertices nearer than delta, and most of those join cells that
+// lighter bridges have already joined:
+//
+//  1. tree_scan_kernel reads every arc but the heavy ones (weight delta or
+//     more) between two vertices nearer than delta: the light part of a row
+//     whose vertex is nearer than delta, the whole row otherwise.  That gives
+//     every predecessor, and every pair whose minimum bridge is below delta
+//     (such a bridge's arc is lighter than delta).
+//  2. The MST of those pairs is the part of Kruskal's tree below delta.  Of
+//     its components the one whose cells hold the most unread arcs (sampled)
+//     is the hub.
+//  3. rest_scan_kernel reads the unread arcs of the vertices outside the
+//     hub's cells.  Every arc between two components has such an end, so the
+//     minimum bridge of every pair of cells in different components is now
+//     in the table; pairs inside a component may have been left at a larger
+//     bridge or none, but the component's own tree joins them by bridges
+//     below delta, so they cannot be in the MST.
+//  4. The MST of all pairs in the table is then the MST of G'_1.
+//
+// A bridge key carries the caller's index of its arc, which a row split by
+// weight does not give: it is searched in the id-ordered row, for proposals
+// that lower the table (first with an index above all, so that few others
+// search).  Narrow labels only: their distances rule out an overflow.
+
+struct TreeScanArgs {
+    const uint32_t *__restrict__ row_ptr;
+    const uint2 *__restrict__ adj;       // rows in the caller's order
+    const uint2 *__restrict__ adj_w;     // rows with the light arcs first
+    const uint32_t *__restrict__ lend;   // end of the light part
+    const uint64_t *__restrict__ heavy_chunks;
+    uint32_t n_heavy_chunks;
+    const uint32_t *__restrict__ items;
+    uint32_t n_items;
+    uint32_t delta;
+    uint32_t near;                       // smallest label of a distance delta
+    const uint32_t *label32;
+    uint32_t lshift;
+    uint32_t *pred_arc;                  // index in adj_w (vertex nearer than delta) or adj
+    uint64_t *pairtab;
+    uint32_t k;
+    const uint32_t *orig_of, *orig_row_ptr;
+    const uint32_t *comp;                // per cell: component of the light pairs' MST
+    const uint32_t *hub;                 // the hub component
+};
+
+// The caller's index of arc x -> y.
+__device__ __forceinline__ uint32_t caller_arc(const TreeScanArgs &a, uint32_t x, uint32_t y) {
+    const uint32_t rs = a.row_ptr[x], want = caller_id(a.orig_of, y);
+    uint32_t lo = rs, hi = a.row_ptr[x + 1];
+    while (hi - lo > 1) {                // largest arc whose head is at or before y
+        const uint32_t mid = lo + (hi - lo) / 2;
+        if (caller_id(a.orig_of, a.adj[mid].x) <= want) lo = mid;
+        else hi = mid;
+    }
+    return caller_arc_base(a.orig_of, a.orig_row_ptr, x, rs) + lo;
+}
+
+// Proposes bridge b over arc x -> y (x in the cell of smaller rank).
+__device__ __forceinline__ void propose_bridge(const TreeScanArgs &a, uint32_t cx, uint32_t cy,
+                                               uint64_t b, uint32_t x, uint32_t y) {
+    auto *slot = reinterpret_cast<unsigned long long *>(&a.pairtab[pair_slot(cx, cy, a.k)]);
+    if (b > __ldg(slot) >> 32) return;
+    if (b > atomicMin(slot, (b << 32) | INF32) >> 32) return;
+    atomicMin(slot, (b << 32) | caller_arc(a, x, y));
+}
+
+__device__ __forceinline__ void tree_arc(const TreeScanArgs &a, uint32_t v, uint32_t lv, bool whole,
+                                         uint32_t cbase, uint32_t arc, uint2 e) {
+    const uint32_t lu = __ldg(&a.label32[e.x]);
+    if (lu == INF32) return;
+    const uint64_t sum = ((uint64_t)e.y << a.lshift) + lu;       // the head's distance + w
+    if (sum == lv) atomicMin(&a.pred_arc[v], arc);
+    const uint32_t mask = (1u << a.lshift) - 1u, cv = lv & mask, cu = lu & mask;
+    if (cv == cu) return;
+    const uint64_t b = (lv >> a.lshift) + (sum >> a.lshift);
+    if (cv < cu) {
+        if (whole) {
+            auto *slot = reinterpret_cast<unsigned long long *>(&a.pairtab[pair_slot(cv, cu, a.k)]);
+            const unsigned long long key = (b << 32) | (uint32_t)(cbase + arc);
+            if (key < __ldg(slot)) atomicMin(slot, key);
+        } else {
+            propose_bridge(a, cv, cu, b, v, e.x);
+        }
+    } else if (whole && e.y >= a.delta && lu < a.near) {
+        propose_bridge(a, cu, cv, b, e.x, v);        // the head does not read this arc
+    }
+}
+
+__global__ void __launch_bounds__(256) tree_scan_kernel(const __grid_constant__ TreeScanArgs a) {
+    const uint32_t lane = lane_id();
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t n_work = a.n_heavy_chunks + a.n_items;
+    for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
+        if (wi < a.n_heavy_chunks) {
+            const uint64_t item = a.heavy_chunks[wi];
+            const uint32_t v = (uint32_t)(item >> 32), c = (uint32_t)item;
+            const uint32_t lv = __ldg(&a.label32[v]);
+            if (lv == INF32) continue;
+            const bool whole = lv >= a.near;
+            const uint32_t rs = a.row_ptr[v], end = whole ? a.row_ptr[v + 1] : a.lend[v];
+            const uint32_t s = rs + c * CHUNK, e = min(end, s + CHUNK);
+            if (s >= end) continue;
+            const uint2 *arcs = whole ? a.adj : a.adj_w;
+            const uint32_t cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, rs);
+            uint2 en = make_uint2(0, 0);
+            if (s + lane < e) en = __ldcs(&arcs[s + lane]);
+            for (uint32_t b = s; b < e; b += 32) {
+                const uint2 ec = en;
+                if (b + 32 + lane < e) en = __ldcs(&arcs[b + 32 + lane]);
+                if (b + lane < e) tree_arc(a, v, lv, whole, cbase, b + lane, ec);
+            }
+            continue;
+        }
+        const uint32_t v1 = __ldg(&a.items[wi - n_work + a.n_items + 1]);
+        for (uint32_t vb = __ldg(&a.items[wi - n_work + a.n_items]); vb < v1; vb += 32) {
+            const uint32_t v = vb + lane;
+            uint32_t s = 0, deg = 0, cbase = 0, lv = INF32;
+            if (v < v1) {
+                lv = __ldg(&a.label32[v]);
+                if (lv != INF32) {
+                    s = a.row_ptr[v];
+                    const uint32_t r1 = a.row_ptr[v + 1];
+                    deg = r1 - s >= HEAVY_DEG ? 0u : (lv >= a.near ? r1 : a.lend[v]) - s;
+                    if (deg && lv >= a.near) cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, s);
+                }
+            }
+            const uint32_t incl = warp_inclusive_scan(deg);
+            const uint32_t excl = incl - deg;
+            const uint32_t total = __shfl_sync(FULL, incl, 31);
+            for (uint32_t b = 0; b < total; b += 32) {
+                const uint32_t j = b + lane;
+                const uint32_t own = warp_owner_search(excl, j < total ? j : 0);
+                const uint32_t arc = __shfl_sync(FULL, s, own) + (j - __shfl_sync(FULL, excl, own));
+                const uint32_t lo = __shfl_sync(FULL, lv, own), co = __shfl_sync(FULL, cbase, own);
+                const bool whole = lo >= a.near;
+                if (j >= total) continue;
+                tree_arc(a, vb + own, lo, whole, co, arc, __ldcs(&(whole ? a.adj : a.adj_w)[arc]));
+            }
+        }
+    }
+}
+
+// The unread arcs (heavy part of a row whose vertex is nearer than delta) of
+// the vertices outside the hub component's cells.
+__global__ void __launch_bounds__(256) rest_scan_kernel(const __grid_constant__ TreeScanArgs a) {
+    const uint32_t lane = lane_id();
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t n_work = a.n_heavy_chunks + a.n_items;
+    const uint32_t hub = *a.hub, mask = (1u << a.lshift) - 1u;
+    auto arc = [&](uint32_t v, uint32_t lv, uint32_t cc, uint2 e) {
+        const uint32_t lu = __ldg(&a.label32[e.x]);
+        if (lu >= a.near || __ldg(&a.comp[lu & mask]) == cc) return;
+        const uint32_t cv = lv & mask, cu = lu & mask;
+        const uint64_t b = (uint64_t)(lv >> a.lshift) + e.y + (lu >> a.lshift);
+        if (cv < cu) propose_bridge(a, cv, cu, b, v, e.x);
+        else propose_bridge(a, cu, cv, b, e.x, v);
+    };
+    for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
+        if (wi < a.n_heavy_chunks) {
+            const uint64_t item = a.heavy_chunks[wi];
+            const uint32_t v = (uint32_t)(item >> 32), c = (uint32_t)item;
+            const uint32_t lv = __ldg(&a.label32[v]);
+            if (lv >= a.near) continue;
+            const uint32_t cc = __ldg(&a.comp[lv & mask]);
+            if (cc == hub) continue;
+            const uint32_t r1 = a.row_ptr[v + 1];
+            const uint32_t s = a.lend[v] + c * CHUNK, e = min(r1, s + CHUNK);
+            for (uint32_t j = s + lane; s < r1 && j < e; j += 32) arc(v, lv, cc, __ldcs(&a.adj_w[j]));
+            continue;
+        }
+        const uint32_t v1 = __ldg(&a.items[wi - n_work + a.n_items + 1]);
+        for (uint32_t vb = __ldg(&a.items[wi - n_work + a.n_items]); vb < v1; vb += 32) {
+            const uint32_t v = vb + lane;
+            uint32_t s = 0, deg = 0, lv = INF32, cc = hub;
+            if (v < v1) {
+                lv = __ldg(&a.label32[v]);
+                if (lv < a.near) cc = __ldg(&a.comp[lv & mask]);
+                if (cc != hub) {
+                    s = a.lend[v];
+                    const uint32_t r1 = a.row_ptr[v + 1];
+                    deg = r1 - a.row_ptr[v] >= HEAVY_DEG ? 0u : r1 - s;
+                }
+            }
+            if (!__any_sync(FULL, deg)) continue;
+            const uint32_t incl = warp_inclusive_scan(deg);
+            const uint32_t excl = incl - deg;
+            const uint32_t total = __shfl_sync(FULL, incl, 31);
+            for (uint32_t b = 0; b < total; b += 32) {
+                const uint32_t j = b + lane;
+                const uint32_t own = warp_owner_search(excl, j < total ? j : 0);
+                const uint32_t at = __shfl_sync(FULL, s, own) + (j - __shfl_sync(FULL, excl, own));
+                const uint32_t lo = __shfl_sync(FULL, lv, own), co = __shfl_sync(FULL, cc, own);
+                if (j < total) arc(vb + own, lo, co, __ldcs(&a.adj_w[at]));
+            }
+        }
+    }
+}
+
+// Unread arcs per component, by a sample of arcs spread over all of them.
+constexpr uint32_t HUB_SAMPLES = 1u << 15;
+__global__ void hub_sample_kernel(const __grid_constant__ TreeScanArgs a, uint32_t n, uint64_t m,
+                                  uint32_t *count) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= HUB_SAMPLES) return;
+    const uint32_t arc = (uint32_t)(m * i / HUB_SAMPLES);
+    uint32_t lo = 0, hi = n;             // largest v with row_ptr[v] <= arc
+    while (hi - lo > 1) {
+        const uint32_t mid = lo + (hi - lo) / 2;
+        if (a.row_ptr[mid] <= arc) lo = mid;
+        else hi = mid;
+    }
+    const uint32_t lv = a.label32[lo];
+    if (lv < a.near && arc >= a.lend[lo]) atomicAdd(&count[a.comp[lv & ((1u << a.lshift) - 1u)]], 1u);
+}
+
+// The component with the largest count (one block).
+__global__ void __launch_bounds__(1024) hub_pick_kernel(const uint32_t *count, uint32_t k, uint32_t *hub) {
+    __shared__ unsigned long long best;
+    if (threadIdx.x == 0) best = 0;
+    __syncthreads();
+    unsigned long long mine = 0;
+    for (uint32_t c = threadIdx.x; c < k; c += blockDim.x) {
+        const unsigned long long x = ((unsigned long long)count[c] << 32) | c;
+        if (x > mine) mine = x;
+    }
+    atomicMax(&best, mine);
+    __syncthreads();
+    if (threadIdx.x == 0) *hub = (uint32_t)best;
+}
+
+// ---------------------------------------------------------------------------
 // ordered compaction of the pair table: entries != INF in slot order,
 // i.e. ascending (rank a, rank b)
 // ---------------------------------------------------------------------------
@@ -304,6 +543,63 @@ cudaError_t launch_compact_pairs(Workspace &ws, uint32_t k, cudaStream_t s) {
     tile_scan_kernel<<<1, 1024, 0, s>>>(ws.tile_off, tiles, &ws.ctl->n_pairs);
     pair_write_kernel<<<tiles, CT_THREADS, 0, s>>>(ws.pairtab, slots, k, ws.tile_off, ws.e_key,
                                                    ws.e_ra, ws.e_rb, ws.e_arc, ws.e_mst);
+    return cudaGetLastError();
+}
+
+// The tree-only scan serves a query whose label width and weights make it
+// exact (narrow labels of two rank bits or more cannot overflow a bridge), with
+// rows split by weight, on a graph large enough for its extra compaction and
+// MST (query times, tree-only against full): R-MAT 26 (degree 8), k = 10,000
+// 8.6 against 11.2 ms, R-MAT 24, k = 10,000 5.3 against 6.1, k = 700 at the
+// default band 6.0 against 6.5, R-MAT 22, k = 300 2.25 against 2.32; R-MAT 20,
+// k = 1000 1.41 against 1.39, 250,000 vertices, k = 3000 1.09 against 0.85.
+bool tree_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t k, uint32_t delta) {
+    const bool exact = ws.narrow && ws.lshift >= 2 && g.max_w < 0x80000000u &&
+                       active_lend(g, delta) && k > 1 && !small_tail(k);
+    if (g.tree_scan >= 0) return exact && g.tree_scan;
+    return exact && g.m >= TREE_SCAN_MIN_ARCS;
+}
+
+static TreeScanArgs tree_scan_args(const DevGraph &g, const Workspace &ws, uint32_t k, uint32_t delta) {
+    TreeScanArgs a;
+    a.row_ptr = g.row_ptr;
+    a.adj = g.adj;
+    a.adj_w = g.adj_w;
+    a.lend = g.lend;
+    a.heavy_chunks = g.heavy_chunks;
+    a.n_heavy_chunks = g.n_heavy_chunks;
+    a.items = g.items;
+    a.n_items = g.n_items;
+    a.delta = delta;
+    a.near = near_label(ws, delta);
+    a.label32 = ws.label32;
+    a.lshift = ws.lshift;
+    a.pred_arc = ws.pred_arc;
+    a.pairtab = ws.pairtab;
+    a.k = k;
+    a.orig_of = g.orig_of;
+    a.orig_row_ptr = g.orig_row_ptr;
+    a.comp = ws.comp;
+    a.hub = ws.hub;
+    return a;
+}
+
+cudaError_t launch_tree_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t delta,
+                             const Geometry &geo, cudaStream_t s) {
+    const TreeScanArgs a = tree_scan_args(g, ws, k, delta);
+    const uint64_t slots = (uint64_t)k * (k - 1) / 2;
+    cudaError_t e = cudaMemsetAsync(ws.pairtab, 0xFF, slots * sizeof(uint64_t), s);
+    if (e != cudaSuccess) return e;
+    const unsigned blocks = (unsigned)current_sm_count() * 32;
+    tree_scan_kernel<<<blocks, 256, 0, s>>>(a);
+    e = launch_compact_pairs(ws, k, s);
+    if (e == cudaSuccess) e = launch_mst(ws, k, geo, (uint64_t)delta << 32, s);
+    // (the MST is done with its hooks: they count the samples)
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws.hook, 0, (size_t)k * 4, s);
+    if (e != cudaSuccess) return e;
+    hub_sample_kernel<<<HUB_SAMPLES / 256, 256, 0, s>>>(a, g.n, g.m, ws.hook);
+    hub_pick_kernel<<<1, 1024, 0, s>>>(ws.hook, k, ws.hub);
+    rest_scan_kernel<<<blocks, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -61,12 +61,28 @@ struct DevGraph {
     // Vertices with ids at or above n_live have no arcs (the degree order
     // puts them last; n without it).
     uint32_t n_live = 0;
+    int tree_scan = -1;              // tree-only scan: -1 chooses, 0 / 1 force it off / on
 };
 
 // The weight-partitioned rows to use for band width delta: built for that
 // width and the split on (delta at or below the largest weight), else null.
 inline const uint32_t *active_lend(const DevGraph &g, uint32_t delta) {
     return (delta <= g.max_w && g.adj_w && g.lend && g.part_delta == delta) ? g.lend : nullptr;
+}
+
+// The first band's inner threshold with the split on for band width delta (0:
+// none).  The default band width is 32 mean weights over the mean degree: on
+// R-MAT graphs the hubs and most of the core settle below half a mean weight
+// over the mean degree, and with them settled the rest of the band improves
+// most vertices once.  R-MAT of 10^6 vertices, k = 101, default band: 54 ->
+// 26 M relaxations, 1.72 -> 1.10 ms (1.06 at a 48th, 1.35 at a 96th of the
+// default width); R-MAT 24, k = 700: 11.2 -> 6.6 ms.  Bands narrowed by
+// tuning gain less and take an eighth of themselves: R-MAT 26 (degree 8),
+// k = 10,000 14.2 -> 13.4 ms, R-MAT 22, weights to 10^5, k = 64 2.35 -> 2.04.
+inline uint32_t first_step(const DevGraph &g, uint32_t delta) {
+    if (delta > g.max_w) return 0;
+    const uint32_t s = delta > g.delta0 / 8 ? g.delta0 / 64 : delta / 8;
+    return s < 2 ? 2 : s;
 }
 
 // Offset from internal to caller arc indices along internal row v (which
@@ -188,6 +204,7 @@ struct Workspace {
     uint32_t tile_cap = 0;
     // MST scratch (k entries)
     uint32_t *comp = nullptr, *hook = nullptr;
+    uint32_t *hub = nullptr;        // component picked by the tree-only scan
     unsigned long long *best = nullptr;
     uint32_t comp_cap = 0;
     // tree output
@@ -238,11 +255,26 @@ int sssp_occupancy(int threads);
 cudaError_t launch_scan(const DevGraph &g, Workspace &ws, uint32_t k, bool pairs,
                         cudaStream_t s);
 cudaError_t launch_compact_pairs(Workspace &ws, uint32_t k, cudaStream_t s);
+// Arcs from which on a query that returns only its tree takes the tree-only
+// scan.
+constexpr uint64_t TREE_SCAN_MIN_ARCS = 1ull << 27;
+bool tree_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t k, uint32_t delta);
+// The smallest 32-bit label of a distance delta (saturating).
+inline uint32_t near_label(const Workspace &ws, uint32_t delta) {
+    const uint64_t l = (uint64_t)delta << ws.lshift;
+    return l < INF32 ? (uint32_t)l : INF32;
+}
+// Predecessors and the part of the pair table that the MST can need.
+cudaError_t launch_tree_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t delta,
+                             const Geometry &geo, cudaStream_t s);
 
 // tree.cu
-cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, cudaStream_t s);
+// limit: pairs whose key (b << 32 | slot) is at or above it are left out.
+cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, uint64_t limit,
+                       cudaStream_t s);
+// split_delta: the band width of a tree-only scan (0: the full scan).
 cudaError_t launch_tree(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t tag,
-                        uint32_t n_bits, cudaStream_t s);
+                        uint32_t n_bits, uint32_t split_delta, cudaStream_t s);
 cudaError_t launch_small_tail(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t tag,
                               uint32_t n_bits, cudaStream_t s);
 int mst_occupancy(int threads);

@@ -30,6 +30,7 @@ struct MstArgs {
     uint32_t *hook;
     unsigned long long *best;
     uint32_t k;
+    uint64_t limit;          // pairs of this key or above are left out
     Control *ctl;
 };
 
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(512) mst_kernel(MstArgs a) {
             uint32_t ca = ldcg_u32(&a.comp[a.e_ra[j]]), cb = ldcg_u32(&a.comp[a.e_rb[j]]);
             if (ca == cb) continue;
             unsigned long long key = a.e_key[j];
+            if (key >= a.limit) continue;
             atomicMin(&a.best[ca], key);
             atomicMin(&a.best[cb], key);
             any = true;
@@ -135,6 +137,8 @@ __global__ void expand_kernel(const uint32_t *__restrict__ row_ptr, const uint2 
                               const uint32_t *__restrict__ orig_of,
                               const uint32_t *__restrict__ new_of,
                               const uint32_t *__restrict__ orig_row_ptr,
+                              const uint2 *__restrict__ adj_near,
+                              const uint32_t *__restrict__ label32, uint32_t near,
                               uint32_t n, const uint32_t *__restrict__ e_arc,
                               const uint32_t *__restrict__ e_mst,
                               const uint32_t *__restrict__ pred_arc, uint32_t pred_stride,
@@ -167,8 +171,11 @@ __global__ void expand_kernel(const uint32_t *__restrict__ row_ptr, const uint2 
         for (uint32_t steps = 0; steps < n; ++steps) {
             uint32_t pa = pred_arc[(uint64_t)x * pred_stride];
             if (pa == SEED_ARC || pa == INF32) break;
+            // the tree-only scan leaves indices in the weight-split rows for
+            // vertices nearer than the band width
+            const uint2 *arcs = label32 && label32[x] < near ? adj_near : adj;
             uint32_t old = atomicExch(&mark[x], tag);
-            uint2 pe = adj[pa];              // independent of the exchange's result
+            uint2 pe = arcs[pa];             // independent of the exchange's result
             if (old == tag) break;           // the rest of the chain is another walker's
             emit_edge(caller_id(orig_of, x), caller_id(orig_of, pe.x), pe.y, nbits, key, wout, cap,
                       ctl);
@@ -566,7 +573,8 @@ cudaError_t launch_small_tail(const DevGraph &g, Workspace &ws, uint32_t k, uint
 
 static int sort_blocks_cache = -1;
 
-cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, cudaStream_t s) {
+cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, uint64_t limit,
+                       cudaStream_t s) {
     if (k < 2) return cudaSuccess;
     MstArgs a;
     a.e_key = ws.e_key;
@@ -577,6 +585,7 @@ cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, cudaStrea
     a.hook = ws.hook;
     a.best = ws.best;
     a.k = k;
+    a.limit = limit;
     a.ctl = ws.ctl;
     uint64_t slots = (uint64_t)k * (k - 1) / 2;
     int blocks = slots <= 65536 ? 1 : geo.mst_blocks;
@@ -587,11 +596,13 @@ cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, cudaStrea
 }
 
 cudaError_t launch_tree(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t tag,
-                        uint32_t n_bits, cudaStream_t s) {
+                        uint32_t n_bits, uint32_t split_delta, cudaStream_t s) {
     if (k < 2) return cudaSuccess;
     uint64_t slots = (uint64_t)k * (k - 1) / 2;
     uint32_t blocks = (uint32_t)std::min<uint64_t>((2 * slots + 255) / 256, (uint64_t)current_sm_count() * 8);
     expand_kernel<<<blocks, 256, 0, s>>>(g.row_ptr, g.adj, g.orig_of, g.new_of, g.orig_row_ptr,
+                                         g.adj_w, split_delta ? ws.label32 : nullptr,
+                                         near_label(ws, split_delta),
                                          g.n, ws.e_arc, ws.e_mst, ws.pred_arc,
                                          ws.pred_stride, ws.mark, tag, n_bits, ws.tree_key,
                                          ws.tree_w, ws.tree_cap, ws.ctl);

@@ -1593,6 +1593,17 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     // one vertex per warp only splits early (0.29 against 0.31 ms).  With
     // local rounds asked for the frontier is rarely latency-bound, and the
     // early split only unsettles it (grid 4096 x 4096: 9.7 against 9.25 ms).
+    a.step0 = p.far_scan ? first_step(g, p.delta) : 0u;
+    // Thin frontiers with the far pile (see the kernel).  Few arcs per vertex
+    // mean a high diameter (grids, paths, trees): below eight vertices per
+    // warp a frontier there also takes 16 warp-local rounds, so that a
+    // barrier is paid every 16 hops (grid 1021 x 733, k = 37: 2.4 ms; split
+    // early without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.64
+    // against 1.21).  On denser graphs a warp's own rounds would relax hub
+    // rows alone (R-MAT 12: 0.93 ms against 0.20); there a frontier below
+    // one vertex per warp only splits early (0.29 against 0.31 ms).  With
+    // local rounds asked for the frontier is rarely latency-bound, and the
+    // early split only unsettles it (grid 4096 x 4096: 9.7 against 9.25 ms).
     // The first band's inner threshold (the default band width is 32 mean
     // weights over the mean degree): on R-MAT graphs the hubs and most of the
     // core settle below half a mean weight over the mean degree, and with

@@ -185,3 +185,29 @@ def test_pull_steps_and_tail_frontier(n, relabel, monkeypatch):
             _check(g, G.seeds_from(np.arange(2 * core), 5, n),
                    [("delta", 30), ("pull", 2), ("tail", tail), ("label_bits", bits)])
 
+
+
+@pytest.mark.parametrize("relabel", ["0", "1"])
+@pytest.mark.parametrize("k", [182, 400, 1500])
+@pytest.mark.parametrize("wmax,delta", [(3, 1), (3, 3), (60, 2), (60, 15), (1000, 40), (1000, 900)])
+def test_tree_only_scan(wmax, delta, k, relabel, monkeypatch):
+    """steiner_query's scan of the arcs that the MST can need (forced on small
+    graphs) gives the oracle's tree: ties (small weights), almost everything
+    left to the rest scan (narrow bands) or nothing, hubs in chunks, forests,
+    and both vertex orders (the bridge's arc is searched in its row)."""
+    monkeypatch.setenv("STEINER_TREE_SCAN", "1")
+    monkeypatch.setenv("STEINER_RELABEL", relabel)
+    graphs = [(wl.rmat(12, 16, wmax=wmax, seed=71), True),
+              (G.random_graph(4000, 5000, 1, wmax, 72), False),
+              (wl.grid(70, 60, wmax, seed=73), False)]
+    for g, core in graphs:
+        seeds = wl.sample_distinct(wl.largest_cc(g) if core else np.arange(g.n, dtype=np.int32), k, 74)
+        ref = oracle.steiner(g, seeds, want_labels=False)
+        with st.SteinerGraph(g) as Gd:
+            Gd.set_param("delta", delta)
+            res = Gd.query(seeds)
+            full = Gd.query_detail(seeds)
+        assert res.status == ref.status == full.status
+        np.testing.assert_array_equal(res.edges, ref.edges)
+        assert res.total == ref.total
+        np.testing.assert_array_equal(full.edges, ref.edges)
