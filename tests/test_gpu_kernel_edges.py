@@ -211,3 +211,17 @@ def test_tree_only_scan(wmax, delta, k, relabel, monkeypatch):
         np.testing.assert_array_equal(res.edges, ref.edges)
         assert res.total == ref.total
         np.testing.assert_array_equal(full.edges, ref.edges)
+
+
+@pytest.mark.parametrize("n", [33, 1024, 1025, 1026, 4098, 9000])
+def test_rows_split_by_weight_around_hub_sizes(n):
+    """Rows split by weight class: hub rows around the size that takes a
+    block, tiles of 4096 arcs and their remainders, and widths that put all,
+    some or none of a row in the light part."""
+    r = G.rng(n)
+    extra = 3 * n
+    g = wl.from_edges(n, np.concatenate([np.zeros(n - 1, int), r.integers(0, n, extra)]),
+                      np.concatenate([np.arange(1, n), r.integers(0, n, extra)]),
+                      r.integers(1, 90, n - 1 + extra))
+    for delta in (1, 30, 89):
+        _check(g, G.seeds_from(np.arange(n), 6, n), [("delta", delta)])
