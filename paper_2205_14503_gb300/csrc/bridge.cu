@@ -164,32 +164,34 @@ __global__ void __launch_bounds__(256) scan_kernel(ScanArgs a) {
 // the scan of a query that returns the tree alone
 // ---------------------------------------------------------------------------
 //
-// A tree needs the MST of G'_1, not all of G'_1, and predecessors only along
-// tight arcs, which are no heavier than their head's distance.  With rows
-// split at band width delta, most arcs of a large graph are heavy arcs
-// between vertices nearer than delta, and most of those join cells that
-// lighter bridges have already joined:
+// A tree needs the MST of G'_1, not all of G'_1, and the predecessors of its
+// own vertices.  With rows split at band width delta, most arcs of a large
+// graph join cells that bridges lighter than delta have joined already:
 //
-//  1. tree_scan_kernel reads every arc but the heavy ones (weight delta or
-//     more) between two vertices nearer than delta: the light part of a row
-//     whose vertex is nearer than delta, the whole row otherwise.  That gives
-//     every predecessor, and every pair whose minimum bridge is below delta
-//     (such a bridge's arc is lighter than delta).
+//  1. tree_scan_kernel reads the light part of the rows of the vertices nearer
+//     than delta: every pair of cells with a bridge below delta gets its
+//     minimum (such a bridge's arc is lighter than delta, its ends nearer),
+//     and these vertices their predecessors (a tight arc is no heavier than
+//     its head's distance).  Hub rows farther out are read for the
+//     predecessor alone; the predecessors of the other vertices beyond delta
+//     are found by the expansion, for those on the tree.
 //  2. The MST of those pairs is the part of Kruskal's tree below delta.  Of
-//     its components the one whose cells hold the most unread arcs (sampled)
-//     is the hub.
-//  3. rest_scan_kernel reads the unread arcs of the vertices outside the
-//     hub's cells.  Every arc between two components has such an end, so the
-//     minimum bridge of every pair of cells in different components is now
-//     in the table; pairs inside a component may have been left at a larger
-//     bridge or none, but the component's own tree joins them by bridges
-//     below delta, so they cannot be in the MST.
+//     its components the one whose cells hold the most arcs (sampled) is the
+//     hub component.
+//  3. rest_scan_kernel reads the rows of the vertices outside the hub
+//     component's cells.  Every arc between two components has such an end,
+//     so the minimum bridge of every pair of cells in different components is
+//     now in the table; pairs inside a component are joined by the
+//     component's own tree, by bridges below delta, and cannot add to it.
 //  4. The MST of all pairs in the table is then the MST of G'_1.
 //
 // A bridge key carries the caller's index of its arc, which a row split by
 // weight does not give: it is searched in the id-ordered row, for proposals
 // that lower the table (first with an index above all, so that few others
 // search).  Narrow labels only: their distances rule out an overflow.
+// Bound by the label gathers and, at k = 10,000, by probes of a 400 MB table:
+// looking at every bridge in step 1, and at every arc of the vertices beyond
+// delta, took it 1.91 ms on R-MAT 26 (degree 8) against 1.08.
 
 struct TreeScanArgs {
     const uint32_t *__restrict__ row_ptr;
@@ -233,29 +235,21 @@ __device__ __forceinline__ void propose_bridge(const TreeScanArgs &a, uint32_t c
     atomicMin(slot, (b << 32) | caller_arc(a, x, y));
 }
 
-__device__ __forceinline__ void tree_arc(const TreeScanArgs &a, uint32_t v, uint32_t lv, bool whole,
-                                         uint32_t cbase, uint32_t arc, uint2 e) {
-    const uint32_t lu = __ldg(&a.label32[e.x]);
+// Arc `arc` = (v, head, w) of step 1, lu the head's label.
+__device__ __forceinline__ void tree_arc(const TreeScanArgs &a, uint32_t v, uint32_t lv,
+                                         uint32_t arc, uint2 e, uint32_t lu) {
     if (lu == INF32) return;
     const uint64_t sum = ((uint64_t)e.y << a.lshift) + lu;       // the head's distance + w
     if (sum == lv) atomicMin(&a.pred_arc[v], arc);
     const uint32_t mask = (1u << a.lshift) - 1u, cv = lv & mask, cu = lu & mask;
-    if (cv == cu) return;
+    if (cv >= cu) return;
     const uint64_t b = (lv >> a.lshift) + (sum >> a.lshift);
-    if (cv < cu) {
-        if (whole) {
-            auto *slot = reinterpret_cast<unsigned long long *>(&a.pairtab[pair_slot(cv, cu, a.k)]);
-            const unsigned long long key = (b << 32) | (uint32_t)(cbase + arc);
-            if (key < __ldg(slot)) atomicMin(slot, key);
-        } else {
-            propose_bridge(a, cv, cu, b, v, e.x);
-        }
-    } else if (whole && e.y >= a.delta && lu < a.near) {
-        propose_bridge(a, cu, cv, b, e.x, v);        // the head does not read this arc
-    }
+    if (b < a.delta) propose_bridge(a, cv, cu, b, v, e.x);
 }
 
-__global__ void __launch_bounds__(256) tree_scan_kernel(const __grid_constant__ TreeScanArgs a) {
+constexpr int TREE_ILP = 2;        // arcs in flight per lane (full occupancy matters more)
+
+__global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant__ TreeScanArgs a) {
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -266,90 +260,120 @@ __global__ void __launch_bounds__(256) tree_scan_kernel(const __grid_constant__ 
             const uint32_t v = (uint32_t)(item >> 32), c = (uint32_t)item;
             const uint32_t lv = __ldg(&a.label32[v]);
             if (lv == INF32) continue;
-            const bool whole = lv >= a.near;
-            const uint32_t rs = a.row_ptr[v], end = whole ? a.row_ptr[v + 1] : a.lend[v];
+            const bool far = lv >= a.near;           // the whole row, for the predecessor alone
+            const uint32_t rs = a.row_ptr[v], end = far ? a.row_ptr[v + 1] : a.lend[v];
             const uint32_t s = rs + c * CHUNK, e = min(end, s + CHUNK);
             if (s >= end) continue;
-            const uint2 *arcs = whole ? a.adj : a.adj_w;
-            const uint32_t cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, rs);
-            uint2 en = make_uint2(0, 0);
-            if (s + lane < e) en = __ldcs(&arcs[s + lane]);
-            for (uint32_t b = s; b < e; b += 32) {
-                const uint2 ec = en;
-                if (b + 32 + lane < e) en = __ldcs(&arcs[b + 32 + lane]);
-                if (b + lane < e) tree_arc(a, v, lv, whole, cbase, b + lane, ec);
+            const uint2 *arcs = far ? a.adj : a.adj_w;
+            for (uint32_t b = s; b < e; b += 32 * TREE_ILP) {
+                uint2 x[TREE_ILP];
+                uint32_t lu[TREE_ILP];
+#pragma unroll
+                for (int q = 0; q < TREE_ILP; ++q) {
+                    x[q] = make_uint2(0, 0);                    // weight 0: no arc
+                    if (b + 32 * q + lane < e) x[q] = __ldcs(&arcs[b + 32 * q + lane]);
+                }
+#pragma unroll
+                for (int q = 0; q < TREE_ILP; ++q) {
+                    // (an arc heavier than the row's distance is not tight)
+                    const bool look = x[q].y && (!far || x[q].y <= lv >> a.lshift);
+                    lu[q] = look ? __ldg(&a.label32[x[q].x]) : INF32;
+                }
+#pragma unroll
+                for (int q = 0; q < TREE_ILP; ++q)
+                    tree_arc(a, v, lv, b + 32 * q + lane, x[q], lu[q]);
             }
             continue;
         }
         const uint32_t v1 = __ldg(&a.items[wi - n_work + a.n_items + 1]);
         for (uint32_t vb = __ldg(&a.items[wi - n_work + a.n_items]); vb < v1; vb += 32) {
             const uint32_t v = vb + lane;
-            uint32_t s = 0, deg = 0, cbase = 0, lv = INF32;
+            uint32_t s = 0, deg = 0, lv = INF32;
             if (v < v1) {
                 lv = __ldg(&a.label32[v]);
-                if (lv != INF32) {
+                if (lv < a.near) {
                     s = a.row_ptr[v];
-                    const uint32_t r1 = a.row_ptr[v + 1];
-                    deg = r1 - s >= HEAVY_DEG ? 0u : (lv >= a.near ? r1 : a.lend[v]) - s;
-                    if (deg && lv >= a.near) cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, s);
+                    deg = a.row_ptr[v + 1] - s >= HEAVY_DEG ? 0u : a.lend[v] - s;
                 }
             }
+            const uint32_t rows = __ballot_sync(FULL, deg != 0);
+            if (rows == 0) continue;
             const uint32_t incl = warp_inclusive_scan(deg);
-            const uint32_t excl = incl - deg;
             const uint32_t total = __shfl_sync(FULL, incl, 31);
-            for (uint32_t b = 0; b < total; b += 32) {
-                const uint32_t j = b + lane;
-                const uint32_t own = warp_owner_search(excl, j < total ? j : 0);
-                const uint32_t arc = __shfl_sync(FULL, s, own) + (j - __shfl_sync(FULL, excl, own));
-                const uint32_t lo = __shfl_sync(FULL, lv, own), co = __shfl_sync(FULL, cbase, own);
-                const bool whole = lo >= a.near;
-                if (j >= total) continue;
-                tree_arc(a, vb + own, lo, whole, co, arc, __ldcs(&(whole ? a.adj : a.adj_w)[arc]));
+            const uint32_t excl = deg ? incl - deg : INF32;
+            uint32_t before = 0;             // rows that start before the window
+            for (uint32_t b = 0; b < total; b += 32 * TREE_ILP) {
+                uint2 x[TREE_ILP];
+                uint32_t lu[TREE_ILP], own[TREE_ILP], at[TREE_ILP];
+#pragma unroll
+                for (int q = 0; q < TREE_ILP; ++q) {
+                    const uint32_t w0 = b + 32 * q, j = w0 + lane;
+                    const uint32_t starts = __reduce_or_sync(FULL, excl - w0 < 32 ? 1u << (excl - w0) : 0u);
+                    own[q] = nth_set_bit(rows, before + (uint32_t)__popc(starts & (FULL >> (31 - lane))) - 1);
+                    before += (uint32_t)__popc(starts);
+                    at[q] = __shfl_sync(FULL, s - excl, own[q]) + j;
+                    x[q] = make_uint2(0, 0);
+                    if (j < total) x[q] = __ldcs(&a.adj_w[at[q]]);
+                }
+#pragma unroll
+                for (int q = 0; q < TREE_ILP; ++q) lu[q] = x[q].y ? __ldg(&a.label32[x[q].x]) : INF32;
+#pragma unroll
+                for (int q = 0; q < TREE_ILP; ++q) {
+                    const uint32_t lo = __shfl_sync(FULL, lv, own[q]);
+                    tree_arc(a, vb + own[q], lo, at[q], x[q], lu[q]);
+                }
             }
         }
     }
 }
 
-// The unread arcs (heavy part of a row whose vertex is nearer than delta) of
-// the vertices outside the hub component's cells.
+// Step 3: the rows of the vertices outside the hub component's cells.
 __global__ void __launch_bounds__(256) rest_scan_kernel(const __grid_constant__ TreeScanArgs a) {
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t n_work = a.n_heavy_chunks + a.n_items;
     const uint32_t hub = *a.hub, mask = (1u << a.lshift) - 1u;
-    auto arc = [&](uint32_t v, uint32_t lv, uint32_t cc, uint2 e) {
+    // arc `at` of row v (the caller's index cbase + at)
+    auto arc = [&](uint32_t v, uint32_t lv, uint32_t cc, uint32_t cbase, uint32_t at) {
+        const uint2 e = __ldcs(&a.adj[at]);
         const uint32_t lu = __ldg(&a.label32[e.x]);
-        if (lu >= a.near || __ldg(&a.comp[lu & mask]) == cc) return;
+        if (lu == INF32 || __ldg(&a.comp[lu & mask]) == cc) return;
         const uint32_t cv = lv & mask, cu = lu & mask;
         const uint64_t b = (uint64_t)(lv >> a.lshift) + e.y + (lu >> a.lshift);
-        if (cv < cu) propose_bridge(a, cv, cu, b, v, e.x);
-        else propose_bridge(a, cu, cv, b, e.x, v);
+        if (cv < cu) {
+            auto *slot = reinterpret_cast<unsigned long long *>(&a.pairtab[pair_slot(cv, cu, a.k)]);
+            const unsigned long long key = (b << 32) | (uint32_t)(cbase + at);
+            if (key < __ldg(slot)) atomicMin(slot, key);
+        } else {
+            propose_bridge(a, cu, cv, b, e.x, v);    // the head's row may not be read
+        }
     };
     for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
         if (wi < a.n_heavy_chunks) {
             const uint64_t item = a.heavy_chunks[wi];
             const uint32_t v = (uint32_t)(item >> 32), c = (uint32_t)item;
             const uint32_t lv = __ldg(&a.label32[v]);
-            if (lv >= a.near) continue;
+            if (lv == INF32) continue;
             const uint32_t cc = __ldg(&a.comp[lv & mask]);
             if (cc == hub) continue;
-            const uint32_t r1 = a.row_ptr[v + 1];
-            const uint32_t s = a.lend[v] + c * CHUNK, e = min(r1, s + CHUNK);
-            for (uint32_t j = s + lane; s < r1 && j < e; j += 32) arc(v, lv, cc, __ldcs(&a.adj_w[j]));
+            const uint32_t rs = a.row_ptr[v], s = rs + c * CHUNK, e = min(a.row_ptr[v + 1], s + CHUNK);
+            const uint32_t cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, rs);
+            for (uint32_t j = s + lane; j < e; j += 32) arc(v, lv, cc, cbase, j);
             continue;
         }
         const uint32_t v1 = __ldg(&a.items[wi - n_work + a.n_items + 1]);
         for (uint32_t vb = __ldg(&a.items[wi - n_work + a.n_items]); vb < v1; vb += 32) {
             const uint32_t v = vb + lane;
-            uint32_t s = 0, deg = 0, lv = INF32, cc = hub;
+            uint32_t s = 0, deg = 0, lv = INF32, cc = hub, cbase = 0;
             if (v < v1) {
                 lv = __ldg(&a.label32[v]);
-                if (lv < a.near) cc = __ldg(&a.comp[lv & mask]);
+                if (lv != INF32) cc = __ldg(&a.comp[lv & mask]);
                 if (cc != hub) {
-                    s = a.lend[v];
-                    const uint32_t r1 = a.row_ptr[v + 1];
-                    deg = r1 - a.row_ptr[v] >= HEAVY_DEG ? 0u : r1 - s;
+                    s = a.row_ptr[v];
+                    deg = a.row_ptr[v + 1] - s;
+                    if (deg >= HEAVY_DEG) deg = 0;   // covered by the chunk list
+                    if (deg) cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, s);
                 }
             }
             if (!__any_sync(FULL, deg)) continue;
@@ -359,15 +383,16 @@ __global__ void __launch_bounds__(256) rest_scan_kernel(const __grid_constant__ 
             for (uint32_t b = 0; b < total; b += 32) {
                 const uint32_t j = b + lane;
                 const uint32_t own = warp_owner_search(excl, j < total ? j : 0);
-                const uint32_t at = __shfl_sync(FULL, s, own) + (j - __shfl_sync(FULL, excl, own));
+                const uint32_t at = __shfl_sync(FULL, s - excl, own) + j;
                 const uint32_t lo = __shfl_sync(FULL, lv, own), co = __shfl_sync(FULL, cc, own);
-                if (j < total) arc(vb + own, lo, co, __ldcs(&a.adj_w[at]));
+                const uint32_t bo = __shfl_sync(FULL, cbase, own);
+                if (j < total) arc(vb + own, lo, co, bo, at);
             }
         }
     }
 }
 
-// Unread arcs per component, by a sample of arcs spread over all of them.
+// Arcs per component, by a sample of arcs spread over all of them.
 constexpr uint32_t HUB_SAMPLES = 1u << 15;
 __global__ void hub_sample_kernel(const __grid_constant__ TreeScanArgs a, uint32_t n, uint64_t m,
                                   uint32_t *count) {
@@ -381,7 +406,7 @@ __global__ void hub_sample_kernel(const __grid_constant__ TreeScanArgs a, uint32
         else hi = mid;
     }
     const uint32_t lv = a.label32[lo];
-    if (lv < a.near && arc >= a.lend[lo]) atomicAdd(&count[a.comp[lv & ((1u << a.lshift) - 1u)]], 1u);
+    if (lv != INF32) atomicAdd(&count[a.comp[lv & ((1u << a.lshift) - 1u)]], 1u);
 }
 
 // The component with the largest count (one block).
@@ -550,9 +575,9 @@ cudaError_t launch_compact_pairs(Workspace &ws, uint32_t k, cudaStream_t s) {
 // exact (narrow labels of two rank bits or more cannot overflow a bridge), with
 // rows split by weight, on a graph large enough for its extra compaction and
 // MST (query times, tree-only against full): R-MAT 26 (degree 8), k = 10,000
-// 8.6 against 11.2 ms, R-MAT 24, k = 10,000 5.3 against 6.1, k = 700 at the
-// default band 6.0 against 6.5, R-MAT 22, k = 300 2.25 against 2.32; R-MAT 20,
-// k = 1000 1.41 against 1.39, 250,000 vertices, k = 3000 1.09 against 0.85.
+// 7.7 against 11.1 ms, R-MAT 24, k = 10,000 4.7 against 6.1, k = 700 at the
+// default band 5.9 against 6.5, R-MAT 22, k = 300 2.23 against 2.33; R-MAT 20,
+// k = 1000 1.42 against 1.42, 250,000 vertices, k = 3000 1.11 against 0.87.
 bool tree_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t k, uint32_t delta) {
     const bool exact = ws.narrow && ws.lshift >= 2 && g.max_w < 0x80000000u &&
                        active_lend(g, delta) && k > 1 && !small_tail(k);

@@ -129,6 +129,21 @@ __device__ __forceinline__ uint32_t warp_inclusive_scan(uint32_t x) {
     return x;
 }
 
+// Index of the t-th set bit (0-based) of a 32-bit word.
+__device__ __forceinline__ uint32_t nth_set_bit(uint32_t x, uint32_t t) {
+    uint32_t pos = 0;
+#pragma unroll
+    for (uint32_t w = 16; w >= 1; w >>= 1) {
+        const uint32_t c = (uint32_t)__popc(x & ((1u << w) - 1u));
+        if (t >= c) {
+            t -= c;
+            x >>= w;
+            pos += w;
+        }
+    }
+    return pos;
+}
+
 // Largest lane L whose value excl[L] <= j (excl non-decreasing across lanes).
 __device__ __forceinline__ uint32_t warp_owner_search(uint32_t excl, uint32_t j) {
     uint32_t lo = 0;

@@ -137,8 +137,6 @@ __global__ void expand_kernel(const uint32_t *__restrict__ row_ptr, const uint2 
                               const uint32_t *__restrict__ orig_of,
                               const uint32_t *__restrict__ new_of,
                               const uint32_t *__restrict__ orig_row_ptr,
-                              const uint2 *__restrict__ adj_near,
-                              const uint32_t *__restrict__ label32, uint32_t near,
                               uint32_t n, const uint32_t *__restrict__ e_arc,
                               const uint32_t *__restrict__ e_mst,
                               const uint32_t *__restrict__ pred_arc, uint32_t pred_stride,
@@ -171,12 +169,91 @@ __global__ void expand_kernel(const uint32_t *__restrict__ row_ptr, const uint2 
         for (uint32_t steps = 0; steps < n; ++steps) {
             uint32_t pa = pred_arc[(uint64_t)x * pred_stride];
             if (pa == SEED_ARC || pa == INF32) break;
-            // the tree-only scan leaves indices in the weight-split rows for
-            // vertices nearer than the band width
-            const uint2 *arcs = label32 && label32[x] < near ? adj_near : adj;
             uint32_t old = atomicExch(&mark[x], tag);
-            uint2 pe = arcs[pa];             // independent of the exchange's result
+            uint2 pe = adj[pa];              // independent of the exchange's result
             if (old == tag) break;           // the rest of the chain is another walker's
+            emit_edge(caller_id(orig_of, x), caller_id(orig_of, pe.x), pe.y, nbits, key, wout, cap,
+                      ctl);
+            x = pe.x;
+        }
+    }
+}
+
+// The expansion after a tree-only scan: as above, a warp for 32 walkers, where
+// the predecessor of a vertex nearer than the band width is an index in the
+// weight-split rows, and that of another vertex may still have to be found
+// (the first tight arc of its row, by the whole warp).
+__global__ void __launch_bounds__(256) expand_found_kernel(
+    const uint32_t *__restrict__ row_ptr, const uint2 *__restrict__ adj,
+    const uint2 *__restrict__ adj_w, const uint32_t *__restrict__ label32, uint32_t lshift,
+    uint32_t near, const uint32_t *__restrict__ orig_of, const uint32_t *__restrict__ new_of,
+    const uint32_t *__restrict__ orig_row_ptr, uint32_t n, const uint32_t *__restrict__ e_arc,
+    const uint32_t *__restrict__ e_mst, const uint32_t *__restrict__ pred_arc, uint32_t *mark,
+    uint32_t tag, uint32_t nbits, uint64_t *key, uint32_t *wout, uint32_t cap, Control *ctl) {
+    const uint32_t lane = lane_id();
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t E = ldcg_u32(&ctl->n_pairs);
+    for (uint64_t t0 = (uint64_t)warp * 32; t0 < 2 * (uint64_t)E; t0 += (uint64_t)nwarps * 32) {
+        const uint64_t t = t0 + lane;
+        const uint32_t j = (uint32_t)(t >> 1);
+        bool walk = t < 2 * (uint64_t)E && e_mst[j];
+        if (!__any_sync(FULL, walk)) continue;
+        uint32_t x = 0;
+        if (walk) {
+            const uint32_t carc = e_arc[j];
+            uint32_t tail, arc;
+            if (orig_of) {
+                const uint32_t ct = arc_owner(orig_row_ptr, n, carc);
+                tail = new_of[ct];
+                arc = row_ptr[tail] + (carc - orig_row_ptr[ct]);
+            } else {
+                tail = arc_owner(row_ptr, n, carc);
+                arc = carc;
+            }
+            const uint2 e = adj[arc];
+            x = e.x;
+            if ((t & 1) == 0) {
+                atomicAdd(&ctl->n_mst, 1u);
+                x = tail;
+                emit_edge(caller_id(orig_of, x), caller_id(orig_of, e.x), e.y, nbits, key, wout,
+                          cap, ctl);
+            }
+        }
+        for (uint32_t steps = 0; steps < n && __any_sync(FULL, walk); ++steps) {
+            uint32_t pa = SEED_ARC, lx = INF32;
+            if (walk) {
+                pa = pred_arc[x];
+                lx = label32[x];
+            }
+            walk = walk && pa != SEED_ARC;
+            for (uint32_t m = __ballot_sync(FULL, walk && pa == INF32); m; m &= m - 1) {
+                const uint32_t l = __ffs(m) - 1;
+                const uint32_t v = __shfl_sync(FULL, x, l), lv = __shfl_sync(FULL, lx, l);
+                const uint32_t r1 = row_ptr[v + 1];
+                uint32_t found = INF32;
+                for (uint32_t b = row_ptr[v]; b < r1 && found == INF32; b += 32) {
+                    bool tight = false;
+                    if (b + lane < r1) {
+                        const uint2 e = adj[b + lane];
+                        tight = ((uint64_t)e.y << lshift) + label32[e.x] == lv;
+                    }
+                    const uint32_t any = __ballot_sync(FULL, tight);
+                    if (any) found = b + __ffs(any) - 1;
+                }
+                if (lane == l) pa = found;
+            }
+            if (!walk) continue;
+            if (pa == INF32) {
+                walk = false;
+                continue;
+            }
+            const uint32_t old = atomicExch(&mark[x], tag);
+            const uint2 pe = (lx < near ? adj_w : adj)[pa];
+            if (old == tag) {                // the rest of the chain is another walker's
+                walk = false;
+                continue;
+            }
             emit_edge(caller_id(orig_of, x), caller_id(orig_of, pe.x), pe.y, nbits, key, wout, cap,
                       ctl);
             x = pe.x;
@@ -600,12 +677,16 @@ cudaError_t launch_tree(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t t
     if (k < 2) return cudaSuccess;
     uint64_t slots = (uint64_t)k * (k - 1) / 2;
     uint32_t blocks = (uint32_t)std::min<uint64_t>((2 * slots + 255) / 256, (uint64_t)current_sm_count() * 8);
-    expand_kernel<<<blocks, 256, 0, s>>>(g.row_ptr, g.adj, g.orig_of, g.new_of, g.orig_row_ptr,
-                                         g.adj_w, split_delta ? ws.label32 : nullptr,
-                                         near_label(ws, split_delta),
-                                         g.n, ws.e_arc, ws.e_mst, ws.pred_arc,
-                                         ws.pred_stride, ws.mark, tag, n_bits, ws.tree_key,
-                                         ws.tree_w, ws.tree_cap, ws.ctl);
+    if (split_delta)
+        expand_found_kernel<<<blocks, 256, 0, s>>>(
+            g.row_ptr, g.adj, g.adj_w, ws.label32, ws.lshift, near_label(ws, split_delta),
+            g.orig_of, g.new_of, g.orig_row_ptr, g.n, ws.e_arc, ws.e_mst, ws.pred_arc, ws.mark, tag,
+            n_bits, ws.tree_key, ws.tree_w, ws.tree_cap, ws.ctl);
+    else
+        expand_kernel<<<blocks, 256, 0, s>>>(g.row_ptr, g.adj, g.orig_of, g.new_of, g.orig_row_ptr,
+                                             g.n, ws.e_arc, ws.e_mst, ws.pred_arc,
+                                             ws.pred_stride, ws.mark, tag, n_bits, ws.tree_key,
+                                             ws.tree_w, ws.tree_cap, ws.ctl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (sort_blocks_cache < 0) {

@@ -558,21 +558,6 @@ __device__ __forceinline__ void band_track(const SsspArgs &a, Stage &st, bool wa
     }
 }
 
-// Index of the t-th set bit (0-based) of a 32-bit word.
-__device__ __forceinline__ uint32_t nth_set_bit(uint32_t x, uint32_t t) {
-    uint32_t pos = 0;
-#pragma unroll
-    for (uint32_t w = 16; w >= 1; w >>= 1) {
-        const uint32_t c = (uint32_t)__popc(x & ((1u << w) - 1u));
-        if (t >= c) {
-            t -= c;
-            x >>= w;
-            pos += w;
-        }
-    }
-    return pos;
-}
-
 // Relaxes the arcs of up to 32 rows, one per lane ([s, s + deg), tail label
 // lab; lanes without work deg = 0), flattened over the lanes.  The lanes'
 // rows are first compacted (no empty row in between), so that the row of
