@@ -56,10 +56,22 @@ uint32_t bit_length(uint32_t x) { return x ? 32u - (uint32_t)__builtin_clz(x) : 
 // counts HEAVY_DEG: longer rows are queued in chunks) and ITEM_SPAN
 // vertices, and into coarser ones of SPARSE_ITEM_FACTOR times the arcs; a
 // single vertex may exceed the arc limit.  at[0] / at[1] receive the range
-// starts followed by n.  Blocks of CUT_BLOCK vertices are cut side by side
-// on the host's threads.
-void cut_items(const uint32_t *row_ptr, uint32_t n, uint64_t arcs, std::vector<uint32_t> (&at)[2]) {
+// starts followed by n.  Without skew (the longest row, max_deg, within a few
+// times the mean) ranges of equal length do; else blocks of CUT_BLOCK
+// vertices are cut side by side on the host's threads.
+void cut_items(const uint32_t *row_ptr, uint32_t n, uint64_t arcs, uint32_t max_deg,
+               std::vector<uint32_t> (&at)[2]) {
     constexpr uint32_t CUT_BLOCK = 1u << 17;
+    const uint64_t mean = std::max<uint64_t>(row_ptr[n] / n, 1);
+    if (max_deg <= 4 * mean) {
+        for (int i = 0; i < 2; ++i) {
+            const uint64_t span = (i ? SPARSE_ITEM_FACTOR : 1) * arcs / mean;
+            const uint32_t step = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(span, 1), ITEM_SPAN);
+            for (uint64_t v = 0; v < n; v += step) at[i].push_back((uint32_t)v);
+            at[i].push_back(n);
+        }
+        return;
+    }
     struct Part {
         std::vector<uint32_t> at[2];
     };
@@ -689,7 +701,7 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
         const uint64_t arcs = std::min<uint64_t>(std::max<uint64_t>(n_arcs / (16 * warps), ITEM_ARCS_MIN),
                                                  ITEM_ARCS_MAX);
         std::vector<uint32_t> at[2];
-        cut_items(irp, std::max(G->g.n_live, 1u), arcs, at);
+        cut_items(irp, std::max(G->g.n_live, 1u), arcs, max_deg, at);
         G->g.n_items = (uint32_t)at[0].size() - 1;
         G->g.n_sparse_items = (uint32_t)at[1].size() - 1;
         e = dalloc(G->g.items, at[0].size());

@@ -361,10 +361,30 @@ __device__ __forceinline__ void push_far(const SsspArgs &a, Stage &st, const Pus
     if (m == INF32) return;              // nothing far
     if (lane_id() == 0) atomicMin(&st.far_min, m);
     if constexpr (!SCAN) {               // (no pile with the scan)
+        // one claim of the block's buffer for the warp's appends; what does
+        // not fit goes to the pile
+        uint32_t mask[N], k = 0;
 #pragma unroll
-        for (int i = 0; i < N; ++i)
-            stage_append(want[i], v[i], st.far_buf, &st.far_n, FAR_STAGE, t.farq, t.far_count, a.n,
-                         &a.ctl->err);
+        for (int i = 0; i < N; ++i) {
+            mask[i] = __ballot_sync(FULL, want[i]);
+            k += (uint32_t)__popc(mask[i]);
+        }
+        if (k == 0) return;
+        uint32_t at = 0;
+        if (lane_id() == 0) at = atomicAdd(&st.far_n, k);
+        at = __shfl_sync(FULL, at, 0);
+        const bool fits = at + k <= FAR_STAGE;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const uint32_t slot = at + (uint32_t)__popc(mask[i] & lanemask_lt());
+            if (want[i] && slot < FAR_STAGE) st.far_buf[slot] = v[i];
+            if (!fits) {
+                const uint32_t g = warp_append(want[i] && slot >= FAR_STAGE, t.far_count, a.n,
+                                               &a.ctl->err);
+                if (g != INF32) t.farq[g] = v[i];
+            }
+            at += (uint32_t)__popc(mask[i]);
+        }
     }
 }
 
@@ -402,33 +422,33 @@ __device__ __forceinline__ uint64_t threshold_label(const SsspArgs &a, uint64_t 
     return T >= INF32 ? INF64 : T << 32;
 }
 
-// One group of up to ILP arcs per lane: the arc records and their tails'
+// One group of up to N arcs per lane: the arc records and their tails'
 // labels (`valid`: this lane has arc u).
-template <bool NARROW>
+template <bool NARROW, int N>
 struct ArcGroup {
-    uint2 e[ILP];
-    typename LabelOf<NARROW>::T lab[ILP];
-    bool valid[ILP];
+    uint2 e[N];
+    typename LabelOf<NARROW>::T lab[N];
+    bool valid[N];
 };
 
 // Relaxes a group's arcs of weight in [wlo, whi).  The loads and atomics of
-// the ILP arcs are issued back to back so their latencies overlap.
+// the N arcs are issued back to back so their latencies overlap.
 // With `precheck` a plain load of the head's label comes first and only
 // improving proposals issue the atomic: right for thick frontiers, where
 // L2 atomic throughput is the limit; thin frontiers are latency-bound and
 // skip the extra dependent load.
 // NARROW kernels flag (narrow_miss) any proposal whose distance does not fit
 // a 32-bit label, which the host answers with a 64-bit rerun.
-template <bool NARROW, bool SCAN>
+template <bool NARROW, bool SCAN, int N>
 __device__ __forceinline__ void relax_group(const SsspArgs &a, Stage &st, const PushTargets &t,
-                                            const ArcGroup<NARROW> &g, bool flush, bool precheck, uint32_t wlo,
+                                            const ArcGroup<NARROW, N> &g, bool flush, bool precheck, uint32_t wlo,
                                             uint32_t whi, uint32_t &attempts,
                                             uint32_t &improved, bool &narrow_miss) {
     using L = typename LabelOf<NARROW>::T;
-    L nl[ILP], cur[ILP];
-    bool want[ILP];
+    L nl[N], cur[N];
+    bool want[N];
 #pragma unroll
-    for (int u = 0; u < ILP; ++u) {
+    for (int u = 0; u < N; ++u) {
         want[u] = g.valid[u] && g.e[u].y >= wlo && g.e[u].y < whi;
         attempts += want[u];
         cur[u] = (L)~0ull;
@@ -447,10 +467,10 @@ __device__ __forceinline__ void relax_group(const SsspArgs &a, Stage &st, const 
         }
         if (precheck && want[u]) cur[u] = raw_label<NARROW>(a, g.e[u].x);
     }
-    bool imp[ILP], fr[ILP];
+    bool imp[N], fr[N];
     bool any = false;
 #pragma unroll
-    for (int u = 0; u < ILP; ++u) {
+    for (int u = 0; u < N; ++u) {
         imp[u] = fr[u] = false;
         if (want[u] && nl[u] < cur[u]) {
             const bool far = SCAN && nl[u] >= (L)t.Tl;
@@ -470,11 +490,11 @@ __device__ __forceinline__ void relax_group(const SsspArgs &a, Stage &st, const 
     }
     // rounds that improve nothing skip the append machinery
     if (!__any_sync(FULL, any)) return;
-    bool to_near[ILP], to_far[ILP], cand[ILP];
-    uint32_t deg[ILP], vs[ILP];
+    bool to_near[N], to_far[N], cand[N];
+    uint32_t deg[N], vs[N];
     uint32_t dn = 0;
 #pragma unroll
-    for (int u = 0; u < ILP; ++u) {
+    for (int u = 0; u < N; ++u) {
         to_near[u] = to_far[u] = false;
         cand[u] = fr[u];         // a fire-and-forget far proposal still bounds far_min
         deg[u] = 0;
@@ -509,10 +529,10 @@ __device__ __forceinline__ void relax_group(const SsspArgs &a, Stage &st, const 
             if (!SCAN) to_far[u] = atomicExch(&a.stamp_far[v], t.tag_far) != t.tag_far;
         }
     }
-    push_far<SCAN, ILP>(a, st, t, to_far, cand, vs, [&](int u) {
+    push_far<SCAN, N>(a, st, t, to_far, cand, vs, [&](int u) {
         return (uint32_t)(NARROW ? nl[u] >> a.lshift : (uint64_t)nl[u] >> 32);
     });
-    push_near<ILP>(a, st, t, flush, to_near, vs, deg);
+    push_near<N>(a, st, t, flush, to_near, vs, deg);
     if (SCAN && t.dense) {
         dn = __reduce_add_sync(FULL, dn);
         if (lane_id() == 0 && dn) st.dn_near[threadIdx.x >> 5] += dn;
@@ -586,12 +606,13 @@ __device__ __forceinline__ void relax_rows(const SsspArgs &a, Stage &st, const P
     const uint32_t total = __shfl_sync(FULL, incl, 31);
     const uint32_t excl = lane < rows ? incl - deg : INF32;
     const uint32_t base = s - excl;      // arc of position j in row r: base(r) + j
-    auto load = [&](uint32_t b, ArcGroup<NARROW> &g) {
+    auto load = [&](uint32_t b, auto &g) {
+        constexpr int N = sizeof(g.e) / sizeof(g.e[0]);
 #pragma unroll
-        for (int q = 0; q < ILP; ++q) {
+        for (int q = 0; q < N; ++q) {
             const uint32_t b0 = b + 32 * q, j = b0 + lane;
             // rows that start in this window, and those before it
-            const uint32_t before = (uint32_t)__popc(__ballot_sync(FULL, excl < b0));
+            const uint32_t before = N == 1 ? 0u : (uint32_t)__popc(__ballot_sync(FULL, excl < b0));
             const uint32_t at = excl - b0;
             const uint32_t starts = __reduce_or_sync(FULL, at < 32 ? 1u << at : 0u);
             const uint32_t row = before + (uint32_t)__popc(starts & (FULL >> (31 - lane))) - 1;
@@ -604,13 +625,23 @@ __device__ __forceinline__ void relax_rows(const SsspArgs &a, Stage &st, const P
             if (g.valid[q]) g.e[q] = stream ? __ldcs(&a.adj[arc]) : __ldg(&a.adj[arc]);
         }
     };
-    ArcGroup<NARROW> g;
+    if (total <= 32) {
+        // a thin frontier's batch: one arc per lane, a quarter of the
+        // instructions (a hop is bound by them as much as by its round trips)
+        ArcGroup<NARROW, 1> g;
+        load(0, g);
+        relax_group<NARROW, SCAN, 1>(a, st, t, g, flush, precheck, wlo, whi, attempts, improved,
+                                     narrow_miss);
+        return;
+    }
+    ArcGroup<NARROW, ILP> g;
     load(0, g);
     for (uint32_t b = 0; b < total; b += 32 * ILP) {
-        ArcGroup<NARROW> next;
+        ArcGroup<NARROW, ILP> next;
         const bool more = b + 32 * ILP < total;
         if (more) load(b + 32 * ILP, next);
-        relax_group<NARROW, SCAN>(a, st, t, g, flush, precheck, wlo, whi, attempts, improved, narrow_miss);
+        relax_group<NARROW, SCAN, ILP>(a, st, t, g, flush, precheck, wlo, whi, attempts, improved,
+                                       narrow_miss);
         if (more) g = next;
     }
 }
@@ -1026,7 +1057,9 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
                     --rounds;
                     __syncwarp();
                     local_hi = min(*(volatile uint32_t *)&st.near_n[wib], NEAR_REGION);
-                    if (local_lo >= local_hi) break;
+                    // (a thin frontier that grew past a batch goes back to
+                    // the queue: the other warps take their share)
+                    if (local_lo >= local_hi || (local_hi - local_lo > 32 && !a.local_rounds)) break;
                     nb = (local_hi - local_lo + 31) / 32;
                 } else {
                     if (wi + nwarps >= n_fixed && n_fixed != n_work && lane == 0)
@@ -1568,41 +1601,18 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.pull = p.far_scan ? p.pull : 0u;
     a.tail = p.tail;
     a.m = g.m;
-    // Thin frontiers with the far pile (see the kernel).  Few arcs per vertex
-    // mean a high diameter (grids, paths, trees): below eight vertices per
-    // warp a frontier there also takes 16 warp-local rounds, so that a
-    // barrier is paid every 16 hops (grid 1021 x 733, k = 37: 2.4 ms; split
-    // early without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.64
-    // against 1.21).  On denser graphs a warp's own rounds would relax hub
-    // rows alone (R-MAT 12: 0.93 ms against 0.20); there a frontier below
-    // one vertex per warp only splits early (0.29 against 0.31 ms).  With
-    // local rounds asked for the frontier is rarely latency-bound, and the
-    // early split only unsettles it (grid 4096 x 4096: 9.7 against 9.25 ms).
     a.step0 = p.far_scan ? first_step(g, p.delta) : 0u;
     // Thin frontiers with the far pile (see the kernel).  Few arcs per vertex
     // mean a high diameter (grids, paths, trees): below eight vertices per
     // warp a frontier there also takes 16 warp-local rounds, so that a
-    // barrier is paid every 16 hops (grid 1021 x 733, k = 37: 2.4 ms; split
-    // early without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.64
-    // against 1.21).  On denser graphs a warp's own rounds would relax hub
-    // rows alone (R-MAT 12: 0.93 ms against 0.20); there a frontier below
-    // one vertex per warp only splits early (0.29 against 0.31 ms).  With
-    // local rounds asked for the frontier is rarely latency-bound, and the
-    // early split only unsettles it (grid 4096 x 4096: 9.7 against 9.25 ms).
-    // The first band's inner threshold (the default band width is 32 mean
-    // weights over the mean degree): on R-MAT graphs the hubs and most of the
-    // core settle below half a mean weight over the mean degree, and with
-    // them settled the rest of the band improves most vertices once.  R-MAT
-    // of 10^6 vertices, k = 101, default band: 54 -> 26 M relaxations, 1.72
-    // -> 1.10 ms (1.06 at a 48th, 1.35 at a 96th of the default width);
-    // R-MAT 24, k = 700: 11.2 -> 6.6 ms.  Bands narrowed by tuning gain less
-    // and take an eighth of themselves: R-MAT 26 (degree 8), k = 10,000 14.2
-    // -> 13.4 ms, R-MAT 22, weights to 10^5, k = 64 2.35 -> 2.04.
-    a.step0 = 0;
-    if (a.defer && p.far_scan) {
-        a.step0 = p.delta > g.delta0 / 8 ? g.delta0 / 64 : p.delta / 8;
-        if (a.step0 < 2) a.step0 = 2;
-    }
+    // barrier is paid every 16 hops, until one has more than a batch to relax
+    // (grid 1021 x 733, k = 37: 2.04 ms; 2.39 without that limit; split early
+    // without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.58 against 1.21).
+    // On denser graphs a warp's own rounds would relax hub rows alone (R-MAT
+    // 12: 0.93 ms against 0.20); there a frontier below one vertex per warp
+    // only splits early (0.29 against 0.31 ms).  With local rounds asked for
+    // the frontier is rarely latency-bound, and the early split only unsettles
+    // it (grid 4096 x 4096: 9.7 against 9.25 ms).
     const uint32_t warps = (uint32_t)(geo.sssp_blocks * (geo.threads / 32));
     const bool sparse_rows = g.m <= 8ull * g.n;
     a.thin = p.local_rounds ? 1u : sparse_rows ? 8 * warps : warps;
