@@ -349,6 +349,8 @@ int run_pipeline_once(steiner_graph *G, const std::vector<int32_t> &ss, bool ful
     CK(mark(2));
     const bool pruned = full && tree_only && tree_scan_applies(G->g, ws, k, G->delta);
     if (pruned) CK(launch_tree_scan(G->g, ws, k, G->delta, G->geo, s));
+    else if (!full && pred_scan_applies(G->g, ws, G->delta))
+        CK(launch_pred_scan(G->g, ws, k, G->delta, s));
     else CK(launch_scan(G->g, ws, k, full, s));
     uint32_t launches = 4;      // init labels, init seeds, SSSP, scan
     const bool small = full && small_tail(k);
@@ -858,7 +860,8 @@ int steiner_voronoi(steiner_graph_t G, const int32_t *seeds, uint32_t k, int32_t
     if (hc) d_cell = reinterpret_cast<int32_t *>(G->ws.tree_key);
     if (hd) d_dist = reinterpret_cast<uint32_t *>(G->ws.tree_key2);
     if (hp) d_pred = reinterpret_cast<int32_t *>(G->ws.tree_w);
-    CK(launch_export(G->g, G->ws, k, d_cell, d_dist, d_pred, s));
+    const uint32_t split = pred_scan_applies(G->g, G->ws, G->delta) ? G->delta : 0u;
+    CK(launch_export(G->g, G->ws, split, d_cell, d_dist, d_pred, s));
     if (hc) CK(cudaMemcpyAsync(cell, d_cell, (size_t)n * 4, cudaMemcpyDeviceToHost, s));
     if (hd) CK(cudaMemcpyAsync(dist, d_dist, (size_t)n * 4, cudaMemcpyDeviceToHost, s));
     if (hp) CK(cudaMemcpyAsync(pred, d_pred, (size_t)n * 4, cudaMemcpyDeviceToHost, s));

@@ -24,6 +24,8 @@
 // batches after the hubs held up to 32 x 255 arcs, read 32 at a time: pairs
 // and predecessors of R-MAT 16 took 0.19 ms, 0.034 in ranges; R-MAT of 10^6
 // vertices 0.26 against 0.14; R-MAT 26 (degree 8) 5.9 against 5.6.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace stn {
@@ -236,11 +238,13 @@ __device__ __forceinline__ void propose_bridge(const TreeScanArgs &a, uint32_t c
 }
 
 // Arc `arc` = (v, head, w) of step 1, lu the head's label.
+template <bool PAIRS>
 __device__ __forceinline__ void tree_arc(const TreeScanArgs &a, uint32_t v, uint32_t lv,
                                          uint32_t arc, uint2 e, uint32_t lu) {
     if (lu == INF32) return;
     const uint64_t sum = ((uint64_t)e.y << a.lshift) + lu;       // the head's distance + w
     if (sum == lv) atomicMin(&a.pred_arc[v], arc);
+    if (!PAIRS) return;
     const uint32_t mask = (1u << a.lshift) - 1u, cv = lv & mask, cu = lu & mask;
     if (cv >= cu) return;
     const uint64_t b = (lv >> a.lshift) + (sum >> a.lshift);
@@ -249,6 +253,9 @@ __device__ __forceinline__ void tree_arc(const TreeScanArgs &a, uint32_t v, uint
 
 constexpr int TREE_ILP = 2;        // arcs in flight per lane (full occupancy matters more)
 
+// PAIRS: step 1.  Else the predecessors of every vertex, for a Voronoi call:
+// the rows of the vertices beyond delta too, whole.
+template <bool PAIRS>
 __global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant__ TreeScanArgs a) {
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -276,12 +283,12 @@ __global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant
 #pragma unroll
                 for (int q = 0; q < TREE_ILP; ++q) {
                     // (an arc heavier than the row's distance is not tight)
-                    const bool look = x[q].y && (!far || x[q].y <= lv >> a.lshift);
+                    const bool look = x[q].y && ((PAIRS && !far) || x[q].y <= lv >> a.lshift);
                     lu[q] = look ? __ldg(&a.label32[x[q].x]) : INF32;
                 }
 #pragma unroll
                 for (int q = 0; q < TREE_ILP; ++q)
-                    tree_arc(a, v, lv, b + 32 * q + lane, x[q], lu[q]);
+                    tree_arc<PAIRS>(a, v, lv, b + 32 * q + lane, x[q], lu[q]);
             }
             continue;
         }
@@ -291,9 +298,10 @@ __global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant
             uint32_t s = 0, deg = 0, lv = INF32;
             if (v < v1) {
                 lv = __ldg(&a.label32[v]);
-                if (lv < a.near) {
+                if (lv < a.near || (!PAIRS && lv != INF32)) {
                     s = a.row_ptr[v];
-                    deg = a.row_ptr[v + 1] - s >= HEAVY_DEG ? 0u : a.lend[v] - s;
+                    const uint32_t r1 = a.row_ptr[v + 1];
+                    deg = r1 - s >= HEAVY_DEG ? 0u : (lv < a.near ? a.lend[v] : r1) - s;
                 }
             }
             const uint32_t rows = __ballot_sync(FULL, deg != 0);
@@ -304,7 +312,7 @@ __global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant
             uint32_t before = 0;             // rows that start before the window
             for (uint32_t b = 0; b < total; b += 32 * TREE_ILP) {
                 uint2 x[TREE_ILP];
-                uint32_t lu[TREE_ILP], own[TREE_ILP], at[TREE_ILP];
+                uint32_t lu[TREE_ILP], own[TREE_ILP], at[TREE_ILP], lo[TREE_ILP];
 #pragma unroll
                 for (int q = 0; q < TREE_ILP; ++q) {
                     const uint32_t w0 = b + 32 * q, j = w0 + lane;
@@ -312,16 +320,19 @@ __global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant
                     own[q] = nth_set_bit(rows, before + (uint32_t)__popc(starts & (FULL >> (31 - lane))) - 1);
                     before += (uint32_t)__popc(starts);
                     at[q] = __shfl_sync(FULL, s - excl, own[q]) + j;
+                    lo[q] = __shfl_sync(FULL, lv, own[q]);
                     x[q] = make_uint2(0, 0);
-                    if (j < total) x[q] = __ldcs(&a.adj_w[at[q]]);
+                    if (j < total) x[q] = __ldcs(&(PAIRS || lo[q] < a.near ? a.adj_w : a.adj)[at[q]]);
                 }
-#pragma unroll
-                for (int q = 0; q < TREE_ILP; ++q) lu[q] = x[q].y ? __ldg(&a.label32[x[q].x]) : INF32;
 #pragma unroll
                 for (int q = 0; q < TREE_ILP; ++q) {
-                    const uint32_t lo = __shfl_sync(FULL, lv, own[q]);
-                    tree_arc(a, vb + own[q], lo, at[q], x[q], lu[q]);
+                    // (an arc heavier than the row's distance is not tight)
+                    const bool look = x[q].y && (PAIRS || x[q].y <= lo[q] >> a.lshift);
+                    lu[q] = look ? __ldg(&a.label32[x[q].x]) : INF32;
                 }
+#pragma unroll
+                for (int q = 0; q < TREE_ILP; ++q)
+                    tree_arc<PAIRS>(a, vb + own[q], lo[q], at[q], x[q], lu[q]);
             }
         }
     }
@@ -616,7 +627,7 @@ cudaError_t launch_tree_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint3
     cudaError_t e = cudaMemsetAsync(ws.pairtab, 0xFF, slots * sizeof(uint64_t), s);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)current_sm_count() * 32;
-    tree_scan_kernel<<<blocks, 256, 0, s>>>(a);
+    tree_scan_kernel<true><<<blocks, 256, 0, s>>>(a);
     e = launch_compact_pairs(ws, k, s);
     if (e == cudaSuccess) e = launch_mst(ws, k, geo, (uint64_t)delta << 32, s);
     // (the MST is done with its hooks: they count the samples)
@@ -625,6 +636,21 @@ cudaError_t launch_tree_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint3
     hub_sample_kernel<<<HUB_SAMPLES / 256, 256, 0, s>>>(a, g.n, g.m, ws.hook);
     hub_pick_kernel<<<1, 1024, 0, s>>>(ws.hook, k, ws.hub);
     rest_scan_kernel<<<blocks, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+// Predecessors alone, by the light part of most rows (R-MAT 22, weights to
+// 10^5, k = 64: Voronoi call 1.62 ms, with the full scan 1.82).
+bool pred_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t delta) {
+    return ws.narrow && active_lend(g, delta);
+}
+
+cudaError_t launch_pred_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t delta,
+                             cudaStream_t s) {
+    const TreeScanArgs a = tree_scan_args(g, ws, k, delta);
+    const uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_items;
+    const uint64_t blocks = std::min<uint64_t>((work + 7) / 8, (uint64_t)current_sm_count() * 32);
+    tree_scan_kernel<false><<<(unsigned)std::max<uint64_t>(blocks, 1), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

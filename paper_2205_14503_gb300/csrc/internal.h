@@ -247,7 +247,8 @@ cudaError_t launch_init(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t d
                         cudaStream_t s);
 cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
                         const SsspParams &p, cudaStream_t s);
-cudaError_t launch_export(const DevGraph &g, Workspace &ws, uint32_t k, int32_t *cell,
+// split_delta: the band width of launch_pred_scan (0: the full scan).
+cudaError_t launch_export(const DevGraph &g, Workspace &ws, uint32_t split_delta, int32_t *cell,
                           uint32_t *dist, int32_t *pred, cudaStream_t s);
 int sssp_occupancy(int threads);
 
@@ -269,6 +270,11 @@ cudaError_t launch_tree_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint3
                              const Geometry &geo, cudaStream_t s);
 
 // tree.cu
+// Predecessors of a Voronoi call on rows split by weight: the pred_arc of a
+// vertex nearer than the band width is then an index in adj_w.
+bool pred_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t delta);
+cudaError_t launch_pred_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t delta,
+                             cudaStream_t s);
 // limit: pairs whose key (b << 32 | slot) is at or above it are left out.
 cudaError_t launch_mst(Workspace &ws, uint32_t k, const Geometry &geo, uint64_t limit,
                        cudaStream_t s);

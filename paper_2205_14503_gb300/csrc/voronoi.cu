@@ -1499,6 +1499,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
 // ---------------------------------------------------------------------------
 
 __global__ void export_kernel(uint32_t n, const uint2 *__restrict__ adj,
+                              const uint2 *__restrict__ adj_near, uint32_t near,
                               const uint64_t *__restrict__ label,
                               const uint32_t *__restrict__ label32, uint32_t lshift,
                               const uint32_t *__restrict__ pred_arc,
@@ -1518,8 +1519,10 @@ __global__ void export_kernel(uint32_t n, const uint2 *__restrict__ adj,
         if (dist) dist[v] = (uint32_t)(lab >> 32);
         if (pred) {
             uint32_t pa = pred_arc[u];
+            // (the near vertices' arcs are indices in the split rows)
             pred[v] = pa == SEED_ARC ? (int32_t)v
-                                     : (pa == INF32 ? -1 : (int32_t)caller_id(orig_of, adj[pa].x));
+                      : pa == INF32 ? -1
+                      : (int32_t)caller_id(orig_of, (label32 && label32[u] < near ? adj_near : adj)[pa].x);
         }
     }
 }
@@ -1637,13 +1640,12 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     return cudaLaunchCooperativeKernel(fn, dim3(geo.sssp_blocks), dim3(geo.threads), args, 0, s);
 }
 
-cudaError_t launch_export(const DevGraph &g, Workspace &ws, uint32_t k, int32_t *cell,
+cudaError_t launch_export(const DevGraph &g, Workspace &ws, uint32_t split_delta, int32_t *cell,
                           uint32_t *dist, int32_t *pred, cudaStream_t s) {
-    (void)k;
-    export_kernel<<<grid_for(g.n, 256), 256, 0, s>>>(g.n, g.adj, ws.label,
-                                                      ws.narrow ? ws.label32 : nullptr, ws.lshift,
-                                                      ws.pred_arc, ws.seeds, g.orig_of, cell,
-                                                      dist, pred);
+    export_kernel<<<grid_for(g.n, 256), 256, 0, s>>>(
+        g.n, g.adj, g.adj_w, split_delta ? near_label(ws, split_delta) : 0u, ws.label,
+        ws.narrow ? ws.label32 : nullptr, ws.lshift, ws.pred_arc, ws.seeds, g.orig_of, cell, dist,
+        pred);
     return cudaGetLastError();
 }
 
