@@ -30,7 +30,7 @@
 namespace stn {
 
 // (arc, slot) pairs in flight per lane, and blocks per SM: R-MAT 22, 64 queries
-// 51 ms at two and six, 55 at four and four to six.
+// 46 ms at two and six, 48 and 51 at two and five or four, 52 at four and five.
 constexpr int MQ_ILP = 2;
 constexpr int MQ_BLOCKS = 6;
 constexpr uint32_t MQ_HOLD = 16;   // iterations a drained first band waits for others
@@ -73,6 +73,14 @@ __device__ __forceinline__ uint32_t *band_list(const MqArgs &a, uint32_t i) {
 constexpr int MQ_WARPS = 256 / 32;
 constexpr int MQ_MAX_BLOCKS = 1024;
 
+struct MqTargets {
+    uint32_t *qn, *qn_count;
+    unsigned long long *act;
+    uint32_t *farq, *far_count;
+    uint32_t *fmin;          // ctl->fmin[pile]
+    uint32_t tag_next;
+};
+
 struct MqStage {
     uint64_t boff[MQ_MAX_BLOCKS];          // pair offset of each block's frontier segment
     uint64_t wtot[MQ_WARPS];
@@ -87,6 +95,13 @@ struct MqStage {
     int32_t fpend[MQ_SLOTS];               // change of far_pending in this segment
     unsigned long long mag[MQ_SLOTS + 1];  // ceil(2^40 / c) for c = 2..64 (divmod by c)
     uint32_t lshift[MQ_SLOTS];             // rank bits of each slot's labels
+    MqTargets t;                           // where this iteration's pushes go
+    unsigned long long miss;               // slots whose distances left the 32-bit labels
+    // each warp's window of work items in the pair pass: {vertex, first arc,
+    // first pair, end of pairs}, {first arc index, last arc index, slot mask},
+    // slots | (window flags)
+    uint4 wa[MQ_WARPS][32], wb[MQ_WARPS][32];
+    uint32_t wc[MQ_WARPS][32];
 };
 
 // Slot q's label of v in the 64-bit form (dist << 32) | rank.
@@ -94,14 +109,6 @@ __device__ __forceinline__ uint64_t mq_label(const uint32_t *label, uint64_t v, 
                                              uint32_t shift) {
     return widen_label(ldcg_u32(&label[v * MQ_SLOTS + q]), shift);
 }
-
-struct MqTargets {
-    uint32_t *qn, *qn_count;
-    unsigned long long *act;
-    uint32_t *farq, *far_count;
-    uint32_t *fmin;          // ctl->fmin[pile]
-    uint32_t tag_next;
-};
 
 __device__ __forceinline__ int popc64(unsigned long long x) { return __popcll(x); }
 
@@ -212,6 +219,7 @@ __device__ __forceinline__ void mq_push_near(const MqArgs &a, MqStage &st, const
 // (as stored) of the vertex being relaxed.
 struct MqLane {
     uint32_t q, sh, lab;
+    uint32_t room, whi;      // arcs of weight `room` on do not fit; from `whi` on are not relaxed
 };
 
 // Sums of label and weight step at or above this do not fit slot labels of
@@ -225,30 +233,29 @@ __device__ __forceinline__ uint32_t mq_threshold_label(unsigned long long T, uin
 
 // Relaxes up to MQ_ILP (arc, slot) pairs per lane: arc record e[i] (weight 0:
 // no pair) for the lane's slot s0, or with TWO slots per lane s0 and s1 in
-// turn.  Only arcs of weight in [wlo, whi) are relaxed.  Labels are compared
-// and sent as stored: lab + (weight << rank bits), in 64 bits for the
-// overflow.  UNIFORM: at every i all lanes have the same arc, so the masks
-// and the stamp of its head take one atomic for the warp.
+// turn.  Only arcs of weight in [wlo, the lane's whi) are relaxed.  Labels are
+// compared and sent as stored: lab + (weight << rank bits), which fits for
+// weights below the lane's room.  UNIFORM: at every i all lanes have the same
+// arc, so the masks and the stamp of its head take one atomic for the warp.
 template <bool TWO, bool UNIFORM>
 __device__ __forceinline__ void mq_relax(const MqArgs &a, MqStage &st, const MqTargets &t,
                                          const uint2 (&e)[MQ_ILP], const MqLane &s0,
-                                         const MqLane &s1, uint32_t wlo, uint32_t whi, uint32_t &attempts,
-                                         uint32_t &improved, unsigned long long &narrow_miss) {
+                                         const MqLane &s1, uint32_t wlo, uint32_t &attempts,
+                                         uint32_t &improved) {
     uint32_t nl[MQ_ILP], cur[MQ_ILP];
 #pragma unroll
     for (int i = 0; i < MQ_ILP; ++i) {
         const MqLane &s = TWO && (i & 1) ? s1 : s0;
         nl[i] = INF32;
         cur[i] = 0;
-        if (e[i].y < wlo || e[i].y >= whi || s.lab == INF32) continue;
+        if (e[i].y < wlo || e[i].y >= s.whi) continue;
         ++attempts;
-        const uint64_t sum = ((uint64_t)e[i].y << s.sh) + s.lab;
-        if (sum >= mq_label_limit(s.sh)) {
-            narrow_miss |= 1ull << s.q;          // the slot is answered by the single-query path
+        if (e[i].y >= s.room) {
+            atomicOr(&st.miss, 1ull << s.q);     // the slot is answered by the single-query path
         } else {
             // read first: most proposals do not improve, and a load costs far
             // less L2 throughput than an atomic
-            nl[i] = (uint32_t)sum;
+            nl[i] = s.lab + (e[i].y << s.sh);
             cur[i] = ldcg_u32(&a.label[(uint64_t)e[i].x * MQ_SLOTS + s.q]);
         }
     }
@@ -335,7 +342,7 @@ __device__ __forceinline__ void mq_relax(const MqArgs &a, MqStage &st, const MqT
 // rows are cut in pieces over the grid: one arc after another, a hub left
 // unsettled in some slot held up the whole sweep (R-MAT 22, 64 queries: the
 // batch took 100 or 205 ms, by whether the draw of seeds left one).  With one
-// shared sweep and the tails behind it the same batch takes 51 ms: Voronoi
+// shared sweep and the tails behind it the same batch took 51 ms: Voronoi
 // part 70 -> 31 ms, 66 -> 23 iterations, 6 -> 1 sweeps.
 constexpr int PULL_ARCS = 4;
 constexpr int PULL_ROWS = 4;       // vertices whose labels are loaded together
@@ -344,8 +351,7 @@ __device__ __forceinline__ void mq_pull_row(const MqArgs &a, MqStage &st, const 
                                             uint32_t v, uint32_t s, uint32_t r1, uint2 mine,
                                             uint2 lv, bool ua,
                                             bool ub, uint32_t sha, uint32_t shb, uint32_t Ta,
-                                            uint32_t Tb, uint32_t &attempts, uint32_t &improved,
-                                            unsigned long long &narrow_miss) {
+                                            uint32_t Tb, uint32_t &attempts, uint32_t &improved) {
     const uint32_t lane = lane_id(), qa = 2 * lane, qb = qa + 1;
     uint32_t ba = INF32, bb = INF32;
     for (uint32_t w0 = s; w0 < r1; w0 += 32) {
@@ -370,13 +376,13 @@ __device__ __forceinline__ void mq_pull_row(const MqArgs &a, MqStage &st, const 
                     ++attempts;
                     const uint64_t sum = ((uint64_t)w << sha) + x[k].x;
                     if (sum < mq_label_limit(sha)) ba = min(ba, (uint32_t)sum);
-                    else if (lv.x == INF32) narrow_miss |= 1ull << qa;
+                    else if (lv.x == INF32) atomicOr(&st.miss, 1ull << qa);
                 }
                 if (ub && x[k].y < Tb) {
                     ++attempts;
                     const uint64_t sum = ((uint64_t)w << shb) + x[k].y;
                     if (sum < mq_label_limit(shb)) bb = min(bb, (uint32_t)sum);
-                    else if (lv.y == INF32) narrow_miss |= 1ull << qb;
+                    else if (lv.y == INF32) atomicOr(&st.miss, 1ull << qb);
                 }
             }
         }
@@ -419,8 +425,7 @@ __device__ __forceinline__ void mq_pull_row(const MqArgs &a, MqStage &st, const 
 __device__ __noinline__ void mq_pull_sweep(const MqArgs &a, MqStage &st, unsigned long long P,
                                            uint32_t *qn, uint32_t *qn_count, uint32_t *farq,
                                            uint32_t *far_count, uint32_t tag_next,
-                                           uint32_t &attempts, uint32_t &improved,
-                                           unsigned long long &narrow_miss) {
+                                           uint32_t &attempts, uint32_t &improved) {
     MqTargets t;
     t.qn = qn;
     t.qn_count = qn_count;
@@ -496,7 +501,7 @@ __device__ __noinline__ void mq_pull_sweep(const MqArgs &a, MqStage &st, unsigne
         for (int r = 0; r < PULL_ROWS; ++r)
             if (e[r] > s[r])
                 mq_pull_row(a, st, t, v0 + r, s[r], e[r], mine[r], lv[r], ua[r], ub[r], sha, shb,
-                            Ta, Tb, attempts, improved, narrow_miss);
+                            Ta, Tb, attempts, improved);
     }
 }
 
@@ -509,7 +514,6 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
     const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const bool first = gtid == 0;
     uint32_t attempts = 0, improved = 0;     // this thread's
-    unsigned long long narrow_miss = 0;
     uint32_t it = ldcg_u32(&ctl->it), fc = ldcg_u32(&ctl->fc);
     unsigned long long infl = __ldcg(&ctl->inflight) & ~__ldcg(&ctl->converged);
     unsigned long long conv_total = 0;
@@ -525,6 +529,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         st.T[threadIdx.x] = __ldcg(&ctl->T[threadIdx.x]);
         st.lshift[threadIdx.x] = ldcg_u32(&ctl->lshift[threadIdx.x]);
     }
+    if (threadIdx.x == 0) st.miss = 0;
     if (threadIdx.x <= MQ_SLOTS) {
         const uint32_t c = threadIdx.x;
         st.mag[c] = c > 1 ? ((1ull << 40) + c - 1) / c : 0ull;
@@ -620,14 +625,17 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             __syncthreads();
         }
         seg_reset(st);
-        MqTargets t;
-        t.qn = odd ? a.q0 : a.q1;
-        t.qn_count = &ctl->near_count[ns];
-        t.act = &ctl->act[ns];
-        t.farq = fc ? a.far1 : a.far0;
-        t.far_count = &ctl->far_count[fc];
-        t.fmin = ctl->fmin[fc];
-        t.tag_next = a.base_near + it + 1;
+        MqTargets &t = st.t;
+        if (threadIdx.x == 0) {
+            t.qn = odd ? a.q0 : a.q1;
+            t.qn_count = &ctl->near_count[ns];
+            t.act = &ctl->act[ns];
+            t.farq = fc ? a.far1 : a.far0;
+            t.far_count = &ctl->far_count[fc];
+            t.fmin = ctl->fmin[fc];
+            t.tag_next = a.base_near + it + 1;
+        }
+        __syncthreads();
 
         // Phase B: the W (arc, slot) pairs, numbered arc-major inside each
         // item (arc j, slot t -> j * |mask| + t), are cut into 32 chunks per
@@ -638,6 +646,14 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         // slides a window of 32 consecutive items (one per lane, loaded in
         // parallel) and spreads the window's pairs over its lanes, MQ_ILP per
         // lane in flight.
+        // Registers bound it: six blocks per SM leave 40 per thread, and with
+        // the window in registers (eight a lane, read by shuffles), pointers
+        // to the push targets and 64-bit label sums a third of the L2 traffic
+        // was spilled registers.  So each lane works out its own item's pair
+        // range and leaves it in shared memory, the targets are in shared
+        // memory too, and a lane compares an arc's weight with the room its
+        // label leaves.  R-MAT 22, 64 queries: Voronoi part 31 -> 26 ms (five
+        // blocks with more registers 28, four 31).
         const uint64_t W = st.W;
         auto gpre = [&](uint32_t i) -> uint64_t {
             return st.boff[i / seg] + __ldcg(reinterpret_cast<const unsigned long long *>(&a.item_pre[i]));
@@ -655,63 +671,78 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             }
             my_i0 = lo;
         }
+        const uint32_t wid = threadIdx.x >> 5;
         for (uint32_t ch = 0; ch < 32; ++ch) {
             uint64_t p = __shfl_sync(FULL, my_p, ch);
             const uint64_t p1 = __shfl_sync(FULL, my_p1, ch);
             uint32_t i0 = __shfl_sync(FULL, my_i0, ch);
             while (p < p1) {
-                uint32_t idx = i0 + lane;
-                uint64_t pre = ~0ull;
-                uint32_t u = 0, s0 = 0, c = 0;
-                unsigned long long M = 0;
-                if (idx < n_all) {
-                    pre = gpre(idx);
-                    u = idx < n_items ? ldcg_u32(&qc[idx]) : ldcg_u32(&blo[idx - n_items]);
-                    M = __ldcg(&a.item_mask[idx]);
-                    s0 = (idx >= n_items && a.lend) ? a.lend[u] : a.row_ptr[u];
-                    c = (uint32_t)popc64(M);
+                // the window's items, one per lane: arcs, slots and the pairs
+                // inside this chunk, left in shared memory for the warp
+                uint32_t live;
+                {
+                    const uint32_t idx = i0 + lane;
+                    const uint64_t wend = i0 + 32 < n_all ? gpre(i0 + 32) : W;
+                    const uint64_t stop = min(p1, wend);
+                    uint64_t pre = wend;
+                    uint32_t u = 0, s0 = 0, c = 0;
+                    unsigned long long M = 0;
+                    const bool hv = idx >= n_items;        // heavy-arc pass item
+                    if (idx < n_all) {
+                        pre = gpre(idx);
+                        u = hv ? ldcg_u32(&blo[idx - n_items]) : ldcg_u32(&qc[idx]);
+                        M = __ldcg(&a.item_mask[idx]);
+                        s0 = (hv && a.lend) ? a.lend[u] : a.row_ptr[u];
+                        c = (uint32_t)popc64(M);
+                    }
+                    uint64_t end = __shfl_down_sync(FULL, pre, 1);
+                    if (lane == 31) end = wend;
+                    end = min(end, stop);
+                    const uint64_t beg = max(p, pre);
+                    const bool has = c != 0 && beg < end;
+                    live = __ballot_sync(FULL, has);
+                    if (has) {
+                        // pair l of the item is (arc l / c, slot l % c)
+                        const uint32_t lo = (uint32_t)(beg - pre), hi = (uint32_t)(end - pre);
+                        const uint64_t mg = st.mag[c] << 24;
+                        const uint32_t jlo = c > 1 ? (uint32_t)__umul64hi((uint64_t)lo, mg) : lo;
+                        const uint32_t jhi = c > 1 ? (uint32_t)__umul64hi((uint64_t)(hi - 1), mg) : hi - 1;
+                        // heavy-arc items relax weights >= delta, light ones
+                        // the rest; bit 8: lower bound, bit 9: upper bound
+                        const uint32_t fl = (hv ? 256u : 0u) | (a.defer && !hv && !(M & tails) ? 512u : 0u);
+                        st.wa[wid][lane] = make_uint4(u, s0, lo, hi);
+                        st.wb[wid][lane] = make_uint4(jlo, jhi, (uint32_t)M, (uint32_t)(M >> 32));
+                        st.wc[wid][lane] = c | fl;
+                    }
+                    __syncwarp();
+                    p = stop;
+                    i0 += 32;
                 }
-                const bool hv = idx >= n_items;        // heavy-arc pass item
-                const bool whole = !hv && (M & tails); // whole row
-                const uint64_t wend = i0 + 32 < n_all ? gpre(i0 + 32) : W;
-                const uint64_t stop = min(p1, wend);
-                // The window's items one after another: an item's pairs are
-                // (arc j, slot t) -> j * c + t; the lanes take fixed slots
+                // The items one after another; the lanes take fixed slots
                 // (and, for c <= 16, several arcs per step), so a lane finds
                 // its slot and loads the tail's label once per item and then
                 // steps over the arcs.
-                for (uint32_t w = 0; w < 32; ++w) {
-                    const uint64_t pre_w = __shfl_sync(FULL, pre, w);
-                    if (pre_w >= stop) break;
-                    uint64_t end_w = w < 31 ? __shfl_sync(FULL, pre, w + 1) : wend;
-                    end_w = min(end_w, stop);
-                    const uint32_t cw = __shfl_sync(FULL, c, w);
-                    if (cw == 0 || end_w <= p || end_w <= pre_w) continue;
-                    const uint32_t uw = __shfl_sync(FULL, u, w);
-                    const uint32_t sw = __shfl_sync(FULL, s0, w);
-                    const unsigned long long Mw = __shfl_sync(FULL, M, w);
-                    const bool hw = __shfl_sync(FULL, hv, w), ww = __shfl_sync(FULL, whole, w);
-                    const uint32_t wlo = hw ? a.delta : 1u;          // (weight 0: no pair)
-                    const uint32_t whi = a.defer && !hw && !ww ? a.delta : 0xFFFFFFFFu;
-                    // the item's pairs inside this chunk: [lo, hi)
-                    const uint32_t lo = (uint32_t)((p > pre_w ? p : pre_w) - pre_w);
-                    const uint32_t hi = (uint32_t)(end_w - pre_w);
-                    const uint64_t mw = st.mag[cw];
-                    const uint32_t jlo = cw > 1 ? (uint32_t)__umul64hi((uint64_t)lo, mw << 24) : lo;
-                    const uint32_t jhi = cw > 1 ? (uint32_t)__umul64hi((uint64_t)(hi - 1), mw << 24) : hi - 1;
+                for (; live; live &= live - 1) {
+                    const uint32_t w = __ffs(live) - 1;
+                    const uint4 ia = st.wa[wid][w], ib = st.wb[wid][w];
+                    const uint32_t ic = st.wc[wid][w], cw = ic & 255u;
+                    const uint32_t wlo = ic & 256u ? a.delta : 1u;   // (weight 0: no pair)
+                    const uint32_t sw = ia.y, lo = ia.z, hi = ia.w, jhi = ib.y;
                     auto lane_slot = [&](uint32_t tq) {
-                        MqLane s{0, 0, INF32};
+                        MqLane s{0, 0, INF32, 0, 0};
                         if (tq < cw) {
-                            s.q = cw == MQ_SLOTS ? tq : nth_bit64(Mw, tq);
+                            s.q = cw == MQ_SLOTS ? tq : nth_bit64(((unsigned long long)ib.w << 32) | ib.z, tq);
                             s.sh = st.lshift[s.q];
-                            s.lab = ldcg_u32(&a.label[(uint64_t)uw * MQ_SLOTS + s.q]);
+                            s.lab = ldcg_u32(&a.label[(uint64_t)ia.x * MQ_SLOTS + s.q]);
+                            s.room = (INF32 >> s.sh) - (s.lab >> s.sh);
+                            s.whi = s.lab == INF32 ? 0u : (ic & 512u ? a.delta : INF32);
                         }
                         return s;
                     };
                     if (cw > 32) {
                         // 33..64 slots: each lane takes slots lane and lane + 32
                         const MqLane s0 = lane_slot(lane), s1 = lane_slot(lane + 32);
-                        for (uint32_t j0 = jlo; j0 <= jhi; j0 += MQ_ILP / 2) {
+                        for (uint32_t j0 = ib.x; j0 <= jhi; j0 += MQ_ILP / 2) {
                             uint2 e[MQ_ILP];
 #pragma unroll
                             for (int k = 0; k < MQ_ILP; k += 2) {
@@ -722,7 +753,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
                                 if (l < lo || l >= hi) e[k].y = 0;
                                 if (lane + 32 >= cw || l + 32 < lo || l + 32 >= hi) e[k + 1].y = 0;
                             }
-                            mq_relax<true, true>(a, st, t, e, s0, s1, wlo, whi, attempts, improved, narrow_miss);
+                            mq_relax<true, true>(a, st, t, e, s0, s1, wlo, attempts, improved);
                         }
                     } else {
                         // g lanes per arc (g = c rounded up to a power of two),
@@ -731,7 +762,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
                         const uint32_t A = 32u >> gsh;
                         const uint32_t tq = lane & ((1u << gsh) - 1u), aoff = lane >> gsh;
                         const MqLane s0 = lane_slot(tq);
-                        for (uint32_t j0 = jlo; j0 <= jhi; j0 += MQ_ILP * A) {
+                        for (uint32_t j0 = ib.x; j0 <= jhi; j0 += MQ_ILP * A) {
                             uint2 e[MQ_ILP];
 #pragma unroll
                             for (int k = 0; k < MQ_ILP; ++k) {
@@ -739,17 +770,16 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
                                 e[k] = make_uint2(0, 0);
                                 if (tq < cw && jj <= jhi && l >= lo && l < hi) e[k] = __ldg(&a.adj[sw + jj]);
                             }
-                            mq_relax<false, false>(a, st, t, e, s0, s0, wlo, whi, attempts, improved, narrow_miss);
+                            mq_relax<false, false>(a, st, t, e, s0, s0, wlo, attempts, improved);
                         }
                     }
                 }
-                p = stop;
-                i0 += 32;
+                __syncwarp();
             }
         }
         if (P) {
             mq_pull_sweep(a, st, P, t.qn, t.qn_count, t.farq, t.far_count, t.tag_next, attempts,
-                          improved, narrow_miss);
+                          improved);
             ++pull_sweeps;
         }
         unsigned long long tm3 = first ? gtimer() : 0;
@@ -899,8 +929,8 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         atomicAdd(&ctl->relax_attempts, sum_a);
         atomicAdd(&ctl->relax_improved, sum_i);
     }
-    narrow_miss = warp_or64(narrow_miss);
-    if (lane == 0 && narrow_miss) atomicOr(&ctl->slot_narrow, narrow_miss);
+    __syncthreads();
+    if (threadIdx.x == 0 && st.miss) atomicOr(&ctl->slot_narrow, st.miss);
     if (first) {
         ctl->it = it;
         ctl->fc = fc;

@@ -225,3 +225,24 @@ def test_rows_split_by_weight_around_hub_sizes(n):
                       r.integers(1, 90, n - 1 + extra))
     for delta in (1, 30, 89):
         _check(g, G.seeds_from(np.arange(n), 6, n), [("delta", delta)])
+
+
+@pytest.mark.parametrize("k", [2, 3, 5])
+@pytest.mark.parametrize("short", [0, 1, 2])
+def test_batch_labels_at_the_last_distance_that_fits(k, short):
+    """A batch slot with b rank bits holds distances below 2^(32-b) - 1: the
+    largest sum of the path, back over its last edge, lies `short` below that,
+    and only short = 0 sends the query to the single-query path."""
+    last = 2 ** (32 - int(k - 1).bit_length()) - 1 - short
+    m = 40
+    base = last // (m + 1)
+    w = [1] * (k - 1) + [last - m * base] + [base] * (m - 1)
+    n = k + m
+    g = wl.from_edges(n, np.arange(n - 1), np.arange(1, n), np.array(w))
+    sets = [np.arange(k, dtype=np.int32)] * 2
+    with st.SteinerGraph(g) as Gd:
+        rc, res = Gd.query_batch(sets)
+        reruns = Gd.get_param("batch_narrow_reruns")
+    assert rc == st.STEINER_OK and reruns == (2 if short == 0 else 0)
+    for r in res:
+        assert r.total == k - 1 and len(r.edges) == k - 1
