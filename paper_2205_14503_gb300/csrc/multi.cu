@@ -33,6 +33,14 @@ namespace stn {
 // 46 ms at two and six, 48 and 51 at two and five or four, 52 at four and five.
 constexpr int MQ_ILP = 2;
 constexpr int MQ_BLOCKS = 6;
+// The last MQ_TAKE of every 32 chunks of the pair pass go to whichever warp is
+// free: the wait at the end of an iteration, up to 0.3 ms of 3, came from warps
+// whose chunks had many improving pairs.  R-MAT 22, 64 queries: waits 5.3 ->
+// 1.9 ms, batch 46.3 -> 44.3 ms (46.5 -> 45.5 at 4 of 32, the same at 16).
+// Chunks of less than MQ_TAKE_PAIRS pairs are left with their warps: there the
+// search for a chunk costs as much as its pairs.
+constexpr uint32_t MQ_TAKE = 8;
+constexpr uint64_t MQ_TAKE_PAIRS = 64;
 constexpr uint32_t MQ_HOLD = 16;   // iterations a drained first band waits for others
 constexpr uint32_t MQ_NEAR_STAGE = 1024;
 constexpr uint32_t MQ_FAR_STAGE = 512;
@@ -557,6 +565,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             uint32_t r = (it + 2) % 3;
             ctl->near_count[r] = 0;
             ctl->act[r] = 0;
+            ctl->take[r] = 0;
             if (H) ctl->bcount[(bc + 2) % 3] = 0;
         }
         const uint32_t *qc = odd ? a.q1 : a.q0;
@@ -672,10 +681,34 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             my_i0 = lo;
         }
         const uint32_t wid = threadIdx.x >> 5;
-        for (uint32_t ch = 0; ch < 32; ++ch) {
-            uint64_t p = __shfl_sync(FULL, my_p, ch);
-            const uint64_t p1 = __shfl_sync(FULL, my_p1, ch);
-            uint32_t i0 = __shfl_sync(FULL, my_i0, ch);
+        const bool on_demand = W >= n_chunks * MQ_TAKE_PAIRS;
+        const uint32_t n_own = on_demand ? 32 - MQ_TAKE : 32;
+        for (uint32_t ch = 0;; ++ch) {
+            uint64_t p, p1;
+            uint32_t i0;
+            if (ch < n_own) {
+                p = __shfl_sync(FULL, my_p, ch);
+                p1 = __shfl_sync(FULL, my_p1, ch);
+                i0 = __shfl_sync(FULL, my_i0, ch);
+            } else {
+                if (!on_demand) break;
+                uint32_t tk = 0;
+                if (lane == 0) tk = atomicAdd(&ctl->take[cs], 1u);
+                tk = __shfl_sync(FULL, tk, 0);
+                if (tk >= MQ_TAKE * nwarps) break;
+                const uint64_t chunk = (uint64_t)n_own * nwarps + tk;
+                p = (uint64_t)((unsigned __int128)W * chunk / n_chunks);
+                p1 = (uint64_t)((unsigned __int128)W * (chunk + 1) / n_chunks);
+                // the same search for one chunk, 32 probes at a time
+                uint32_t hi = n_all;
+                i0 = 0;
+                while (hi - i0 > 1) {
+                    const uint32_t step = (hi - i0 + 31) / 32, x = i0 + lane * step;
+                    const uint32_t b = __ballot_sync(FULL, x < hi && gpre(x) <= p);
+                    i0 += (31 - __clz(b)) * step;           // (lane 0 always holds)
+                    hi = min(hi, i0 + step);
+                }
+            }
             while (p < p1) {
                 // the window's items, one per lane: arcs, slots and the pairs
                 // inside this chunk, left in shared memory for the warp

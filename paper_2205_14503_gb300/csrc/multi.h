@@ -29,6 +29,7 @@ struct MqControl {
     // never sees block 0 overwrite it with the next iteration's)
     uint32_t stop_req[2];
     uint32_t near_count[3];
+    uint32_t take[3];             // chunks of the pair pass handed out on demand
     uint32_t far_count[2];
     unsigned long long act[3];    // slots with near work queued, per iteration slot
     unsigned long long inflight;  // admitted, not yet converged (host-written)

@@ -246,3 +246,19 @@ def test_batch_labels_at_the_last_distance_that_fits(k, short):
     assert rc == st.STEINER_OK and reruns == (2 if short == 0 else 0)
     for r in res:
         assert r.total == k - 1 and len(r.edges) == k - 1
+
+
+@pytest.mark.parametrize("queries", [33, 64])
+def test_batch_chunks_handed_out_on_demand(queries):
+    """Iterations of tens of millions of (arc, slot) pairs, whose last chunks
+    go to whichever warp is free."""
+    g = wl.rmat(16, 16, wmax=1000, seed=61)
+    pool = wl.largest_cc(g)
+    sets = [wl.sample_distinct(pool, 2 + 5 * i, 700 + i) for i in range(queries)]
+    with st.SteinerGraph(g) as Gd:
+        rc, res = Gd.query_batch(sets)
+    assert rc == st.STEINER_OK
+    for s, r in list(zip(sets, res))[::5]:
+        ref = oracle.steiner(g, s)
+        np.testing.assert_array_equal(r.edges, ref.edges)
+        assert r.total == ref.total
