@@ -22,9 +22,10 @@
 //    current band (vertices with any bit set are kept in a band list), and
 //    when a slot's near work drains its heavy arcs are relaxed once, in the
 //    next shared iteration, for the listed vertices with its bit;
-//  * a slot whose first heavy-arc pass ran in the pull form finishes as one
-//    unbounded band over whole rows (its tail), as in the single-query
-//    kernel.
+//  * a slot whose band holds most of the graph (its first one as a rule, its
+//    second at the latest) runs the heavy-arc pass in the pull form and
+//    finishes as one unbounded band over whole rows (its tail), as in the
+//    single-query kernel.
 #include "multi.h"
 
 namespace stn {
@@ -103,6 +104,7 @@ struct MqStage {
     int32_t fpend[MQ_SLOTS];               // change of far_pending in this segment
     unsigned long long mag[MQ_SLOTS + 1];  // ceil(2^40 / c) for c = 2..64 (divmod by c)
     uint32_t lshift[MQ_SLOTS];             // rank bits of each slot's labels
+    uint32_t cov[MQ_SLOTS];                // sampled arcs with a settled end, then the grid's sum
     MqTargets t;                           // where this iteration's pushes go
     unsigned long long miss;               // slots whose distances left the 32-bit labels
     // each warp's window of work items in the pair pass: {vertex, first arc,
@@ -332,10 +334,11 @@ __device__ __forceinline__ void mq_relax(const MqArgs &a, MqStage &st, const MqT
     }
 }
 
-// Pull form of the first heavy-arc pass of the slots in P.  A slot in its
-// first band has threshold delta; once its near work drained, every label
-// below it is final, and a heavy arc (weight delta or more) brings a vertex
-// still at or above it only a proposal at or above it.  So instead of
+// Pull form of the heavy-arc pass of the slots in P.  A slot in its first band
+// has threshold delta; once its near work drained, every label below it is
+// final, and a heavy arc (weight delta or more) brings a vertex still at or
+// above it only a proposal at or above it.  (In a second band the same holds
+// for the band's vertices, and the first band's heavy arcs have been pushed.)  So instead of
 // pushing the heavy arcs of the band's vertices, every vertex unsettled in
 // some slot of P reads its own heavy arcs and, per arc, the label run of the
 // other end.  Lane l serves slots 2l and 2l + 1 (one 8-byte load of a run per
@@ -513,6 +516,46 @@ __device__ __noinline__ void mq_pull_sweep(const MqArgs &a, MqStage &st, unsigne
     }
 }
 
+// Which of the slots in `ask` have settled most arcs' ends, by a sample of one
+// arc per warp, spread evenly over the arcs (a slot asks only if some arc
+// weighs delta or more, so there are arcs).  One grid barrier; all blocks get
+// the same answer.  A failed barrier sets `reason`.
+// Why the pull form and the tail wait for that: they pay where little of the
+// graph is left.  A slot whose seeds lie off the core settled next to nothing
+// in its first band, made the sweep read every row (2.4 -> 9.6 ms) and then
+// carried the whole graph through its tail, alone in its label runs.  Such a
+// slot has its heavy arcs pushed instead and gets a second band, once (its
+// threshold starts at the nearest vertex it left out).  R-MAT 22, 64 queries,
+// draws with one to five such slots: 61-72 -> 44-51 ms, the others the same
+// (44-47); each ask costs 20 us.
+__device__ __noinline__ unsigned long long mq_wide_bands(const MqArgs &a, MqStage &st,
+                                                         unsigned long long ask, uint32_t &bar_target,
+                                                         uint32_t &reason) {
+    const uint32_t lane = lane_id();
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    MqControl *ctl = a.ctl;
+    if (threadIdx.x < MQ_SLOTS) st.cov[threadIdx.x] = 0;
+    __syncthreads();
+    const uint32_t arcs = a.row_ptr[a.n];
+    const uint32_t v = a.adj[(uint64_t)arcs * warp / nwarps].x;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t q = lane + 32 * h;
+        if (((ask >> q) & 1ull) &&
+            ldcg_u32(&a.label[(uint64_t)v * MQ_SLOTS + q]) < mq_threshold_label(st.T[q], st.lshift[q]))
+            atomicAdd(&st.cov[q], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < MQ_SLOTS && st.cov[threadIdx.x]) atomicAdd(&ctl->cov[threadIdx.x], st.cov[threadIdx.x]);
+    if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; return 0ull; }
+    if (threadIdx.x < MQ_SLOTS) st.cov[threadIdx.x] = ldcg_u32(&ctl->cov[threadIdx.x]);
+    __syncthreads();
+    const uint32_t lo = __ballot_sync(FULL, 2 * st.cov[lane] >= nwarps);
+    const uint32_t hi = __ballot_sync(FULL, 2 * st.cov[lane + 32] >= nwarps);
+    return (((unsigned long long)hi << 32) | lo) & ask;
+}
+
 __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_constant__ MqArgs a) {
     __shared__ MqStage st;
     MqControl *ctl = a.ctl;
@@ -529,6 +572,8 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
     unsigned long long H = __ldcg(&ctl->hpass) & infl;
     unsigned long long hp_done = __ldcg(&ctl->hp_done);
     unsigned long long band0 = __ldcg(&ctl->band0);
+    unsigned long long wide = __ldcg(&ctl->wide);       // slots whose band holds most arcs
+    unsigned long long late = __ldcg(&ctl->late);       // slots with a narrow band behind them
     unsigned long long tails = __ldcg(&ctl->tails);     // slots in their unbounded tail
     uint32_t held = ldcg_u32(&ctl->held);               // iterations that drained slots waited
     uint32_t pull_sweeps = 0;
@@ -555,7 +600,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         // survivors, with this iteration's new listings, to list bc + 1;
         // list bc + 2 (read by the previous pass) is cleared for the next.
         // slots of H in their first band run the pass in the pull form
-        const unsigned long long P = a.pull ? (H & band0) : 0ull;
+        const unsigned long long P = a.pull ? (H & band0 & wide) : 0ull;
         const uint32_t n_band = H ? min(ldcg_u32(&ctl->bcount[bc]), a.n) : 0u;
         const uint32_t n_all = n_items + n_band;
         const uint32_t tgt = H ? (bc + 1) % 3 : bc;
@@ -618,6 +663,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         unsigned long long tm1 = first ? gtimer() : 0;
         if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; break; }
         unsigned long long tm2 = first ? gtimer() : 0;
+        if (blockIdx.x == 0 && threadIdx.x < MQ_SLOTS) ctl->cov[threadIdx.x] = 0;
         // block offsets and the total
         {
             uint64_t carry = 0;
@@ -680,6 +726,16 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             }
             my_i0 = lo;
         }
+        // the same search by the whole warp for one pair, 32 probes at a time
+        auto item_of = [&](uint64_t p, uint32_t i) {
+            for (uint32_t hi = n_all; hi - i > 1;) {
+                const uint32_t step = (hi - i + 31) / 32, x = i + lane * step;
+                const uint32_t b = __ballot_sync(FULL, x < hi && gpre(x) <= p);
+                i += (31 - __clz(b)) * step;                // (lane 0 always holds)
+                hi = min(hi, i + step);
+            }
+            return i;
+        };
         const uint32_t wid = threadIdx.x >> 5;
         const bool on_demand = W >= n_chunks * MQ_TAKE_PAIRS;
         const uint32_t n_own = on_demand ? 32 - MQ_TAKE : 32;
@@ -699,15 +755,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
                 const uint64_t chunk = (uint64_t)n_own * nwarps + tk;
                 p = (uint64_t)((unsigned __int128)W * chunk / n_chunks);
                 p1 = (uint64_t)((unsigned __int128)W * (chunk + 1) / n_chunks);
-                // the same search for one chunk, 32 probes at a time
-                uint32_t hi = n_all;
-                i0 = 0;
-                while (hi - i0 > 1) {
-                    const uint32_t step = (hi - i0 + 31) / 32, x = i0 + lane * step;
-                    const uint32_t b = __ballot_sync(FULL, x < hi && gpre(x) <= p);
-                    i0 += (31 - __clz(b)) * step;           // (lane 0 always holds)
-                    hi = min(hi, i0 + step);
-                }
+                i0 = item_of(p, 0);
             }
             while (p < p1) {
                 // the window's items, one per lane: arcs, slots and the pairs
@@ -750,6 +798,14 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
                     __syncwarp();
                     p = stop;
                     i0 += 32;
+                }
+                // no pair in the window: jump over the items without any.  A
+                // band list that one slot of many passes over is full of
+                // them, and a warp that walked over a million held up its
+                // iteration for 7 to 17 ms.
+                if (!live && p < p1) {
+                    i0 = item_of(p, i0);
+                    continue;
                 }
                 // The items one after another; the lanes take fixed slots
                 // (and, for c <= 16, several arcs per step), so a lane finds
@@ -841,14 +897,23 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         hp_done &= ~act_next;
         unsigned long long idle = infl & ~act_next, S = 0, conv = 0;
         H = a.defer ? (idle & ~hp_done & ~tails) : 0ull;
-        // A pull sweep visits every vertex however few slots it serves, so
-        // drained first bands wait (up to MQ_HOLD iterations) for the other
-        // slots' and share one sweep.
-        if (a.pull && (H & band0) && (infl & band0 & act_next) && held < MQ_HOLD) {
-            idle &= ~(H & band0);
-            H &= ~band0;
+        // A pull sweep pays for a slot whose band holds most of the graph.
+        const unsigned long long ask = a.pull ? H & band0 & ~wide : 0ull;
+        if (ask) {
+            const unsigned long long most = mq_wide_bands(a, st, ask, bar_target, reason);
+            if (reason) break;
+            wide |= ask & (most | late);
+            late |= ask;
+        }
+        // The sweep visits every vertex however few slots it serves, so
+        // drained bands wait (up to MQ_HOLD iterations) for the other slots'
+        // and share one sweep.
+        const unsigned long long ready = a.pull ? H & band0 & wide : 0ull;
+        if (ready && (infl & band0 & (act_next | ~wide)) && held < MQ_HOLD) {
+            idle &= ~ready;
+            H &= ~ready;
             ++held;
-        } else if (H & band0) {
+        } else if (ready) {
             held = 0;
         }
         hp_done |= H;
@@ -858,9 +923,10 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             else S |= 1ull << q;
         }
         hp_done &= ~S;                      // a split opens a new band
-        const unsigned long long to_tail = a.pull ? S & band0 : 0ull;
+        const unsigned long long to_tail = a.pull ? S & band0 & wide : 0ull;
         tails |= to_tail;
-        band0 &= ~S;
+        if (a.pull) band0 &= ~to_tail;
+        else band0 &= ~S;
         infl &= ~conv;
         conv_total |= conv;
         if (!infl) { reason = 1; break; }
@@ -970,6 +1036,8 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         ctl->hpass = H & infl;
         ctl->hp_done = hp_done;
         ctl->band0 = band0;
+        ctl->wide = wide;
+        ctl->late = late;
         ctl->tails = tails;
         ctl->held = held;
         ctl->pull_sweeps += pull_sweeps;
@@ -1028,6 +1096,8 @@ __global__ void mq_seed_kernel(const uint32_t *__restrict__ row_ptr, uint32_t n,
         ctl->hp_done &= ~bit;
         ctl->hpass &= ~bit;
         ctl->band0 |= bit;
+        ctl->wide &= ~bit;
+        ctl->late &= ~bit;
         ctl->tails &= ~bit;
     }
     if (r >= k) return;

@@ -57,6 +57,10 @@ struct MqControl {
     // slots still in their first band (set at admission, cleared by the
     // slot's first split): their heavy-arc pass may run in the pull form
     unsigned long long band0;
+    // slots of band0 whose band holds most of the graph (their heavy-arc pass
+    // takes the pull form), and those that asked before; sampled counts
+    unsigned long long wide, late;
+    uint32_t cov[MQ_SLOTS];
     // slots in their tail: after the pull-form pass the rest runs as one
     // unbounded band over whole rows
     unsigned long long tails;

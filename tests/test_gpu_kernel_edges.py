@@ -262,3 +262,30 @@ def test_batch_chunks_handed_out_on_demand(queries):
         ref = oracle.steiner(g, s)
         np.testing.assert_array_equal(r.edges, ref.edges)
         assert r.total == ref.total
+
+
+@pytest.mark.parametrize("far", [5, 50, 5000])
+@pytest.mark.parametrize("queries", [1, 2, 40, 64])
+def test_batch_slots_whose_first_band_covers_little(queries, far):
+    """Slots with seeds on a path that hangs off the core by an edge lighter
+    or heavier than a band, among slots with seeds in the core: their heavy
+    arcs are pushed, then they get a second band, and the band list that only
+    they pass over is left out in between."""
+    g = wl.rmat(11, 12, wmax=60, seed=71)
+    pool = wl.largest_cc(g)
+    src = np.repeat(np.arange(g.n), np.diff(g.row_ptr.astype(np.int64)))
+    keep = src < g.col
+    u = np.concatenate([src[keep], [pool[0], g.n, g.n + 1]])
+    v = np.concatenate([g.col[keep], [g.n, g.n + 1, g.n + 2]])
+    w = np.concatenate([g.w[keep], [far, 3, far]])
+    g = wl.from_edges(g.n + 3, u, v, w)
+    tail = np.array([g.n - 3, g.n - 1])
+    sets = [tail if i % 7 == 0 else wl.sample_distinct(pool, 2 + i % 9, 800 + i) for i in range(queries)]
+    with st.SteinerGraph(g) as Gd:
+        Gd.set_param("batch_delta", 15)
+        rc, res = Gd.query_batch(sets)
+    assert rc == st.STEINER_OK
+    for s, r in zip(sets, res):
+        ref = oracle.steiner(g, s)
+        np.testing.assert_array_equal(r.edges, ref.edges)
+        assert r.total == ref.total
