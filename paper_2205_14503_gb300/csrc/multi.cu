@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             const unsigned long long most = mq_wide_bands(a, st, ask, bar_target, reason);
             if (reason) break;
             wide |= ask & (most | late);
-            late |= ask;
+            late |= ask & ~most;
         }
         // The sweep visits every vertex however few slots it serves, so
         // drained bands wait (up to MQ_HOLD iterations) for the other slots'
@@ -1332,6 +1332,242 @@ __global__ void __launch_bounds__(256, 5) mq_scan_kernel(MqScanArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// the scan of slots that return the tree alone
+// ---------------------------------------------------------------------------
+//
+// As in the single-query tree-only scan: mq_tree_scan_kernel reads the light
+// part of the rows, for the predecessors of the (vertex, slot) pairs nearer
+// than delta and for every bridge below delta, and whole rows only for the
+// predecessors of the vertices that are farther in some slot; the batched
+// tails form each slot's MST of those pairs; mq_rest_scan_kernel then reads
+// the rows of the (vertex, slot) pairs outside the cells of the slot's hub
+// component (the one with most arcs), and the MST of all pairs found is the
+// slot's MST of G'_1.  A predecessor is an index in the rows split by weight
+// for a pair nearer than delta, in the caller's order for another.
+//
+// The full scan evaluates every (arc, slot) pair and is bound by that; here a
+// light arc is a few 32-bit operations and most bridges fail b < delta before
+// the table is probed.  R-MAT 22, 64 queries: scan 17.1 -> 4.3 ms, tails with
+// the rest scan and the second MST 0.5 -> 1.3 ms, batch 44.0 -> 32.2 ms; R-MAT
+// 20, serving 90: 28-36 -> 25-34 ms.  It pays from about ten slots on: 8 slots
+// R-MAT 20 6.1 against 5.8 ms, R-MAT 22 19.2 against 20.3; 12 slots 6.7 against
+// 7.0 and 22.5 against 25.4.  Slots whose first band covered little are left
+// to the full scan: each would have nearly every whole row read (scan 4.3 ->
+// 9.5 ms with one to five of them, 7.5 with the full scan for these).  Exact as
+// in the single-query path: two rank bits or more rule out that a bridge
+// overflows.
+
+struct MqTreeArgs {
+    const uint32_t *__restrict__ row_ptr;
+    const uint2 *__restrict__ adj;
+    const uint2 *__restrict__ adj_w;
+    const uint32_t *__restrict__ lend;
+    const uint64_t *__restrict__ heavy_chunks;
+    uint32_t n_heavy_chunks;
+    const uint32_t *__restrict__ items;
+    uint32_t n_items;
+    uint32_t delta;
+    const uint32_t *label;
+    const uint32_t *lshift;
+    uint32_t *pred;
+    uint64_t *const *pairtab;
+    const uint32_t *k;
+    unsigned long long slots;
+    const uint32_t *orig_of, *orig_row_ptr;
+    const TailSlot *tails;           // rest scan: the retiring slots,
+    const TailOut *out;              // their hub components
+    const uint32_t *comp;            // and the component of every cell
+    uint32_t r;
+};
+
+// Proposes bridge b over arc x -> y for a table entry (x in the cell of smaller
+// rank); the key's arc is searched only if the entry goes down.
+__device__ __forceinline__ void mq_propose(const MqTreeArgs &a, uint64_t *entry, uint64_t b,
+                                           uint32_t x, uint32_t y) {
+    auto *slot = reinterpret_cast<unsigned long long *>(entry);
+    if (b > __ldg(slot) >> 32) return;
+    if (b > atomicMin(slot, (b << 32) | INF32) >> 32) return;
+    const uint32_t rs = a.row_ptr[x], want = caller_id(a.orig_of, y);
+    uint32_t lo = rs, hi = a.row_ptr[x + 1];
+    while (hi - lo > 1) {                // largest arc whose head is at or before y
+        const uint32_t mid = lo + (hi - lo) / 2;
+        if (caller_id(a.orig_of, a.adj[mid].x) <= want) lo = mid;
+        else hi = mid;
+    }
+    atomicMin(slot, (b << 32) | (uint32_t)(caller_arc_base(a.orig_of, a.orig_row_ptr, x, rs) + lo));
+}
+
+// A slot served by a lane for the whole launch.
+struct TreeSlot {
+    uint32_t q, sh, k;
+    uint64_t *tab;
+    bool on;
+};
+
+__device__ __forceinline__ TreeSlot tree_slot(const MqTreeArgs &a, uint32_t q) {
+    TreeSlot t{q, 1u, 0u, nullptr, ((a.slots >> q) & 1ull) != 0};
+    if (t.on) {
+        t.sh = a.lshift[q];
+        t.k = a.k[q];
+        t.tab = a.pairtab[q];
+    }
+    return t;
+}
+
+// Light arc `arc` = (v, y, w) for a slot with v's label lv below the near
+// limit: `limit` is that limit, or 0 for a slot that does not look.
+__device__ __forceinline__ void tree_light(const MqTreeArgs &a, const TreeSlot &t, uint32_t lv,
+                                           uint32_t limit, uint32_t v, uint32_t y, uint32_t w,
+                                           uint32_t lu, uint32_t arc, uint32_t &pmin) {
+    if (lu >= limit) return;
+    const uint32_t sum = lu + (w << t.sh);           // (both below 2^31)
+    if (sum == lv) pmin = min(pmin, arc);
+    const uint32_t b = (lv >> t.sh) + (sum >> t.sh);
+    if (b >= a.delta) return;
+    const uint32_t mask = (1u << t.sh) - 1u, cv = lv & mask, cu = lu & mask;
+    if (cv < cu) mq_propose(a, t.tab + pair_slot(cv, cu, t.k), b, v, y);
+}
+
+// Arcs [s0, s1) of `arcs`, every lane walking every arc: fn(arc, head, w,
+// labels of the head for the lane's two slots).
+template <class F>
+__device__ __forceinline__ void tree_arcs(const MqTreeArgs &a, const uint2 *__restrict__ arcs,
+                                          uint32_t s0, uint32_t s1, bool look, F fn) {
+    const uint32_t lane = lane_id();
+    for (uint32_t w0 = s0; w0 < s1; w0 += 32) {
+        uint2 mine = make_uint2(0, 0);
+        if (w0 + lane < s1) mine = __ldcs(&arcs[w0 + lane]);
+        const uint32_t got = min(32u, s1 - w0);
+        for (uint32_t i = 0; i < got; i += SCAN_ARCS) {
+            uint2 lu[SCAN_ARCS];
+#pragma unroll
+            for (int j = 0; j < SCAN_ARCS; ++j) {
+                const uint32_t head = __shfl_sync(FULL, mine.x, i + j);
+                lu[j] = make_uint2(INF32, INF32);
+                if (look && i + j < got)
+                    lu[j] = __ldg(reinterpret_cast<const uint2 *>(
+                        &a.label[(uint64_t)head * MQ_SLOTS + 2 * lane]));
+            }
+#pragma unroll
+            for (int j = 0; j < SCAN_ARCS; ++j) {
+                const uint32_t y = __shfl_sync(FULL, mine.x, i + j), w = __shfl_sync(FULL, mine.y, i + j);
+                if (i + j < got) fn(w0 + i + j, y, w, lu[j]);
+            }
+        }
+    }
+}
+
+// Calls fn(v, row start, row end, first arc offset, whole row?, v's labels)
+// for every row that is not empty, hub rows in CHUNK-arc pieces; the labels of
+// a row are fetched a row ahead.
+template <class F>
+__device__ __forceinline__ void tree_rows(const MqTreeArgs &a, F fn) {
+    const uint32_t lane = lane_id();
+    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t n_work = a.n_heavy_chunks + a.n_items;
+    auto labels = [&](uint32_t v) {
+        return __ldg(reinterpret_cast<const uint2 *>(&a.label[(uint64_t)v * MQ_SLOTS + 2 * lane]));
+    };
+    for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
+        if (wi < a.n_heavy_chunks) {
+            const uint64_t item = a.heavy_chunks[wi];
+            const uint32_t v = (uint32_t)(item >> 32);
+            fn(v, a.row_ptr[v], a.row_ptr[v + 1], (uint32_t)item * CHUNK, CHUNK, labels(v));
+            continue;
+        }
+        const uint32_t v1 = __ldg(&a.items[wi - a.n_heavy_chunks + 1]);
+        for (uint32_t v0 = __ldg(&a.items[wi - a.n_heavy_chunks]); v0 < v1; v0 += 32) {
+            const uint32_t vl = v0 + lane;
+            const uint32_t rs = vl < v1 ? a.row_ptr[vl] : 0;
+            const uint32_t re = vl < v1 ? a.row_ptr[vl + 1] : 0;
+            uint32_t rows = __ballot_sync(FULL, re - rs < HEAVY_DEG && re != rs);
+            uint2 next = rows ? labels(v0 + __ffs(rows) - 1) : make_uint2(0, 0);
+            while (rows) {
+                const uint32_t l = __ffs(rows) - 1;
+                const uint2 lv = next;
+                rows &= rows - 1;
+                if (rows) next = labels(v0 + __ffs(rows) - 1);
+                fn(v0 + l, __shfl_sync(FULL, rs, l), __shfl_sync(FULL, re, l), 0u, 0u, lv);
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256, 5) mq_tree_scan_kernel(const __grid_constant__ MqTreeArgs a) {
+    const TreeSlot t0 = tree_slot(a, 2 * lane_id()), t1 = tree_slot(a, 2 * lane_id() + 1);
+    const uint32_t n0 = t0.on ? a.delta << t0.sh : 0u, n1 = t1.on ? a.delta << t1.sh : 0u;
+    tree_rows(a, [&](uint32_t v, uint32_t rs, uint32_t re, uint32_t at, uint32_t piece, uint2 lv) {
+        const uint32_t l0 = lv.x < n0 ? n0 : 0u, l1 = lv.y < n1 ? n1 : 0u;
+        const bool f0 = t0.on && lv.x >= n0 && lv.x != INF32, f1 = t1.on && lv.y >= n1 && lv.y != INF32;
+        uint32_t p0 = INF32, p1 = INF32;
+        const uint32_t s = rs + at;
+        if (__any_sync(FULL, l0 | l1)) {
+            const uint32_t le = a.lend[v], e = piece ? min(le, s + piece) : le;
+            tree_arcs(a, a.adj_w, s, e, l0 | l1, [&](uint32_t arc, uint32_t y, uint32_t w, uint2 lu) {
+                tree_light(a, t0, lv.x, l0, v, y, w, lu.x, arc, p0);
+                tree_light(a, t1, lv.y, l1, v, y, w, lu.y, arc, p1);
+            });
+        }
+        if (__any_sync(FULL, f0 || f1)) {
+            const uint32_t e = piece ? min(re, s + piece) : re;
+            tree_arcs(a, a.adj, s, e, f0 || f1, [&](uint32_t arc, uint32_t, uint32_t w, uint2 lu) {
+                if (f0 && w <= lv.x >> t0.sh && lv.x - (w << t0.sh) == lu.x) p0 = min(p0, arc);
+                if (f1 && w <= lv.y >> t1.sh && lv.y - (w << t1.sh) == lu.y) p1 = min(p1, arc);
+            });
+        }
+        uint32_t *pp = &a.pred[(uint64_t)v * MQ_SLOTS + t0.q];
+        if (p0 != INF32) { if (piece) atomicMin(pp, p0); else *pp = p0; }
+        if (p1 != INF32) { if (piece) atomicMin(pp + 1, p1); else pp[1] = p1; }
+    });
+}
+
+__global__ void __launch_bounds__(256, 5) mq_rest_scan_kernel(const __grid_constant__ MqTreeArgs a) {
+    __shared__ uint32_t s_hub[MQ_SLOTS], s_comp0[MQ_SLOTS];
+    if (threadIdx.x < a.r) {
+        const TailSlot &sl = a.tails[threadIdx.x];
+        s_hub[sl.q] = a.out[threadIdx.x].hub;
+        s_comp0[sl.q] = sl.comp0;
+    }
+    __syncthreads();
+    const TreeSlot t0 = tree_slot(a, 2 * lane_id()), t1 = tree_slot(a, 2 * lane_id() + 1);
+    auto comp = [&](const TreeSlot &t, uint32_t l) {
+        return __ldg(&a.comp[s_comp0[t.q] + (l & ((1u << t.sh) - 1u))]);
+    };
+    tree_rows(a, [&](uint32_t v, uint32_t rs, uint32_t re, uint32_t at, uint32_t piece, uint2 lv) {
+        uint32_t c0 = 0, c1 = 0;
+        bool o0 = t0.on && lv.x != INF32, o1 = t1.on && lv.y != INF32;
+        if (o0) o0 = (c0 = comp(t0, lv.x)) != s_hub[t0.q];
+        if (o1) o1 = (c1 = comp(t1, lv.y)) != s_hub[t1.q];
+        if (!__any_sync(FULL, o0 || o1)) return;
+        auto arc_of = [&](const TreeSlot &t, uint32_t l, uint32_t c, uint32_t y, uint32_t w, uint32_t lu) {
+            if (lu == INF32 || comp(t, lu) == c) return;
+            const uint32_t mask = (1u << t.sh) - 1u, cv = l & mask, cu = lu & mask;
+            const uint64_t b = (uint64_t)(l >> t.sh) + w + (lu >> t.sh);
+            // (in the other cell's row the arc may not be read)
+            if (cv < cu) mq_propose(a, t.tab + pair_slot(cv, cu, t.k), b, v, y);
+            else mq_propose(a, t.tab + pair_slot(cu, cv, t.k), b, y, v);
+        };
+        const uint32_t s = rs + at, e = piece ? min(re, s + piece) : re;
+        tree_arcs(a, a.adj, s, e, o0 || o1, [&](uint32_t, uint32_t y, uint32_t w, uint2 lu) {
+            if (o0) arc_of(t0, lv.x, c0, y, w, lu.x);
+            if (o1) arc_of(t1, lv.y, c1, y, w, lu.y);
+        });
+    });
+}
+
+// Takes the slots' predecessors and pairs back to none, before the full scan.
+__global__ void mq_forget_kernel(uint32_t n, const uint32_t *label, const uint32_t *lshift, uint32_t *pred,
+                                 unsigned long long mask) {
+    const uint64_t total = (uint64_t)n * MQ_SLOTS;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t q = (uint32_t)i & (MQ_SLOTS - 1);
+        if ((mask >> q) & 1ull) pred[i] = label[i] >> lshift[q] ? INF32 : SEED_ARC;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 
@@ -1491,6 +1727,70 @@ cudaError_t mq_launch_scan(const DevGraph &g, MqState &m, unsigned long long slo
     uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>((work + 7) / 8, (uint64_t)current_sm_count() * 32));
     mq_scan_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
     return cudaGetLastError();
+}
+
+static MqTreeArgs mq_tree_args(const DevGraph &g, MqState &m, unsigned long long slots, uint32_t delta) {
+    MqTreeArgs a{};
+    a.row_ptr = g.row_ptr;
+    a.adj = g.adj;
+    a.adj_w = g.adj_w;
+    a.lend = active_lend(g, delta);
+    a.heavy_chunks = g.heavy_chunks;
+    a.n_heavy_chunks = g.n_heavy_chunks;
+    a.items = g.items;
+    a.n_items = g.n_items;
+    a.delta = delta;
+    a.label = m.label;
+    a.lshift = m.ctl->lshift;
+    a.pred = m.pred;
+    a.pairtab = m.d_pairtab;
+    a.k = m.d_k;
+    a.slots = slots;
+    a.orig_of = g.orig_of;
+    a.orig_row_ptr = g.orig_row_ptr;
+    return a;
+}
+
+static unsigned mq_tree_blocks(const DevGraph &g) {
+    const uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_items;
+    return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((work + 7) / 8, (uint64_t)current_sm_count() * 32));
+}
+
+bool mq_tree_scan_applies(const DevGraph &g, uint32_t k, uint32_t delta) {
+    uint32_t b = 1;
+    while (b < 31 && (1u << b) < k) ++b;
+    return b >= 2 && g.max_w < 0x80000000u && active_lend(g, delta) && delta < 1ull << (31 - b);
+}
+
+cudaError_t mq_launch_tree_scan(const DevGraph &g, MqState &m, unsigned long long slots, uint32_t delta,
+                                cudaStream_t s) {
+    const MqTreeArgs a = mq_tree_args(g, m, slots, delta);
+    mq_tree_scan_kernel<<<mq_tree_blocks(g), 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t mq_launch_rest_scan(const DevGraph &g, MqState &m, unsigned long long slots, uint32_t delta,
+                                const TailSlot *tails, const TailOut *out, const uint32_t *comp, uint32_t r,
+                                cudaStream_t s) {
+    MqTreeArgs a = mq_tree_args(g, m, slots, delta);
+    a.tails = tails;
+    a.out = out;
+    a.comp = comp;
+    a.r = r;
+    mq_rest_scan_kernel<<<mq_tree_blocks(g), 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t mq_launch_forget(const DevGraph &g, MqState &m, unsigned long long slots, const uint32_t *ks,
+                             cudaStream_t s) {
+    mq_forget_kernel<<<current_sm_count() * 8, 256, 0, s>>>(g.n, m.label, m.ctl->lshift, m.pred, slots);
+    cudaError_t e = cudaGetLastError();
+    for (unsigned long long mm = slots; mm && e == cudaSuccess; mm &= mm - 1) {
+        const int q = __builtin_ctzll(mm);
+        const uint64_t n_slots = (uint64_t)ks[q] * (ks[q] - 1) / 2;
+        if (n_slots) e = cudaMemsetAsync(m.pairtab[q], 0xFF, n_slots * 8, s);
+    }
+    return e;
 }
 
 }  // namespace stn

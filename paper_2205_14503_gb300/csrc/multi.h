@@ -109,6 +109,7 @@ struct TailOut {
     uint32_t n_mst;              // MST pairs
     uint32_t n_edges;            // distinct tree edges
     unsigned long long total;    // D(G_S)
+    uint32_t hub;                // the MST component whose cells hold most arcs
 };
 
 // Device workspace of the batched tails, grown on demand.
@@ -138,8 +139,10 @@ void tail_ws_free(TailWs &t);
 // step.  Fills res[i] (edges allocated with malloc) and returns STEINER_OK;
 // on a buffer shortfall returns STEINER_ENOMEM with no results, and the
 // caller runs those slots one at a time.
+// tree_delta > 0: the slots went through mq_launch_tree_scan at that band
+// width; the rest scan and a second MST follow the first one.
 int run_batched_tails(steiner_graph *G, MqState &m, TailWs &t, const int *qs, const uint32_t *ks,
-                      int r, steiner_result_t *res);
+                      int r, uint32_t tree_delta, steiner_result_t *res);
 
 cudaError_t mq_alloc(const DevGraph &g, MqState &m, cudaStream_t s);
 void mq_free(MqState &m);
@@ -159,6 +162,19 @@ cudaError_t mq_launch_sssp(const DevGraph &g, MqState &m, int blocks, uint32_t d
                            cudaStream_t s);
 // Clears the shared frontier state (after an error).
 cudaError_t mq_reset(MqState &m, cudaStream_t s);
+// The scan of slots that return the tree alone, in two parts (the rest scan
+// after a first MST), where mq_tree_scan_applies to every slot.
+cudaError_t mq_launch_tree_scan(const DevGraph &g, MqState &m, unsigned long long slots, uint32_t delta,
+                                cudaStream_t s);
+cudaError_t mq_launch_rest_scan(const DevGraph &g, MqState &m, unsigned long long slots, uint32_t delta,
+                                const TailSlot *tails, const TailOut *out, const uint32_t *comp, uint32_t r,
+                                cudaStream_t s);
+// Slots that retire together from which on the tree scan is the faster one.
+constexpr int MQ_TREE_SLOTS = 9;
+bool mq_tree_scan_applies(const DevGraph &g, uint32_t k, uint32_t delta);
+// Undoes a tree scan's predecessors and pairs (slot q has ks[q] seeds).
+cudaError_t mq_launch_forget(const DevGraph &g, MqState &m, unsigned long long slots, const uint32_t *ks,
+                             cudaStream_t s);
 // Predecessors and per-slot bridge tables for the slots in `slots`.
 cudaError_t mq_launch_scan(const DevGraph &g, MqState &m, unsigned long long slots,
                            cudaStream_t s);

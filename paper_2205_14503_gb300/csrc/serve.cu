@@ -287,33 +287,65 @@ struct BatchEngine {
         if (!mask) return;
         cudaStream_t s = api_stream(G);
         double t0 = now_s();
-        cudaError_t e = mq_launch_scan(api_graph(G), m, mask, s);
+        // slots whose trees the tree scan can find; the others, and those that
+        // the batched tails turn away, take the full scan
+        const uint32_t delta = cur_delta();
+        unsigned long long tree = 0;
+        uint32_t ks[MQ_SLOTS] = {};
+        for (unsigned long long mm = mask; mm; mm &= mm - 1) {
+            const int q = __builtin_ctzll(mm);
+            ks[q] = slots[q].k;
+            if (batched_tails && mq_tree_scan_applies(api_graph(G), ks[q], delta)) tree |= 1ull << q;
+        }
+        tree &= ~h_ctl->late;      // little of the graph lies within their first band
+        if (__builtin_popcountll(tree) < MQ_TREE_SLOTS) tree = 0;
+        cudaError_t e = cudaSuccess;
+        if (tree) e = mq_launch_tree_scan(api_graph(G), m, tree, delta, s);
+        if (e == cudaSuccess) e = mq_launch_scan(api_graph(G), m, mask & ~tree, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(h_ctl, m.ctl, sizeof(MqControl), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         double t1 = now_s();
         ms_scan += 1e3 * (t1 - t0);
-        // slots without overflow: their tails all at once
-        int bq[MQ_SLOTS];
-        uint32_t bk[MQ_SLOTS];
-        int nb = 0;
+        // slots without overflow: their tails all at once (those with a tree
+        // scan and the others apart)
         const unsigned long long narrow = e == cudaSuccess ? h_ctl->slot_narrow : 0ull;
-        if (e == cudaSuccess && batched_tails)
-            for (unsigned long long mm = mask & ~narrow; mm; mm &= mm - 1) {
+        steiner_result_t bres[MQ_SLOTS];
+        unsigned long long batched = 0;
+        for (int pass = 0; pass < 2 && e == cudaSuccess && batched_tails; ++pass) {
+            int bq[MQ_SLOTS];
+            uint32_t bk[MQ_SLOTS];
+            int nb = 0;
+            unsigned long long set = 0;
+            for (unsigned long long mm = (pass ? mask & ~tree : tree) & ~narrow; mm; mm &= mm - 1) {
                 const int q = __builtin_ctzll(mm);
                 if (!((h_ctl->slot_overflow >> q) & 1ull) && slots[q].k > 1) {
                     bq[nb] = q;
                     bk[nb++] = slots[q].k;
+                    set |= 1ull << q;
                 }
             }
-        steiner_result_t bres[MQ_SLOTS];
-        const bool batched = nb > 0 && run_batched_tails(G, m, tails, bq, bk, nb, bres) == STEINER_OK;
-        if (batched) ++tail_batches;
-        int bi = 0;
+            steiner_result_t res[MQ_SLOTS];
+            if (nb && run_batched_tails(G, m, tails, bq, bk, nb, pass ? 0u : delta, res) == STEINER_OK) {
+                ++tail_batches;
+                batched |= set;
+                for (int i = 0; i < nb; ++i) bres[bq[i]] = res[i];
+            }
+        }
+        const unsigned long long again = tree & ~narrow & ~batched;
+        if (e == cudaSuccess && again) {
+            e = mq_launch_forget(api_graph(G), m, again, ks, s);
+            if (e == cudaSuccess) e = mq_launch_scan(api_graph(G), m, again, s);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(h_ctl, m.ctl, sizeof(MqControl), cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        }
         for (unsigned long long mm = mask; mm; mm &= mm - 1) {
             int q = __builtin_ctzll(mm);
             steiner_result_t r{};
-            if (e != cudaSuccess) {
+            if ((batched >> q) & 1ull) {
+                r = bres[q];
+            } else if (e != cudaSuccess) {
                 r.status = STEINER_ECUDA;
                 api_set_error(std::string("batched scan: ") + cudaGetErrorString(e));
             } else if ((narrow >> q) & 1ull) {
@@ -321,8 +353,6 @@ struct BatchEngine {
                 // alone through the single-query path (64-bit labels as needed)
                 ++narrow_reruns;
                 api_query_locked(G, slot_seeds[q].data(), slots[q].k, &r);
-            } else if (batched && bi < nb && bq[bi] == q) {
-                r = bres[bi++];
             } else {
                 bool ovf = (h_ctl->slot_overflow >> q) & 1ull;
                 api_run_tail(G, m.pairtab[q], m.pred + q, MQ_SLOTS, slots[q].k, ovf, &r);

@@ -9,6 +9,8 @@
 //  * MST: one block per slot runs Boruvka on its segment under the strict
 //    order (b, rank a, rank b) (block barriers only), so each slot's MST is
 //    the unique one Kruskal finds on the same order;
+//  * after a tree scan the steps so far run twice: the first MST gives each
+//    slot's hub component, and the rest scan adds the pairs outside it;
 //  * expansion: two walkers per MST pair, as in the single-query path, on
 //    the slot's predecessor column; the walkers of all slots share one mark
 //    array with a tag per slot, so a walker stops only where its own slot
@@ -28,6 +30,7 @@ namespace stn {
 
 constexpr uint32_t BT_THREADS = 256;
 constexpr uint32_t BT_PER_THREAD = 8;
+constexpr uint32_t BT_HUB_SAMPLES = 2048;
 constexpr uint32_t BT_TILE = BT_THREADS * BT_PER_THREAD;
 
 // Slot index of global tile `tile`: the last slot whose first tile is at or
@@ -153,14 +156,24 @@ __global__ void __launch_bounds__(BT_THREADS) bt_write_kernel(const TailSlot *__
     }
 }
 
+// For the hub components after a tree scan: the arcs to sample (0: none
+// wanted) of the m, and the engine's labels.
+struct BtHub {
+    const uint2 *__restrict__ adj;
+    uint64_t m;
+    uint32_t samples;
+    const uint32_t *label, *lshift;
+};
+
 // One block per slot: Boruvka on the slot's segment with block barriers.
 // comp / hook / best hold the slot's k entries at comp0.
 __global__ void __launch_bounds__(512) bt_mst_kernel(const TailSlot *__restrict__ slots,
                                                      BtPairs p, TailOut *out, uint32_t *comp_all,
                                                      uint32_t *hook_all,
                                                      unsigned long long *best_all,
-                                                     Control *ctl) {
+                                                     BtHub h, Control *ctl) {
     __shared__ int any_s;
+    __shared__ unsigned long long most_s;
     const TailSlot sl = slots[blockIdx.x];
     const uint32_t k = sl.k;
     const uint32_t e0 = out[blockIdx.x].pair0, E = out[blockIdx.x].n_pairs;
@@ -224,6 +237,24 @@ __global__ void __launch_bounds__(512) bt_mst_kernel(const TailSlot *__restrict_
         }
         __syncthreads();
     }
+    // after a tree scan, the component whose cells hold most arcs, by a sample
+    // of arcs spread evenly (hook counts them)
+    if (h.samples) {
+        for (uint32_t c = threadIdx.x; c < k; c += blockDim.x) hook[c] = 0;
+        if (threadIdx.x == 0) most_s = 0;
+        __syncthreads();
+        const uint32_t sh = h.lshift[sl.q];
+        for (uint32_t i = threadIdx.x; i < h.samples; i += blockDim.x) {
+            const uint32_t v = h.adj[h.m * i / h.samples].x;
+            const uint32_t l = h.label[(uint64_t)v * MQ_SLOTS + sl.q];
+            if (l != INF32) atomicAdd(&hook[comp[l & ((1u << sh) - 1u)]], 1u);
+        }
+        __syncthreads();
+        for (uint32_t c = threadIdx.x; c < k; c += blockDim.x)
+            if (hook[c]) atomicMax(&most_s, (unsigned long long)hook[c] << 32 | c);
+        __syncthreads();
+        if (threadIdx.x == 0) out[blockIdx.x].hub = (uint32_t)most_s;
+    }
     uint32_t cnt = 0;
     for (uint32_t j = e0 + threadIdx.x; j < e0 + E; j += blockDim.x) cnt += p.mst[j];
 #pragma unroll
@@ -251,6 +282,11 @@ struct BtExpandArgs {
     const TailSlot *slots;
     BtPairs p;
     const uint32_t *pred;       // the engine's pred columns, MQ_SLOTS per vertex
+    // after a tree scan, the preds of labels below `near << rank bits` are
+    // indexes in these rows (else null)
+    const uint2 *__restrict__ adj_w;
+    const uint32_t *__restrict__ label, *__restrict__ lshift;
+    uint32_t near;
     uint32_t *mark;
     uint32_t tag0;              // slot i marks with tag0 + i
     uint32_t nbits;
@@ -313,7 +349,8 @@ __global__ void __launch_bounds__(256) bt_expand_kernel(BtExpandArgs a) {
                     active = false;
                 } else {
                     const uint32_t old = atomicExch(&a.mark[x], tag);
-                    const uint2 pe = a.adj[pa];
+                    const bool split = a.adj_w && a.label[(uint64_t)x * MQ_SLOTS + q] >> a.lshift[q] < a.near;
+                    const uint2 pe = (split ? a.adj_w : a.adj)[pa];
                     if (old == tag) {
                         active = false;        // this slot walked on from here already
                     } else {
@@ -409,7 +446,7 @@ static cudaError_t bt_setup(TailWs &t) {
     } while (0)
 
 int run_batched_tails(steiner_graph *G, MqState &m, TailWs &t, const int *qs,
-                      const uint32_t *ks, int r, steiner_result_t *res) {
+                      const uint32_t *ks, int r, uint32_t tree_delta, steiner_result_t *res) {
     if (r <= 0) return STEINER_OK;
     if (r > MQ_SLOTS) return STEINER_EINVAL;
     const DevGraph &g = api_graph(G);
@@ -432,26 +469,36 @@ int run_batched_tails(steiner_graph *G, MqState &m, TailWs &t, const int *qs,
     BT_CK(bt_grow(t.tile_cap, tiles, t.tile_cnt));
     BT_CK(bt_grow(t.comp_cap, comps, t.comp, t.hook, t.best));
     BT_CK(cudaMemcpyAsync(t.d_slots, t.h_slots, r * sizeof(TailSlot), cudaMemcpyHostToDevice, s));
-    BT_CK(cudaMemsetAsync(t.d_out, 0, MQ_SLOTS * sizeof(TailOut), s));
-    BT_CK(cudaMemsetAsync(t.ctl, 0, sizeof(Control), s));
-    bt_count_kernel<<<(unsigned)tiles, BT_THREADS, 0, s>>>(t.d_slots, r, t.tile_cnt);
-    bt_scan_kernel<<<1, 1024, 0, s>>>(t.tile_cnt, (uint32_t)tiles, t.d_slots, r, t.d_out, t.ctl);
-    BT_CK(cudaGetLastError());
-    BT_CK(cudaMemcpyAsync(t.h_ctl, t.ctl, sizeof(Control), cudaMemcpyDeviceToHost, s));
-    BT_CK(cudaStreamSynchronize(s));
-    const uint32_t n_pairs = t.h_ctl->n_pairs;
-    BT_CK(bt_grow(t.e_cap, n_pairs, t.e_key, t.e_ra, t.e_rb, t.e_arc, t.e_mst, t.e_owner));
+    unsigned long long mask = 0;
+    for (int i = 0; i < r; ++i) mask |= 1ull << qs[i];
+    uint32_t n_pairs = 0;
+    BtPairs p{};
+    for (int pass = tree_delta ? 0 : 1; pass < 2; ++pass) {
+        if (pass && tree_delta)
+            BT_CK(mq_launch_rest_scan(g, m, mask, tree_delta, t.d_slots, t.d_out, t.comp, (uint32_t)r, s));
+        BT_CK(cudaMemsetAsync(t.d_out, 0, MQ_SLOTS * sizeof(TailOut), s));
+        BT_CK(cudaMemsetAsync(t.ctl, 0, sizeof(Control), s));
+        bt_count_kernel<<<(unsigned)tiles, BT_THREADS, 0, s>>>(t.d_slots, r, t.tile_cnt);
+        bt_scan_kernel<<<1, 1024, 0, s>>>(t.tile_cnt, (uint32_t)tiles, t.d_slots, r, t.d_out, t.ctl);
+        BT_CK(cudaGetLastError());
+        BT_CK(cudaMemcpyAsync(t.h_ctl, t.ctl, sizeof(Control), cudaMemcpyDeviceToHost, s));
+        BT_CK(cudaStreamSynchronize(s));
+        n_pairs = t.h_ctl->n_pairs;
+        BT_CK(bt_grow(t.e_cap, n_pairs, t.e_key, t.e_ra, t.e_rb, t.e_arc, t.e_mst, t.e_owner));
+        p = BtPairs{t.e_key, t.e_ra, t.e_rb, t.e_arc, t.e_mst, t.e_owner};
+        bt_write_kernel<<<(unsigned)tiles, BT_THREADS, 0, s>>>(t.d_slots, r, t.tile_cnt, p,
+                                                                (uint32_t)t.e_cap, t.ctl);
+        bt_mst_kernel<<<r, 512, 0, s>>>(t.d_slots, p, t.d_out, t.comp, t.hook, t.best,
+                                         BtHub{g.adj, g.m, pass ? 0u : BT_HUB_SAMPLES, m.label, m.ctl->lshift},
+                                         t.ctl);
+        BT_CK(cudaGetLastError());
+    }
     // edge capacity: every slot's tree has at most n - 1 edges, and the
     // walkers of a typical batch emit a few edges per seed; start at 4M and
     // grow after a capacity miss
     if (!t.tree_cap) t.tree_cap = std::min<uint64_t>(1ull << 22, (uint64_t)g.n * r + 64);
     BT_CK(bt_grow(t.key_cap, t.tree_cap, t.key0, t.key1, t.w0, t.w1));
     const uint32_t cap = (uint32_t)std::min<uint64_t>(t.key_cap, 0xFFFFFFF0ull);
-    BtPairs p{t.e_key, t.e_ra, t.e_rb, t.e_arc, t.e_mst, t.e_owner};
-    bt_write_kernel<<<(unsigned)tiles, BT_THREADS, 0, s>>>(t.d_slots, r, t.tile_cnt, p,
-                                                            (uint32_t)t.e_cap, t.ctl);
-    bt_mst_kernel<<<r, 512, 0, s>>>(t.d_slots, p, t.d_out, t.comp, t.hook, t.best, t.ctl);
-    BT_CK(cudaGetLastError());
     uint32_t *mark = nullptr;
     const uint32_t tag0 = api_reserve_mark_tags(G, (uint32_t)r, &mark);
     if (!mark) return STEINER_ENOMEM;
@@ -460,7 +507,7 @@ int run_batched_tails(steiner_graph *G, MqState &m, TailWs &t, const int *qs,
     while ((1u << rbits) < (uint32_t)r) ++rbits;
     if (2 * nbits + rbits > 64) return STEINER_ENOMEM;    // keys do not fit: one slot at a time
     BtExpandArgs xa{g.row_ptr, g.adj, g.orig_of, g.new_of, g.orig_row_ptr, g.n, t.d_slots, p,
-                    m.pred, mark, tag0, nbits, 2 * nbits, t.key0, t.w0, cap, t.ctl};
+                    m.pred, tree_delta ? g.adj_w : nullptr, m.label, m.ctl->lshift, tree_delta, mark, tag0, nbits, 2 * nbits, t.key0, t.w0, cap, t.ctl};
     const uint64_t walkers = 2ull * n_pairs;
     const unsigned xb = (unsigned)std::max<uint64_t>(
         1, std::min<uint64_t>((walkers + 255) / 256, (uint64_t)current_sm_count() * 8));

@@ -289,3 +289,42 @@ def test_batch_slots_whose_first_band_covers_little(queries, far):
         ref = oracle.steiner(g, s)
         np.testing.assert_array_equal(r.edges, ref.edges)
         assert r.total == ref.total
+
+
+@pytest.mark.parametrize("relabel", ["0", "1"])
+@pytest.mark.parametrize("wmax,delta", [(3, 1), (3, 3), (60, 2), (60, 15), (1000, 40), (1000, 900)])
+def test_batch_tree_scan(wmax, delta, relabel, monkeypatch):
+    """Slots that return the tree alone: trees of light bridges, trees that
+    need the rest scan or are forests, hub rows in pieces, and slots too small
+    for that scan among them."""
+    monkeypatch.setenv("STEINER_RELABEL", relabel)
+    g = wl.rmat(12, 40, wmax=wmax, seed=81)
+    deg = np.diff(g.row_ptr.astype(np.int64))
+    assert deg.max() > 1024
+    pool = np.flatnonzero(deg > 0) if delta % 2 else np.arange(g.n)
+    sets = [wl.sample_distinct(pool, 2 + (i * i) % 60, 900 + i) for i in range(40)]
+    with st.SteinerGraph(g) as Gd:
+        Gd.set_param("batch_delta", delta)
+        rc, res = Gd.query_batch(sets)
+    for s, r in list(zip(sets, res))[::2]:
+        ref = oracle.steiner(g, s)
+        assert r.status == ref.status
+        np.testing.assert_array_equal(r.edges, ref.edges)
+        assert r.total == ref.total
+
+
+def test_batch_tree_scan_turned_away_by_the_tails():
+    """More tree edges than the batched tails hold: the slots' tree scans are
+    undone and each slot takes the full scan and its own tail."""
+    n = 100_000
+    rng = np.random.default_rng(91)
+    w = rng.integers(1, 51, n - 1)
+    g = wl.from_edges(n, np.arange(n - 1), np.arange(1, n), w)
+    sets = [np.unique(np.concatenate([[0, n - 1], rng.integers(0, n, 300)])) for _ in range(64)]
+    with st.SteinerGraph(g) as Gd:
+        Gd.set_param("batch_delta", 20)
+        rc, res = Gd.query_batch(sets)
+        assert Gd.get_param("batch_tail_batches") == 0
+    assert rc == st.STEINER_OK
+    for r in res:
+        assert len(r.edges) == n - 1 and r.total == w.sum()
