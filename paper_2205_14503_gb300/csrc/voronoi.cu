@@ -1025,6 +1025,48 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
         const uint32_t n_work = n_hitems + (dense_in ? (sparse ? a.n_sparse_items : a.n_items)
                                                      : (n_light + bsz - 1) / bsz);
         if (a.trace && lane == 0) trace_snap[threadIdx.x >> 5][2] = global_ns();
+        if (!SCAN && split) {
+            // The pile of the phase that this iteration ended (see the
+            // decision below): a vertex below the old threshold was settled
+            // while parked; one below the new threshold joins the next
+            // frontier, the rest the new pile.  Vertices that this
+            // iteration's relaxations push as well are kept apart by the
+            // stamps (a region without stamps may hold a vertex twice).
+            // Before the frontier, and the pile dealt out to the warps one
+            // vertex each in turn, so that the warp-local rounds follow its
+            // vertices at once, on all warps alike (grid 4096 x 4096, 32
+            // rounds: 9.2 ms split after the rounds, 8.1 before them, 7.8
+            // with the early split; from pieces of 32 the few warps that had
+            // one held up the others, 12.1).
+            const uint32_t *pile = fc ? a.far0 : a.far1;
+            for (uint64_t b = 0; b * nwarps + warp < n_far; b += 32 * SPLIT_ILP) {
+                uint32_t v[SPLIT_ILP], deg[SPLIT_ILP];
+                uint64_t d[SPLIT_ILP];
+                bool to_near[SPLIT_ILP], keep[SPLIT_ILP], to_far[SPLIT_ILP];
+#pragma unroll
+                for (int c = 0; c < SPLIT_ILP; ++c) {
+                    const uint64_t i = (b + 32u * c + lane) * nwarps + warp;
+                    v[c] = i < n_far ? ldcg_u32(&pile[i]) : INF32;
+                }
+#pragma unroll
+                for (int c = 0; c < SPLIT_ILP; ++c)
+                    d[c] = v[c] != INF32 ? sssp_label<NARROW>(a, v[c]) >> 32 : 0ull;
+#pragma unroll
+                for (int c = 0; c < SPLIT_ILP; ++c) {
+                    to_near[c] = d[c] >= T_old && d[c] < T;
+                    deg[c] = 0;
+                    if (to_near[c]) {
+                        if (v[c] < a.n_big) deg[c] = a.row_ptr[v[c] + 1] - a.row_ptr[v[c]];
+                        if (!t.nostamp || deg[c] >= HEAVY_DEG)
+                            to_near[c] = atomicExch(&a.stamp_near[v[c]], t.tag_next) != t.tag_next;
+                    }
+                    keep[c] = d[c] >= T;
+                    to_far[c] = keep[c] && atomicExch(&a.stamp_far[v[c]], t.tag_far) != t.tag_far;
+                }
+                push_far<SCAN, SPLIT_ILP>(a, st, t, to_far, keep, v, [&](int c) { return (uint32_t)d[c]; });
+                push_near<SPLIT_ILP>(a, st, t, !t.nostamp, to_near, v, deg);
+            }
+        }
         if (SCAN && hp && pull) {
             uint32_t *pile = fc ? a.far1 : a.far0;
             // with the tail to follow, the pass pushes its first frontier
@@ -1152,45 +1194,6 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
                                                                      : n_fixed + __shfl_sync(FULL, grab, 0);
             }
             if (lane == 0) st.local_lo[wib] = local_lo;
-        }
-        if (!SCAN && split) {
-            // The pile of the phase that this iteration ended (see the
-            // decision below): a vertex below the old threshold was settled
-            // while parked; one below the new threshold joins the next
-            // frontier, the rest the new pile.  Vertices that this
-            // iteration's relaxations push as well are kept apart by the
-            // stamps (a region without stamps may hold a vertex twice).
-            // After the warp-local rounds: only the warps that read the pile
-            // would follow its vertices there, and the others wait (grid
-            // 4096 x 4096, 32 rounds: Voronoi phase 11.4 against 8.5 ms).
-            const uint32_t *pile = fc ? a.far0 : a.far1;
-            for (uint32_t b = warp * 32 * SPLIT_ILP; b < n_far; b += nwarps * 32 * SPLIT_ILP) {
-                uint32_t v[SPLIT_ILP], deg[SPLIT_ILP];
-                uint64_t d[SPLIT_ILP];
-                bool to_near[SPLIT_ILP], keep[SPLIT_ILP], to_far[SPLIT_ILP];
-#pragma unroll
-                for (int c = 0; c < SPLIT_ILP; ++c) {
-                    const uint32_t i = b + 32u * c + lane;
-                    v[c] = i < n_far ? ldcg_u32(&pile[i]) : INF32;
-                }
-#pragma unroll
-                for (int c = 0; c < SPLIT_ILP; ++c)
-                    d[c] = v[c] != INF32 ? sssp_label<NARROW>(a, v[c]) >> 32 : 0ull;
-#pragma unroll
-                for (int c = 0; c < SPLIT_ILP; ++c) {
-                    to_near[c] = d[c] >= T_old && d[c] < T;
-                    deg[c] = 0;
-                    if (to_near[c]) {
-                        if (v[c] < a.n_big) deg[c] = a.row_ptr[v[c] + 1] - a.row_ptr[v[c]];
-                        if (!t.nostamp || deg[c] >= HEAVY_DEG)
-                            to_near[c] = atomicExch(&a.stamp_near[v[c]], t.tag_next) != t.tag_next;
-                    }
-                    keep[c] = d[c] >= T;
-                    to_far[c] = keep[c] && atomicExch(&a.stamp_far[v[c]], t.tag_far) != t.tag_far;
-                }
-                push_far<SCAN, SPLIT_ILP>(a, st, t, to_far, keep, v, [&](int c) { return (uint32_t)d[c]; });
-                push_near<SPLIT_ILP>(a, st, t, !t.nostamp, to_near, v, deg);
-            }
         }
         if (a.trace && it < TRACE_LEN) {
             // per warp: busy time of this iteration's relaxation (sum, max)
@@ -1609,16 +1612,16 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     // mean a high diameter (grids, paths, trees): below eight vertices per
     // warp a frontier there also takes 16 warp-local rounds, so that a
     // barrier is paid every 16 hops, until one has more than a batch to relax
-    // (grid 1021 x 733, k = 37: 2.04 ms; 2.39 without that limit; split early
+    // (grid 1021 x 733, k = 37: 1.98 ms; 2.39 without that limit; split early
     // without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.58 against 1.21).
     // On denser graphs a warp's own rounds would relax hub rows alone (R-MAT
     // 12: 0.93 ms against 0.20); there a frontier below one vertex per warp
     // only splits early (0.29 against 0.31 ms).  With local rounds asked for
-    // the frontier is rarely latency-bound, and the early split only unsettles
-    // it (grid 4096 x 4096: 9.7 against 9.25 ms).
+    // the same lines hold for the early split (grid 4096 x 4096: 7.8 ms; 8.1
+    // without, 7.9 at one vertex per warp, 8.2 at 32).
     const uint32_t warps = (uint32_t)(geo.sssp_blocks * (geo.threads / 32));
     const bool sparse_rows = g.m <= 8ull * g.n;
-    a.thin = p.local_rounds ? 1u : sparse_rows ? 8 * warps : warps;
+    a.thin = sparse_rows ? 8 * warps : warps;
     a.thin_rounds = sparse_rows ? 16u : 0u;
     a.n_big = g.n_big;
     a.n_live = g.n_live;

@@ -328,3 +328,20 @@ def test_batch_tree_scan_turned_away_by_the_tails():
     assert rc == st.STEINER_OK
     for r in res:
         assert len(r.edges) == n - 1 and r.total == w.sum()
+
+
+@pytest.mark.parametrize("local_rounds", [0, 1, 16])
+@pytest.mark.parametrize("n", [200, 4000, 600_000])
+def test_far_pile_dealt_out_to_the_warps(n, local_rounds):
+    """A far pile of a few vertices per block to several batches per warp (the
+    leaves of a broom, all beyond the first band), split and followed in the
+    same iteration, with and without warp-local rounds asked for."""
+    rng = np.random.default_rng(95)
+    u = np.concatenate([[0], np.ones(n - 2, dtype=np.int64)])
+    v = np.concatenate([[1], np.arange(2, n)])
+    w = np.concatenate([[1000], rng.integers(2, 1001, n - 2)])
+    # pairs of leaves joined, so that the next hop matters
+    a = np.arange(2, n - 1, 2)
+    g = wl.from_edges(n, np.concatenate([u, a]), np.concatenate([v, a + 1]),
+                      np.concatenate([w, rng.integers(1, 400, len(a))]))
+    _check(g, np.array([0, n // 2, n - 1]), (("delta", 1001), ("local_rounds", local_rounds)))
