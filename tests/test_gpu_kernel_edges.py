@@ -56,6 +56,9 @@ def _noalloc_graphs():
     yield "disconnected", G.random_graph(4000, 3000, 1, 20, 6)
     yield "dense", G.complete(300, 1, 40, 7)            # every row a hub
     yield "rmat", wl.rmat(12, 16, wmax=1000, seed=8)    # hubs of several pieces
+    yield "hubs", wl.rmat(14, 64, wmax=1000, seed=9)    # more hubs than a block loads at a time
+    yield "spread", G.random_tree(3000, 1, 2**20, 10)   # many bands
+    yield "wide", G.path(40, 2**25, 2**26, 11)          # thresholds near 2^32
 
 
 NOALLOC = list(_noalloc_graphs())
