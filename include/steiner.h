@@ -203,7 +203,8 @@ int steiner_serve_stop(steiner_graph_t g);
  * Tuning parameters of a graph handle (used by the autotuner):
  *   "delta"        near/far band width of the Voronoi phase (>= 1)
  *   "sssp_blocks"  blocks of the persistent Voronoi kernel (0 = every
- *                  co-resident block; at most "sssp_max_blocks")
+ *                  co-resident block; at most "sssp_max_blocks").  Forms of
+ *                  the kernel that run two blocks per SM cap it there
  *   "local_rounds" local relaxation rounds per frontier iteration
  *                  (0 = off): each warp keeps relaxing the vertices it
  *                  just queued, a hop per round, before the grid barrier.

@@ -139,6 +139,7 @@ struct Control {
     unsigned long long band_hsum;
     unsigned long long pull_hsum;
     uint32_t trace[TRACE_LEN][4];  // first iterations: near items, heavy chunks, far pile, T
+    uint32_t trace_warps;                // of the Voronoi kernel's grid
     unsigned long long trace_ns[TRACE_LEN];   // their start times (global timer, ns)
     unsigned long long trace_relax[TRACE_LEN][2];   // relaxations, improvements (traced)
     unsigned long long trace_busy[TRACE_LEN][2];    // warps' relaxation time: sum, max (ns)

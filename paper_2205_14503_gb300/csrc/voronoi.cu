@@ -36,6 +36,9 @@
 // holds most of the vertices and nearly all heavy arcs, while the vertices
 // left unsettled have few (direction-optimising search, Beamer et al.,
 // applied to delta-stepping's heavy-arc phase).
+#include <algorithm>
+#include <type_traits>
+
 #include "internal.h"
 
 namespace stn {
@@ -891,8 +894,10 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st, PullScratch
 // ---------------------------------------------------------------------------
 
 // SCAN: splits scan the labels (a.far_scan), else there is a far pile.
-template <bool NARROW, bool SCAN>
-__global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ SsspArgs a) {
+// BLOCKS per SM: three (80 registers), or two, where nothing is spilled.
+constexpr int SSSP_BLOCKS = 3;
+template <bool NARROW, bool SCAN, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS) sssp_kernel(const __grid_constant__ SsspArgs a) {
     __shared__ Stage st;
     __shared__ PushTargets t;      // this iteration's (shared: off the hot loops' registers)
     const uint32_t lane = lane_id();
@@ -946,6 +951,7 @@ __global__ void __launch_bounds__(256, 3) sssp_kernel(const __grid_constant__ Ss
             ctl->heavy_count[(it + 2) % 3] = 0;
             ctl->work_next[(it + 2) % 3] = 0;
             if (hp && pull) ++ctl->pulls;
+            ctl->trace_warps = nwarps;
             if (it < TRACE_LEN) {
                 ctl->trace[it][0] = n_light;
                 ctl->trace[it][1] = n_heavy;
@@ -1558,8 +1564,10 @@ cudaError_t launch_init(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t d
 
 // Co-resident blocks per SM that every form of the kernel reaches.
 int sssp_occupancy(int threads) {
-    const void *forms[] = {(const void *)sssp_kernel<false, false>, (const void *)sssp_kernel<false, true>,
-                           (const void *)sssp_kernel<true, false>, (const void *)sssp_kernel<true, true>};
+    const void *forms[] = {(const void *)sssp_kernel<false, false, SSSP_BLOCKS>,
+                           (const void *)sssp_kernel<false, true, SSSP_BLOCKS>,
+                           (const void *)sssp_kernel<true, false, SSSP_BLOCKS>,
+                           (const void *)sssp_kernel<true, true, SSSP_BLOCKS>};
     int least = 0;
     for (const void *fn : forms) {
         int n = 0;
@@ -1608,6 +1616,15 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.tail = p.tail;
     a.m = g.m;
     a.step0 = p.far_scan ? first_step(g, p.delta) : 0u;
+    // Three blocks per SM spill registers, two do not.  Two go faster through
+    // the chain of loads of a hop, three keep more arcs in flight.  Two, of
+    // three: R-MAT 12 0.224 ms of 0.257, 10^6 vertices (k = 101) 1.04 of 1.07,
+    // R-MAT 22 (k = 64) 1.50 of 1.58; grid 1021 x 733 1.85 of 1.96, 2048 x 1900
+    // 10.4 of 11.1.  Three, of two: R-MAT 24 5.6 ms of 6.2, R-MAT 26 (degree 8)
+    // 7.9 of 8.1; with local rounds asked for, where every warp has a chain of
+    // its own, grid 4096 x 4096 7.8 of 8.05.
+    const bool two = p.far_scan ? g.m < 1ull << 28 : !p.local_rounds;
+    const int blocks = two ? std::min(geo.sssp_blocks, 2 * geo.sm_count) : geo.sssp_blocks;
     // Thin frontiers with the far pile (see the kernel).  Few arcs per vertex
     // mean a high diameter (grids, paths, trees): below eight vertices per
     // warp a frontier there also takes 16 warp-local rounds, so that a
@@ -1619,7 +1636,7 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     // only splits early (0.29 against 0.31 ms).  With local rounds asked for
     // the same lines hold for the early split (grid 4096 x 4096: 7.8 ms; 8.1
     // without, 7.9 at one vertex per warp, 8.2 at 32).
-    const uint32_t warps = (uint32_t)(geo.sssp_blocks * (geo.threads / 32));
+    const uint32_t warps = (uint32_t)(blocks * (geo.threads / 32));
     const bool sparse_rows = g.m <= 8ull * g.n;
     a.thin = sparse_rows ? 8 * warps : warps;
     a.thin_rounds = sparse_rows ? 16u : 0u;
@@ -1636,11 +1653,15 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.lend = active_lend(g, p.delta);
     if (a.lend) a.adj = g.adj_w;        // rows partitioned by weight class
     void *args[] = {&a};
-    const void *fn = ws.narrow ? (p.far_scan ? (const void *)sssp_kernel<true, true>
-                                             : (const void *)sssp_kernel<true, false>)
-                               : (p.far_scan ? (const void *)sssp_kernel<false, true>
-                                             : (const void *)sssp_kernel<false, false>);
-    return cudaLaunchCooperativeKernel(fn, dim3(geo.sssp_blocks), dim3(geo.threads), args, 0, s);
+    auto form = [&](auto b) {
+        constexpr int B = decltype(b)::value;
+        return ws.narrow ? (p.far_scan ? (const void *)sssp_kernel<true, true, B>
+                                       : (const void *)sssp_kernel<true, false, B>)
+                         : (p.far_scan ? (const void *)sssp_kernel<false, true, B>
+                                       : (const void *)sssp_kernel<false, false, B>);
+    };
+    const void *fn = two ? form(std::integral_constant<int, 2>()) : form(std::integral_constant<int, SSSP_BLOCKS>());
+    return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(geo.threads), args, 0, s);
 }
 
 cudaError_t launch_export(const DevGraph &g, Workspace &ws, uint32_t split_delta, int32_t *cell,
