@@ -30,8 +30,9 @@
 
 namespace stn {
 
-// (arc, slot) pairs in flight per lane, and blocks per SM: R-MAT 22, 64 queries
-// 46 ms at two and six, 48 and 51 at two and five or four, 52 at four and five.
+// (arc, slot) pairs in flight per lane, and blocks per SM: R-MAT 22, 64 queries,
+// Voronoi part 26 ms at two and six (24 with the chunks on demand), 28 and 31 at
+// two and five or four, 32 at four and five.
 constexpr int MQ_ILP = 2;
 constexpr int MQ_BLOCKS = 6;
 // The last MQ_TAKE of every 32 chunks of the pair pass go to whichever warp is
@@ -1075,10 +1076,19 @@ __global__ void mq_clear_rows_kernel(uint32_t n, uint32_t *label, uint32_t *pred
     }
 }
 
-__global__ void mq_seed_kernel(const uint32_t *__restrict__ row_ptr, uint32_t n, const int32_t *seeds,
-                               const uint32_t *__restrict__ new_of, uint32_t k, uint32_t q,
-                               uint32_t delta, MqState m) {
+// The slots admitted together, one per blockIdx.y: one launch for all (with a
+// launch per slot admitting 64 queries took 0.77 ms, now 0.39).
+struct MqSeedArgs {
+    const int32_t *seeds[MQ_SLOTS];
+    uint32_t k[MQ_SLOTS];
+    uint32_t q[MQ_SLOTS];
+};
+
+__global__ void mq_seed_kernel(uint32_t n, const uint32_t *__restrict__ new_of, uint32_t delta,
+                               const __grid_constant__ MqSeedArgs a, const __grid_constant__ MqState m) {
     MqControl *ctl = m.ctl;
+    const int32_t *seeds = a.seeds[blockIdx.y];
+    const uint32_t k = a.k[blockIdx.y], q = a.q[blockIdx.y];
     uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t it = ctl->it;
     const unsigned long long bit = 1ull << q;
@@ -1086,19 +1096,15 @@ __global__ void mq_seed_kernel(const uint32_t *__restrict__ row_ptr, uint32_t n,
         uint32_t b = 1;
         while (b < 31 && (1u << b) < k) ++b;
         ctl->lshift[q] = b;
-        ctl->slot_narrow &= ~bit;
         ctl->T[q] = delta;
         ctl->fmin[0][q] = INF32;
         ctl->fmin[1][q] = INF32;
         ctl->far_pending[q] = 0;
         atomicOr(&ctl->act[it % 3], bit);
-        ctl->slot_overflow &= ~bit;
-        ctl->hp_done &= ~bit;
-        ctl->hpass &= ~bit;
-        ctl->band0 |= bit;
-        ctl->wide &= ~bit;
-        ctl->late &= ~bit;
-        ctl->tails &= ~bit;
+        atomicOr(&ctl->band0, bit);
+        for (unsigned long long *mask : {&ctl->slot_narrow, &ctl->slot_overflow, &ctl->hp_done, &ctl->hpass,
+                                         &ctl->wide, &ctl->late, &ctl->tails})
+            atomicAnd(mask, ~bit);
     }
     if (r >= k) return;
     uint32_t s = internal_id(new_of, (uint32_t)seeds[r]);
@@ -1653,10 +1659,19 @@ cudaError_t mq_launch_clear(const DevGraph &g, MqState &m, unsigned long long ma
     return cudaGetLastError();
 }
 
-cudaError_t mq_launch_seed(const DevGraph &g, MqState &m, int q, uint32_t k, uint32_t delta,
-                           cudaStream_t s) {
-    mq_seed_kernel<<<(k + 255) / 256, 256, 0, s>>>(g.row_ptr, g.n, m.seeds[q], g.new_of, k, (uint32_t)q,
-                                                    delta, m);
+cudaError_t mq_launch_seed(const DevGraph &g, MqState &m, unsigned long long slots, const uint32_t *ks,
+                           uint32_t delta, cudaStream_t s) {
+    MqSeedArgs a{};
+    uint32_t r = 0, most = 1;
+    for (unsigned long long mm = slots; mm; mm &= mm - 1, ++r) {
+        const int q = __builtin_ctzll(mm);
+        a.seeds[r] = m.seeds[q];
+        a.k[r] = ks[q];
+        a.q[r] = (uint32_t)q;
+        most = std::max(most, ks[q]);
+    }
+    if (!r) return cudaSuccess;
+    mq_seed_kernel<<<dim3((most + 255) / 256, r), 256, 0, s>>>(g.n, g.new_of, delta, a, m);
     return cudaGetLastError();
 }
 

@@ -149,11 +149,12 @@ void mq_free(MqState &m);
 int mq_occupancy(int threads);
 
 // Admission: clear the label/pred columns of the slots in `mask`, then
-// seed slot q from the k sorted seeds already copied to m.seeds[q].
+// seed each slot q in `slots` from the ks[q] sorted seeds already copied to
+// m.seeds[q].
 cudaError_t mq_launch_clear(const DevGraph &g, MqState &m, unsigned long long mask,
                             cudaStream_t s);
-cudaError_t mq_launch_seed(const DevGraph &g, MqState &m, int q, uint32_t k, uint32_t delta,
-                           cudaStream_t s);
+cudaError_t mq_launch_seed(const DevGraph &g, MqState &m, unsigned long long slots, const uint32_t *ks,
+                           uint32_t delta, cudaStream_t s);
 // Runs the persistent multi-query SSSP.  yield > 0: return once `yield`
 // slots converged or *doorbell (host-mapped) is set; yield = 0: run until
 // every in-flight slot converged.  max_iters caps this launch.

@@ -167,10 +167,9 @@ struct BatchEngine {
         double t0 = now_s();
         cudaStream_t s = api_stream(G);
         cudaError_t e = mq_launch_clear(api_graph(G), m, staged, s);
-        for (unsigned long long mm = staged; mm && e == cudaSuccess; mm &= mm - 1) {
-            int q = __builtin_ctzll(mm);
-            e = mq_launch_seed(api_graph(G), m, q, slots[q].k, cur_delta(), s);
-        }
+        uint32_t ks[MQ_SLOTS];
+        for (int q = 0; q < MQ_SLOTS; ++q) ks[q] = slots[q].k;
+        if (e == cudaSuccess) e = mq_launch_seed(api_graph(G), m, staged, ks, cur_delta(), s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         unsigned long long done = staged;
         staged = 0;

@@ -1629,8 +1629,8 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     // mean a high diameter (grids, paths, trees): below eight vertices per
     // warp a frontier there also takes 16 warp-local rounds, so that a
     // barrier is paid every 16 hops, until one has more than a batch to relax
-    // (grid 1021 x 733, k = 37: 1.98 ms; 2.39 without that limit; split early
-    // without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.58 against 1.21).
+    // (grid 1021 x 733, k = 37, three blocks per SM: 1.98 ms; 2.39 without that
+    // limit; split early without rounds 4.9, neither 6.7; 300 x 333, k = 200: 0.58 against 1.21).
     // On denser graphs a warp's own rounds would relax hub rows alone (R-MAT
     // 12: 0.93 ms against 0.20); there a frontier below one vertex per warp
     // only splits early (0.29 against 0.31 ms).  With local rounds asked for
