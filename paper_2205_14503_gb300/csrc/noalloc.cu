@@ -37,15 +37,19 @@ constexpr uint32_t NA_MAX_VERTICES = STEINER_NOALLOC_MAX_VERTICES;
 
 struct NaControl {
     GridBarrier bar;
-    uint32_t err;            // ERR_* bits, plus NA_BAD_INPUT
+    uint32_t err;            // ERR_* bits
+    // Rejected input.  The blocks leave together on a word only if nothing
+    // writes it after the barrier that they read it behind, so each check has
+    // a word of its own: row offsets (written before the first barrier),
+    // seeds (between the first and the second), neighbour ids (while the
+    // iterations run, read after the last).
+    uint32_t bad_rows, bad_seeds, bad_arcs;
     uint32_t count[3];       // frontier: short rows, rotating by iteration
     uint32_t hubs[3];        // frontier: rows of NA_HUB_DEG arcs or more
     uint32_t iterations;
     uint32_t far_min[3];     // smallest distance left beyond the threshold, by phase
     unsigned long long wsum; // sum of the sampled weights
 };
-
-constexpr uint32_t NA_BAD_INPUT = 1u << 8;   // seed list, row offsets or arc out of range
 
 // Layout of the scratch array: control block, then per-vertex arrays.
 constexpr size_t CTL_BYTES = 256;
@@ -184,7 +188,7 @@ __device__ __forceinline__ void na_relax(const NaArgs &a, NaControl *c, const Na
             cur[i] = ldcg_u64(&label[cv[i]]);
         }
     }
-    if (bad) atomicOr(&c->err, NA_BAD_INPUT);
+    if (bad) atomicOr(&c->bad_arcs, 1u);
 #pragma unroll
     for (int i = 0; i < NA_ILP; ++i) {
         imp[i] = false;
@@ -302,7 +306,7 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
             stamp[v] = 0;
             bad |= a.row_ptr[v] > a.row_ptr[v + 1];
         }
-        if (bad) atomicOr(&c->err, NA_BAD_INPUT);
+        if (bad) atomicOr(&c->bad_rows, 1u);
         if (first) c->far_min[0] = c->far_min[1] = c->far_min[2] = INF32;
         // one weight per thread, spread evenly over the arcs
         unsigned long long wt = a.n_arcs ? a.w[a.n_arcs * gtid / nth] : 0u;
@@ -311,8 +315,7 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
         if (lane == 0) atomicAdd(&c->wsum, wt);
     }
     if (!grid_sync(&c->bar, &c->err, bar_target)) return;
-    // set before the barrier: all blocks agree
-    if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;
+    if (ldcg_u32(&c->bad_rows)) return;
     // Seeds (ascending, distinct, in range) at distance 0 on the first
     // frontier (iteration 0, tag 1).
     for (uint32_t r0 = warp * 32; r0 < a.k; r0 += nwarps * 32) {
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
         if (ok) {
             s = a.seeds[r];
             if (s < 0 || (uint32_t)s >= a.n || (r && a.seeds[r - 1] >= s)) {
-                atomicOr(&c->err, NA_BAD_INPUT);
+                atomicOr(&c->bad_seeds, 1u);
                 ok = false;
             } else {
                 label[s] = (uint64_t)r;
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
         na_queue(a, NaFront{queue_of(a, 0), &c->count[0], &c->hubs[0], 1u}, ok, (uint32_t)s, &c->err);
     }
     if (!grid_sync(&c->bar, &c->err, bar_target)) return;
-    if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;
+    if (ldcg_u32(&c->bad_seeds)) return;
 
     // Iteration `it` relaxes the arcs of its frontier, queueing every vertex
     // whose label drops below the threshold T (once per iteration, by stamp).
@@ -468,7 +471,7 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
     // input leaves the caller's outputs untouched.  A block takes 256 rows,
     // a warp 32 of them with their arcs flattened over its lanes; rows of
     // NA_BLOCK_DEG arcs or more are then scanned by the whole block.
-    if (ldcg_u32(&c->err) & NA_BAD_INPUT) return;
+    if (ldcg_u32(&c->bad_arcs)) return;
     bool overflow = false;
     for (uint32_t v0 = blockIdx.x * 256; v0 < a.n; v0 += gridDim.x * 256) {
         if (threadIdx.x == 0) big_n = 0;
@@ -621,30 +624,33 @@ extern "C" int steiner_voronoi_noalloc(const uint32_t *row_ptr, const int32_t *c
         void *args[] = {&a};
         e = cudaLaunchCooperativeKernel((const void *)na_kernel, dim3(blocks), dim3(256), args, 0, s);
     }
-    uint32_t err = 0;
+    struct {
+        uint32_t err, bad_rows, bad_seeds, bad_arcs;
+    } r = {};
+    static_assert(offsetof(NaControl, bad_arcs) == offsetof(NaControl, err) + 12, "read back as one");
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&err, su.scratch + offsetof(NaControl, err), sizeof(err),
+        e = cudaMemcpyAsync(&r, su.scratch + offsetof(NaControl, err), sizeof(r),
                             cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         api_set_error(std::string("steiner_voronoi_noalloc: ") + cudaGetErrorString(e));
         return STEINER_ECUDA;
     }
-    if (err & NA_BAD_INPUT) {
+    if (r.bad_rows | r.bad_seeds | r.bad_arcs) {
         api_set_error("steiner_voronoi_noalloc: seeds must be distinct, ascending and below n, "
                       "row_ptr must run from 0 to n_arcs without decreasing, and every "
                       "neighbour id must be below n");
         return STEINER_EINVAL;
     }
-    if (err & (ERR_BARRIER | ERR_TIMEOUT)) {
+    if (r.err & (ERR_BARRIER | ERR_TIMEOUT)) {
         api_set_error("steiner_voronoi_noalloc: device loop or barrier hit its cap");
         return STEINER_ETIMEOUT;
     }
-    if (err & ERR_OVERFLOW) {
+    if (r.err & ERR_OVERFLOW) {
         api_set_error("steiner_voronoi_noalloc: a distance reached 2^32 - 1");
         return STEINER_EOVERFLOW;
     }
-    if (err & ERR_CAPACITY) {
+    if (r.err & ERR_CAPACITY) {
         api_set_error("steiner_voronoi_noalloc: frontier capacity exceeded");
         return STEINER_ENOMEM;
     }

@@ -85,6 +85,55 @@ def test_noalloc_rows_and_rounds(name, g):
         np.testing.assert_array_equal(out[2].cpu().numpy(), ref.pred)
 
 
+def _dev(a):
+    """numpy 4-byte array -> CUDA int32 tensor with the same bits."""
+    import torch
+
+    return torch.from_numpy(np.ascontiguousarray(a).view(np.int32).copy()).cuda()
+
+
+@pytest.mark.parametrize("fault", ["rows_first", "rows_last", "seeds_first", "seeds_last", "seeds_many",
+                                   "arc_first", "arc_last", "arcs_many"])
+def test_noalloc_rejects_on_every_block(fault):
+    """Hundreds of blocks leave a rejected call together, whichever of them
+    meets the fault first: EINVAL, outputs untouched, and the next call runs.
+    (Verdicts of one check kept in a word that a later check writes too would
+    let a slow block leave on a fast block's next verdict.)"""
+    import torch
+
+    n = 400_000
+    g = wl.grid(800, 500, 100, seed=31)
+    rp, col, w = (a.copy() for a in (g.row_ptr, g.col, g.w))
+    good = np.arange(0, n, 40, dtype=np.int32)
+    seeds = good.copy()
+    if fault == "rows_first":
+        rp[1] = rp[3]
+    elif fault == "rows_last":
+        rp[n - 1] = rp[n] + 1
+    elif fault == "seeds_first":
+        seeds[1] = seeds[0]
+    elif fault == "seeds_last":
+        seeds[-1] = n
+    elif fault == "seeds_many":
+        seeds[1::2] = 7
+    elif fault == "arc_first":
+        col[0] = n
+    elif fault == "arc_last":
+        col[-1] = -1
+    else:
+        col[::3] = n
+    rows, cols, ws, ok = _dev(g.row_ptr), _dev(g.col), _dev(g.w), _dev(good)
+    bad = _dev(rp), _dev(col), _dev(w), _dev(seeds)
+    ref = oracle.voronoi(g, good)
+    for _ in range(5):
+        out = [torch.full((n,), -7, dtype=torch.int32, device="cuda") for _ in range(3)]
+        assert st.steiner_voronoi_noalloc(*bad, *out) == st.STEINER_EINVAL
+        assert all(bool((o == -7).all()) for o in out)
+        assert st.steiner_voronoi_noalloc(rows, cols, ws, ok, *out) == st.STEINER_OK, st.last_error()
+        for o, r in zip(out, (ref.cell, ref.dist, ref.pred)):
+            np.testing.assert_array_equal(o.cpu().numpy().view(r.dtype), r)
+
+
 def _sparse_graphs():
     yield "grid", wl.grid(150, 111, 1000, seed=21), 30
     yield "grid_unit", wl.grid(64, 65, 1, seed=22), 9
