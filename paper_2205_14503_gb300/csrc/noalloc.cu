@@ -308,14 +308,17 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
         }
         if (bad) atomicOr(&c->bad_rows, 1u);
         if (first) c->far_min[0] = c->far_min[1] = c->far_min[2] = INF32;
-        // one weight per thread, spread evenly over the arcs
+    }
+    if (!grid_sync(&c->bar, &c->err, bar_target)) return;
+    if (ldcg_u32(&c->bad_rows)) return;
+    // One weight per thread, spread evenly over the arcs (only now: the arc
+    // count is known to be the row offsets').
+    {
         unsigned long long wt = a.n_arcs ? a.w[a.n_arcs * gtid / nth] : 0u;
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) wt += __shfl_xor_sync(FULL, wt, o);
         if (lane == 0) atomicAdd(&c->wsum, wt);
     }
-    if (!grid_sync(&c->bar, &c->err, bar_target)) return;
-    if (ldcg_u32(&c->bad_rows)) return;
     // Seeds (ascending, distinct, in range) at distance 0 on the first
     // frontier (iteration 0, tag 1).
     for (uint32_t r0 = warp * 32; r0 < a.k; r0 += nwarps * 32) {

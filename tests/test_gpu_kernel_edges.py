@@ -134,6 +134,25 @@ def test_noalloc_rejects_on_every_block(fault):
             np.testing.assert_array_equal(o.cpu().numpy().view(r.dtype), r)
 
 
+@pytest.mark.parametrize("n_arcs", [0, 2, 2**20, 2**31, 2**32 - 2])
+def test_noalloc_reads_no_arc_before_the_arc_count_is_checked(n_arcs):
+    """An arc count that the row offsets do not end at is rejected before any
+    arc or weight is read: counts far beyond the arrays behind the pointers."""
+    import torch
+
+    g = wl.grid(60, 50, 9, seed=32)
+    lib = st.load_library()
+    rp, col, w, seeds = _dev(g.row_ptr), _dev(g.col), _dev(g.w), _dev(np.array([3, 900], np.int32))
+    out = torch.full((g.n,), -7, dtype=torch.int32, device="cuda")
+    args = rp.data_ptr(), col.data_ptr(), w.data_ptr(), g.n
+    rest = seeds.data_ptr(), 2, out.data_ptr(), None, None, None
+    torch.cuda.synchronize()
+    assert lib.steiner_voronoi_noalloc(*args, n_arcs, *rest) == st.STEINER_EINVAL
+    assert "row_ptr" in st.last_error() and bool((out == -7).all())
+    assert lib.steiner_voronoi_noalloc(*args, g.n_arcs, *rest) == st.STEINER_OK, st.last_error()
+    np.testing.assert_array_equal(out.cpu().numpy(), oracle.voronoi(g, np.array([3, 900], np.int32)).cell)
+
+
 def _sparse_graphs():
     yield "grid", wl.grid(150, 111, 1000, seed=21), 30
     yield "grid_unit", wl.grid(64, 65, 1, seed=22), 9
