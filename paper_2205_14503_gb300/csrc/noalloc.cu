@@ -390,23 +390,23 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
             for (uint32_t g = 0; g < 256 && h0 + g < nh; g += 32) {
                 const uint32_t s = hub_s[g + lane], deg = hub_deg_s[g + lane];
                 const uint64_t lab = hub_lab_s[g + lane];
-                const uint32_t pieces = (deg + NA_CHUNK - 1) / NA_CHUNK;
+                const uint32_t pieces = deg / NA_CHUNK + (deg % NA_CHUNK != 0);
                 const uint32_t p0 = (warp + nwarps - (h0 + g + lane) * 97u % nwarps) % nwarps;
                 for (uint32_t m = __ballot_sync(FULL, p0 < pieces); m; m &= m - 1) {
                     const uint32_t l = __ffs(m) - 1;
                     const uint32_t sl = __shfl_sync(FULL, s, l), dl = __shfl_sync(FULL, deg, l);
                     const uint64_t ll = __shfl_sync(FULL, lab, l);
                     for (uint64_t p = __shfl_sync(FULL, p0, l); p * NA_CHUNK < dl; p += nwarps) {
-                        const uint32_t lo = (uint32_t)p * NA_CHUNK, hi = min(dl, lo + NA_CHUNK);
-                        for (uint32_t b = lo; b < hi; b += 32 * NA_ILP) {
+                        const uint32_t lo = (uint32_t)p * NA_CHUNK, len = min(dl - lo, NA_CHUNK);
+                        for (uint32_t b = 0; b < len; b += 32 * NA_ILP) {
                             bool valid[NA_ILP];
                             uint32_t arc[NA_ILP];
                             uint64_t labs[NA_ILP];
-    #pragma unroll
+#pragma unroll
                             for (int i = 0; i < NA_ILP; ++i) {
                                 const uint32_t j = b + lane + 32 * i;
-                                valid[i] = j < hi;
-                                arc[i] = sl + j;
+                                valid[i] = j < len;
+                                arc[i] = sl + lo + j;
                                 labs[i] = ll;
                             }
                             na_relax(a, c, f, region, region_n, valid, arc, labs, T, fmin);
@@ -521,10 +521,11 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
             const uint64_t lu = ldcg_u64(&label[u]);
             const uint32_t r1 = a.row_ptr[u + 1];
             uint32_t best = INF32;
-            for (uint32_t e0 = a.row_ptr[u] + threadIdx.x; e0 < r1; e0 += 256 * NA_ILP) {
+            // (64-bit: a row may end next to 2^32)
+            for (uint64_t e0 = (uint64_t)a.row_ptr[u] + threadIdx.x; e0 < r1; e0 += 256 * NA_ILP) {
 #pragma unroll
                 for (int q = 0; q < NA_ILP; ++q) {
-                    const uint64_t e = (uint64_t)e0 + 256u * q;
+                    const uint64_t e = e0 + 256u * q;
                     if (e < r1) best = min(best, na_tight(a, lu, (uint32_t)e, overflow));
                 }
             }

@@ -153,6 +153,31 @@ def test_noalloc_reads_no_arc_before_the_arc_count_is_checked(n_arcs):
     np.testing.assert_array_equal(out.cpu().numpy(), oracle.voronoi(g, np.array([3, 900], np.int32)).cell)
 
 
+@pytest.mark.parametrize("last", [1, 255, 257, 1024, 2000, 5000])
+def test_noalloc_rows_that_end_at_the_last_arc_index(last):
+    """The largest arc count (2^32 - 2): a row of `last` arcs, relaxed in
+    pieces and derived by a whole block from 256 and 1024 arcs on, ends at the
+    last index.  The arcs before it belong to a vertex that no seed reaches."""
+    import torch
+
+    if torch.cuda.mem_get_info()[0] < 48 << 30:
+        pytest.skip("needs 34 GB of device memory")
+    m = 2**32 - 2
+    col = torch.empty(m, dtype=torch.int32, device="cuda")
+    w = torch.full((m,), 9, dtype=torch.int32, device="cuda")
+    col[:2] = 3                                  # 0 -> 3 (5), 1 -> 3 (7), filler in row 2
+    w[0], w[1] = 5, 7
+    col[m - last:], w[m - last:] = 0, 5          # 3 -> 0 (5), again and again,
+    col[m - 1], w[m - 1] = 1, 7                  # and 3 -> 1 (7) last of all
+    row_ptr = _dev(np.array([0, 1, 2, m - last, m], np.uint32))
+    out = [torch.full((4,), -7, dtype=torch.int32, device="cuda") for _ in range(3)]
+    rc = st.steiner_voronoi_noalloc(row_ptr, col, w, _dev(np.array([0], np.int32)), *out)
+    del col, w
+    assert rc == st.STEINER_OK, st.last_error()
+    assert out[0].tolist() == [0, 0, -1, 0] and out[1].tolist() == [0, 12, -1, 5]
+    assert out[2].tolist() == [0, 3, -1, 0 if last > 1 else -1]
+
+
 def _sparse_graphs():
     yield "grid", wl.grid(150, 111, 1000, seed=21), 30
     yield "grid_unit", wl.grid(64, 65, 1, seed=22), 9
