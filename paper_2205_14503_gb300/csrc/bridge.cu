@@ -107,17 +107,18 @@ __global__ void __launch_bounds__(256) scan_kernel(ScanArgs a) {
             uint64_t item = a.heavy_chunks[wi / a.subs];
             uint32_t v = (uint32_t)(item >> 32), c = (uint32_t)item;
             uint32_t rs = a.row_ptr[v];
-            uint32_t s = rs + c * CHUNK + wi % a.subs * (CHUNK / SCAN_SUBS);
-            uint32_t e = min(a.row_ptr[v + 1], s + CHUNK / a.subs);
+            const RowPiece p = row_piece(rs, a.row_ptr[v + 1], c * CHUNK + wi % a.subs * (CHUNK / SCAN_SUBS),
+                                         CHUNK / a.subs);
+            if (p.count == 0) continue;
             uint64_t lv = scan_label<NARROW>(a, v);
             uint32_t cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, rs);
             // the next 32 arcs' records are loaded while these are scanned
             uint2 en = make_uint2(0, 0);
-            if (s + lane < e) en = __ldcs(&a.adj[s + lane]);    // streamed once: evict first
-            for (uint32_t b = s; b < e; b += 32) {
+            if (lane < p.count) en = __ldcs(&a.adj[p.first + lane]);    // streamed once: evict first
+            for (uint32_t j = lane; j < p.count + lane; j += 32) {
                 const uint2 ec = en;
-                if (b + 32 + lane < e) en = __ldcs(&a.adj[b + 32 + lane]);
-                scan_arc<NARROW>(a, b + lane < e, v, lv, cbase, b + lane, ec, overflow);
+                if (j + 32 < p.count) en = __ldcs(&a.adj[p.first + j + 32]);
+                scan_arc<NARROW>(a, j < p.count, v, lv, cbase, p.first + j, ec, overflow);
             }
             continue;
         }
@@ -268,17 +269,15 @@ __global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant
             const uint32_t lv = __ldg(&a.label32[v]);
             if (lv == INF32) continue;
             const bool far = lv >= a.near;           // the whole row, for the predecessor alone
-            const uint32_t rs = a.row_ptr[v], end = far ? a.row_ptr[v + 1] : a.lend[v];
-            const uint32_t s = rs + c * CHUNK, e = min(end, s + CHUNK);
-            if (s >= end) continue;
+            RowPiece p = row_piece(a.row_ptr[v], far ? a.row_ptr[v + 1] : a.lend[v], c * CHUNK, CHUNK);
             const uint2 *arcs = far ? a.adj : a.adj_w;
-            for (uint32_t b = s; b < e; b += 32 * TREE_ILP) {
+            for (; p.count; skip_arcs(p, 32 * TREE_ILP)) {
                 uint2 x[TREE_ILP];
                 uint32_t lu[TREE_ILP];
 #pragma unroll
                 for (int q = 0; q < TREE_ILP; ++q) {
                     x[q] = make_uint2(0, 0);                    // weight 0: no arc
-                    if (b + 32 * q + lane < e) x[q] = __ldcs(&arcs[b + 32 * q + lane]);
+                    if (32 * q + lane < p.count) x[q] = __ldcs(&arcs[p.first + 32 * q + lane]);
                 }
 #pragma unroll
                 for (int q = 0; q < TREE_ILP; ++q) {
@@ -288,7 +287,7 @@ __global__ void __launch_bounds__(256, 8) tree_scan_kernel(const __grid_constant
                 }
 #pragma unroll
                 for (int q = 0; q < TREE_ILP; ++q)
-                    tree_arc<PAIRS>(a, v, lv, b + 32 * q + lane, x[q], lu[q]);
+                    tree_arc<PAIRS>(a, v, lv, p.first + 32 * q + lane, x[q], lu[q]);
             }
             continue;
         }
@@ -368,9 +367,10 @@ __global__ void __launch_bounds__(256) rest_scan_kernel(const __grid_constant__ 
             if (lv == INF32) continue;
             const uint32_t cc = __ldg(&a.comp[lv & mask]);
             if (cc == hub) continue;
-            const uint32_t rs = a.row_ptr[v], s = rs + c * CHUNK, e = min(a.row_ptr[v + 1], s + CHUNK);
+            const uint32_t rs = a.row_ptr[v];
+            const RowPiece p = row_piece(rs, a.row_ptr[v + 1], c * CHUNK, CHUNK);
             const uint32_t cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, v, rs);
-            for (uint32_t j = s + lane; j < e; j += 32) arc(v, lv, cc, cbase, j);
+            for (uint32_t j = lane; j < p.count; j += 32) arc(v, lv, cc, cbase, p.first + j);
             continue;
         }
         const uint32_t v1 = __ldg(&a.items[wi - n_work + a.n_items + 1]);

@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "rows.h"
+
 namespace stn {
 
 constexpr uint32_t INF32 = 0xFFFFFFFFu;

@@ -366,9 +366,9 @@ __device__ __forceinline__ void mq_pull_row(const MqArgs &a, MqStage &st, const 
                                             uint32_t Tb, uint32_t &attempts, uint32_t &improved) {
     const uint32_t lane = lane_id(), qa = 2 * lane, qb = qa + 1;
     uint32_t ba = INF32, bb = INF32;
-    for (uint32_t w0 = s; w0 < r1; w0 += 32) {
-        if (w0 != s) mine = w0 + lane < r1 ? __ldcs(&a.adj[w0 + lane]) : make_uint2(0, 0);
-        const uint32_t cnt = min(32u, r1 - w0);
+    for (uint32_t w0 = s, cnt; w0 != r1; w0 += cnt) {        // (r1 + 31 may wrap)
+        cnt = min(32u, r1 - w0);
+        if (w0 != s) mine = lane < cnt ? __ldcs(&a.adj[w0 + lane]) : make_uint2(0, 0);
         for (uint32_t i = 0; i < cnt; i += PULL_ARCS) {
             uint2 x[PULL_ARCS];
 #pragma unroll
@@ -491,8 +491,9 @@ __device__ __noinline__ void mq_pull_sweep(const MqArgs &a, MqStage &st, unsigne
             e[r] = __shfl_sync(FULL, off, r + 1);
             s[r] = __shfl_sync(FULL, off, 8 + r);
             if (hub) {
-                s[r] += c * CHUNK;
-                e[r] = r == 0 && s[r] < e[r] ? min(e[r], s[r] + CHUNK) : s[r];
+                const RowPiece p = row_piece(s[r], e[r], c * CHUNK, r == 0 ? CHUNK : 0u);
+                s[r] = p.first;
+                e[r] = p.first + p.count;
             } else if ((uint32_t)r >= rows || e[r] - r0 >= HEAVY_DEG) {
                 e[r] = s[r];
             }
@@ -507,7 +508,7 @@ __device__ __noinline__ void mq_pull_sweep(const MqArgs &a, MqStage &st, unsigne
             ub[r] = e[r] > s[r] && pb && lv[r].y >= Tb;
             mine[r] = make_uint2(0, 0);
             if (!__any_sync(FULL, ua[r] || ub[r])) e[r] = s[r];
-            else if (s[r] + lane < e[r]) mine[r] = __ldcs(&a.adj[s[r] + lane]);
+            else if (lane < e[r] - s[r]) mine[r] = __ldcs(&a.adj[s[r] + lane]);
         }
 #pragma unroll
         for (int r = 0; r < PULL_ROWS; ++r)
@@ -1219,7 +1220,7 @@ struct LaneSlots {
     uint64_t *t0, *t1;
 };
 
-// One vertex's arcs [s0, s1) for every slot of the launch.  Each lane keeps
+// A piece of one vertex's arcs for every slot of the launch.  Each lane keeps
 // its slots' row state in registers and stores v's pred once per slot
 // (atomically when the row is split into chunks over several warps).
 // Over 32 slots: lane l takes slots 2l and 2l + 1 (one 16-byte load of the
@@ -1228,7 +1229,7 @@ struct LaneSlots {
 // takes one arc, lane t of the group the t-th slot; the groups' minima meet
 // by shuffles.
 __device__ __forceinline__ void mq_scan_row(const MqScanArgs &a, const LaneSlots &ls, uint32_t v,
-                                            uint32_t rs, uint32_t s0, uint32_t s1, bool whole_row,
+                                            uint32_t rs, RowPiece p, bool whole_row,
                                             uint32_t cnt, uint32_t gsh,
                                             unsigned long long &overflow) {
     const uint32_t lane = lane_id();
@@ -1239,10 +1240,11 @@ __device__ __forceinline__ void mq_scan_row(const MqScanArgs &a, const LaneSlots
         ScanSlot r0 = mq_row_slot(ls.q0, ls.t0, ls.k0, ls.sh0, lv.x);
         ScanSlot r1 = mq_row_slot(ls.q0 + 1, ls.t1, ls.k1, ls.sh1, lv.y);
         // the arc records 32 at a time, one per lane, streamed
-        for (uint32_t w0 = s0; w0 < s1; w0 += 32) {
+        const uint32_t end = p.first + p.count;
+        for (uint32_t w0 = p.first, got; w0 != end; w0 += got) {     // (end + 31 may wrap)
+            got = min(32u, end - w0);
             uint2 mine = make_uint2(0, 0);
-            if (w0 + lane < s1) mine = __ldcs(&a.adj[w0 + lane]);
-            const uint32_t got = min(32u, s1 - w0);
+            if (lane < got) mine = __ldcs(&a.adj[w0 + lane]);
             for (uint32_t i = 0; i < got; i += SCAN_ARCS) {
                 uint2 lu[SCAN_ARCS];
 #pragma unroll
@@ -1269,11 +1271,11 @@ __device__ __forceinline__ void mq_scan_row(const MqScanArgs &a, const LaneSlots
     const uint32_t g = 1u << gsh, apr = 32 >> gsh, grp = lane >> gsh;
     const bool has_slot = ls.h0;
     ScanSlot r = mq_row_slot(ls.q0, ls.t0, ls.k0, ls.sh0, has_slot ? __ldg(&lrow[ls.q0]) : INF32);
-    for (uint32_t j0 = s0; j0 < s1; j0 += apr * 4) {
+    for (; p.count; skip_arcs(p, apr * 4)) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            uint32_t arc = j0 + k * apr + grp;
-            if (has_slot && arc < s1) {
+            const uint32_t j = k * apr + grp, arc = p.first + j;
+            if (has_slot && j < p.count) {
                 uint2 e = __ldg(&a.adj[arc]);
                 const uint32_t lu = __ldg(&a.label[(uint64_t)e.x * MQ_SLOTS + ls.q0]);
                 mq_scan_eval(r, arc, e.y, lu, cbase, overflow);
@@ -1315,9 +1317,8 @@ __global__ void __launch_bounds__(256, 5) mq_scan_kernel(MqScanArgs a) {
             uint64_t item = a.heavy_chunks[wi];
             uint32_t v = (uint32_t)(item >> 32), c = (uint32_t)item;
             uint32_t rs = a.row_ptr[v];
-            uint32_t s = rs + c * CHUNK;
-            uint32_t e = min(a.row_ptr[v + 1], s + CHUNK);
-            mq_scan_row(a, ls, v, rs, s, e, false, cnt, gsh, overflow);
+            mq_scan_row(a, ls, v, rs, row_piece(rs, a.row_ptr[v + 1], c * CHUNK, CHUNK), false, cnt, gsh,
+                        overflow);
         } else {
             const uint32_t v1 = __ldg(&a.items[wi - a.n_heavy_chunks + 1]);
             for (uint32_t v0 = __ldg(&a.items[wi - a.n_heavy_chunks]); v0 < v1; v0 += 32) {
@@ -1328,7 +1329,7 @@ __global__ void __launch_bounds__(256, 5) mq_scan_kernel(MqScanArgs a) {
                     const uint32_t s = __shfl_sync(FULL, rs, l), e = __shfl_sync(FULL, re, l);
                     // hubs are covered by the chunk list; no arcs, nothing to scan
                     if (e - s >= HEAVY_DEG || e == s) continue;
-                    mq_scan_row(a, ls, v0 + l, s, s, e, true, cnt, gsh, overflow);
+                    mq_scan_row(a, ls, v0 + l, s, RowPiece{s, e - s}, true, cnt, gsh, overflow);
                 }
             }
         }
@@ -1440,7 +1441,7 @@ template <class F>
 __device__ __forceinline__ void tree_arcs(const MqTreeArgs &a, const uint2 *__restrict__ arcs,
                                           uint32_t s0, uint32_t s1, bool look, F fn) {
     const uint32_t lane = lane_id();
-    for (uint32_t w0 = s0; w0 < s1; w0 += 32) {
+    for (uint32_t w0 = s0; w0 < s1; w0 += 32) {      // (cannot wrap: MQ_TREE_MAX_ARCS)
         uint2 mine = make_uint2(0, 0);
         if (w0 + lane < s1) mine = __ldcs(&arcs[w0 + lane]);
         const uint32_t got = min(32u, s1 - w0);
@@ -1463,8 +1464,8 @@ __device__ __forceinline__ void tree_arcs(const MqTreeArgs &a, const uint2 *__re
     }
 }
 
-// Calls fn(v, row start, row end, first arc offset, whole row?, v's labels)
-// for every row that is not empty, hub rows in CHUNK-arc pieces; the labels of
+// Calls fn(v, first arc, row end, hub piece?, v's labels) for every row that is
+// not empty and for every CHUNK-arc piece of a hub row; the labels of
 // a row are fetched a row ahead.
 template <class F>
 __device__ __forceinline__ void tree_rows(const MqTreeArgs &a, F fn) {
@@ -1479,7 +1480,7 @@ __device__ __forceinline__ void tree_rows(const MqTreeArgs &a, F fn) {
         if (wi < a.n_heavy_chunks) {
             const uint64_t item = a.heavy_chunks[wi];
             const uint32_t v = (uint32_t)(item >> 32);
-            fn(v, a.row_ptr[v], a.row_ptr[v + 1], (uint32_t)item * CHUNK, CHUNK, labels(v));
+            fn(v, a.row_ptr[v] + (uint32_t)item * CHUNK, a.row_ptr[v + 1], true, labels(v));
             continue;
         }
         const uint32_t v1 = __ldg(&a.items[wi - a.n_heavy_chunks + 1]);
@@ -1494,7 +1495,7 @@ __device__ __forceinline__ void tree_rows(const MqTreeArgs &a, F fn) {
                 const uint2 lv = next;
                 rows &= rows - 1;
                 if (rows) next = labels(v0 + __ffs(rows) - 1);
-                fn(v0 + l, __shfl_sync(FULL, rs, l), __shfl_sync(FULL, re, l), 0u, 0u, lv);
+                fn(v0 + l, __shfl_sync(FULL, rs, l), __shfl_sync(FULL, re, l), false, lv);
             }
         }
     }
@@ -1503,28 +1504,25 @@ __device__ __forceinline__ void tree_rows(const MqTreeArgs &a, F fn) {
 __global__ void __launch_bounds__(256, 5) mq_tree_scan_kernel(const __grid_constant__ MqTreeArgs a) {
     const TreeSlot t0 = tree_slot(a, 2 * lane_id()), t1 = tree_slot(a, 2 * lane_id() + 1);
     const uint32_t n0 = t0.on ? a.delta << t0.sh : 0u, n1 = t1.on ? a.delta << t1.sh : 0u;
-    tree_rows(a, [&](uint32_t v, uint32_t rs, uint32_t re, uint32_t at, uint32_t piece, uint2 lv) {
+    tree_rows(a, [&](uint32_t v, uint32_t s, uint32_t re, bool hub, uint2 lv) {
         const uint32_t l0 = lv.x < n0 ? n0 : 0u, l1 = lv.y < n1 ? n1 : 0u;
         const bool f0 = t0.on && lv.x >= n0 && lv.x != INF32, f1 = t1.on && lv.y >= n1 && lv.y != INF32;
         uint32_t p0 = INF32, p1 = INF32;
-        const uint32_t s = rs + at;
         if (__any_sync(FULL, l0 | l1)) {
-            const uint32_t le = a.lend[v], e = piece ? min(le, s + piece) : le;
-            tree_arcs(a, a.adj_w, s, e, l0 | l1, [&](uint32_t arc, uint32_t y, uint32_t w, uint2 lu) {
+            tree_arcs(a, a.adj_w, s, piece_end(s, a.lend[v], CHUNK), l0 | l1, [&](uint32_t arc, uint32_t y, uint32_t w, uint2 lu) {
                 tree_light(a, t0, lv.x, l0, v, y, w, lu.x, arc, p0);
                 tree_light(a, t1, lv.y, l1, v, y, w, lu.y, arc, p1);
             });
         }
         if (__any_sync(FULL, f0 || f1)) {
-            const uint32_t e = piece ? min(re, s + piece) : re;
-            tree_arcs(a, a.adj, s, e, f0 || f1, [&](uint32_t arc, uint32_t, uint32_t w, uint2 lu) {
+            tree_arcs(a, a.adj, s, piece_end(s, re, CHUNK), f0 || f1, [&](uint32_t arc, uint32_t, uint32_t w, uint2 lu) {
                 if (f0 && w <= lv.x >> t0.sh && lv.x - (w << t0.sh) == lu.x) p0 = min(p0, arc);
                 if (f1 && w <= lv.y >> t1.sh && lv.y - (w << t1.sh) == lu.y) p1 = min(p1, arc);
             });
         }
         uint32_t *pp = &a.pred[(uint64_t)v * MQ_SLOTS + t0.q];
-        if (p0 != INF32) { if (piece) atomicMin(pp, p0); else *pp = p0; }
-        if (p1 != INF32) { if (piece) atomicMin(pp + 1, p1); else pp[1] = p1; }
+        if (p0 != INF32) { if (hub) atomicMin(pp, p0); else *pp = p0; }
+        if (p1 != INF32) { if (hub) atomicMin(pp + 1, p1); else pp[1] = p1; }
     });
 }
 
@@ -1540,7 +1538,7 @@ __global__ void __launch_bounds__(256, 5) mq_rest_scan_kernel(const __grid_const
     auto comp = [&](const TreeSlot &t, uint32_t l) {
         return __ldg(&a.comp[s_comp0[t.q] + (l & ((1u << t.sh) - 1u))]);
     };
-    tree_rows(a, [&](uint32_t v, uint32_t rs, uint32_t re, uint32_t at, uint32_t piece, uint2 lv) {
+    tree_rows(a, [&](uint32_t v, uint32_t s, uint32_t re, bool hub, uint2 lv) {
         uint32_t c0 = 0, c1 = 0;
         bool o0 = t0.on && lv.x != INF32, o1 = t1.on && lv.y != INF32;
         if (o0) o0 = (c0 = comp(t0, lv.x)) != s_hub[t0.q];
@@ -1554,8 +1552,7 @@ __global__ void __launch_bounds__(256, 5) mq_rest_scan_kernel(const __grid_const
             if (cv < cu) mq_propose(a, t.tab + pair_slot(cv, cu, t.k), b, v, y);
             else mq_propose(a, t.tab + pair_slot(cu, cv, t.k), b, y, v);
         };
-        const uint32_t s = rs + at, e = piece ? min(re, s + piece) : re;
-        tree_arcs(a, a.adj, s, e, o0 || o1, [&](uint32_t, uint32_t y, uint32_t w, uint2 lu) {
+        tree_arcs(a, a.adj, s, piece_end(s, re, CHUNK), o0 || o1, [&](uint32_t, uint32_t y, uint32_t w, uint2 lu) {
             if (o0) arc_of(t0, lv.x, c0, y, w, lu.x);
             if (o1) arc_of(t1, lv.y, c1, y, w, lu.y);
         });
@@ -1774,7 +1771,8 @@ static unsigned mq_tree_blocks(const DevGraph &g) {
 bool mq_tree_scan_applies(const DevGraph &g, uint32_t k, uint32_t delta) {
     uint32_t b = 1;
     while (b < 31 && (1u << b) < k) ++b;
-    return b >= 2 && g.max_w < 0x80000000u && active_lend(g, delta) && delta < 1ull << (31 - b);
+    return b >= 2 && g.max_w < 0x80000000u && active_lend(g, delta) && delta < 1ull << (31 - b) &&
+           g.m <= MQ_TREE_MAX_ARCS;
 }
 
 cudaError_t mq_launch_tree_scan(const DevGraph &g, MqState &m, unsigned long long slots, uint32_t delta,

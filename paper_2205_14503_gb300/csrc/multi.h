@@ -172,6 +172,10 @@ cudaError_t mq_launch_rest_scan(const DevGraph &g, MqState &m, unsigned long lon
                                 cudaStream_t s);
 // Slots that retire together from which on the tree scan is the faster one.
 constexpr int MQ_TREE_SLOTS = 9;
+// Its kernels step 32 arcs at a time with 32-bit arc indexes, past a row's end;
+// larger graphs take the full scan (loops that cannot wrap, in its registers:
+// scan 4.41 -> 4.83 ms on R-MAT 22, 64 queries).
+constexpr uint64_t MQ_TREE_MAX_ARCS = (1ull << 32) - 64;
 bool mq_tree_scan_applies(const DevGraph &g, uint32_t k, uint32_t delta);
 // Undoes a tree scan's predecessors and pairs (slot q has ks[q] seeds).
 cudaError_t mq_launch_forget(const DevGraph &g, MqState &m, unsigned long long slots, const uint32_t *ks,

@@ -230,16 +230,16 @@ __global__ void __launch_bounds__(256) expand_found_kernel(
             for (uint32_t m = __ballot_sync(FULL, walk && pa == INF32); m; m &= m - 1) {
                 const uint32_t l = __ffs(m) - 1;
                 const uint32_t v = __shfl_sync(FULL, x, l), lv = __shfl_sync(FULL, lx, l);
-                const uint32_t r1 = row_ptr[v + 1];
+                const uint32_t r0 = row_ptr[v], deg = row_ptr[v + 1] - r0;
                 uint32_t found = INF32;
-                for (uint32_t b = row_ptr[v]; b < r1 && found == INF32; b += 32) {
+                for (uint32_t b = 0; b < deg && found == INF32; b += 32) {
                     bool tight = false;
-                    if (b + lane < r1) {
-                        const uint2 e = adj[b + lane];
+                    if (b + lane < deg) {
+                        const uint2 e = adj[r0 + b + lane];
                         tight = ((uint64_t)e.y << lshift) + label32[e.x] == lv;
                     }
                     const uint32_t any = __ballot_sync(FULL, tight);
-                    if (any) found = b + __ffs(any) - 1;
+                    if (any) found = r0 + b + __ffs(any) - 1;
                 }
                 if (lane == l) pa = found;
             }
