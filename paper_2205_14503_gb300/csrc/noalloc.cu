@@ -397,16 +397,20 @@ __global__ void __launch_bounds__(256, 4) na_kernel(NaArgs a) {
                     const uint32_t sl = __shfl_sync(FULL, s, l), dl = __shfl_sync(FULL, deg, l);
                     const uint64_t ll = __shfl_sync(FULL, lab, l);
                     for (uint64_t p = __shfl_sync(FULL, p0, l); p * NA_CHUNK < dl; p += nwarps) {
-                        const uint32_t lo = (uint32_t)p * NA_CHUNK, len = min(dl - lo, NA_CHUNK);
-                        for (uint32_t b = 0; b < len; b += 32 * NA_ILP) {
+                        const uint32_t lo = (uint32_t)p * NA_CHUNK, hi = lo + min(dl - lo, NA_CHUNK);
+                        // (steps counted from the piece's start: in a row of almost
+                        // 2^32 arcs b and j may wrap, to arcs of the same row)
+                        for (uint32_t h = 0; h < NA_CHUNK; h += 32 * NA_ILP) {
+                            const uint32_t b = lo + h;
+                            if (b >= hi) break;
                             bool valid[NA_ILP];
                             uint32_t arc[NA_ILP];
                             uint64_t labs[NA_ILP];
 #pragma unroll
                             for (int i = 0; i < NA_ILP; ++i) {
                                 const uint32_t j = b + lane + 32 * i;
-                                valid[i] = j < len;
-                                arc[i] = sl + lo + j;
+                                valid[i] = j < hi;
+                                arc[i] = sl + j;
                                 labs[i] = ll;
                             }
                             na_relax(a, c, f, region, region_n, valid, arc, labs, T, fmin);
