@@ -640,9 +640,12 @@ cudaError_t launch_tree_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint3
 }
 
 // Predecessors alone, by the light part of most rows (R-MAT 22, weights to
-// 10^5, k = 64: Voronoi call 1.62 ms, with the full scan 1.82).
+// 10^5, k = 64: Voronoi call 1.62 ms, with the full scan 1.82).  It sees no
+// overflow.  A distance that does not fit a narrow label is found while it is
+// relaxed, but the relaxation leaves out arcs of weight 2^32 - 1: with one in
+// the graph the full scan looks for reached vertices next to unreached ones.
 bool pred_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t delta) {
-    return ws.narrow && active_lend(g, delta);
+    return ws.narrow && active_lend(g, delta) && g.max_w < INF32;
 }
 
 cudaError_t launch_pred_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t delta,

@@ -441,3 +441,28 @@ def test_far_pile_dealt_out_to_the_warps(n, local_rounds):
     g = wl.from_edges(n, np.concatenate([u, a]), np.concatenate([v, a + 1]),
                       np.concatenate([w, rng.integers(1, 400, len(a))]))
     _check(g, np.array([0, n // 2, n - 1]), (("delta", 1001), ("local_rounds", local_rounds)))
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("pull,tail", [(0, 0), (1, 1), (2, 0), (2, 1)])
+@pytest.mark.parametrize("w", [2**31, 2**32 - 2, 2**32 - 1])
+def test_overflow_over_the_largest_weights(w, pull, tail, bits):
+    """A vertex that only an arc too heavy for any distance leads to is an
+    overflow in every form of the Voronoi call (an arc of weight 2^32 - 1 is
+    never relaxed, so only a scan of whole rows can tell), and a vertex that
+    has a lighter way is not."""
+    u, v = np.array([0, 1, 2, 3]), np.array([1, 2, 3, 4])
+    g = wl.from_edges(5, u, v, np.array([5, 7, w, 3]))
+    ring = wl.from_edges(5, np.append(u, 0), np.append(v, 4), np.array([5, 7, w, 3, 9]))
+    for graph, status in ((g, st.STEINER_EOVERFLOW if w + 12 >= 2**32 - 1 else st.STEINER_OK), (ring, st.STEINER_OK)):
+        with st.SteinerGraph(graph) as Gd:
+            for key, value in (("label_bits", bits), ("pull", pull), ("tail", tail), ("delta", 10)):
+                Gd.set_param(key, value)
+            rc, cell, dist, pred = Gd.voronoi(np.array([0]))
+            res = Gd.query_detail(np.array([0, 4]))
+        assert rc == status
+        assert res.status == oracle.steiner(graph, np.array([0, 4])).status
+        if rc == st.STEINER_OK:
+            ref = oracle.voronoi(graph, np.array([0]))
+            np.testing.assert_array_equal(dist, ref.dist)
+            np.testing.assert_array_equal(pred, ref.pred)
