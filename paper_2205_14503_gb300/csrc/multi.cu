@@ -924,11 +924,6 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             if (__ldcg(&ctl->far_pending[q]) <= 0) conv |= 1ull << q;
             else S |= 1ull << q;
         }
-        hp_done &= ~S;                      // a split opens a new band
-        const unsigned long long to_tail = a.pull ? S & band0 & wide : 0ull;
-        tails |= to_tail;
-        if (a.pull) band0 &= ~to_tail;
-        else band0 &= ~S;
         infl &= ~conv;
         conv_total |= conv;
         if (!infl) { reason = 1; break; }
@@ -936,6 +931,12 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         if (a.yield && ldcg_u32(&ctl->stop_req[(it - 1) & 1])) { reason = 3; break; }
         if (iters >= a.max_iters) { reason = 4; break; }
         if (!S) continue;
+        // (a launch that left above finds S as it was: the next one decides again)
+        hp_done &= ~S;                      // a split opens a new band
+        const unsigned long long to_tail = a.pull ? S & band0 & wide : 0ull;
+        tails |= to_tail;
+        if (a.pull) band0 &= ~to_tail;
+        else band0 &= ~S;
 
         unsigned long long tm5 = first ? gtimer() : 0;
         // Split the far pile for the slots in S.  A barrier first: every

@@ -466,3 +466,39 @@ def test_overflow_over_the_largest_weights(w, pull, tail, bits):
             ref = oracle.voronoi(graph, np.array([0]))
             np.testing.assert_array_equal(dist, ref.dist)
             np.testing.assert_array_equal(pred, ref.pred)
+
+
+@pytest.mark.parametrize("pull", [0, 1])
+def test_batch_tails_survive_a_yield(pull):
+    """With queries waiting, the engine leaves its kernel as soon as one slot
+    of many converged (batch_yield_div 64), here at the very iteration in which
+    the others' first bands closed and their far vertices, spread over hundreds
+    of bands, are about to join one unbounded band.  They still do: the
+    iterations stay near those of whole waves.  In the push form there is no
+    such band, and yields change nothing but the trees' order of retirement."""
+    core, leaves, delta = wl.rmat(10, 16, wmax=2, seed=77), 150, 10
+    pool = wl.largest_cc(core)
+    src = np.repeat(np.arange(core.n), np.diff(core.row_ptr.astype(np.int64)))
+    keep = src < core.col
+    ends = core.n + np.arange(leaves)
+    g = wl.from_edges(core.n + leaves, np.concatenate([src[keep], pool[:leaves]]),
+                      np.concatenate([core.col[keep], ends]),
+                      np.concatenate([core.w[keep], 100 + 40 * np.arange(leaves)]))
+    done = np.concatenate([pool[:3], ends]).astype(np.int32)     # nothing is far: converges first
+    sets = [done] + [wl.sample_distinct(pool, 2 + i % 7, 500 + i) for i in range(99)]
+    iterations = {}
+    with st.SteinerGraph(g) as Gd:
+        Gd.set_param("batch_delta", delta)
+        Gd.set_param("batch_pull", pull)
+        for div in (1, 64):
+            Gd.set_param("batch_yield_div", div)
+            Gd.get_param("batch_reset")
+            rc, res = Gd.query_batch(sets)
+            iterations[div] = Gd.get_param("batch_iterations")
+            assert rc == st.STEINER_OK
+            for s, r in zip(sets, res):
+                ref = oracle.steiner(g, s)
+                np.testing.assert_array_equal(r.edges, ref.edges)
+                assert r.total == ref.total
+    if pull:
+        assert iterations[64] < leaves
