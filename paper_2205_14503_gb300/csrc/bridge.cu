@@ -195,6 +195,10 @@ __global__ void __launch_bounds__(256) scan_kernel(ScanArgs a) {
 // Bound by the label gathers and, at k = 10,000, by probes of a 400 MB table:
 // looking at every bridge in step 1, and at every arc of the vertices beyond
 // delta, took it 1.91 ms on R-MAT 26 (degree 8) against 1.08.
+// Where few bridges are lighter than delta the rest scan reads most rows:
+// proposing an arc between two cells from the cell of larger rank only where
+// the other's row is not read, and turning ties away before the search, took
+// a query of R-MAT 24 (weights to 20, delta 2, k = 10,000) from 11.4 to 8.3 ms.
 
 struct TreeScanArgs {
     const uint32_t *__restrict__ row_ptr;
@@ -217,25 +221,32 @@ struct TreeScanArgs {
     const uint32_t *hub;                 // the hub component
 };
 
-// The caller's index of arc x -> y.
-__device__ __forceinline__ uint32_t caller_arc(const TreeScanArgs &a, uint32_t x, uint32_t y) {
-    const uint32_t rs = a.row_ptr[x], want = caller_id(a.orig_of, y);
+// The caller's index of arc x -> y (row x starts at rs, at cbase + rs in the
+// caller's order).
+__device__ __forceinline__ uint32_t caller_arc(const TreeScanArgs &a, uint32_t x, uint32_t rs,
+                                               uint32_t cbase, uint32_t y) {
+    const uint32_t want = caller_id(a.orig_of, y);
     uint32_t lo = rs, hi = a.row_ptr[x + 1];
     while (hi - lo > 1) {                // largest arc whose head is at or before y
         const uint32_t mid = lo + (hi - lo) / 2;
         if (caller_id(a.orig_of, a.adj[mid].x) <= want) lo = mid;
         else hi = mid;
     }
-    return caller_arc_base(a.orig_of, a.orig_row_ptr, x, rs) + lo;
+    return cbase + lo;
 }
 
-// Proposes bridge b over arc x -> y (x in the cell of smaller rank).
+// Proposes bridge b over arc x -> y (x in the cell of smaller rank).  Weights
+// of a narrow range make many bridges of a pair equal, and only the smallest
+// arc counts: an arc of a later row is turned away before the search.
 __device__ __forceinline__ void propose_bridge(const TreeScanArgs &a, uint32_t cx, uint32_t cy,
                                                uint64_t b, uint32_t x, uint32_t y) {
     auto *slot = reinterpret_cast<unsigned long long *>(&a.pairtab[pair_slot(cx, cy, a.k)]);
-    if (b > __ldg(slot) >> 32) return;
-    if (b > atomicMin(slot, (b << 32) | INF32) >> 32) return;
-    atomicMin(slot, (b << 32) | caller_arc(a, x, y));
+    unsigned long long cur = __ldg(slot);        // (a stale value is only larger)
+    if (b < cur >> 32) cur = atomicMin(slot, (b << 32) | INF32);
+    if (b > cur >> 32) return;
+    const uint32_t rs = a.row_ptr[x], cbase = caller_arc_base(a.orig_of, a.orig_row_ptr, x, rs);
+    if (b == cur >> 32 && (uint32_t)cur < cbase + rs) return;    // a tie with an earlier row's arc
+    atomicMin(slot, (b << 32) | caller_arc(a, x, rs, cbase, y));
 }
 
 // Arc `arc` = (v, head, w) of step 1, lu the head's label.
@@ -348,15 +359,16 @@ __global__ void __launch_bounds__(256) rest_scan_kernel(const __grid_constant__ 
     auto arc = [&](uint32_t v, uint32_t lv, uint32_t cc, uint32_t cbase, uint32_t at) {
         const uint2 e = __ldcs(&a.adj[at]);
         const uint32_t lu = __ldg(&a.label32[e.x]);
-        if (lu == INF32 || __ldg(&a.comp[lu & mask]) == cc) return;
+        const uint32_t cm = lu == INF32 ? cc : __ldg(&a.comp[lu & mask]);
+        if (cm == cc) return;
         const uint32_t cv = lv & mask, cu = lu & mask;
         const uint64_t b = (uint64_t)(lv >> a.lshift) + e.y + (lu >> a.lshift);
         if (cv < cu) {
             auto *slot = reinterpret_cast<unsigned long long *>(&a.pairtab[pair_slot(cv, cu, a.k)]);
             const unsigned long long key = (b << 32) | (uint32_t)(cbase + at);
             if (key < __ldg(slot)) atomicMin(slot, key);
-        } else {
-            propose_bridge(a, cu, cv, b, e.x, v);    // the head's row may not be read
+        } else if (cm == hub) {
+            propose_bridge(a, cu, cv, b, e.x, v);    // the head's row is not read
         }
     };
     for (uint32_t wi = warp; wi < n_work; wi += nwarps) {
