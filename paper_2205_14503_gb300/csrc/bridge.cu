@@ -596,16 +596,12 @@ cudaError_t launch_compact_pairs(Workspace &ws, uint32_t k, cudaStream_t s) {
 
 // The tree-only scan serves a query whose label width and weights make it
 // exact (narrow labels of two rank bits or more cannot overflow a bridge), with
-// rows split by weight, on a graph large enough for its extra compaction and
-// MST (query times, tree-only against full): R-MAT 26 (degree 8), k = 10,000
-// 7.7 against 11.1 ms, R-MAT 24, k = 10,000 4.7 against 6.1, k = 700 at the
-// default band 5.9 against 6.5, R-MAT 22, k = 300 2.23 against 2.33; R-MAT 20,
-// k = 1000 1.42 against 1.42, 250,000 vertices, k = 3000 1.11 against 0.87.
+// rows split by weight, where it pays.
 bool tree_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t k, uint32_t delta) {
     const bool exact = ws.narrow && ws.lshift >= 2 && g.max_w < 0x80000000u &&
                        active_lend(g, delta) && k > 1 && !small_tail(k);
     if (g.tree_scan >= 0) return exact && g.tree_scan;
-    return exact && g.m >= TREE_SCAN_MIN_ARCS;
+    return exact && tree_scan_pays(g.m, k, delta, g.max_w);
 }
 
 static TreeScanArgs tree_scan_args(const DevGraph &g, const Workspace &ws, uint32_t k, uint32_t delta) {

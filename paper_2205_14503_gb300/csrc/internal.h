@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "rules.h"
 
 namespace stn {
 
@@ -257,9 +258,6 @@ int sssp_occupancy(int threads);
 cudaError_t launch_scan(const DevGraph &g, Workspace &ws, uint32_t k, bool pairs,
                         cudaStream_t s);
 cudaError_t launch_compact_pairs(Workspace &ws, uint32_t k, cudaStream_t s);
-// Arcs from which on a query that returns only its tree takes the tree-only
-// scan.
-constexpr uint64_t TREE_SCAN_MIN_ARCS = 1ull << 27;
 bool tree_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t k, uint32_t delta);
 // The smallest 32-bit label of a distance delta (saturating).
 inline uint32_t near_label(const Workspace &ws, uint32_t delta) {
