@@ -517,7 +517,7 @@ int query_locked(steiner_graph *G, const int32_t *seeds, uint32_t k, steiner_res
         stats->relax_attempts = c.relax_attempts;
         stats->relax_improved = c.relax_improved;
         stats->iterations = c.iterations;
-        stats->phases = c.phases;
+        stats->phases = c.advances;
         stats->n_pairs = k > 1 ? c.n_pairs : 0;
         stats->n_tree_edges = c.n_tree;
         stats->gpu_launches = (uint32_t)ms[5];

@@ -115,7 +115,8 @@ struct Control {
     uint32_t far_count[3];       // by phase % 3 (the piles alternate by phase & 1)
     uint32_t far_min[3];
     uint32_t iterations;
-    uint32_t phases;
+    uint32_t phases;             // ended ones: each uses a tag of the far stamps
+    uint32_t advances;           // of the threshold (ended phases with something left)
     unsigned long long relax_attempts;
     unsigned long long relax_improved;
     // bridge / tree phases

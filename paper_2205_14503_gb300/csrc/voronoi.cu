@@ -1286,6 +1286,7 @@ __global__ void __launch_bounds__(256, BLOCKS) sssp_kernel(const __grid_constant
                 ctl->far_min[(phase + 1) % 3] = INF32;
             }
             if (n_far) {
+                if (first) atomicAdd(&ctl->advances, 1u);
                 T_old = T;
                 T = (fmin_now != INF32 && (uint64_t)fmin_now > T ? (uint64_t)fmin_now : T) +
                     a.delta;
@@ -1357,6 +1358,7 @@ __global__ void __launch_bounds__(256, BLOCKS) sssp_kernel(const __grid_constant
             ctl->near_count[(its + 1) % 3] = 0;
             ctl->heavy_count[(its + 1) % 3] = 0;
             ctl->work_next[(its + 1) % 3] = 0;
+            atomicAdd(&ctl->advances, 1u);
             if (!step) {
                 ctl->band_count = 0;
                 ctl->band_hcount = 0;

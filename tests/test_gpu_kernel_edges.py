@@ -502,3 +502,21 @@ def test_batch_tails_survive_a_yield(pull):
                 assert r.total == ref.total
     if pull:
         assert iterations[64] < leaves
+
+
+@pytest.mark.parametrize("far_scan", [0, 1])
+@pytest.mark.parametrize("delta", [100, 1001, 5000, 10**6])
+def test_phases_count_threshold_advances(delta, far_scan):
+    """stats.phases: every advance raises the threshold by the band width at
+    least (by less inside the first band alone), so a query has no more of them
+    than its largest distance holds bands, and one for a pile whose vertices
+    were all settled while parked."""
+    g = wl.grid(150, 111, 1000, seed=21)
+    seeds = G.seeds_from(np.arange(g.n), 7, 5)
+    top = int(oracle.voronoi(g, seeds).dist.max())
+    with st.SteinerGraph(g) as Gd:
+        Gd.set_param("delta", delta)
+        Gd.set_param("far_scan", far_scan)
+        stats = Gd.query_detail(seeds).stats
+    assert (1 if top >= delta else 0) <= stats["phases"] <= top // delta + 2
+    assert stats["phases"] <= stats["iterations"]
