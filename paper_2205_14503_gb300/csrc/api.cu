@@ -11,7 +11,6 @@
 #include <deque>
 #include <mutex>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -51,68 +50,6 @@ cudaError_t dalloc(T *&p, uint64_t count) {
 }
 
 uint32_t bit_length(uint32_t x) { return x ? 32u - (uint32_t)__builtin_clz(x) : 0u; }
-
-// Cuts the vertices into consecutive ranges of at most `arcs` arcs (a hub
-// counts HEAVY_DEG: longer rows are queued in chunks) and ITEM_SPAN
-// vertices, and into coarser ones of SPARSE_ITEM_FACTOR times the arcs; a
-// single vertex may exceed the arc limit.  at[0] / at[1] receive the range
-// starts followed by n.  Without skew (the longest row, max_deg, within a few
-// times the mean) ranges of equal length do; else blocks of CUT_BLOCK
-// vertices are cut side by side on the host's threads.
-void cut_items(const uint32_t *row_ptr, uint32_t n, uint64_t arcs, uint32_t max_deg,
-               std::vector<uint32_t> (&at)[2]) {
-    constexpr uint32_t CUT_BLOCK = 1u << 17;
-    const uint64_t mean = std::max<uint64_t>(row_ptr[n] / n, 1);
-    if (max_deg <= 4 * mean) {
-        for (int i = 0; i < 2; ++i) {
-            const uint64_t span = (i ? SPARSE_ITEM_FACTOR : 1) * arcs / mean;
-            const uint32_t step = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(span, 1), ITEM_SPAN);
-            for (uint64_t v = 0; v < n; v += step) at[i].push_back((uint32_t)v);
-            at[i].push_back(n);
-        }
-        return;
-    }
-    struct Part {
-        std::vector<uint32_t> at[2];
-    };
-    const uint32_t blocks = (uint32_t)(((uint64_t)n + CUT_BLOCK - 1) / CUT_BLOCK);
-    std::vector<Part> part(blocks);
-    std::atomic<uint32_t> next{0};
-    auto work = [&] {
-        for (uint32_t b; (b = next.fetch_add(1)) < blocks;) {
-            const uint32_t lo = b * CUT_BLOCK, hi = (uint32_t)std::min<uint64_t>(n, (uint64_t)lo + CUT_BLOCK);
-            const uint64_t limit[2] = {arcs, SPARSE_ITEM_FACTOR * arcs};
-            uint64_t sum[2] = {0, 0};
-            uint32_t from[2] = {lo, lo};
-            for (int i = 0; i < 2; ++i) part[b].at[i].push_back(lo);
-            for (uint32_t v = lo; v < hi; ++v) {
-                const uint32_t d = std::min(row_ptr[v + 1] - row_ptr[v], HEAVY_DEG);
-                for (int i = 0; i < 2; ++i) {
-                    if (v > from[i] && (sum[i] + d > limit[i] || v - from[i] == ITEM_SPAN)) {
-                        part[b].at[i].push_back(from[i] = v);
-                        sum[i] = 0;
-                    }
-                    sum[i] += d;
-                }
-            }
-        }
-    };
-    std::vector<std::thread> pool;
-    const uint32_t threads = std::min(blocks, std::min(16u, std::max(1u, std::thread::hardware_concurrency())));
-    for (uint32_t t = 1; t < threads; ++t) {
-        try {
-            pool.emplace_back(work);
-        } catch (const std::system_error &) {
-            break;          // fewer threads do the same work
-        }
-    }
-    work();
-    for (auto &t : pool) t.join();
-    for (int i = 0; i < 2; ++i) {
-        for (auto &p : part) at[i].insert(at[i].end(), p.at[i].begin(), p.at[i].end());
-        at[i].push_back(n);
-    }
-}
 
 uint32_t bits_for(uint32_t n) {
     uint32_t b = 1;
@@ -698,12 +635,11 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     G->geo.sssp_max_blocks = G->geo.sssp_blocks;
     int mst_sm = mst_occupancy(512);
     G->geo.mst_blocks = std::max(1, mst_sm) * G->geo.sm_count;
-    {   // dense work items: some sixteen per warp of the persistent grid
-        const uint64_t warps = (uint64_t)G->geo.sssp_max_blocks * (G->geo.threads / 32);
-        const uint64_t arcs = std::min<uint64_t>(std::max<uint64_t>(n_arcs / (16 * warps), ITEM_ARCS_MIN),
-                                                 ITEM_ARCS_MAX);
+    {
         std::vector<uint32_t> at[2];
-        cut_items(irp, std::max(G->g.n_live, 1u), arcs, max_deg, at);
+        const uint64_t warps = (uint64_t)G->geo.sssp_max_blocks * (G->geo.threads / 32);
+        if (!cut_items(irp, std::max(G->g.n_live, 1u), max_deg, warps, at))
+            return bail(fail(STEINER_ENOMEM, "host allocation of the work items failed"));
         G->g.n_items = (uint32_t)at[0].size() - 1;
         G->g.n_sparse_items = (uint32_t)at[1].size() - 1;
         e = dalloc(G->g.items, at[0].size());

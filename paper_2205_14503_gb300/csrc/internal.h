@@ -6,24 +6,10 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "items.h"
 #include "rules.h"
 
 namespace stn {
-
-// Degree at or above which a vertex's adjacency is processed in chunks of
-// CHUNK arcs (one warp per chunk) instead of inside a 32-vertex batch.
-constexpr uint32_t HEAVY_DEG = 256;
-constexpr uint32_t CHUNK = 512;
-// Largest vertex range of a dense work item: whatever its alignment it
-// touches at most 32 bitmap words, one per lane.
-constexpr uint32_t ITEM_SPAN = 992;
-// Arcs per dense work item: some sixteen items per warp of the grid, within
-// these bounds (below one relax_group a smaller item saves nothing; above
-// the upper one the slowest item shows).  Voronoi query, R-MAT 22, weights
-// to 10^5, k = 64: 2.76 ms; four items per warp up to 8192 arcs 3.30 ms.
-constexpr uint64_t ITEM_ARCS_MIN = 128, ITEM_ARCS_MAX = 4096;
-// A sparse bitmap's items may hold this many times the arcs (few are set).
-constexpr uint64_t SPARSE_ITEM_FACTOR = 8;
 
 // Resident graph: row offsets and interleaved (neighbour, weight) arcs.
 struct DevGraph {

@@ -1,0 +1,103 @@
+// Work items of the dense frontiers and the scans: consecutive vertex ranges.
+// Host code only, apart from the CUDA headers.
+#pragma once
+#include <algorithm>
+#include <atomic>
+#include <cstdint>
+#include <thread>
+#include <vector>
+
+namespace stn {
+
+// Degree at or above which a vertex's adjacency is processed in chunks of
+// CHUNK arcs (one warp per chunk) instead of inside a 32-vertex batch.
+constexpr uint32_t HEAVY_DEG = 256;
+constexpr uint32_t CHUNK = 512;
+// Largest vertex range of a dense work item: whatever its alignment it
+// touches at most 32 bitmap words, one per lane.
+constexpr uint32_t ITEM_SPAN = 992;
+// Arcs per dense work item where rows are uneven: some sixteen items per warp
+// of the grid, within these bounds (below one relax_group a smaller item saves
+// nothing; above the upper one the slowest item shows).  R-MAT 22, weights to
+// 10^5, k = 64, when the rule was drawn: 2.76 ms; four items per warp up to
+// 8192 arcs 3.30.
+constexpr uint64_t ITEM_ARCS_MIN = 128, ITEM_ARCS_MAX = 4096;
+// A sparse bitmap's items may hold this many times the arcs (few are set).
+constexpr uint64_t SPARSE_ITEM_FACTOR = 8;
+// Cuts the vertices into consecutive ranges of about equal arcs (a hub counts
+// HEAVY_DEG: longer rows are queued in chunks) and at most ITEM_SPAN vertices,
+// and into coarser ones for sparse bitmaps, for a grid of `warps` warps (three
+// blocks per SM); a single vertex may exceed the arc limit.  at[0] / at[1]
+// receive the range starts followed by n.  Without skew (the longest row within
+// a few times the mean) ranges of equal length do; else blocks of CUT_BLOCK
+// vertices are cut side by side on the host's threads.  False: out of memory
+// (nothing is thrown, on any thread).
+inline bool cut_items(const uint32_t *row_ptr, uint32_t n, uint32_t max_deg, uint64_t warps,
+                      std::vector<uint32_t> (&at)[2]) noexcept try {
+    constexpr uint32_t CUT_BLOCK = 1u << 17;
+    const uint64_t m = row_ptr[n], mean = std::max<uint64_t>(m / n, 1);
+    const uint64_t arcs = std::min(std::max(m / (16 * warps), ITEM_ARCS_MIN), ITEM_ARCS_MAX);
+    if (max_deg <= 4 * mean) {
+        for (int i = 0; i < 2; ++i) {
+            const uint64_t span = (i ? SPARSE_ITEM_FACTOR : 1) * arcs / mean;
+            const uint32_t step = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(span, 1), ITEM_SPAN);
+            at[i].reserve(n / step + 2);
+            for (uint64_t v = 0; v < n; v += step) at[i].push_back((uint32_t)v);
+            at[i].push_back(n);
+        }
+        return true;
+    }
+    struct Part {
+        std::vector<uint32_t> at[2];
+    };
+    const uint32_t blocks = (uint32_t)(((uint64_t)n + CUT_BLOCK - 1) / CUT_BLOCK);
+    std::vector<Part> part(blocks);
+    std::atomic<uint32_t> next{0};
+    std::atomic<bool> failed{false};
+    auto work = [&]() noexcept {
+        try {
+            for (uint32_t b; (b = next.fetch_add(1)) < blocks;) {
+                const uint32_t lo = b * CUT_BLOCK, hi = (uint32_t)std::min<uint64_t>(n, (uint64_t)lo + CUT_BLOCK);
+                const uint64_t limit[2] = {arcs, SPARSE_ITEM_FACTOR * arcs};
+                uint64_t sum[2] = {0, 0};
+                uint32_t from[2] = {lo, lo};
+                for (int i = 0; i < 2; ++i) part[b].at[i].push_back(lo);
+                for (uint32_t v = lo; v < hi; ++v) {
+                    const uint32_t d = std::min(row_ptr[v + 1] - row_ptr[v], HEAVY_DEG);
+                    for (int i = 0; i < 2; ++i) {
+                        if (v > from[i] && (sum[i] + d > limit[i] || v - from[i] == ITEM_SPAN)) {
+                            part[b].at[i].push_back(from[i] = v);
+                            sum[i] = 0;
+                        }
+                        sum[i] += d;
+                    }
+                }
+            }
+        } catch (...) {
+            failed = true;
+        }
+    };
+    std::vector<std::thread> pool;
+    const uint32_t threads = std::min(blocks, std::min(16u, std::max(1u, std::thread::hardware_concurrency())));
+    try {
+        pool.reserve(threads);
+        for (uint32_t t = 1; t < threads; ++t) pool.emplace_back(work);
+    } catch (...) {
+        // fewer threads do the same work
+    }
+    work();
+    for (auto &t : pool) t.join();
+    if (failed) return false;
+    for (int i = 0; i < 2; ++i) {
+        size_t total = 1;
+        for (auto &p : part) total += p.at[i].size();
+        at[i].reserve(total);
+        for (auto &p : part) at[i].insert(at[i].end(), p.at[i].begin(), p.at[i].end());
+        at[i].push_back(n);
+    }
+    return true;
+} catch (...) {
+    return false;
+}
+
+}  // namespace stn
