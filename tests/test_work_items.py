@@ -101,6 +101,16 @@ def test_items_cover_the_vertices(cut, kind, n):
             assert np.all((arcs <= lim) | (np.diff(at) == 1))
 
 
+@pytest.mark.parametrize("kind", ["grid", "uniform"])
+@pytest.mark.parametrize("n", [20000, 400000, 1500000])
+def test_even_rows_have_few_items(cut, kind, n):
+    """Even rows need no finer cut than the grid has warps: at most five items
+    per warp of the two-block grid, and one for a sparse bitmap (an item costs
+    a warp about 2 us whether or not it finds anything to relax)."""
+    dense, sparse = cut(_degrees(kind, n))
+    assert len(dense) - 1 <= 5 * 2432 and len(sparse) - 1 <= 2432
+
+
 @pytest.mark.parametrize("kind", ["grid", "power"])
 def test_items_without_memory(cut, kind):
     """Whichever allocation fails first, on whichever thread: the call says so
