@@ -571,6 +571,7 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     G->g.n_live = n;
     if (relabel)
         G->g.n_live = (uint32_t)(std::lower_bound(irp, irp + n, (uint32_t)n_arcs) - irp);
+    G->g.even = even_rows(max_deg, n_arcs / std::max(G->g.n_live, 1u));
     G->g.heavy_chunk_cap = (uint32_t)std::max<uint64_t>(cap, 1);
     if ((e = dalloc(G->g.row_ptr, (uint64_t)n + 1)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     if ((e = dalloc(G->g.adj, n_arcs)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));

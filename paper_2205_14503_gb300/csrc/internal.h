@@ -22,6 +22,7 @@ struct DevGraph {
     uint32_t heavy_chunk_cap = 0;   // bound on chunk entries a frontier can hold
     uint32_t max_w = 0;             // largest arc weight
     uint32_t delta0 = 0;            // default band width
+    bool even = false;              // rows of about the same length
     // Internal vertex order.  On a skewed degree distribution the vertices
     // are renumbered by descending degree (ties by id), so the labels of
     // the hubs that most arcs point to share L2 sectors; rows keep the
@@ -55,21 +56,6 @@ struct DevGraph {
 // width and the split on (delta at or below the largest weight), else null.
 inline const uint32_t *active_lend(const DevGraph &g, uint32_t delta) {
     return (delta <= g.max_w && g.adj_w && g.lend && g.part_delta == delta) ? g.lend : nullptr;
-}
-
-// The first band's inner threshold with the split on for band width delta (0:
-// none).  The default band width is 32 mean weights over the mean degree: on
-// R-MAT graphs the hubs and most of the core settle below half a mean weight
-// over the mean degree, and with them settled the rest of the band improves
-// most vertices once.  R-MAT of 10^6 vertices, k = 101, default band: 54 ->
-// 26 M relaxations, 1.72 -> 1.10 ms (1.06 at a 48th, 1.35 at a 96th of the
-// default width); R-MAT 24, k = 700: 11.2 -> 6.6 ms.  Bands narrowed by
-// tuning gain less and take an eighth of themselves: R-MAT 26 (degree 8),
-// k = 10,000 14.2 -> 13.4 ms, R-MAT 22, weights to 10^5, k = 64 2.35 -> 2.04.
-inline uint32_t first_step(const DevGraph &g, uint32_t delta) {
-    if (delta > g.max_w) return 0;
-    const uint32_t s = delta > g.delta0 / 8 ? g.delta0 / 64 : delta / 8;
-    return s < 2 ? 2 : s;
 }
 
 // Offset from internal to caller arc indices along internal row v (which

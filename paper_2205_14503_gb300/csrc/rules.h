@@ -29,4 +29,26 @@ inline bool tree_scan_pays(uint64_t m, uint32_t k, uint32_t delta, uint32_t max_
     return (double)m * (1.0 - 1.5 * delta / max_w) >= 3.0 * slots;
 }
 
+// The first band's inner threshold with the split on for band width delta (0:
+// none), delta0 being the default.  The default band width is 32 mean weights
+// over the mean degree: on R-MAT graphs the hubs and most of the core settle
+// below half a mean weight over the mean degree, and with them settled the rest
+// of the band improves most vertices once.  R-MAT of 10^6 vertices, k = 101,
+// default band: 54 -> 26 M relaxations, 1.72 -> 1.10 ms (1.06 at a 48th, 1.35
+// at a 96th of the default width); R-MAT 24, k = 700: 11.2 -> 6.6 ms.  Bands
+// narrowed by tuning gain less and take an eighth of themselves: R-MAT 26
+// (degree 8), k = 10,000 14.2 -> 13.4 ms, R-MAT 22, weights to 10^5, k = 64 2.35
+// -> 2.04.  Without hubs (even rows) a narrowed band gains nothing, and its
+// fewer listings can keep the heavy pass from its pull form: uniform random
+// graphs of lognormal weights at a 16th of the default, 30,000 vertices, k =
+// 1000 0.96 -> 0.46 ms in one step, 1.5 * 10^6, k = 37 1.11 -> 1.09, 3 * 10^6,
+// k = 2 1.74 -> 1.70.
+inline uint32_t first_step(uint32_t delta, uint32_t delta0, uint32_t max_w, bool even) {
+    if (delta > max_w) return 0;
+    const bool narrowed = delta <= delta0 / 8;
+    if (narrowed && even) return 0;
+    const uint32_t s = narrowed ? delta / 8 : delta0 / 64;
+    return s < 2 ? 2 : s;
+}
+
 }  // namespace stn

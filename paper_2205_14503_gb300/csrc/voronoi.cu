@@ -1617,7 +1617,7 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.pull = p.far_scan ? p.pull : 0u;
     a.tail = p.tail;
     a.m = g.m;
-    a.step0 = p.far_scan ? first_step(g, p.delta) : 0u;
+    a.step0 = p.far_scan ? first_step(p.delta, g.delta0, g.max_w, g.even) : 0u;
     // Three blocks per SM spill registers, two do not.  Two go faster through
     // the chain of loads of a hop, three keep more arcs in flight.  Two, of
     // three: R-MAT 12 0.224 ms of 0.257, 10^6 vertices (k = 101) 1.04 of 1.07,

@@ -31,16 +31,25 @@ TREE_SCAN = [
 
 
 @pytest.fixture(scope="module")
-def pays(tmp_path_factory):
+def rules(tmp_path_factory):
     d = tmp_path_factory.mktemp("rules")
     src, lib = str(d / "shim.cpp"), str(d / "shim.so")
     with open(src, "w") as f:
         f.write('#include "rules.h"\nextern "C" int pays(uint64_t m, uint32_t k, uint32_t delta, uint32_t w) '
-                "{ return stn::tree_scan_pays(m, k, delta, w); }\n")
+                "{ return stn::tree_scan_pays(m, k, delta, w); }\n"
+                'extern "C" uint32_t step(uint32_t delta, uint32_t delta0, uint32_t w, int even) '
+                "{ return stn::first_step(delta, delta0, w, even != 0); }\n")
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, src, "-o", lib], check=True)
-    fn = ctypes.CDLL(lib).pays
-    fn.argtypes = [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint32]
-    return fn
+    so = ctypes.CDLL(lib)
+    so.pays.argtypes = [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint32]
+    so.step.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int]
+    so.step.restype = ctypes.c_uint32
+    return so
+
+
+@pytest.fixture
+def pays(rules):
+    return rules.pays
 
 
 @pytest.mark.parametrize("call,full,tree", TREE_SCAN, ids=[str(c[0]) for c in TREE_SCAN])
@@ -53,3 +62,19 @@ def test_tree_scan_lines(pays):
     assert not pays(1 << 32, 300, 3, 60) and pays(1 << 32, 300, 4, 60)
     assert not pays(1 << 32, 300, 1000, 1000)            # every arc light: nothing to spare
     assert not pays(1 << 32, 23000, 2**32 - 2, 2**32 - 1)
+
+
+@pytest.mark.parametrize("delta0", [2, 64, 500, 2191])
+def test_first_band_steps(rules, delta0):
+    """The first band of even rows is reached in one step once it is narrower
+    than an eighth of the default; without the split there is no step."""
+    for delta in (1, delta0 // 16, delta0 // 8, delta0 // 8 + 1, delta0, 4 * delta0):
+        if delta == 0:
+            continue
+        for even in (0, 1):
+            assert rules.step(delta, delta0, delta - 1, even) == 0
+            got = rules.step(delta, delta0, 10**6, even)
+            if delta > delta0 // 8:
+                assert got == max(2, delta0 // 64)
+            else:
+                assert got == (0 if even else max(2, delta // 8))
