@@ -520,3 +520,16 @@ def test_phases_count_threshold_advances(delta, far_scan):
         stats = Gd.query_detail(seeds).stats
     assert (1 if top >= delta else 0) <= stats["phases"] <= top // delta + 2
     assert stats["phases"] <= stats["iterations"]
+
+
+@pytest.mark.parametrize("n,k,launches", [(3000, 1, 4), (2049, 2, 5), (2050, 2, 6), (5000, 3, 6), (3000, 182, 10)])
+def test_launches_are_counted(n, k, launches):
+    """stats.gpu_launches on a path between its ends: labels, seeds, Voronoi
+    and scan, then one kernel for the rest, and a sort when the tree (n - 1
+    edges) outgrows it; six kernels above 181 seeds."""
+    g = G.path(n, 1, 9, 42)
+    seeds = np.unique(np.concatenate([[0], [n - 1] if k > 1 else [], np.arange(1, k - 1)])).astype(np.int32)
+    with st.SteinerGraph(g) as Gd:
+        res = Gd.query_detail(seeds)
+    assert len(seeds) == k and len(res.edges) == (n - 1 if k > 1 else 0)
+    assert res.stats["gpu_launches"] == launches
