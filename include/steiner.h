@@ -99,7 +99,9 @@ typedef struct {
      * init = labels and seeds, voronoi = the near/far SSSP kernel alone,
      * bridges = pred + bridge scan and pair compaction, mst = Boruvka,
      * tree = expansion, sort and total; seed sets of up to 181 run all of
-     * the steps after the scan as one kernel, counted as tree */
+     * the steps after the scan as one kernel, counted as tree.  A call that
+     * asks for counters or pairs scans every arc; steiner_query may read only
+     * the arcs that its tree can need, in less time than ms_bridges */
     float ms_init, ms_voronoi, ms_bridges, ms_mst, ms_tree;
 } steiner_stats_t;
 
@@ -212,11 +214,15 @@ int steiner_serve_stop(steiner_graph_t g);
  *                  still takes some on graphs of few arcs per vertex
  *   "batch_delta"  band width of the multi-query engine (0 = w_max / 8 when
  *                  "delta" is at most the largest weight w_max, else "delta")
- *   "batch_pull"   1 (default): a query's first heavy-arc pass in the
- *                  multi-query engine runs in the pull form (each vertex
- *                  unsettled in that query reads its own heavy arcs and the
- *                  labels at their other ends); 0: it pushes the heavy arcs
- *                  of the band's vertices
+ *   "batch_pull"   1 (default): once a query's band holds most of the graph
+ *                  (by a sample of the arcs; the second band is taken as
+ *                  such in any case), its heavy-arc pass in the multi-query
+ *                  engine runs in the pull form (each vertex unsettled in
+ *                  that query reads its own heavy arcs and the labels at
+ *                  their other ends) and the rest of the query as one
+ *                  unbounded band; a first band that holds less pushes the
+ *                  heavy arcs of its vertices.  0: every band pushes them,
+ *                  and there is no unbounded band
  *   "batch_tails"  1 (default): the tails (MST, expansion, sorted edges) of
  *                  the queries that finish together run as one launch per
  *                  step for all of them; 0: one query at a time

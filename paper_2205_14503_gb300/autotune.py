@@ -21,6 +21,12 @@ fingerprint of the graph and the GPU name, so later handles of the same
 graph start tuned (``apply_cached``).  Results never depend on these
 settings, only the time does.  Tune on sample queries other than the ones
 to be timed.
+
+The timed queries ask for counters, so they take the full bridge scan, whose
+time does not depend on the band width, also where ``steiner_query`` reads
+fewer arcs.  Forms of the kernel that run two blocks per SM (label scans below
+2^28 arcs, far piles without local rounds) cap the grid there: the default block
+candidates are then the same launch, timed twice.
 """
 from __future__ import annotations
 

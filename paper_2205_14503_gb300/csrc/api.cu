@@ -401,10 +401,11 @@ int query_locked(steiner_graph *G, const int32_t *seeds, uint32_t k, steiner_res
                 c.err, c.exit_reason, c.iterations, c.phases, c.relax_attempts);
         const int nt = std::min<int>(TRACE_LEN, (int)c.iterations);
         for (int i = 0; i < nt; ++i) {
-            // a far-pile split takes an iteration index of its own and is
-            // not traced; its time counts with the iteration before it
+            // a split of a band with light and heavy arcs takes an iteration
+            // index of its own and is not traced; its time counts with the
+            // iteration before it
             if (!c.trace_ns[i]) {
-                fprintf(stderr, "[steiner]   it %d: far-pile split\n", i);
+                fprintf(stderr, "[steiner]   it %d: split\n", i);
                 continue;
             }
             unsigned long long t1 = (int)c.iterations <= TRACE_LEN ? c.end_ns : 0;

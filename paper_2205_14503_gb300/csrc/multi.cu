@@ -71,7 +71,7 @@ struct MqArgs {
     // with the split: end of each row's light part in the weight-partitioned
     // adjacency `adj` (null: rows are unpartitioned and arcs are filtered)
     const uint32_t *lend;
-    uint32_t pull;           // first heavy-arc pass of a slot in the pull form
+    uint32_t pull;           // a slot whose band holds most of the graph takes the pull form and the tail
     const uint64_t *__restrict__ heavy_chunks;   // hub rows in CHUNK-arc pieces
     uint32_t n_heavy_chunks;
 };
@@ -123,12 +123,6 @@ __device__ __forceinline__ uint64_t mq_label(const uint32_t *label, uint64_t v, 
 
 __device__ __forceinline__ int popc64(unsigned long long x) { return __popcll(x); }
 
-__device__ __forceinline__ unsigned long long gtimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // Inclusive scan of one 64-bit value per thread over a 256-thread block;
 // wtot[] receives the per-warp inclusive totals (wtot[MQ_WARPS-1] = block
 // total after the call).  Every thread of the block must call it.
@@ -152,24 +146,9 @@ __device__ __forceinline__ uint64_t block_inclusive_scan64(uint64_t x, uint64_t 
     return x + (w ? wtot[w - 1] : 0);
 }
 
-// Index of the t-th set bit (0-based) of a 32-bit word.
-__device__ __forceinline__ uint32_t nth_bit32(uint32_t x, uint32_t t) {
-    uint32_t pos = 0;
-#pragma unroll
-    for (uint32_t w = 16; w >= 1; w >>= 1) {
-        uint32_t c = __popc(x & ((1u << w) - 1u));
-        if (t >= c) {
-            t -= c;
-            x >>= w;
-            pos += w;
-        }
-    }
-    return pos;
-}
-
 __device__ __forceinline__ uint32_t nth_bit64(unsigned long long m, uint32_t t) {
     uint32_t lo = (uint32_t)m, pl = (uint32_t)__popc(lo);
-    return t < pl ? nth_bit32(lo, t) : 32 + nth_bit32((uint32_t)(m >> 32), t - pl);
+    return t < pl ? nth_set_bit(lo, t) : 32 + nth_set_bit((uint32_t)(m >> 32), t - pl);
 }
 
 __device__ __forceinline__ unsigned long long warp_or64(unsigned long long x) {
@@ -601,7 +580,8 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         // heavy-arc pass) the band list.  A pass reads list bc and moves the
         // survivors, with this iteration's new listings, to list bc + 1;
         // list bc + 2 (read by the previous pass) is cleared for the next.
-        // slots of H in their first band run the pass in the pull form
+        // slots of H whose band holds most of the graph (or their second band)
+        // run the pass in the pull form
         const unsigned long long P = a.pull ? (H & band0 & wide) : 0ull;
         const uint32_t n_band = H ? min(ldcg_u32(&ctl->bcount[bc]), a.n) : 0u;
         const uint32_t n_all = n_items + n_band;
@@ -617,7 +597,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         }
         const uint32_t *qc = odd ? a.q1 : a.q0;
 
-        unsigned long long tm0 = first ? gtimer() : 0;
+        unsigned long long tm0 = first ? global_ns() : 0;
         // Phase A: every frontier vertex takes its pending slot mask; its
         // work is deg x |mask| (arc, slot) pairs; prefix sums per block
         // segment of the frontier.
@@ -662,9 +642,9 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
             __syncthreads();
         }
         if (threadIdx.x == 0) a.bsum[blockIdx.x] = st.carry;
-        unsigned long long tm1 = first ? gtimer() : 0;
+        unsigned long long tm1 = first ? global_ns() : 0;
         if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; break; }
-        unsigned long long tm2 = first ? gtimer() : 0;
+        unsigned long long tm2 = first ? global_ns() : 0;
         if (blockIdx.x == 0 && threadIdx.x < MQ_SLOTS) ctl->cov[threadIdx.x] = 0;
         // block offsets and the total
         {
@@ -873,13 +853,13 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
                           improved);
             ++pull_sweeps;
         }
-        unsigned long long tm3 = first ? gtimer() : 0;
+        unsigned long long tm3 = first ? global_ns() : 0;
         seg_flush(st, t, ctl, a.n);
         if (first)
             ctl->stop_req[it & 1] = (a.yield && a.doorbell) ? *(volatile const uint32_t *)a.doorbell : 0u;
         if (!grid_sync(&ctl->bar, &ctl->err, bar_target)) { reason = 5; break; }
         if (first) {
-            unsigned long long tm4 = gtimer();
+            unsigned long long tm4 = global_ns();
             ctl->t_part[0] += tm1 - tm0;
             ctl->t_part[1] += tm2 - tm1;
             ctl->t_part[2] += tm3 - tm2;
@@ -938,7 +918,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         if (a.pull) band0 &= ~to_tail;
         else band0 &= ~S;
 
-        unsigned long long tm5 = first ? gtimer() : 0;
+        unsigned long long tm5 = first ? global_ns() : 0;
         // Split the far pile for the slots in S.  A barrier first: every
         // block has read the decision inputs before the split appends to
         // them.  Near pushes go to this iteration's queue (slot it % 3).
@@ -1018,7 +998,7 @@ __global__ void __launch_bounds__(256, MQ_BLOCKS) mq_sssp_kernel(const __grid_co
         if (threadIdx.x < MQ_SLOTS) st.T[threadIdx.x] = st.Tnew[threadIdx.x];
         __syncthreads();
         fc ^= 1;
-        if (first) ctl->t_part[4] += gtimer() - tm5;
+        if (first) ctl->t_part[4] += global_ns() - tm5;
     }
     if (!infl && reason == 0) reason = 1;
     unsigned long long sum_a = attempts, sum_i = improved;
@@ -1224,7 +1204,7 @@ struct LaneSlots {
 // A piece of one vertex's arcs for every slot of the launch.  Each lane keeps
 // its slots' row state in registers and stores v's pred once per slot
 // (atomically when the row is split into chunks over several warps).
-// Over 32 slots: lane l takes slots 2l and 2l + 1 (one 16-byte load of the
+// Over 32 slots: lane l takes slots 2l and 2l + 1 (one 8-byte load of the
 // pair's labels per arc), and every lane walks every arc.
 // Otherwise lanes are grouped as in the SSSP kernel: a group of g lanes
 // takes one arc, lane t of the group the t-th slot; the groups' minima meet
@@ -1357,9 +1337,11 @@ __global__ void __launch_bounds__(256, 5) mq_scan_kernel(MqScanArgs a) {
 // light arc is a few 32-bit operations and most bridges fail b < delta before
 // the table is probed.  R-MAT 22, 64 queries: scan 17.1 -> 4.3 ms, tails with
 // the rest scan and the second MST 0.5 -> 1.3 ms, batch 44.0 -> 32.2 ms; R-MAT
-// 20, serving 90: 28-36 -> 25-34 ms.  It pays from about ten slots on: 8 slots
-// R-MAT 20 6.1 against 5.8 ms, R-MAT 22 19.2 against 20.3; 12 slots 6.7 against
-// 7.0 and 22.5 against 25.4.  Slots whose first band covered little are left
+// 20, serving 90: 28-36 -> 25-34 ms.  It pays from about eight slots on, a
+// little later on small graphs: 8 slots R-MAT 20 6.1 against 5.8 ms, R-MAT 22
+// 19.2 against 20.3; 12 slots 6.7 against 7.0 and 22.5 against 25.4 (the line,
+// MQ_TREE_SLOTS, lies between).  24 and 64 slots, weights to 20 and up to 1000:
+// 1.00 to 1.45 times as fast.  Slots whose first band covered little are left
 // to the full scan: each would have nearly every whole row read (scan 4.3 ->
 // 9.5 ms with one to five of them, 7.5 with the full scan for these).  Exact as
 // in the single-query path: two rank bits or more rule out that a bridge

@@ -54,8 +54,9 @@ struct MqControl {
     uint32_t bcount[3];
     uint32_t lshift[MQ_SLOTS];          // rank bits of each slot's 32-bit labels
     unsigned long long slot_narrow;     // slots with a distance too large for their labels
-    // slots still in their first band (set at admission, cleared by the
-    // slot's first split): their heavy-arc pass may run in the pull form
+    // slots whose heavy-arc pass may yet run in the pull form: set at
+    // admission, cleared when the slot enters its tail (without the pull form
+    // by its first split)
     unsigned long long band0;
     // slots of band0 whose band holds most of the graph (their heavy-arc pass
     // takes the pull form), and those that asked before; sampled counts

@@ -50,7 +50,6 @@ struct SsspArgs {
     uint64_t *label;         // 64-bit labels (the wide kernel)
     uint32_t *label32;       // narrow labels (the narrow kernel)
     uint32_t lshift;         // rank bits of a narrow label
-    uint32_t ldmax;          // largest distance a narrow label holds
     uint32_t lstep;          // 1 << lshift: a narrow label's step per unit of distance
     uint64_t lmiss;          // sums of label and step at or above this do not fit
     uint32_t *stamp_near;
@@ -818,7 +817,7 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st, PullScratch
                         nl = (uint32_t)sum;
                         if (sum >= a.lmiss) {
                             // only an unreached vertex could take it (a narrow
-                            // label's distance is at most ldmax): the host
+                            // label holds no such distance): the host
                             // reruns the query with 64-bit labels
                             if (sc.best[slot[q]] == UNREACHED) narrow_miss = true;
                             continue;
@@ -894,7 +893,9 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st, PullScratch
 // ---------------------------------------------------------------------------
 
 // SCAN: splits scan the labels (a.far_scan), else there is a far pile.
-// BLOCKS per SM: three (80 registers), or two, where nothing is spilled.
+// BLOCKS per SM: three (80 registers, 298 to 378 bytes of spill stores), or two:
+// the far-pile forms then spill nothing, the label-scan forms 122 (narrow) and
+// 216 bytes.
 constexpr int SSSP_BLOCKS = 3;
 template <bool NARROW, bool SCAN, int BLOCKS>
 __global__ void __launch_bounds__(256, BLOCKS) sssp_kernel(const __grid_constant__ SsspArgs a) {
@@ -1268,8 +1269,9 @@ __global__ void __launch_bounds__(256, BLOCKS) sssp_kernel(const __grid_constant
             // Far pile, no light/heavy split: the next iteration splits the
             // pile as well (no iteration and barrier of its own) when the
             // frontier drained, and already when it is thin (a.thin): the
-            // grid's warps would idle through the last hops of every band.  Every block decides on near_count, which no
-            // iteration writes before all have read it.  A thin frontier
+            // grid's warps would idle through the last hops of every band.
+            // Every block decides on near_count, which no iteration writes
+            // before all have read it.  A thin frontier
             // always ends the phase (the threshold stays if the pile is
             // empty): an ended phase's pile takes no more pushes, so every
             // block reads the same count and minimum of it.
@@ -1589,9 +1591,8 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.label = ws.label;
     a.label32 = ws.label32;
     a.lshift = ws.lshift;
-    a.ldmax = (uint32_t)((1ull << (32 - ws.lshift)) - 2);
     a.lstep = 1u << ws.lshift;
-    a.lmiss = ((uint64_t)a.ldmax + 1) << ws.lshift;
+    a.lmiss = (1ull << 32) - a.lstep;        // distances up to 2^(32 - rank bits) - 2 fit
     a.stamp_near = ws.stamp_near;
     a.stamp_far = ws.stamp_far;
     a.q0 = ws.q[0];
@@ -1618,8 +1619,8 @@ cudaError_t launch_sssp(const DevGraph &g, Workspace &ws, const Geometry &geo,
     a.tail = p.tail;
     a.m = g.m;
     a.step0 = p.far_scan ? first_step(p.delta, g.delta0, g.max_w, g.even) : 0u;
-    // Three blocks per SM spill registers, two do not.  Two go faster through
-    // the chain of loads of a hop, three keep more arcs in flight.  Two, of
+    // Two blocks per SM spill little or nothing (see SSSP_BLOCKS) and go faster
+    // through the chain of loads of a hop, three keep more arcs in flight.  Two, of
     // three: R-MAT 12 0.224 ms of 0.257, 10^6 vertices (k = 101) 1.04 of 1.07,
     // R-MAT 22 (k = 64) 1.50 of 1.58; grid 1021 x 733 1.85 of 1.96, 2048 x 1900
     // 10.4 of 11.1.  Three, of two: R-MAT 24 5.6 ms of 6.2, R-MAT 26 (degree 8)
