@@ -49,7 +49,8 @@ GRID = 2                # the 4096^2 grid, 256 seeds
 TUNE_SALT = 0x7E57      # seed-set salt of the autotuner's held-out sample
 REF_BUDGET_S = 300.0    # reference arm: whole oracle queries within this time
 SSSP_SOURCES = ["paper_2205_14503_gb300/csrc/voronoi.cu", "paper_2205_14503_gb300/csrc/common.cuh",
-                "paper_2205_14503_gb300/csrc/internal.h"]
+                "paper_2205_14503_gb300/csrc/internal.h", "paper_2205_14503_gb300/csrc/items.h",
+                "paper_2205_14503_gb300/csrc/rules.h"]
 
 
 def _code_only(src: str) -> str:

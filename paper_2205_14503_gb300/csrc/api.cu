@@ -573,7 +573,7 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     G->g.n_live = n;
     if (relabel)
         G->g.n_live = (uint32_t)(std::lower_bound(irp, irp + n, (uint32_t)n_arcs) - irp);
-    G->g.even = even_rows(max_deg, n_arcs / std::max(G->g.n_live, 1u));
+    G->g.even = even_rows(max_deg, n_arcs, std::max(G->g.n_live, 1u));
     G->g.heavy_chunk_cap = (uint32_t)std::max<uint64_t>(cap, 1);
     if ((e = dalloc(G->g.row_ptr, (uint64_t)n + 1)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     if ((e = dalloc(G->g.adj, n_arcs)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
@@ -639,19 +639,19 @@ int steiner_load_graph(const uint32_t *row_ptr, const int32_t *col, const uint32
     int mst_sm = mst_occupancy(512);
     G->geo.mst_blocks = std::max(1, mst_sm) * G->geo.sm_count;
     {
-        std::vector<uint32_t> at[2];
+        std::vector<uint32_t> at[3];
         const uint64_t warps = (uint64_t)G->geo.sssp_max_blocks * (G->geo.threads / 32);
         if (!cut_items(irp, std::max(G->g.n_live, 1u), max_deg, warps, at))
             return bail(fail(STEINER_ENOMEM, "host allocation of the work items failed"));
-        G->g.n_items = (uint32_t)at[0].size() - 1;
-        G->g.n_sparse_items = (uint32_t)at[1].size() - 1;
-        e = dalloc(G->g.items, at[0].size());
-        if (e == cudaSuccess) e = dalloc(G->g.sparse_items, at[1].size());
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(G->g.items, at[0].data(), at[0].size() * 4, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(G->g.sparse_items, at[1].data(), at[1].size() * 4,
-                                cudaMemcpyHostToDevice, s);
+        uint32_t **list[3] = {&G->g.items, &G->g.sparse_items, &G->g.own_scan_items};
+        uint32_t *count[3] = {&G->g.n_items, &G->g.n_sparse_items, &G->g.n_own_scan_items};
+        for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
+            if (at[i].empty()) continue;
+            *count[i] = (uint32_t)at[i].size() - 1;
+            e = dalloc(*list[i], at[i].size());
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(*list[i], at[i].data(), at[i].size() * 4, cudaMemcpyHostToDevice, s);
+        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return bail(cuda_fail(e, "work items"));
     }
@@ -687,7 +687,7 @@ void steiner_free_graph(steiner_graph_t G) {
                     ws.e_key, ws.e_ra, ws.e_rb, ws.e_arc, ws.e_mst, ws.tile_off, ws.comp, ws.hook, ws.hub,
                     ws.best, ws.tree_key, ws.tree_key2, ws.tree_w, ws.tree_w2, G->g.row_ptr,
                     G->g.adj, G->g.heavy_chunks, G->g.orig_row_ptr, G->g.orig_of, G->g.new_of,
-                    G->g.adj_w, G->g.lend, G->g.items, G->g.sparse_items};
+                    G->g.adj_w, G->g.lend, G->g.items, G->g.sparse_items, G->g.own_scan_items};
     for (void *p : bufs)
         if (p) cudaFree(p);
     for (auto &ev : G->ev)

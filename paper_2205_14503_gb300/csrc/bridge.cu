@@ -572,9 +572,9 @@ cudaError_t launch_scan(const DevGraph &g, Workspace &ws, uint32_t k, bool pairs
     const uint64_t cap = (uint64_t)current_sm_count() * 32;
     // hub chunks in pieces while they leave most of the grid's warps idle
     a.subs = g.n_heavy_chunks * (uint64_t)SCAN_SUBS <= cap * 8 ? SCAN_SUBS : 1u;
-    a.items = g.items;
-    a.n_items = g.n_items;
-    uint64_t work = (uint64_t)g.n_heavy_chunks * a.subs + g.n_items;
+    a.items = g.scan_items();
+    a.n_items = g.n_scan_items();
+    uint64_t work = (uint64_t)g.n_heavy_chunks * a.subs + g.n_scan_items();
     uint64_t blocks = (work + 7) / 8;          // 8 warps per block
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
@@ -612,8 +612,8 @@ static TreeScanArgs tree_scan_args(const DevGraph &g, const Workspace &ws, uint3
     a.lend = g.lend;
     a.heavy_chunks = g.heavy_chunks;
     a.n_heavy_chunks = g.n_heavy_chunks;
-    a.items = g.items;
-    a.n_items = g.n_items;
+    a.items = g.scan_items();
+    a.n_items = g.n_scan_items();
     a.delta = delta;
     a.near = near_label(ws, delta);
     a.label32 = ws.label32;
@@ -659,7 +659,7 @@ bool pred_scan_applies(const DevGraph &g, const Workspace &ws, uint32_t delta) {
 cudaError_t launch_pred_scan(const DevGraph &g, Workspace &ws, uint32_t k, uint32_t delta,
                              cudaStream_t s) {
     const TreeScanArgs a = tree_scan_args(g, ws, k, delta);
-    const uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_items;
+    const uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_scan_items();
     const uint64_t blocks = std::min<uint64_t>((work + 7) / 8, (uint64_t)current_sm_count() * 32);
     tree_scan_kernel<false><<<(unsigned)std::max<uint64_t>(blocks, 1), 256, 0, s>>>(a);
     return cudaGetLastError();

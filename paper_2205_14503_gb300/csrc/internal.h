@@ -43,6 +43,10 @@ struct DevGraph {
     // vertices each; a sparse bitmap is read through the coarser list.
     uint32_t *items = nullptr, *sparse_items = nullptr;
     uint32_t n_items = 0, n_sparse_items = 0;
+    uint32_t *own_scan_items = nullptr;    // where the scans' ranges are others
+    uint32_t n_own_scan_items = 0;
+    const uint32_t *scan_items() const { return own_scan_items ? own_scan_items : items; }
+    uint32_t n_scan_items() const { return own_scan_items ? n_own_scan_items : n_items; }
     // Vertices with ids at or above n_big have fewer than HEAVY_DEG arcs
     // (the descending-degree order puts the hubs first; n without it).
     uint32_t n_big = 0;

@@ -32,26 +32,30 @@ constexpr uint64_t SPARSE_ITEM_FACTOR = 8;
 // the default band 1.61 -> 1.07.
 constexpr uint64_t EVEN_ITEMS = 4;
 
+// Arcs per row, rounded, at least one.
+inline uint64_t mean_row(uint64_t m, uint32_t n) { return std::max<uint64_t>((m + n / 2) / n, 1); }
 // Rows of about the same length: cut by vertices alone.
-inline bool even_rows(uint32_t max_deg, uint64_t mean_deg) { return max_deg <= 4 * mean_deg + 32; }
+inline bool even_rows(uint32_t max_deg, uint64_t m, uint32_t n) { return max_deg <= 4 * mean_row(m, n) + 32; }
 
 // Cuts the vertices into consecutive ranges of about equal arcs (a hub counts
 // HEAVY_DEG: longer rows are queued in chunks) and at most ITEM_SPAN vertices,
 // and into coarser ones for sparse bitmaps, for a grid of `warps` warps (three
 // blocks per SM); a single vertex may exceed the arc limit.  at[0] / at[1]
-// receive the range starts followed by n.  Even rows are cut into ranges of
+// receive the range starts followed by n, at[2] those of the scans, which run
+// eight blocks per SM and take the finer ranges everywhere (empty: at[0]; grid
+// 4096 x 4096, scan 0.355 ms in the ranges of the frontiers, 0.335).  Even rows are cut into ranges of
 // equal length; else blocks of CUT_BLOCK vertices are cut side by side on the
 // host's threads.  False: out of memory (nothing is thrown, on any thread).
 inline bool cut_items(const uint32_t *row_ptr, uint32_t n, uint32_t max_deg, uint64_t warps,
-                      std::vector<uint32_t> (&at)[2]) noexcept try {
+                      std::vector<uint32_t> (&at)[3]) noexcept try {
     constexpr uint32_t CUT_BLOCK = 1u << 17;
-    const uint64_t m = row_ptr[n], mean = std::max<uint64_t>(m / n, 1);
+    const uint64_t m = row_ptr[n], mean = mean_row(m, n);
     const uint64_t arcs = std::min(std::max(m / (16 * warps), ITEM_ARCS_MIN), ITEM_ARCS_MAX);
-    if (even_rows(max_deg, mean)) {
+    if (even_rows(max_deg, m, n)) {
         const uint64_t two = std::max<uint64_t>(warps * 2 / 3, 1);     // warps of the two-block form
-        const uint64_t span[2] = {std::max(arcs / mean, std::min(ITEM_ARCS_MAX / mean, n / (EVEN_ITEMS * two) + 1)),
-                                  std::max(SPARSE_ITEM_FACTOR * arcs / mean, n / two + 1)};
-        for (int i = 0; i < 2; ++i) {
+        const uint64_t span[3] = {std::max(arcs / mean, std::min(ITEM_ARCS_MAX / mean, n / (EVEN_ITEMS * two) + 1)),
+                                  std::max(SPARSE_ITEM_FACTOR * arcs / mean, n / two + 1), arcs / mean};
+        for (int i = 0; i < 3; ++i) {
             const uint32_t step = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(span[i], 1), ITEM_SPAN);
             at[i].reserve(n / step + 2);
             for (uint64_t v = 0; v < n; v += step) at[i].push_back((uint32_t)v);

@@ -1706,8 +1706,8 @@ cudaError_t mq_launch_scan(const DevGraph &g, MqState &m, unsigned long long slo
     a.adj = g.adj;
     a.heavy_chunks = g.heavy_chunks;
     a.n_heavy_chunks = g.n_heavy_chunks;
-    a.items = g.items;
-    a.n_items = g.n_items;
+    a.items = g.scan_items();
+    a.n_items = g.n_scan_items();
     a.n = g.n;
     a.label = m.label;
     a.lshift = m.ctl->lshift;
@@ -1718,7 +1718,7 @@ cudaError_t mq_launch_scan(const DevGraph &g, MqState &m, unsigned long long slo
     a.ctl = m.ctl;
     a.orig_of = g.orig_of;
     a.orig_row_ptr = g.orig_row_ptr;
-    uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_items;
+    uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_scan_items();
     uint64_t blocks = std::max<uint64_t>(1, std::min<uint64_t>((work + 7) / 8, (uint64_t)current_sm_count() * 32));
     mq_scan_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
     return cudaGetLastError();
@@ -1732,8 +1732,8 @@ static MqTreeArgs mq_tree_args(const DevGraph &g, MqState &m, unsigned long long
     a.lend = active_lend(g, delta);
     a.heavy_chunks = g.heavy_chunks;
     a.n_heavy_chunks = g.n_heavy_chunks;
-    a.items = g.items;
-    a.n_items = g.n_items;
+    a.items = g.scan_items();
+    a.n_items = g.n_scan_items();
     a.delta = delta;
     a.label = m.label;
     a.lshift = m.ctl->lshift;
@@ -1747,7 +1747,7 @@ static MqTreeArgs mq_tree_args(const DevGraph &g, MqState &m, unsigned long long
 }
 
 static unsigned mq_tree_blocks(const DevGraph &g) {
-    const uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_items;
+    const uint64_t work = (uint64_t)g.n_heavy_chunks + g.n_scan_items();
     return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((work + 7) / 8, (uint64_t)current_sm_count() * 32));
 }
 

@@ -39,13 +39,14 @@ int main(int, char **argv) {
     if (!f || fread(rp, 4, (size_t)n + 1, f) != (size_t)n + 1) return 3;
     fclose(f);
     for (long grant = atol(argv[5]), step = 0; step < (grant < 0 ? 1 : grant); ++step) {
-        std::vector<uint32_t> at[2];
+        std::vector<uint32_t> at[3];
         left = grant < 0 ? -1 : step;
         const bool ok = stn::cut_items(rp, n, max_deg, (uint64_t)atol(argv[4]), at);
         left = -1;
         if (grant >= 0) printf("%d", ok ? 1 : 0);
         else if (!ok) return 4;
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 3; ++i) {
+            if (ok && i == 2 && at[2].empty()) at[2] = at[0];
             if (ok && (at[i].empty() || at[i].front() != 0 || at[i].back() != n)) return 5;
             if (grant >= 0) continue;
             for (uint32_t v : at[i]) printf("%u ", v);
@@ -88,15 +89,15 @@ def test_items_cover_the_vertices(cut, kind, n):
     more arcs than the limit except in an item of one vertex."""
     deg = _degrees(kind, n)
     rp = np.concatenate([[0], np.cumsum(np.minimum(deg, 256))])
-    dense, sparse = cut(deg)
-    for at in (dense, sparse):
+    dense, sparse, scan = cut(deg)
+    for at in (dense, sparse, scan):
         assert at[0] == 0 and at[-1] == n
         span = np.diff(at)
         assert span.min() >= 1 and span.max() <= 992
-    assert len(sparse) <= len(dense)
+    assert len(sparse) <= len(dense) <= len(scan)
     if kind == "power" and deg.max() > 4 * max(1, deg.mean()) + 32:
         limit = min(max(int(deg.sum()) // (16 * 3648), 128), 4096)
-        for at, lim in ((dense, limit), (sparse, 8 * limit)):
+        for at, lim in ((dense, limit), (sparse, 8 * limit), (scan, limit)):
             arcs = rp[at[1:]] - rp[at[:-1]]
             assert np.all((arcs <= lim) | (np.diff(at) == 1))
 
@@ -107,8 +108,9 @@ def test_even_rows_have_few_items(cut, kind, n):
     """Even rows need no finer cut than the grid has warps: at most five items
     per warp of the two-block grid, and one for a sparse bitmap (an item costs
     a warp about 2 us whether or not it finds anything to relax)."""
-    dense, sparse = cut(_degrees(kind, n))
+    dense, sparse, scan = cut(_degrees(kind, n))
     assert len(dense) - 1 <= 5 * 2432 and len(sparse) - 1 <= 2432
+    assert len(scan) - 1 >= min(n // 50, 3 * 2432)       # the scans keep theirs
 
 
 @pytest.mark.parametrize("kind", ["grid", "power"])
