@@ -893,7 +893,7 @@ __device__ __noinline__ void pull_pass(const SsspArgs &a, Stage &st, PullScratch
 // ---------------------------------------------------------------------------
 
 // SCAN: splits scan the labels (a.far_scan), else there is a far pile.
-// BLOCKS per SM: three (80 registers, 298 to 378 bytes of spill stores), or two:
+// BLOCKS per SM: three (80 registers, 318 to 378 bytes of spill stores), or two:
 // the far-pile forms then spill nothing, the label-scan forms 122 (narrow) and
 // 216 bytes.
 constexpr int SSSP_BLOCKS = 3;
