@@ -382,9 +382,20 @@ static void *cc_unite(void *pp) {
     return NULL;
 }
 
+/* Each thread writes its own entries only, and nothing but roots: a find that
+ * halves paths could store an ancestor over an entry that its owner has
+ * flattened meanwhile. */
 static void *cc_flatten(void *pp) {
     cc_job_t *j = (cc_job_t *)pp;
-    for (uint32_t u = j->lo; u < j->hi; ++u) j->parent[u] = uf_find(j->parent, u);
+    for (uint32_t u = j->lo; u < j->hi; ++u) {
+        uint32_t x = u;
+        for (;;) {
+            uint32_t px = __atomic_load_n(&j->parent[x], __ATOMIC_RELAXED);
+            if (px == x) break;
+            x = px;
+        }
+        __atomic_store_n(&j->parent[u], x, __ATOMIC_RELAXED);
+    }
     return NULL;
 }
 

@@ -173,6 +173,7 @@ def test_noalloc_rows_that_end_at_the_last_arc_index(last):
     out = [torch.full((4,), -7, dtype=torch.int32, device="cuda") for _ in range(3)]
     rc = st.steiner_voronoi_noalloc(row_ptr, col, w, _dev(np.array([0], np.int32)), *out)
     del col, w
+    torch.cuda.empty_cache()
     assert rc == st.STEINER_OK, st.last_error()
     assert out[0].tolist() == [0, 0, -1, 0] and out[1].tolist() == [0, 12, -1, 5]
     assert out[2].tolist() == [0, 3, -1, 0 if last > 1 else -1]
